@@ -21,8 +21,7 @@
 // before and one after on a face volume's level 0, where the mass term of the
 // Helmholtz operator makes the smoothing strong enough that the second costs more
 // than the iterations it saves. The
-// coarsest level (small enough for shared memory) takes a fixed number of sweeps
-// in one block. Every step is linear in r with symmetric smoothing and restriction
+// coarsest level (small enough for shared memory) takes a fixed number of sweeps. Every step is linear in r with symmetric smoothing and restriction
 // proportional to the transposed prolongation, so M is symmetric, as CG needs.
 //
 // The sweeps, the residual and the transfers take four elements per thread and
@@ -76,41 +75,59 @@ struct MgLevel {
     float scale = 1.f;  // 4^-l times the operator's coefficient
     float mass = 0.f;   // identity term (1 for the Helmholtz operator)
     uint8_t *fl = nullptr;
-    float *r = nullptr, *a = nullptr, *b = nullptr, *c = nullptr;  // right-hand side and three work arrays
-    int *ql = nullptr;  // active quads (every level but the coarsest)
-    int nqa = 0;
-    int *pl = nullptr;  // active restriction pairs of this level as the coarse one (levels >= 1)
-    int npa = 0;
+    float *r = nullptr, *a = nullptr, *b = nullptr;  // levels >= 1 (of the set's arrays): right-hand side, result, field
 };
 
+// The levels of one volume (the cell space, or one face component).
 struct MgState {
     int nlev = 0;
     MgLevel lev[MG_MAX_LEVELS];
     long long epoch = -1;  // mask epoch the hierarchy was built for
     float coef = 0.f;      // operator coefficient it was built for
-    bool own0 = true;      // level 0 work arrays belong to this hierarchy
-    const int *done = nullptr;  // the calling solve's convergence flag (nullable)
-    int cl = 0;                 // first level of the single-cluster launch (0: none)
-    bool one0 = false;          // one smoothing sweep each side on level 0 (the face volumes)
-    // r.z in the last level-0 sweep of the current apply (rzs null: not formed)
-    SolveScal *rzs = nullptr;
-    int rz_first = 0, rz_boff = 0, rz_btot = 0;
-    int ctas = 0;               // CTAs of that cluster
-    long long calls = 0;        // applies so far (profiling samples every prof_period-th)
-    // algorithmic bytes of the level-0 kernels, in the order of K_MG0_SMOOTH2 ..
-    // K_MG0_SMOOTH_Z (profiled when the first is > 0)
-    double by0[6] = {0, 0, 0, 0, 0, 0};
+    int lb = 0;            // first level of the single-block launch
 };
 
-// The pressure hierarchy and one per face volume (viscosity). The face volumes
-// share two level-0 work arrays of face-space length, and their V-cycles are
-// independent: volumes 1 and 2 run on two side streams, forked from and joined
-// back to the context's stream.
+// The volumes of one level: each volume's grid and the first element of its array
+// in the level's arrays, which hold the volumes one after another.
+struct MgSpace {
+    MgGrid g[3];
+    int base[3];
+    int nv;
+};
+
+// Volumes whose V-cycles run together, launch by launch: the cell space alone, or
+// the three face components (one by one when one of them is its own coarsest
+// level). Level 0 lies in the arrays of the whole cell or face space; the arrays of
+// a level below belong to the set. The first levels take one launch per step over
+// lists: the active quads (those holding an unknown) and, below level 0, the active
+// restriction pairs, both counted in the level's arrays, volume after volume. The
+// levels from `lf` on take the tile kernels of fs_mg_coarse.cuh.
+struct MgSetLevel {
+    MgSpace sp;
+    uint8_t *fl = nullptr;
+    float *r = nullptr, *a = nullptr, *b = nullptr, *c = nullptr;
+    int *ql = nullptr, *pl = nullptr;
+    int nq = 0, np = 0;
+};
+struct MgSet {
+    int nv = 0, lf = 1;
+    MgState *s[3] = {nullptr, nullptr, nullptr};
+    MgSetLevel lev[MG_MAX_LEVELS];
+    uint8_t *blob = nullptr;  // flags and lists of the single-block levels, volume after volume
+    bool one = false;         // one smoothing sweep each side on level 0 (the face volumes)
+    long long calls = 0;      // applies so far (profiling samples every prof_period-th)
+    // algorithmic bytes of the level-0 kernels, in the order of K_MG0_SMOOTH2 ..
+    // K_MG0_SMOOTH_Z (counted when first profiled; negative before)
+    double by0[6] = {-1, 0, 0, 0, 0, 0};
+};
+
+// The pressure hierarchy and one per face volume (viscosity). The work arrays of
+// level 0 belong here: one pair of cell-space length, one of face-space length.
 struct MgAll {
     MgState cell, face[3];
-    float *fb = nullptr, *fc = nullptr;
-    cudaStream_t side[2] = {nullptr, nullptr};
-    cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
+    MgSet cset, fset[3];
+    int nfset = 0;
+    float *cb = nullptr, *cc = nullptr, *fb = nullptr, *fc = nullptr;
 };
 
 namespace {
@@ -171,37 +188,20 @@ __device__ __forceinline__ float sweep1(uint8_t f, float c, float nb, float rv, 
          mg_i < (na) && ((mg_next = mg_i + mg_st < (na) ? __ldg((list) + mg_i + mg_st) : 0), true);     \
          mg_i += mg_st, q = mg_next)
 
-// Vector loads of the item functions: through the non-coherent path for a launch
-// that does not write what it reads (CG = false), or at L2 (CG = true) for the
-// cluster launch, whose CTAs read what others wrote before a cluster barrier.
-template <bool CG>
-__device__ __forceinline__ float4 ldv4(const float *p, int t)
-{
-    if constexpr (CG)
-        return __ldcg(reinterpret_cast<const float4 *>(p + t));
-    else
-        return __ldg(reinterpret_cast<const float4 *>(p + t));
-}
-template <bool CG>
-__device__ __forceinline__ float ldv1(const float *p, int t)
-{
-    if constexpr (CG)
-        return __ldcg(p + t);
-    else
-        return __ldg(p + t);
-}
+// Vector loads through the non-coherent path: no launch writes what it reads.
+__device__ __forceinline__ float4 ldv4(const float *p, int t) { return __ldg(reinterpret_cast<const float4 *>(p + t)); }
+__device__ __forceinline__ float ldv1(const float *p, int t) { return __ldg(p + t); }
 
 // one damped Jacobi sweep on quad q: eout from ein; returns r.eout over the quad
-template <bool CG>
 __device__ __forceinline__ float smooth_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
                                           const float *ein, float *eout, const float *wt, float scale, float m, int q)
 {
     const int t = q << 2;
     const uchar4 f = ldf4(fl, t);
-    const float4 c = ldv4<CG>(ein, t), rv = ldv4<CG>(r, t);
-    const float4 dn = ldv4<CG>(ein, t - g.sy), up = ldv4<CG>(ein, t + g.sy);
-    const float4 bk = ldv4<CG>(ein, t - g.sz), fw = ldv4<CG>(ein, t + g.sz);
-    const float lf = ldv1<CG>(ein, t - 1), rt = ldv1<CG>(ein, t + 4);
+    const float4 c = ldv4(ein, t), rv = ldv4(r, t);
+    const float4 dn = ldv4(ein, t - g.sy), up = ldv4(ein, t + g.sy);
+    const float4 bk = ldv4(ein, t - g.sz), fw = ldv4(ein, t + g.sz);
+    const float lf = ldv1(ein, t - 1), rt = ldv1(ein, t + 4);
     float4 v;
     v.x = sweep1(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, wt, scale, m);
     v.y = sweep1(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, wt, scale, m);
@@ -212,16 +212,15 @@ __device__ __forceinline__ float smooth_q(const MgGrid &g, const uint8_t *__rest
 }
 
 // res = r - A e on quad q
-template <bool CG>
 __device__ __forceinline__ void resid_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
                                         const float *ev, float *res, float scale, float m, int q)
 {
     const int t = q << 2;
     const uchar4 f = ldf4(fl, t);
-    const float4 c = ldv4<CG>(ev, t), rv = ldv4<CG>(r, t);
-    const float4 dn = ldv4<CG>(ev, t - g.sy), up = ldv4<CG>(ev, t + g.sy);
-    const float4 bk = ldv4<CG>(ev, t - g.sz), fw = ldv4<CG>(ev, t + g.sz);
-    const float lf = ldv1<CG>(ev, t - 1), rt = ldv1<CG>(ev, t + 4);
+    const float4 c = ldv4(ev, t), rv = ldv4(r, t);
+    const float4 dn = ldv4(ev, t - g.sy), up = ldv4(ev, t + g.sy);
+    const float4 bk = ldv4(ev, t - g.sz), fw = ldv4(ev, t + g.sz);
+    const float lf = ldv1(ev, t - 1), rt = ldv1(ev, t + 4);
     auto one = [&](uint8_t fe, float ce, float nb, float re) {
         return liq(fe) ? re - m * ce - scale * ((float)(fe & CF_D) * ce - nb) : 0.f;
     };
@@ -234,7 +233,6 @@ __device__ __forceinline__ void resid_q(const MgGrid &g, const uint8_t *__restri
 }
 
 // the first two sweeps from e = 0 on quad q: e1 = omega D^-1 r on the fly, then one sweep
-template <bool CG>
 __device__ __forceinline__ void smooth2_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r, float *eo,
                                           const float *wt, float scale, float m, int q)
 {
@@ -242,15 +240,15 @@ __device__ __forceinline__ void smooth2_q(const MgGrid &g, const uint8_t *__rest
     const uchar4 f = ldf4(fl, t);
     auto e1q = [&](int u) {  // e1 on the quad at u
         const uchar4 fu = ldf4(fl, u);
-        const float4 ru = ldv4<CG>(r, u);
+        const float4 ru = ldv4(r, u);
         return make_float4(liq(fu.x) ? wt[fu.x & CF_D] * ru.x : 0.f, liq(fu.y) ? wt[fu.y & CF_D] * ru.y : 0.f,
                            liq(fu.z) ? wt[fu.z & CF_D] * ru.z : 0.f, liq(fu.w) ? wt[fu.w & CF_D] * ru.w : 0.f);
     };
     auto e1s = [&](int u) {
         const uint8_t fu = fl[u];
-        return liq(fu) ? wt[fu & CF_D] * ldv1<CG>(r, u) : 0.f;
+        return liq(fu) ? wt[fu & CF_D] * ldv1(r, u) : 0.f;
     };
-    const float4 c = e1q(t), rv = ldv4<CG>(r, t);
+    const float4 c = e1q(t), rv = ldv4(r, t);
     const float4 dn = e1q(t - g.sy), up = e1q(t + g.sy), bk = e1q(t - g.sz), fw = e1q(t + g.sz);
     const float lf = e1s(t - 1), rt = e1s(t + 4);
     float4 v;
@@ -265,7 +263,6 @@ __device__ __forceinline__ void smooth2_q(const MgGrid &g, const uint8_t *__rest
 // elements i .. i + 3 (i a multiple of 4) take their x samples from coarse
 // I0 - 1 .. I0 + 2 (I0 = i / 2); indices past the coarse halo are clamped to it
 // (a sample that only padding elements use).
-template <bool CG>
 __device__ __forceinline__ void prolong_q(const MgGrid &gf, const uint8_t *__restrict__ fl, float *ef,
                                           const MgGrid &gc, const float *ec, int q)
 {
@@ -286,14 +283,14 @@ __device__ __forceinline__ void prolong_q(const MgGrid &gf, const uint8_t *__res
         for (int a = 0; a < 2; a++) {
             const int base = gc.idx(0, jj[a], kk[b]);
             const float w = wy[a] * wy[b];
-            const float cm = ldv1<CG>(ec, base + xs[0]), c0 = ldv1<CG>(ec, base + xs[1]);
-            const float c1 = ldv1<CG>(ec, base + xs[2]), c2 = ldv1<CG>(ec, base + xs[3]);
+            const float cm = ldv1(ec, base + xs[0]), c0 = ldv1(ec, base + xs[1]);
+            const float c1 = ldv1(ec, base + xs[2]), c2 = ldv1(ec, base + xs[3]);
             s0 += w * (0.75f * c0 + 0.25f * cm);
             s1 += w * (0.75f * c0 + 0.25f * c1);
             s2 += w * (0.75f * c1 + 0.25f * c0);
             s3 += w * (0.75f * c1 + 0.25f * c2);
         }
-    float4 v = CG ? __ldcg(reinterpret_cast<const float4 *>(ef + t)) : *reinterpret_cast<const float4 *>(ef + t);
+    float4 v = *reinterpret_cast<const float4 *>(ef + t);
     if (liq(f.x)) v.x += s0;
     if (liq(f.y)) v.y += s1;
     if (liq(f.z)) v.z += s2;
@@ -306,7 +303,6 @@ __device__ __forceinline__ void prolong_q(const MgGrid &gf, const uint8_t *__res
 // row of the 4 x 4 window it reads the aligned quad 4m .. 4m + 3 and the scalars
 // at 4m - 1 and 4m + 4 (excluded at or past nx, where the next row begins), and
 // forms both cells' x weights from them.
-template <bool CG>
 __device__ __forceinline__ void restrict_pair(const MgGrid &gf, const float *res, const MgGrid &gc,
                                               const uint8_t *__restrict__ flc, float *rc, int t0)
 {
@@ -316,23 +312,25 @@ __device__ __forceinline__ void restrict_pair(const MgGrid &gf, const float *res
     const int m = I0 >> 1;
     const bool l0 = liq(flc[t0]), l1 = I0 + 1 < gc.nx && liq(flc[t0 + 1]);
     float a0 = 0.f, a1 = 0.f;
-    // unrolled, so the 16 row loads are issued together
+    // A row off the grid counts nothing: its weight is zero and the pair's own row
+    // is read in its place, so that no branch stands between the 16 rows' loads
+    // (with a skip per row each waited for the one before it: 12 us for the 64^3
+    // level of the three face volumes of 128^3, and the sweeps 4).
 #pragma unroll
     for (int c = 0; c < 4; c++) {
         const int k = 2 * K - 1 + c;
-        if (k < 0 || k >= gf.nz) continue;
+        const bool kin = k >= 0 && k < gf.nz;
 #pragma unroll
         for (int b = 0; b < 4; b++) {
             const int j = 2 * J - 1 + b;
-            if (j < 0 || j >= gf.ny) continue;
-            const int row = gf.idx(0, j, k) + 4 * m;  // a multiple of 4
-            const float4 qd = ldv4<CG>(res, row);
-            const float lf = m > 0 ? ldv1<CG>(res, row - 1) : 0.f;
-            const float rt = 4 * m + 4 < gf.nx ? ldv1<CG>(res, row + 4) : 0.f;
-            const float wyz = w[c] * w[b];
+            const bool in = kin && j >= 0 && j < gf.ny;
+            const int row = gf.idx(0, in ? j : 2 * J, in ? k : 2 * K) + 4 * m;  // a multiple of 4
+            const float4 qd = ldv4(res, row);
+            const float lf = ldv1(res, row - 1), rt = ldv1(res, row + 4);
+            const float wyz = in ? w[c] * w[b] : 0.f;
             // coarse 2m: fine 4m - 1 .. 4m + 2; coarse 2m + 1: fine 4m + 1 .. 4m + 4
-            a0 += wyz * (0.25f * lf + 0.75f * qd.x + 0.75f * qd.y + 0.25f * qd.z);
-            a1 += wyz * (0.25f * qd.y + 0.75f * qd.z + 0.75f * qd.w + 0.25f * rt);
+            a0 += wyz * (0.25f * (m > 0 ? lf : 0.f) + 0.75f * qd.x + 0.75f * qd.y + 0.25f * qd.z);
+            a1 += wyz * (0.25f * qd.y + 0.75f * qd.z + 0.75f * qd.w + 0.25f * (4 * m + 4 < gf.nx ? rt : 0.f));
         }
     }
     if (l0) rc[t0] = 0.125f * a0;
@@ -349,15 +347,15 @@ __device__ __forceinline__ void pre1_q(const MgGrid &g, const uint8_t *__restric
     const uchar4 f = ldf4(fl, t);
     auto e1q = [&](int u) {  // e1 on the quad at u
         const uchar4 fu = ldf4(fl, u);
-        const float4 ru = ldv4<false>(r, u);
+        const float4 ru = ldv4(r, u);
         return make_float4(liq(fu.x) ? wt[fu.x & CF_D] * ru.x : 0.f, liq(fu.y) ? wt[fu.y & CF_D] * ru.y : 0.f,
                            liq(fu.z) ? wt[fu.z & CF_D] * ru.z : 0.f, liq(fu.w) ? wt[fu.w & CF_D] * ru.w : 0.f);
     };
     auto e1s = [&](int u) {
         const uint8_t fu = fl[u];
-        return liq(fu) ? wt[fu & CF_D] * ldv1<false>(r, u) : 0.f;
+        return liq(fu) ? wt[fu & CF_D] * ldv1(r, u) : 0.f;
     };
-    const float4 c = e1q(t), rv = ldv4<false>(r, t);
+    const float4 c = e1q(t), rv = ldv4(r, t);
     const float4 dn = e1q(t - g.sy), up = e1q(t + g.sy), bk = e1q(t - g.sz), fw = e1q(t + g.sz);
     const float lf = e1s(t - 1), rt = e1s(t + 4);
     auto one = [&](uint8_t fe, float ce, float nb, float re) {
@@ -373,27 +371,33 @@ __device__ __forceinline__ void pre1_q(const MgGrid &g, const uint8_t *__restric
 }
 
 // ---- one launch per step ------------------------------------------------------
+// Each walks one list over every volume of a level.
+
+// the volume of an element of a level's arrays
+__device__ __forceinline__ int vol_of(const MgSpace &S, int t)
+{
+    return S.nv > 1 ? (t >= S.base[1]) + (t >= S.base[2]) : 0;
+}
 
 // One sweep over the active quads. With rzs (the last sweep of a V-cycle's level
 // 0), it also forms r.eout, which is the solver's r.z: each block's compensated
 // sum goes to the partials as block boff + blockIdx.x of btot (the blocks of the
 // face volumes' launches together), and the last block to arrive sets beta =
 // rz_new / rz (first: 0) and rz, as the solver's separate r.z pass does.
-__global__ void __launch_bounds__(256) k_mg0_smooth(MgGrid g, const int *__restrict__ qlist, int na,
+__global__ void __launch_bounds__(256) k_mg0_smooth(const MgSpace S, const int *__restrict__ qlist, int na,
                                                     const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                     const float *__restrict__ ein, float *eout, float scale, float m,
-                                                    const int *done, SolveScal *rzs, double *partials, int first,
-                                                    int boff, int btot)
+                                                    const int *done, SolveScal *rzs, double *partials, int first)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
     KSum acc;
-    MG_FOR_LIST(qlist, na) acc.add(smooth_q<false>(g, fl, r, ein, eout, wt, scale, m, q));
+    MG_FOR_LIST(qlist, na) acc.add(smooth_q(S.g[vol_of(S, 4 * q)], fl, r, ein, eout, wt, scale, m, q));
     if (!rzs || *(volatile const int *)&rzs->done) return;  // (a timed sweep runs after convergence too)
     KSum v[1] = {acc};
     double tot[1];
-    if (multi_reduce<1>(v, partials, &rzs->ticket, tot, boff + (int)blockIdx.x, btot) && threadIdx.x == 0) {
+    if (grid_reduce<1>(v, partials, &rzs->ticket, tot) && threadIdx.x == 0) {
         if (!isfinite(tot[0])) {
             rzs->done = 1;
             rzs->status = FS_ENONFINITE;
@@ -404,50 +408,58 @@ __global__ void __launch_bounds__(256) k_mg0_smooth(MgGrid g, const int *__restr
     }
 }
 
-__global__ void __launch_bounds__(256) k_mg0_pre1(MgGrid g, const int *__restrict__ qlist, int na,
+__global__ void __launch_bounds__(256) k_mg0_pre1(const MgSpace S, const int *__restrict__ qlist, int na,
                                                   const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                   float *eb, float *res, float scale, float m, const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
-    MG_FOR_LIST(qlist, na) pre1_q(g, fl, r, eb, res, wt, scale, m, q);
+    MG_FOR_LIST(qlist, na) pre1_q(S.g[vol_of(S, 4 * q)], fl, r, eb, res, wt, scale, m, q);
 }
 
-__global__ void __launch_bounds__(256, 8) k_mg0_residual(MgGrid g, const int *__restrict__ qlist, int na,
+__global__ void __launch_bounds__(256, 8) k_mg0_residual(const MgSpace S, const int *__restrict__ qlist, int na,
                                                       const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                       const float *__restrict__ ev, float *res, float scale, float m,
                                                       const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    MG_FOR_LIST(qlist, na) resid_q<false>(g, fl, r, ev, res, scale, m, q);
+    MG_FOR_LIST(qlist, na) resid_q(S.g[vol_of(S, 4 * q)], fl, r, ev, res, scale, m, q);
 }
 
-__global__ void __launch_bounds__(256) k_mg0_smooth2(MgGrid g, const int *__restrict__ qlist, int na,
+__global__ void __launch_bounds__(256) k_mg0_smooth2(const MgSpace S, const int *__restrict__ qlist, int na,
                                                      const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                      float *eo, float scale, float m, const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
-    MG_FOR_LIST(qlist, na) smooth2_q<false>(g, fl, r, eo, wt, scale, m, q);
+    MG_FOR_LIST(qlist, na) smooth2_q(S.g[vol_of(S, 4 * q)], fl, r, eo, wt, scale, m, q);
 }
 
-__global__ void __launch_bounds__(256) k_mg0_prolong(MgGrid gf, const int *__restrict__ qlist, int na,
-                                                     const uint8_t *__restrict__ fl, float *ef, MgGrid gc,
+__global__ void __launch_bounds__(256) k_mg0_prolong(const MgSpace S, const MgSpace Sc, const int *__restrict__ qlist,
+                                                     int na, const uint8_t *__restrict__ fl, float *ef,
                                                      const float *__restrict__ ec, const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    MG_FOR_LIST(qlist, na) prolong_q<false>(gf, fl, ef, gc, ec, q);
+    MG_FOR_LIST(qlist, na)
+    {
+        const int v = vol_of(S, 4 * q), base = S.base[v];
+        prolong_q(S.g[v], fl + base, ef + base, Sc.g[v], ec + Sc.base[v], q - (base >> 2));
+    }
 }
 
 // restriction over the coarse level's list of active pairs
-__global__ void __launch_bounds__(256) k_mg0_restrict(MgGrid gf, const float *__restrict__ res, MgGrid gc,
+__global__ void __launch_bounds__(256) k_mg0_restrict(const MgSpace S, const float *__restrict__ res, const MgSpace Sc,
                                                       const int *__restrict__ plist, int np,
                                                       const uint8_t *__restrict__ flc, float *rc, const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    MG_FOR_LIST(plist, np) restrict_pair<false>(gf, res, gc, flc, rc, q);
+    MG_FOR_LIST(plist, np)
+    {
+        const int v = vol_of(Sc, q), base = Sc.base[v];
+        restrict_pair(S.g[v], res + S.base[v], Sc.g[v], flc + base, rc + base, q - base);
+    }
 }
 
 // ---- lists of the active quads and restriction pairs ------------------------------
@@ -457,19 +469,21 @@ __global__ void __launch_bounds__(256) k_mg0_restrict(MgGrid gf, const float *__
 // at its offset.
 constexpr int LB_TH = 256, LB_PER = 4, LB_ITEMS = LB_TH * LB_PER;
 
-struct QuadPred {  // a quad of the level holds an unknown
+struct QuadPred {  // a quad of the volume holds an unknown; listed as a quad of the level's arrays
     MgGrid g;
     const uint8_t *fl;
+    int base;
     __device__ long long items() const { return g.n >> 2; }
     __device__ bool keep(long long q, int &out) const
     {
-        out = (int)q;
+        out = (base >> 2) + (int)q;
         return any_liq(ldf4(fl, (int)q << 2));
     }
 };
-struct PairPred {  // a restriction pair (2m, 2m + 1) of the coarse level holds an unknown
+struct PairPred {  // a restriction pair (2m, 2m + 1) of the coarse level holds an unknown; its first element
     MgGrid g;
     const uint8_t *fl;
+    int base;
     __device__ long long items() const { return (long long)((g.nx + 1) >> 1) * g.ny * g.nz; }
     __device__ bool keep(long long it, int &out) const
     {
@@ -477,8 +491,9 @@ struct PairPred {  // a restriction pair (2m, 2m + 1) of the coarse level holds 
         const int m = (int)(it % npair);
         const long long jk = it / npair;
         const int J = (int)(jk % g.ny), K = (int)(jk / g.ny);
-        out = g.idx(2 * m, J, K);
-        return liq(fl[out]) || (2 * m + 1 < g.nx && liq(fl[out + 1]));
+        const int t = g.idx(2 * m, J, K);
+        out = base + t;
+        return liq(fl[t]) || (2 * m + 1 < g.nx && liq(fl[t + 1]));
     }
 };
 
@@ -565,156 +580,21 @@ __global__ void k_mg_count(MgGrid g, uint8_t *fl)
     }
 }
 
-// The coarsest level: MG_COARSE_SWEEPS damped Jacobi sweeps from zero in the
-// shared memory `sm` of one block (13 bytes per element), the result written to
-// e on every element; wt is the level's weight table. Each sweep reads only the
-// previous one, so the result does not depend on the block size.
-template <bool CG>
-__device__ void coarse_block(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r, float *e,
-                             const float *wt, float scale, float m, float *sm)
-{
-    float *e0 = sm, *e1 = sm + g.n, *rs = sm + 2 * g.n;
-    uint8_t *fs = reinterpret_cast<uint8_t *>(sm + 3 * g.n);
-    for (int t = threadIdx.x; t < g.n; t += blockDim.x) {
-        const uint8_t f = fl[t];
-        const float rv = ldv1<CG>(r, t);
-        fs[t] = f;
-        rs[t] = liq(f) ? rv : 0.f;
-        e0[t] = liq(f) ? wt[f & CF_D] * rv : 0.f;
-        e1[t] = 0.f;
-    }
-    __syncthreads();
-    for (int s = 1; s < MG_COARSE_SWEEPS; s++) {
-        const float *ein = (s & 1) ? e0 : e1;
-        float *eout = (s & 1) ? e1 : e0;
-        for (int t = threadIdx.x; t < g.n; t += blockDim.x) {
-            const uint8_t f = fs[t];
-            eout[t] = liq(f) ? ein[t] + wt[f & CF_D] * (rs[t] - m * ein[t] - scale * lap(ein, t, f, g)) : 0.f;
-        }
-        __syncthreads();
-    }
-    const float *res = (MG_COARSE_SWEEPS & 1) ? e0 : e1;  // the last sweep's output
-    for (int t = threadIdx.x; t < g.n; t += blockDim.x) e[t] = res[t];
-}
+#include "fs_mg_coarse.cuh"
 
-constexpr int COARSE_TH = 1024;  // threads of the block that solves the coarsest level
-
-__global__ void __launch_bounds__(COARSE_TH) k_mg_coarse(MgGrid g, const uint8_t *__restrict__ fl,
-                                                         const float *__restrict__ r, float *e, float scale, float m,
-                                                         const int *done)
-{
-    if (done && *(volatile const int *)done) return;  // the solve has converged
-    extern __shared__ float sm[];
-    __shared__ float wt[8];
-    fill_wtab(wt, scale, m);
-    coarse_block<false>(g, fl, r, e, wt, scale, m, sm);
-}
-
-// ---- the small levels in one cluster -------------------------------------------
-// The levels whose active quads number at most MGC_MAX_QUADS take one launch of a
-// single thread-block cluster (MGC_CTAS CTAs of MGC_TH threads): the same steps as
-// the per-level kernels, level by level, with the cluster's hardware barrier in
-// place of each kernel boundary. What one CTA writes another reads after the
-// barrier (release, then acquire at cluster scope), through L2 (ld.global.cg:
-// no SM's L1 can hold a stale copy). CTA 0 solves the coarsest level.
-constexpr int MGC_TH = 1024;
-constexpr int MGC_MAXLEV = 8;
-constexpr int MGC_MAX_QUADS = 49152;
-
-struct MgcLevel {
-    MgGrid g;
-    const uint8_t *fl;
-    float *r, *a, *b, *c;
-    const int *ql, *pl;
-    int nqa, npa;
-    float scale, mass;
-};
-
-struct MgClusterArgs {
-    MgcLevel lev[MGC_MAXLEV];
-    int nlev;
-    const int *done;
-};
-
-__device__ __forceinline__ void cluster_barrier()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ int cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return (int)r;
-}
-__device__ __forceinline__ int cluster_ctas()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return (int)r;
-}
-
-// The V-cycle on a.lev[0] .. a.lev[nlev - 1]: r in lev[0].r, result in lev[0].a.
-__global__ void __launch_bounds__(MGC_TH) k_mg_cluster(const MgClusterArgs a)
-{
-    if (a.done && *(volatile const int *)a.done) return;  // the solve has converged (every CTA alike)
-    extern __shared__ float sm[];
-    __shared__ float wts[MGC_MAXLEV][8];
-    for (int i = threadIdx.x; i < MGC_MAXLEV * 8; i += blockDim.x)
-        if (i / 8 < a.nlev) wts[i / 8][i % 8] = wtab_entry(a.lev[i / 8].scale, a.lev[i / 8].mass, i % 8);
-    __syncthreads();
-    const int tid = cluster_rank() * blockDim.x + threadIdx.x, st = cluster_ctas() * blockDim.x;
-    for (int l = 0; l + 1 < a.nlev; l++) {
-        const MgcLevel &L = a.lev[l], &W = a.lev[l + 1];
-        for (int i = tid; i < L.nqa; i += st)
-            smooth2_q<true>(L.g, L.fl, L.r, L.b, wts[l], L.scale, L.mass, __ldg(L.ql + i));
-        cluster_barrier();
-        for (int i = tid; i < L.nqa; i += st) resid_q<true>(L.g, L.fl, L.r, L.b, L.c, L.scale, L.mass, __ldg(L.ql + i));
-        cluster_barrier();
-        for (int i = tid; i < W.npa; i += st) restrict_pair<true>(L.g, L.c, W.g, W.fl, W.r, __ldg(W.pl + i));
-        cluster_barrier();
-    }
-    if (cluster_rank() == 0) {
-        const MgcLevel &L = a.lev[a.nlev - 1];
-        coarse_block<true>(L.g, L.fl, L.r, L.a, wts[a.nlev - 1], L.scale, L.mass, sm);
-    }
-    cluster_barrier();
-    for (int l = a.nlev - 2; l >= 0; l--) {
-        const MgcLevel &L = a.lev[l], &W = a.lev[l + 1];
-        for (int i = tid; i < L.nqa; i += st) prolong_q<true>(L.g, L.fl, L.b, W.g, W.a, __ldg(L.ql + i));
-        cluster_barrier();
-        for (int i = tid; i < L.nqa; i += st)
-            smooth_q<true>(L.g, L.fl, L.r, L.b, L.c, wts[l], L.scale, L.mass, __ldg(L.ql + i));
-        cluster_barrier();
-        for (int i = tid; i < L.nqa; i += st)
-            smooth_q<true>(L.g, L.fl, L.r, L.c, L.a, wts[l], L.scale, L.mass, __ldg(L.ql + i));
-        if (l > 0) cluster_barrier();
-    }
-}
-
-// r.z over the active quads of one or three level-0 lists (r is zero off the
-// unknowns, so no other quad adds to it), in the lists' fixed order: beta =
-// rz_new / rz (first: beta = 0), as the dense pass of the solver does.
-struct RzLists {
-    const int *ql[3];
-    int n[3];
-    long long base[3];
-    int nv;
-};
-
-__global__ void __launch_bounds__(TH) k_mg_rz(RzLists L, const float *__restrict__ r, const float *__restrict__ z,
-                                             int first, SolveScal *s, double *partials)
+// r.z over the active quads of a set's level 0 (r is zero off the unknowns, so no
+// other quad adds to it), in the list's order: beta = rz_new / rz (first: beta =
+// 0), as the dense pass of the solver does.
+__global__ void __launch_bounds__(TH) k_mg_rz(const int *__restrict__ qlist, int na, const float *__restrict__ r,
+                                             const float *__restrict__ z, int first, SolveScal *s, double *partials)
 {
     if (s->done) return;
     KSum acc;
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x, st = gridDim.x * blockDim.x;
-    for (int v = 0; v < L.nv; v++) {
-        const float4 *r4 = reinterpret_cast<const float4 *>(r + L.base[v]);
-        const float4 *z4 = reinterpret_cast<const float4 *>(z + L.base[v]);
-        for (int i = tid; i < L.n[v]; i += st) {
-            const int q = __ldg(L.ql[v] + i);
-            const float4 a = __ldg(r4 + q), b = __ldg(z4 + q);
-            acc.add(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
-        }
+    const float4 *r4 = reinterpret_cast<const float4 *>(r), *z4 = reinterpret_cast<const float4 *>(z);
+    MG_FOR_LIST(qlist, na)
+    {
+        const float4 a = __ldg(r4 + q), b = __ldg(z4 + q);
+        acc.add(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
     }
     KSum v[1] = {acc};
     double tot[1];
@@ -737,8 +617,6 @@ __global__ void k_mg_count_liq(MgGrid g, const uint8_t *__restrict__ fl, unsigne
     for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
     if ((threadIdx.x & 31) == 0 && k) atomicAdd(out, k);
 }
-
-size_t coarse_smem(const MgGrid &g) { return (size_t)g.n * 13 + 16; }
 
 int row_blocks(fs_ctx *c, const MgGrid &g) { return grid_blocks(c, g.rows, 8); }
 
@@ -784,95 +662,24 @@ MgGrid coarse_grid(int nx, int ny, int nz)
     return g;
 }
 
-void free_levels(MgState *s)
+void free_set(MgSet *t)
 {
-    for (int l = 0; l < s->nlev; l++) {
-        cudaFree(s->lev[l].ql);
-        cudaFree(s->lev[l].pl);
-        s->lev[l].ql = s->lev[l].pl = nullptr;
-        s->lev[l].nqa = s->lev[l].npa = 0;
-    }
-    for (int l = 1; l < s->nlev; l++) {
-        MgLevel &v = s->lev[l];
-        cudaFree(v.fl);
-        cudaFree(v.r);
-        cudaFree(v.a);
-        cudaFree(v.b);
-        cudaFree(v.c);
-        v = MgLevel();
-    }
-    if (s->own0) {
-        cudaFree(s->lev[0].b);
-        cudaFree(s->lev[0].c);
-    }
-    s->lev[0] = MgLevel();
-    s->nlev = 0;
-    s->epoch = -1;
-}
-
-// The V-cycle on level l: r in lev[l].r, result in lev[l].a. With `sample`, the
-// last level-0 sweep is timed.
-// The V-cycle on level l: r in lev[l].r, result in lev[l].a. With `sample`
-// (level 0 of a pressure V-cycle on the context's stream), every level-0 kernel
-// and the coarse levels as a whole are timed; a timed kernel always runs in full
-// (an early exit would record work not done).
-// levels cl .. nlev - 1 of a hierarchy in one cluster launch
-int launch_cluster(fs_ctx *c, MgState *s, int cl, cudaStream_t st)
-{
-    MgClusterArgs a;
-    std::memset(&a, 0, sizeof(a));
-    a.nlev = s->nlev - cl;
-    for (int l = cl; l < s->nlev; l++) {
-        const MgLevel &v = s->lev[l];
-        a.lev[l - cl] = MgcLevel{v.g, v.fl, v.r, v.a, v.b, v.c, v.ql, v.pl, v.nqa, v.npa, v.scale, v.mass};
-    }
-    a.done = s->done;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(s->ctas);
-    cfg.blockDim = dim3(MGC_TH);
-    cfg.dynamicSmemBytes = coarse_smem(s->lev[s->nlev - 1].g);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = s->ctas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    FS_CUDA(cudaLaunchKernelEx(&cfg, k_mg_cluster, a));
-    c->n_launches += 1;
-    return FS_OK;
-}
-
-// CTAs of the single-cluster launch on this device: 16 where the device allows
-// that non-portable size, else 8, else 0 (no cluster launch)
-int cluster_ctas_here()
-{
-    static int cached = -1;
-    if (cached >= 0) return cached;
-    cached = 0;
-    if (cudaFuncSetAttribute(k_mg_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        cudaGetLastError();
-    for (int n : {16, 8}) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(n);
-        cfg.blockDim = dim3(MGC_TH);
-        cfg.dynamicSmemBytes = (size_t)MG_COARSE_CELLS * 13 + 16;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = n;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, k_mg_cluster, &cfg) == cudaSuccess && clusters > 0) {
-            cached = n;
-            break;
+    for (int l = 0; l < MG_MAX_LEVELS; l++) {
+        MgSetLevel &v = t->lev[l];
+        cudaFree(v.ql);
+        cudaFree(v.pl);
+        if (l > 0) {  // level 0 lies in the context's arrays and in MgAll's
+            cudaFree(v.fl);
+            for (float *p : {v.r, v.a, v.b, v.c}) cudaFree(p);
         }
-        cudaGetLastError();
+        v = MgSetLevel();
     }
-    return cached;
+    cudaFree(t->blob);
+    t->blob = nullptr;
+    for (MgState *s : t->s)
+        if (s) *s = MgState();
+    t->nv = 0;
+    t->by0[0] = -1.0;
 }
 
 // Resident blocks per SM of the list-walking kernels, for one-wave grids.
@@ -890,127 +697,215 @@ const MgResidency &mg_residency()
     return r;
 }
 
-// blocks of the sweeps k_mg0_smooth over a level's nqa active quads (also the
-// block count of the r.z reduction the last level-0 sweep forms)
-int smooth_blocks(const fs_ctx *c, int nqa) { return wave_blocks(c, nqa, mg_residency().smooth); }
+MgcLevel coarse_level(const MgLevel &v) { return MgcLevel{v.g, v.fl, v.r, v.a, v.b, v.scale, v.mass}; }
 
-int vcycle(fs_ctx *c, MgState *s, int l, bool sample, cudaStream_t st)
+// One leg (down or up) of level l >= 1 for the volumes of the set that hold it
+// above their single-block levels.
+int launch_leg(fs_ctx *c, const MgSet &t, int l, bool down, const int *done)
 {
-    if (s->cl > 0 && l == s->cl) return launch_cluster(c, s, l, st);
-    MgLevel &v = s->lev[l];
-    const MgGrid &g = v.g;
-    if (l == s->nlev - 1) {
-        k_mg_coarse<<<1, COARSE_TH, coarse_smem(g), st>>>(g, v.fl, v.r, v.a, v.scale, v.mass, s->done);
-        c->n_launches += 1;
-        return FS_OK;
+    MgLegArgs a;
+    std::memset((void *)&a, 0, sizeof(a));
+    a.done = done;
+    int nv = 0, tiles = 0;
+    size_t sm = 0;
+    for (int v = 0; v < t.nv; v++) {
+        const MgState &s = *t.s[v];
+        if (l >= s.lb) continue;
+        MgLegVol &x = a.v[nv++];
+        x.f = coarse_level(s.lev[l]);
+        x.c = coarse_level(s.lev[l + 1]);
     }
-    const bool timed = sample && l == 0 && s->by0[0] > 0.0;
-    const int *done = timed ? nullptr : s->done;
+    for (int v = 0; v < nv; v++) {
+        MgLegVol &x = a.v[v];
+        x.t = make_tiles(x.f.g, nv, c->num_sms);
+        tiles = std::max(tiles, x.t.ntx * x.t.nty * x.t.ntz);
+        sm = std::max(sm, leg_smem(x.t, down));
+    }
+    if (!nv) return FS_OK;
+    if (down)
+        k_mg_down<<<dim3(tiles, nv), MGT_TH, sm, c->stream>>>(a);
+    else
+        k_mg_up<<<dim3(tiles, nv), MGT_TH, sm, c->stream>>>(a);
+    c->n_launches += 1;
+    return FS_OK;
+}
+
+// The arguments of the single-block levels lb .. nlev - 1 of every volume of the
+// set (level 0's right-hand side and result left out), and their shared memory.
+size_t bottom_args(const MgSet &t, MgBottomArgs &a)
+{
+    std::memset((void *)&a, 0, sizeof(a));
+    size_t sm = 0, blob = 0;
+    for (int v = 0; v < t.nv; v++) {
+        const MgState &s = *t.s[v];
+        MgBottomVol &x = a.v[v];
+        x.nlev = s.nlev - s.lb;
+        size_t off = 0, n = 0;
+        for (int l = s.lb; l < s.nlev; l++) n += (size_t)s.lev[l].g.n;
+        size_t foff = MGB_HEAD, qoff = foff + n;
+        for (int l = s.lb; l < s.nlev; l++) {
+            MgBottomLevel &b = x.lev[l - s.lb];
+            b.l = coarse_level(s.lev[l]);
+            b.off = (int)off;
+            b.foff = (int)foff;
+            b.qoff = (int)qoff;
+            b.dsy = FastDiv(b.l.g.sy);
+            b.dsz = FastDiv(b.l.g.sz);
+            off += 3 * (size_t)b.l.g.n;
+            foff += (size_t)b.l.g.n;
+            qoff += (size_t)b.l.g.n / 2;
+        }
+        x.n = (int)n;
+        x.bytes = (int)bottom_blob(n);
+        x.blob = t.blob ? t.blob + blob : nullptr;
+        blob += (size_t)x.bytes;
+        sm = std::max(sm, bottom_smem(n));
+    }
+    return sm;
+}
+
+// One block for each volume's single-block levels. For a volume whose level 0 is
+// its coarsest one, r0 and z0 are that level's arrays.
+int launch_bottom(fs_ctx *c, const MgSet &t, const float *r0, float *z0, const int *done)
+{
+    MgBottomArgs a;
+    const size_t sm = bottom_args(t, a);
+    a.done = done;
+    for (int v = 0; v < t.nv; v++)
+        if (t.s[v]->lb == 0) {
+            a.v[v].lev[0].l.r = const_cast<float *>(r0) + t.lev[0].sp.base[v];
+            a.v[v].lev[0].l.a = z0 + t.lev[0].sp.base[v];
+        }
+    k_mg_bottom<<<t.nv, MGB_TH, sm, c->stream>>>(a);
+    c->n_launches += 1;
+    return FS_OK;
+}
+
+// unknowns of levels 0 and 1, for the profiled byte counts: the least each level-0
+// kernel must move is the list entry and the flags of each active quad (or pair)
+// it visits and 4 bytes per unknown for each vector it reads or writes there
+int count_bytes(fs_ctx *c, MgSet &t)
+{
+    unsigned long long *cnt = reinterpret_cast<unsigned long long *>(c->partials), nl[2] = {0, 0};
+    FS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(nl), c->stream));
+    for (int v = 0; v < t.nv; v++) {
+        const MgState &s = *t.s[v];
+        k_mg_count_liq<<<grid_blocks(c, s.lev[0].g.n, TH), TH, 0, c->stream>>>(s.lev[0].g, s.lev[0].fl, cnt);
+        if (s.nlev > 1)
+            k_mg_count_liq<<<grid_blocks(c, s.lev[1].g.n, TH), TH, 0, c->stream>>>(s.lev[1].g, s.lev[1].fl, cnt + 1);
+    }
+    FS_CUDA(cudaMemcpyAsync(nl, cnt, sizeof(nl), cudaMemcpyDeviceToHost, c->stream));
+    FS_CUDA(cudaStreamSynchronize(c->stream));
+    const double u0 = (double)nl[0], u1 = (double)nl[1], q0 = (double)t.lev[0].nq, p1 = (double)t.lev[1].np;
+    t.by0[0] = 8.0 * q0 + 8.0 * u0;             // smooth2: read r, write e
+    t.by0[1] = 8.0 * q0 + 12.0 * u0;            // residual: read r, e, write res
+    t.by0[2] = 6.0 * p1 + 4.0 * u0 + 4.0 * u1;  // restrict: pair list and flags, read res, write level-1 r
+    t.by0[3] = 8.0 * q0 + 8.0 * u0 + 4.0 * u1;  // prolong: read and write e, read the level-1 e
+    t.by0[4] = 8.0 * q0 + 12.0 * u0;            // smooth: read r, e, write e
+    t.by0[5] = 8.0 * q0 + 12.0 * u0;            // last smooth: read r, e, write z
+    return FS_OK;
+}
+
+// One V-cycle of a set: z = M r (whole-space arrays). With `sample` (the pressure
+// V-cycle), every level-0 kernel and the coarse levels as a whole are timed; a
+// timed kernel always runs in full (an early exit would record work not done).
+// With rzs, r.z of the solver is formed in the last level-0 sweep.
+int vcycle(fs_ctx *c, MgSet &t, const float *r, float *z, const int *done_, bool sample, SolveScal *rzs, int first)
+{
+    const MgState &s0 = *t.s[0];
+    if (s0.nlev == 1) return launch_bottom(c, t, r, z, done_);
+    if (sample && t.by0[0] < 0.0)
+        if (int rc = count_bytes(c, t)) return rc;
     // an event pair around each timed launch (an event belongs to one pair)
     cudaEvent_t e0 = nullptr;
-    auto begin = [&]() {
-        if (timed) e0 = prof_mark(c);
+    auto begin = [&](int l) {
+        if (sample && l == 0) e0 = prof_mark(c);
     };
-    auto end = [&](int kind, double bytes) {
-        if (timed) prof_add(c, kind, e0, prof_mark(c), bytes);
+    auto end = [&](int l, int kind, double bytes) {
+        if (sample && l == 0) prof_add(c, kind, e0, prof_mark(c), bytes);
     };
-    // four elements per thread: every level but the coarsest has quad-aligned rows;
-    // each kernel over the active quads in one wave of its resident blocks
+    // four elements per thread, each kernel over the active quads in one wave of
+    // its resident blocks (the volumes of a set share their scale)
     const MgResidency &res = mg_residency();
-    const int nb = smooth_blocks(c, v.nqa);
-    MgLevel &w = s->lev[l + 1];
-    // one sweep each side on level 0 of a face volume (the viscosity solve), two
-    // elsewhere
-    const bool one = l == 0 && s->one0;
-    if (one) {  // the sweep from zero and the residual it leaves, in one pass
-        k_mg0_pre1<<<wave_blocks(c, v.nqa, res.pre1), TH, 0, st>>>(g, v.ql, v.nqa, v.fl, v.r, v.b, v.c, v.scale, v.mass, done);
+    cudaStream_t st = c->stream;
+    for (int l = 0; l < t.lf; l++) {
+        MgSetLevel &v = t.lev[l], &w = t.lev[l + 1];
+        const float *rl = l == 0 ? r : v.r, scale = s0.lev[l].scale, mass = s0.lev[l].mass;
+        const int *done = sample && l == 0 ? nullptr : done_;
+        if (l == 0 && t.one) {  // the sweep from zero and the residual it leaves, in one pass
+            k_mg0_pre1<<<wave_blocks(c, v.nq, res.pre1), TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass,
+                                                                      done);
+            c->n_launches += 1;
+        } else {
+            begin(l);
+            k_mg0_smooth2<<<wave_blocks(c, v.nq, res.smooth2), TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, scale,
+                                                                            mass, done);
+            end(l, K_MG0_SMOOTH2, t.by0[0]);
+            begin(l);
+            k_mg0_residual<<<wave_blocks(c, v.nq, res.residual), TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c,
+                                                                              scale, mass, done);
+            end(l, K_MG0_RESIDUAL, t.by0[1]);
+            c->n_launches += 2;
+        }
+        begin(l);
+        k_mg0_restrict<<<wave_blocks(c, w.np, res.restrict_), TH, 0, st>>>(v.sp, v.c, w.sp, w.pl, w.np, w.fl, w.r,
+                                                                           done);
+        end(l, K_MG0_RESTRICT, t.by0[2]);
         c->n_launches += 1;
-    } else {
-        begin();
-        k_mg0_smooth2<<<wave_blocks(c, v.nqa, res.smooth2), TH, 0, st>>>(g, v.ql, v.nqa, v.fl, v.r, v.b, v.scale, v.mass, done);
-        end(K_MG0_SMOOTH2, s->by0[0]);
-        begin();
-        k_mg0_residual<<<wave_blocks(c, v.nqa, res.residual), TH, 0, st>>>(g, v.ql, v.nqa, v.fl, v.r, v.b, v.c, v.scale, v.mass, done);
-        end(K_MG0_RESIDUAL, s->by0[1]);
+        begin(l);
+    }
+    int lb = 0;
+    for (int v = 0; v < t.nv; v++) lb = std::max(lb, t.s[v]->lb);
+    for (int l = t.lf; l < lb; l++)
+        if (int rc = launch_leg(c, t, l, true, done_)) return rc;
+    if (int rc = launch_bottom(c, t, r, z, done_)) return rc;
+    for (int l = lb - 1; l >= t.lf; l--)
+        if (int rc = launch_leg(c, t, l, false, done_)) return rc;
+    for (int l = t.lf - 1; l >= 0; l--) {
+        MgSetLevel &v = t.lev[l], &w = t.lev[l + 1];
+        const float *rl = l == 0 ? r : v.r, scale = s0.lev[l].scale, mass = s0.lev[l].mass;
+        const int *done = sample && l == 0 ? nullptr : done_;
+        const int nb = wave_blocks(c, v.nq, res.smooth);
+        end(l, K_MG_COARSE, 0.0);
+        begin(l);
+        k_mg0_prolong<<<wave_blocks(c, v.nq, res.prolong), TH, 0, st>>>(v.sp, w.sp, v.ql, v.nq, v.fl, v.b, w.a, done);
+        end(l, K_MG0_PROLONG, t.by0[3]);
+        const float *ez = v.c;  // the input of the last sweep
+        if (l == 0 && t.one) {
+            ez = v.b;
+        } else {
+            begin(l);
+            k_mg0_smooth<<<nb, TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass, done, nullptr, nullptr,
+                                            0);
+            end(l, K_MG0_SMOOTH, t.by0[4]);
+            c->n_launches += 1;
+        }
+        begin(l);
+        k_mg0_smooth<<<nb, TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, ez, l == 0 ? z : v.a, scale, mass, done,
+                                        l == 0 ? rzs : nullptr, c->partials, first);
+        end(l, K_MG0_SMOOTH_Z, t.by0[5]);
         c->n_launches += 2;
     }
-    begin();
-    k_mg0_restrict<<<wave_blocks(c, w.npa, res.restrict_), TH, 0, st>>>(g, v.c, w.g, w.pl, w.npa, w.fl, w.r, done);
-    end(K_MG0_RESTRICT, s->by0[2]);
-    c->n_launches += 1;
-    begin();
-    if (int rc = vcycle(c, s, l + 1, false, st)) return rc;
-    end(K_MG_COARSE, 0.0);
-    begin();
-    k_mg0_prolong<<<wave_blocks(c, v.nqa, res.prolong), TH, 0, st>>>(g, v.ql, v.nqa, v.fl, v.b, w.g, w.a, done);
-    end(K_MG0_PROLONG, s->by0[3]);
-    SolveScal *rzs = l == 0 ? s->rzs : nullptr;  // r.z of the solver in the last level-0 sweep
-    const float *ez = v.c;                        // the input of the last sweep
-    if (one) {
-        ez = v.b;
-    } else {
-        begin();
-        k_mg0_smooth<<<nb, TH, 0, st>>>(g, v.ql, v.nqa, v.fl, v.r, v.b, v.c, v.scale, v.mass, done, nullptr,
-                                        nullptr, 0, 0, 0);
-        end(K_MG0_SMOOTH, s->by0[4]);
-        c->n_launches += 1;
-    }
-    begin();
-    k_mg0_smooth<<<nb, TH, 0, st>>>(g, v.ql, v.nqa, v.fl, v.r, ez, v.a, v.scale, v.mass, done, rzs, c->partials,
-                                    s->rz_first, s->rz_boff, s->rz_btot);
-    end(K_MG0_SMOOTH_Z, s->by0[5]);
-    c->n_launches += 2;
     FS_CUDA(cudaGetLastError());
     return FS_OK;
 }
 
-// Builds a hierarchy under level 0 (grid g0, flags fl0, work arrays b0 and c0 of
-// the level-0 length, or allocated here when null).
-int mg_build(fs_ctx *c, MgState *s, const MgGrid &g0, uint8_t *fl0, float *b0, float *c0, float coef, float mass)
+// The grids of a volume's levels under level 0 (grid g0), and its single-block levels.
+int plan_levels(fs_ctx *c, MgState *s, const MgGrid &g0, float coef, float mass)
 {
-    free_levels(s);
-    MgLevel &l0 = s->lev[0];
-    l0.g = g0;
-    l0.scale = coef;
-    l0.mass = mass;
-    l0.fl = fl0;
+    *s = MgState();
+    s->lev[0].g = g0;
     s->nlev = 1;
-    s->own0 = b0 == nullptr;
-    auto fail = [&](const char *what) {
-        cudaGetLastError();
-        free_levels(s);
-        return set_error(FS_ENOMEM, "multigrid %s", what);
-    };
-    if (s->own0) {
-        if (cudaMalloc(&l0.b, (size_t)g0.n * 4) != cudaSuccess || cudaMalloc(&l0.c, (size_t)g0.n * 4) != cudaSuccess)
-            return fail("level-0 work arrays");
-        FS_CUDA(cudaMemsetAsync(l0.b, 0, (size_t)g0.n * 4, c->stream));
-        FS_CUDA(cudaMemsetAsync(l0.c, 0, (size_t)g0.n * 4, c->stream));
-    } else {
-        l0.b = b0;
-        l0.c = c0;
-    }
     while (s->lev[s->nlev - 1].g.n > MG_COARSE_CELLS && s->nlev < MG_MAX_LEVELS) {
         const MgGrid &gf = s->lev[s->nlev - 1].g;
-        MgLevel &v = s->lev[s->nlev];
+        MgLevel &v = s->lev[s->nlev++];
         v.g = coarse_grid((gf.nx + 1) / 2, (gf.ny + 1) / 2, (gf.nz + 1) / 2);
-        v.scale = s->lev[s->nlev - 1].scale * 0.25f;
-        v.mass = mass;
-        const size_t nb = (size_t)v.g.n;
-        if (cudaMalloc(&v.fl, nb) != cudaSuccess || cudaMalloc(&v.r, nb * 4) != cudaSuccess ||
-            cudaMalloc(&v.a, nb * 4) != cudaSuccess || cudaMalloc(&v.b, nb * 4) != cudaSuccess ||
-            cudaMalloc(&v.c, nb * 4) != cudaSuccess) {
-            s->nlev += 1;  // free what was allocated
-            return fail("level arrays");
-        }
-        s->nlev += 1;
-        for (float *p : {v.r, v.a, v.b, v.c}) FS_CUDA(cudaMemsetAsync(p, 0, nb * 4, c->stream));
-        const int blocks = row_blocks(c, v.g);
-        k_mg_coarsen<<<blocks, RT, 0, c->stream>>>(gf, s->lev[s->nlev - 2].fl, v.g, v.fl);
-        k_mg_count<<<blocks, RT, 0, c->stream>>>(v.g, v.fl);
-        c->n_launches += 2;
-        FS_CUDA(cudaGetLastError());
         if (v.g.nx == 1 && v.g.ny == 1 && v.g.nz == 1) break;
+    }
+    float sc = coef;
+    for (int l = 0; l < s->nlev; l++, sc *= 0.25f) {
+        s->lev[l].scale = sc;
+        s->lev[l].mass = mass;
     }
     if (s->lev[s->nlev - 1].g.n > MG_COARSE_CELLS)
         return set_error(FS_EINVAL, "multigrid: the coarsest level does not fit in shared memory");
@@ -1019,119 +914,161 @@ int mg_build(fs_ctx *c, MgState *s, const MgGrid &g0, uint8_t *fl0, float *b0, f
         if (g.sy % 4 || g.sz % 4 || g.origin % 4 || g.n % 4)
             return set_error(FS_EINVAL, "multigrid: level %d rows are not quad-aligned", l);
     }
-    // the lists of active quads (every level but the coarsest) and of active
-    // restriction pairs (every level but the finest): counted, allocated, filled
-    auto make_list = [&](bool pairs, int l, int **list, int *count) -> int {
-        const MgGrid &g = s->lev[l].g;
-        const long long items = pairs ? (long long)((g.nx + 1) >> 1) * g.ny * g.nz : g.n / 4;
-        const int blocks = (int)std::max(1LL, (items + LB_ITEMS - 1) / LB_ITEMS);
-        int *dcnt = nullptr;
-        std::vector<int> hcnt(blocks);
-        if (cudaMalloc(&dcnt, sizeof(int) * (size_t)blocks * 2) != cudaSuccess) {
-            cudaGetLastError();
-            return FS_ENOMEM;
-        }
-        auto launch = [&](const int *offs, int *out) {
-            if (pairs)
-                k_list_build<<<blocks, LB_TH, 0, c->stream>>>(PairPred{g, s->lev[l].fl}, offs, dcnt, out);
-            else
-                k_list_build<<<blocks, LB_TH, 0, c->stream>>>(QuadPred{g, s->lev[l].fl}, offs, dcnt, out);
-            c->n_launches += 1;
-        };
-        int rc = FS_OK;
-        launch(nullptr, nullptr);
-        if ((rc = check_cuda(cudaGetLastError(), "k_list_build")) ||
-            (rc = check_cuda(cudaMemcpyAsync(hcnt.data(), dcnt, sizeof(int) * (size_t)blocks,
-                                             cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync")) ||
-            (rc = check_cuda(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize"))) {
-            cudaFree(dcnt);
-            return rc;
-        }
-        int total = 0;
-        for (int b = 0; b < blocks; b++) {  // exclusive scan of the block counts
-            const int n = hcnt[b];
-            hcnt[b] = total;
-            total += n;
-        }
-        *count = total;
-        if (cudaMalloc(list, sizeof(int) * (size_t)std::max(total, 1)) != cudaSuccess) {
-            cudaGetLastError();
-            *list = nullptr;
-            cudaFree(dcnt);
-            return FS_ENOMEM;
-        }
-        if (!(rc = check_cuda(cudaMemcpyAsync(dcnt + blocks, hcnt.data(), sizeof(int) * (size_t)blocks,
-                                              cudaMemcpyHostToDevice, c->stream), "cudaMemcpyAsync"))) {
-            launch(dcnt + blocks, *list);
-            rc = check_cuda(cudaGetLastError(), "k_list_build");
-        }
-        // the host counts must outlive the copy above
-        if (!rc) rc = check_cuda(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-        cudaFree(dcnt);
-        return rc;
-    };
-    for (int l = 0; l < s->nlev; l++) {
-        MgLevel &v = s->lev[l];
-        int rc = FS_OK;
-        if (l + 1 < s->nlev) rc = make_list(false, l, &v.ql, &v.nqa);
-        if (!rc && l >= 1) rc = make_list(true, l, &v.pl, &v.npa);
-        if (rc == FS_ENOMEM) return fail("active lists");
-        if (rc) {
-            free_levels(s);
-            return rc;
-        }
+    // the single-block launch takes the levels from the first one below level 0
+    // (or the only level) that fits in shared memory with all below it
+    size_t n = (size_t)s->lev[s->nlev - 1].g.n;
+    s->lb = s->nlev - 1;
+    while (s->lb > 1 && s->nlev - s->lb < MGB_MAXLEV && bottom_smem(n + (size_t)s->lev[s->lb - 1].g.n) <= MGB_SMEM) {
+        s->lb -= 1;
+        n += (size_t)s->lev[s->lb].g.n;
     }
-    // the small levels in one cluster launch: from the first level below level 0
-    // whose active quads fit the cluster's threads a few times over, when at
-    // least one level above the coarsest is among them
-    s->cl = 0;
-    s->ctas = cluster_ctas_here();
-    if (s->ctas > 0)
-        for (int l = 1; l + 1 < s->nlev; l++)
-            if (s->lev[l].nqa <= MGC_MAX_QUADS && s->nlev - l <= MGC_MAXLEV) {
-                s->cl = l;
-                break;
-            }
-    // The least each level-0 kernel must move (its algorithmic bytes): the list
-    // entry and the flags of each active quad (or pair) it visits and 4 bytes per
-    // unknown for each vector it reads or writes on the unknowns.
-    // q0: the active quads of level 0; p1: level 1's active pairs;
-    // u0, u1: the unknowns of levels 0 and 1.
-    unsigned long long *cnt = reinterpret_cast<unsigned long long *>(c->partials), nl[2] = {0, 0};
-    FS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(nl), c->stream));
-    k_mg_count_liq<<<grid_blocks(c, g0.n, TH), TH, 0, c->stream>>>(g0, fl0, cnt);
-    if (s->nlev > 1)
-        k_mg_count_liq<<<grid_blocks(c, s->lev[1].g.n, TH), TH, 0, c->stream>>>(s->lev[1].g, s->lev[1].fl, cnt + 1);
-    FS_CUDA(cudaMemcpyAsync(nl, cnt, sizeof(nl), cudaMemcpyDeviceToHost, c->stream));
-    FS_CUDA(cudaStreamSynchronize(c->stream));
-    const double u0 = (double)nl[0], u1 = (double)nl[1];
-    const double q0 = (double)s->lev[0].nqa, p1 = s->nlev > 1 ? (double)s->lev[1].npa : 0.0;
-    s->by0[0] = 8.0 * q0 + 8.0 * u0;             // smooth2: read r, write e
-    s->by0[1] = 8.0 * q0 + 12.0 * u0;            // residual: read r, e, write res
-    s->by0[2] = 6.0 * p1 + 4.0 * u0 + 4.0 * u1;  // restrict: pair list and flags, read res, write level-1 r
-    s->by0[3] = 8.0 * q0 + 8.0 * u0 + 4.0 * u1;  // prolong: read and write e, read the level-1 e
-    s->by0[4] = 8.0 * q0 + 12.0 * u0;            // smooth: read r, e, write e
-    s->by0[5] = 8.0 * q0 + 12.0 * u0;            // last smooth: read r, e, write z
     s->epoch = c->mask_epoch;
     s->coef = coef;
     return FS_OK;
 }
 
-int apply_on(fs_ctx *c, MgState *s, const float *r, float *z, const int *done, bool sample, cudaStream_t st,
-             SolveScal *rzs = nullptr, int first = 0, int boff = 0, int btot = 0)
+// A list over the volumes of a level of a set, in order: counted, allocated, filled.
+template <class P>
+int make_list(fs_ctx *c, const MgSetLevel &v, long long (*items)(const MgGrid &), int **list, int *count)
 {
-    s->done = done;
-    s->rzs = rzs;
-    s->rz_first = first;
-    s->rz_boff = boff;
-    s->rz_btot = btot;
-    MgLevel &l0 = s->lev[0];
-    l0.r = const_cast<float *>(r);
-    l0.a = z;
-    const int rc = vcycle(c, s, 0, sample, st);
-    l0.r = nullptr;
-    l0.a = nullptr;
+    int *dcnt = nullptr;
+    std::vector<int> hcnt;
+    int blocks[3] = {0, 0, 0}, boff[4] = {0, 0, 0, 0};
+    for (int k = 0; k < v.sp.nv; k++) {
+        blocks[k] = (int)std::max(1LL, (items(v.sp.g[k]) + LB_ITEMS - 1) / LB_ITEMS);
+        boff[k + 1] = boff[k] + blocks[k];
+    }
+    const int nb = boff[v.sp.nv];
+    hcnt.resize((size_t)nb);
+    if (cudaMalloc(&dcnt, sizeof(int) * (size_t)nb * 2) != cudaSuccess) {
+        cudaGetLastError();
+        return FS_ENOMEM;
+    }
+    auto launch = [&](const int *offs, int *out) {
+        for (int k = 0; k < v.sp.nv; k++) {
+            k_list_build<<<blocks[k], LB_TH, 0, c->stream>>>(P{v.sp.g[k], v.fl + v.sp.base[k], v.sp.base[k]},
+                                                             offs ? offs + boff[k] : nullptr, dcnt + boff[k], out);
+            c->n_launches += 1;
+        }
+    };
+    int rc = FS_OK;
+    launch(nullptr, nullptr);
+    if ((rc = check_cuda(cudaGetLastError(), "k_list_build")) ||
+        (rc = check_cuda(cudaMemcpyAsync(hcnt.data(), dcnt, sizeof(int) * (size_t)nb, cudaMemcpyDeviceToHost,
+                                         c->stream), "cudaMemcpyAsync")) ||
+        (rc = check_cuda(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize"))) {
+        cudaFree(dcnt);
+        return rc;
+    }
+    int total = 0;
+    for (int b = 0; b < nb; b++) {  // exclusive scan of the block counts
+        const int n = hcnt[b];
+        hcnt[b] = total;
+        total += n;
+    }
+    *count = total;
+    if (cudaMalloc(list, sizeof(int) * (size_t)std::max(total, 1)) != cudaSuccess) {
+        cudaGetLastError();
+        *list = nullptr;
+        cudaFree(dcnt);
+        return FS_ENOMEM;
+    }
+    if (!(rc = check_cuda(cudaMemcpyAsync(dcnt + nb, hcnt.data(), sizeof(int) * (size_t)nb, cudaMemcpyHostToDevice,
+                                          c->stream), "cudaMemcpyAsync"))) {
+        launch(dcnt + nb, *list);
+        rc = check_cuda(cudaGetLastError(), "k_list_build");
+    }
+    // the host counts must outlive the copy above
+    if (!rc) rc = check_cuda(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+    cudaFree(dcnt);
     return rc;
+}
+
+// Arrays, flags and lists of a set whose volumes' levels are planned and whose
+// level 0 is given (flags, work arrays, bases).
+int build_set(fs_ctx *c, MgSet &t)
+{
+    int nlev = 1, minlb = MG_MAX_LEVELS;
+    for (int v = 0; v < t.nv; v++) {
+        nlev = std::max(nlev, t.s[v]->nlev);
+        minlb = std::min(minlb, t.s[v]->lb);
+    }
+    for (int l = 0; l < nlev; l++) {
+        MgSetLevel &x = t.lev[l];
+        x.sp.nv = t.nv;
+        size_t n = 0;
+        for (int v = 0; v < t.nv; v++) {
+            x.sp.g[v] = t.s[v]->lev[l].g;
+            if (l == 0) continue;
+            x.sp.base[v] = (int)n;
+            if (l < t.s[v]->nlev) n += (size_t)x.sp.g[v].n;
+        }
+        if (l == 0) {
+            for (int v = 0; v < t.nv; v++) t.s[v]->lev[0].fl = x.fl + x.sp.base[v];
+            continue;
+        }
+        bool ok = cudaMalloc(&x.fl, n) == cudaSuccess;
+        for (float **p : {&x.r, &x.a, &x.b, &x.c}) ok = ok && cudaMalloc(p, n * 4) == cudaSuccess;
+        if (!ok) {
+            cudaGetLastError();
+            return set_error(FS_ENOMEM, "multigrid level arrays");
+        }
+        for (float *p : {x.r, x.a, x.b, x.c}) FS_CUDA(cudaMemsetAsync(p, 0, n * 4, c->stream));
+        for (int v = 0; v < t.nv; v++) {
+            if (l >= t.s[v]->nlev) continue;
+            MgLevel &L = t.s[v]->lev[l];
+            L.fl = x.fl + x.sp.base[v];
+            L.r = x.r + x.sp.base[v];
+            L.a = x.a + x.sp.base[v];
+            L.b = x.b + x.sp.base[v];
+            const int blocks = row_blocks(c, L.g);
+            k_mg_coarsen<<<blocks, RT, 0, c->stream>>>(t.s[v]->lev[l - 1].g, t.s[v]->lev[l - 1].fl, L.g, L.fl);
+            k_mg_count<<<blocks, RT, 0, c->stream>>>(L.g, L.fl);
+            c->n_launches += 2;
+        }
+        FS_CUDA(cudaGetLastError());
+    }
+    {
+        MgBottomArgs a;
+        bottom_args(t, a);
+        size_t bytes = 0;
+        for (int v = 0; v < t.nv; v++) bytes += (size_t)a.v[v].bytes;
+        if (cudaMalloc(&t.blob, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            t.blob = nullptr;
+            return set_error(FS_ENOMEM, "multigrid coarse lists");
+        }
+        bottom_args(t, a);
+        k_mg_bottom_lists<<<t.nv, MGB_TH, 0, c->stream>>>(a);
+        c->n_launches += 1;
+        FS_CUDA(cudaGetLastError());
+    }
+    if (nlev == 1) return FS_OK;
+    // A level takes the tile kernels where its tiles run in one wave: at 64^3 with
+    // one volume a leg takes 7 us, the three list kernels with their gaps 14; with
+    // three volumes (648 tiles on 304 slots) 20 us against 17.
+    t.lf = 1;
+    while (t.lf < minlb) {
+        long long tiles = 0;
+        for (int v = 0; v < t.nv; v++) {
+            const MgTiles m = make_tiles(t.s[v]->lev[t.lf].g, t.nv, c->num_sms);
+            tiles += (long long)m.ntx * m.nty * m.ntz;
+        }
+        if (tiles <= (long long)MGT_PER_SM * c->num_sms) break;
+        t.lf += 1;
+    }
+    for (int l = 0; l <= t.lf; l++) {
+        MgSetLevel &x = t.lev[l];
+        int rc = FS_OK;
+        if (l < t.lf)
+            rc = make_list<QuadPred>(c, x, [](const MgGrid &g) { return (long long)(g.n / 4); }, &x.ql, &x.nq);
+        if (!rc && l > 0)
+            rc = make_list<PairPred>(
+                c, x, [](const MgGrid &g) { return (long long)((g.nx + 1) >> 1) * g.ny * g.nz; }, &x.pl, &x.np);
+        if (rc == FS_ENOMEM) return set_error(FS_ENOMEM, "multigrid active lists");
+        if (rc) return rc;
+    }
+    return FS_OK;
 }
 
 MgAll *state(fs_ctx *c)
@@ -1144,43 +1081,76 @@ MgAll *state(fs_ctx *c)
     return m;
 }
 
+// shared memory limits of the coarse-level kernels on the current device
+int coarse_attributes()
+{
+    const int most = 218 * 1024;  // beside the static shared memory
+    for (const void *f : {(const void *)k_mg_down, (const void *)k_mg_up, (const void *)k_mg_bottom})
+        FS_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    return FS_OK;
+}
+
+// two zeroed work arrays of n floats, allocated once
+int work_arrays(fs_ctx *c, float **a, float **b, size_t n, bool zero)
+{
+    if (!*a) {
+        if (cudaMalloc(a, n * 4) != cudaSuccess || cudaMalloc(b, n * 4) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(*a);
+            *a = nullptr;
+            return set_error(FS_ENOMEM, "multigrid level-0 work arrays");
+        }
+        zero = true;
+    }
+    if (zero) {
+        FS_CUDA(cudaMemsetAsync(*a, 0, n * 4, c->stream));
+        FS_CUDA(cudaMemsetAsync(*b, 0, n * 4, c->stream));
+    }
+    return FS_OK;
+}
+
 }  // namespace
 
 void mg_free(fs_ctx *c)
 {
     MgAll *m = static_cast<MgAll *>(c->mg);
     if (!m) return;
-    free_levels(&m->cell);
-    for (MgState &f : m->face) free_levels(&f);
-    cudaFree(m->fb);
-    cudaFree(m->fc);
-    for (int k = 0; k < 2; k++) {
-        if (m->side[k]) cudaStreamDestroy(m->side[k]);
-        if (m->join[k]) cudaEventDestroy(m->join[k]);
-    }
-    if (m->fork) cudaEventDestroy(m->fork);
+    free_set(&m->cset);
+    for (MgSet &t : m->fset) free_set(&t);
+    for (float *p : {m->cb, m->cc, m->fb, m->fc}) cudaFree(p);
     delete m;
     c->mg = nullptr;
 }
 
-// z = M r on the cell space (r and z of length nC, zero off the liquid).
-// z = M r on the cell space; with rzs, r.z in the last level-0 sweep when the
-// hierarchy has one (*fused tells)
+// z = M r on the cell space (r and z of length nC, zero off the liquid); with
+// rzs, r.z in the last level-0 sweep when the hierarchy has one (*fused tells)
 static int apply_cell(fs_ctx *c, const float *r, float *z, const int *done, SolveScal *rzs, int first, bool *fused)
 {
     if (fused) *fused = false;
     MgAll *m = state(c);
     if (!m) return set_error(FS_ENOMEM, "host allocation failed");
     const Layout &L = c->L;
-    if (m->cell.epoch != c->mask_epoch)
-        if (int rc = mg_build(c, &m->cell, level0_grid(L, L.nx, L.ny, L.nz), c->cflag, nullptr, nullptr, 1.f, 0.f))
+    int rc;
+    if (m->cell.epoch != c->mask_epoch) {
+        MgSet &t = m->cset;
+        free_set(&t);
+        if ((rc = coarse_attributes()) || (rc = work_arrays(c, &m->cb, &m->cc, (size_t)L.nC, true)) ||
+            (rc = plan_levels(c, &m->cell, level0_grid(L, L.nx, L.ny, L.nz), 1.f, 0.f)))
             return rc;
+        t.nv = 1;
+        t.s[0] = &m->cell;
+        t.lev[0].fl = c->cflag;
+        t.lev[0].b = m->cb;
+        t.lev[0].c = m->cc;
+        if ((rc = build_set(c, t))) {
+            free_set(&t);
+            return rc;
+        }
+    }
     const bool fuse = rzs && m->cell.nlev >= 2;
-    const bool sample = c->prof_on && (m->cell.calls++ % std::max(1, c->prof_period)) == 0;
+    const bool sample = c->prof_on && (m->cset.calls++ % std::max(1, c->prof_period)) == 0;
     cudaEvent_t e0 = sample ? prof_mark(c) : nullptr;
-    const int rc = fuse ? apply_on(c, &m->cell, r, z, done, sample, c->stream, rzs, first, 0,
-                                   smooth_blocks(c, m->cell.lev[0].nqa))
-                        : apply_on(c, &m->cell, r, z, done, sample, c->stream);
+    rc = vcycle(c, m->cset, r, z, done, sample, fuse ? rzs : nullptr, first);
     if (sample) prof_add(c, K_MG_VCYCLE_P, e0, prof_mark(c), 0.0);
     if (fused) *fused = fuse && rc == FS_OK;
     return rc;
@@ -1198,76 +1168,70 @@ bool mg_apply_rz(fs_ctx *c, const float *r, float *z, const int *done, SolveScal
     return fused;
 }
 
+// The three face hierarchies and their sets for the current mask.
+static int build_faces(fs_ctx *c, MgAll *m, float cc)
+{
+    const Layout &L = c->L;
+    int rc;
+    for (MgSet &t : m->fset) free_set(&t);
+    m->nfset = 0;
+    if ((rc = coarse_attributes()) || (rc = work_arrays(c, &m->fb, &m->fc, (size_t)L.nF, true))) return rc;
+    bool all = true;
+    for (int k = 0; k < 3; k++) {
+        if ((rc = plan_levels(c, &m->face[k], level0_grid(L, L.nx + (k == 0), L.ny + (k == 1), L.nz + (k == 2)), cc,
+                              1.f)))
+            return rc;
+        all = all && m->face[k].nlev >= 2;
+    }
+    const int nset = all ? 1 : 3;
+    for (int n = 0; n < nset; n++) {
+        MgSet &t = m->fset[n];
+        t.nv = all ? 3 : 1;
+        t.lev[0].fl = c->fflag;
+        t.lev[0].b = m->fb;
+        t.lev[0].c = m->fc;
+        t.one = true;
+        for (int v = 0; v < t.nv; v++) {
+            const int k = all ? v : n;
+            t.s[v] = &m->face[k];
+            t.lev[0].sp.base[v] = L.face_origin(k) - L.PL;  // the volume's leading guard plane
+        }
+        if ((rc = build_set(c, t))) {
+            for (MgSet &f : m->fset) free_set(&f);
+            return rc;
+        }
+    }
+    m->nfset = nset;
+    return FS_OK;
+}
+
 // z = M r on the face space for the Helmholtz operator I + cc L of the viscosity
-// solve, one V-cycle per velocity component (r and z of length nF, zero off the
-// unknown faces). With `done` set, every kernel returns at once once *done != 0.
+// solve (r and z of length nF, zero off the unknown faces), the three velocity
+// components' V-cycles launch by launch together. With `done` set, every kernel
+// returns at once once *done != 0.
 static int apply_faces(fs_ctx *c, const float *r, float *z, float cc, const int *done, SolveScal *rzs, int first,
                        bool *fused)
 {
     if (fused) *fused = false;
     MgAll *m = state(c);
     if (!m) return set_error(FS_ENOMEM, "host allocation failed");
-    const Layout &L = c->L;
-    if (!m->fb) {
-        if (cudaMalloc(&m->fb, (size_t)L.nF * 4) != cudaSuccess || cudaMalloc(&m->fc, (size_t)L.nF * 4) != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(m->fb);
-            m->fb = nullptr;
-            return set_error(FS_ENOMEM, "multigrid face work arrays");
+    if (m->nfset == 0 || m->face[0].epoch != c->mask_epoch) {
+        if (int rc = build_faces(c, m, cc)) {
+            m->nfset = 0;
+            return rc;
         }
-        FS_CUDA(cudaMemsetAsync(m->fb, 0, (size_t)L.nF * 4, c->stream));
-        FS_CUDA(cudaMemsetAsync(m->fc, 0, (size_t)L.nF * 4, c->stream));
-    }
-    if (!m->fork) {  // the side streams and their events, once (the fork event last)
-        for (int k = 0; k < 2; k++) {
-            if (!m->side[k]) FS_CUDA(cudaStreamCreateWithFlags(&m->side[k], cudaStreamNonBlocking));
-            if (!m->join[k]) FS_CUDA(cudaEventCreateWithFlags(&m->join[k], cudaEventDisableTiming));
-        }
-        FS_CUDA(cudaEventCreateWithFlags(&m->fork, cudaEventDisableTiming));
-    }
-    if (m->face[0].epoch != c->mask_epoch) {  // new mask: the shared work arrays start from zero again
-        FS_CUDA(cudaMemsetAsync(m->fb, 0, (size_t)L.nF * 4, c->stream));
-        FS_CUDA(cudaMemsetAsync(m->fc, 0, (size_t)L.nF * 4, c->stream));
-    }
-    const bool sample = c->prof_on && (m->face[0].calls++ % std::max(1, c->prof_period)) == 0;
-    cudaEvent_t e0 = sample ? prof_mark(c) : nullptr;
-    for (int k = 0; k < 3; k++) {
-        MgState &s = m->face[k];
-        const size_t base = (size_t)L.face_origin(k) - L.PL;  // the volume's leading guard plane
-        if (s.epoch != c->mask_epoch) {
-            const MgGrid g0 = level0_grid(L, L.nx + (k == 0), L.ny + (k == 1), L.nz + (k == 2));
-            if (int rc = mg_build(c, &s, g0, c->fflag + base, m->fb + base, m->fc + base, cc, 1.f)) return rc;
-            s.one0 = true;
-        } else if (s.coef != cc) {  // a new viscosity or time step: rescale the levels only
+    } else if (m->face[0].coef != cc) {  // a new viscosity or time step: rescale the levels only
+        for (MgState &s : m->face) {
             float sc = cc;
             for (int l = 0; l < s.nlev; l++, sc *= 0.25f) s.lev[l].scale = sc;
             s.coef = cc;
         }
     }
-    // r.z in the three last level-0 sweeps together: their blocks are numbered
-    // one after another for one reduction (volume k's from boff[k])
-    bool fuse = rzs != nullptr;
-    int boff[3] = {0, 0, 0}, btot = 0;
-    for (int k = 0; k < 3 && fuse; k++) {
-        fuse = m->face[k].nlev >= 2;
-        boff[k] = btot;
-        btot += smooth_blocks(c, m->face[k].lev[0].nqa);
-    }
-    // volume 0 on the context's stream, 1 and 2 beside it (their sweeps share the
-    // GPU, so none is timed alone: the profiled sweep is the pressure V-cycle's)
-    FS_CUDA(cudaEventRecord(m->fork, c->stream));
-    for (int k = 0; k < 2; k++) FS_CUDA(cudaStreamWaitEvent(m->side[k], m->fork, 0));
-    for (int k = 2; k >= 0; k--) {
-        const size_t base = (size_t)L.face_origin(k) - L.PL;
-        cudaStream_t st = k == 0 ? c->stream : m->side[k - 1];
-        const int rc = fuse ? apply_on(c, &m->face[k], r + base, z + base, done, false, st, rzs, first, boff[k], btot)
-                            : apply_on(c, &m->face[k], r + base, z + base, done, false, st);
-        if (rc) return rc;
-    }
-    for (int k = 0; k < 2; k++) {
-        FS_CUDA(cudaEventRecord(m->join[k], m->side[k]));
-        FS_CUDA(cudaStreamWaitEvent(c->stream, m->join[k], 0));
-    }
+    const bool fuse = rzs && m->nfset == 1;
+    const bool sample = c->prof_on && (m->fset[0].calls++ % std::max(1, c->prof_period)) == 0;
+    cudaEvent_t e0 = sample ? prof_mark(c) : nullptr;
+    for (int n = 0; n < m->nfset; n++)
+        if (int rc = vcycle(c, m->fset[n], r, z, done, false, fuse ? rzs : nullptr, first)) return rc;
     if (sample) prof_add(c, K_MG_VCYCLE_V, e0, prof_mark(c), 0.0);
     if (fused) *fused = fuse;
     return FS_OK;
@@ -1287,20 +1251,29 @@ bool mg_apply_faces_rz(fs_ctx *c, const float *r, float *z, float cc, const int 
 }
 
 // Launch counts of the level-0 kernels (fs_profile): `vcycles` V-cycles that did
-// work on the pressure hierarchy, or on each of the three face volumes.
+// work on the pressure hierarchy, or on the face volumes together.
 void mg_count(fs_ctx *c, long long vcycles, bool faces)
 {
     const MgAll *m = static_cast<const MgAll *>(c->mg);
     if (!m || !c->prof_on) return;
     const int nlev = faces ? m->face[0].nlev : m->cell.nlev;
     if (nlev < 2) return;
-    const long long k = faces ? 3 * vcycles : vcycles;
-    const bool one = faces && m->face[0].one0;  // the face volumes' level 0 skips three of the six kinds
     for (int id : {K_MG0_SMOOTH2, K_MG0_RESIDUAL, K_MG0_SMOOTH})
-        if (!one) prof_count(c, id, k);
-    for (int id : {K_MG0_RESTRICT, K_MG0_PROLONG, K_MG0_SMOOTH_Z}) prof_count(c, id, k);
+        if (!faces) prof_count(c, id, vcycles);  // the face volumes' level 0 skips three of the six kinds
+    for (int id : {K_MG0_RESTRICT, K_MG0_PROLONG, K_MG0_SMOOTH_Z}) prof_count(c, id, vcycles);
     prof_count(c, faces ? K_MG_VCYCLE_V : K_MG_VCYCLE_P, vcycles);
     if (!faces) prof_count(c, K_MG_COARSE, vcycles);
+}
+
+// the set with level-0 lists for the current mask (of the pressure, or of the
+// face volumes together), or null
+static const MgSet *listed_set(const fs_ctx *c, bool faces)
+{
+    const MgAll *m = static_cast<const MgAll *>(c->mg);
+    if (!m) return nullptr;
+    const MgState &h = faces ? m->face[0] : m->cell;
+    if (h.epoch != c->mask_epoch || h.nlev < 2 || (faces && m->nfset != 1)) return nullptr;
+    return faces ? &m->fset[0] : &m->cset;
 }
 
 // r.z over the active quads of the pressure hierarchy's level 0 (or of the three
@@ -1308,40 +1281,22 @@ void mg_count(fs_ctx *c, long long vcycles, bool faces)
 // own coarsest level), and the caller takes the dense pass
 bool mg_rz(fs_ctx *c, bool faces, const float *r, const float *z, int first, SolveScal *s)
 {
-    const MgAll *m = static_cast<const MgAll *>(c->mg);
-    if (!m) return false;
-    RzLists L;
-    std::memset(&L, 0, sizeof(L));
-    long long total = 0;
-    L.nv = faces ? 3 : 1;
-    for (int v = 0; v < L.nv; v++) {
-        const MgState &h = faces ? m->face[v] : m->cell;
-        if (h.nlev < 2 || h.epoch != c->mask_epoch || !h.lev[0].ql) return false;
-        L.ql[v] = h.lev[0].ql;
-        L.n[v] = h.lev[0].nqa;
-        L.base[v] = faces ? (long long)c->L.face_origin(v) - c->L.PL : 0;
-        total += L.n[v];
-    }
-    k_mg_rz<<<grid_blocks(c, total, TH), TH, 0, c->stream>>>(L, r, z, first, s, c->partials);
+    const MgSet *t = listed_set(c, faces);
+    if (!t) return false;
+    k_mg_rz<<<grid_blocks(c, t->lev[0].nq, TH), TH, 0, c->stream>>>(t->lev[0].ql, t->lev[0].nq, r, z, first, s, c->partials);
     c->n_launches += 1;
     return cudaPeekAtLastError() == cudaSuccess;
 }
 
-// The level-0 lists of active quads of the pressure hierarchy (one) or of the
-// three face volumes, with each volume's first element; false when a hierarchy
-// has no lists for the current mask.
-bool mg_level0_lists(const fs_ctx *c, bool faces, const int **ql, int *n, long long *base)
+// The level-0 list of active quads of the pressure hierarchy, or of the three
+// face volumes together (quads of the whole face space); false when a hierarchy
+// has no list for the current mask.
+bool mg_level0_list(const fs_ctx *c, bool faces, const int **ql, int *n)
 {
-    const MgAll *m = static_cast<const MgAll *>(c->mg);
-    if (!m) return false;
-    const int nv = faces ? 3 : 1;
-    for (int v = 0; v < nv; v++) {
-        const MgState &h = faces ? m->face[v] : m->cell;
-        if (h.nlev < 2 || h.epoch != c->mask_epoch || !h.lev[0].ql) return false;
-        ql[v] = h.lev[0].ql;
-        n[v] = h.lev[0].nqa;
-        base[v] = faces ? (long long)c->L.face_origin(v) - c->L.PL : 0;
-    }
+    const MgSet *t = listed_set(c, faces);
+    if (!t) return false;
+    *ql = t->lev[0].ql;
+    *n = t->lev[0].nq;
     return true;
 }
 

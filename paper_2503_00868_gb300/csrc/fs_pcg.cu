@@ -41,22 +41,14 @@ __device__ __forceinline__ float inv_diag(uint8_t f, float cc)
     return d > 0.f ? __frcp_rn(d) : 0.f;
 }
 
-// The operator apply over lists of active quads (those holding an unknown; the
-// multigrid hierarchy's level-0 lists, one per volume, volume v from element
-// base[v]): per quad, p_new = z + beta p_old on the quad and its six neighbours
-// (inactive elements hold z = p_old = 0, so p_new = 0 there), q = A p_new on the
-// quad, both written whole, and p_new . q. A thread strides through the lists
-// with the next entry fetched a step ahead, so only quads with an unknown are
-// read or written, where a 128 x 8 tile carries many without.
-struct QuadLists {
-    const int *ql[3];
-    int n[3];
-    long long base[3];
-    int nv;
-};
-
+// The operator apply over a list of active quads (those holding an unknown; the
+// multigrid hierarchy's level-0 list): per quad, p_new = z + beta p_old on the
+// quad and its six neighbours (inactive elements hold z = p_old = 0, so p_new = 0
+// there), q = A p_new on the quad, both written whole, and p_new . q. A thread
+// strides through the list with the next entry fetched a step ahead, so only quads
+// with an unknown are read or written, where a 128 x 8 tile carries many without.
 template <class Op>
-__global__ void __launch_bounds__(TH) k_spmv_list(QuadLists Ls, const float *__restrict__ src,
+__global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, int na, const float *__restrict__ src,
                                                   const float *__restrict__ pold, float *__restrict__ pnew,
                                                   float *__restrict__ q, const uint8_t *__restrict__ fl, int P,
                                                   int PL, float cc, SolveScal *s, double *partials)
@@ -66,36 +58,31 @@ __global__ void __launch_bounds__(TH) k_spmv_list(QuadLists Ls, const float *__r
     const float off = Op::offc(cc);
     KSum acc;
     const int st = gridDim.x * blockDim.x;
-    for (int v = 0; v < Ls.nv; v++) {
-        const long long base = Ls.base[v];
-        const int *ql = Ls.ql[v];
-        const int na = Ls.n[v];
-        int i = blockIdx.x * blockDim.x + threadIdx.x;
-        int qn = i < na ? __ldg(ql + i) : 0;
-        for (; i < na; i += st) {
-            const long long t = base + 4LL * qn;
-            qn = i + st < na ? __ldg(ql + i + st) : 0;
-            const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
-            auto pn4 = [&](long long u) {
-                const float4 a = __ldg(reinterpret_cast<const float4 *>(src + u));
-                const float4 b = __ldg(reinterpret_cast<const float4 *>(pold + u));
-                return make_float4(a.x + beta * b.x, a.y + beta * b.y, a.z + beta * b.z, a.w + beta * b.w);
-            };
-            auto pn1 = [&](long long u) { return __ldg(src + u) + beta * __ldg(pold + u); };
-            const float4 c = pn4(t), dn = pn4(t - P), up = pn4(t + P), bk = pn4(t - PL), fw = pn4(t + PL);
-            const float lf = pn1(t - 1), rt = pn1(t + 4);
-            auto one = [&](uint8_t fe, float ce, float nb) {
-                return (fe & Op::ACTIVE) ? Op::diag(fe, cc) * ce - off * nb : 0.f;
-            };
-            float4 qv;
-            qv.x = one(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x));
-            qv.y = one(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y));
-            qv.z = one(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z));
-            qv.w = one(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w));
-            acc.add(c.x * qv.x + c.y * qv.y + c.z * qv.z + c.w * qv.w);
-            *reinterpret_cast<float4 *>(pnew + t) = c;
-            *reinterpret_cast<float4 *>(q + t) = qv;
-        }
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int qn = i < na ? __ldg(ql + i) : 0;
+    for (; i < na; i += st) {
+        const int t = 4 * qn;
+        qn = i + st < na ? __ldg(ql + i + st) : 0;
+        const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
+        auto pn4 = [&](int u) {
+            const float4 a = __ldg(reinterpret_cast<const float4 *>(src + u));
+            const float4 b = __ldg(reinterpret_cast<const float4 *>(pold + u));
+            return make_float4(a.x + beta * b.x, a.y + beta * b.y, a.z + beta * b.z, a.w + beta * b.w);
+        };
+        auto pn1 = [&](int u) { return __ldg(src + u) + beta * __ldg(pold + u); };
+        const float4 c = pn4(t), dn = pn4(t - P), up = pn4(t + P), bk = pn4(t - PL), fw = pn4(t + PL);
+        const float lf = pn1(t - 1), rt = pn1(t + 4);
+        auto one = [&](uint8_t fe, float ce, float nb) {
+            return (fe & Op::ACTIVE) ? Op::diag(fe, cc) * ce - off * nb : 0.f;
+        };
+        float4 qv;
+        qv.x = one(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x));
+        qv.y = one(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y));
+        qv.z = one(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z));
+        qv.w = one(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w));
+        acc.add(c.x * qv.x + c.y * qv.y + c.z * qv.z + c.w * qv.w);
+        *reinterpret_cast<float4 *>(pnew + t) = c;
+        *reinterpret_cast<float4 *>(q + t) = qv;
     }
     KSum vv[1] = {acc};
     double tot[1];
@@ -914,11 +901,10 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     double by_spmv = (double)L.nC + 16.0 * (double)c->n_liquid;
     const double by_upd = (double)L.nC + 24.0 * (double)c->n_liquid;
     const bool tiled = c->act_cell != nullptr;
-    // with multigrid, the operator apply walks the V-cycle's lists of active quads
-    QuadLists qls{};
-    qls.nv = 1;
-    const bool listed = c->prm.precond == FS_PRECOND_MG && mg_level0_lists(c, false, qls.ql, qls.n, qls.base);
-    const long long nlisted = listed ? qls.n[0] : 0;
+    // with multigrid, the operator apply walks the V-cycle's list of active quads
+    const int *ql = nullptr;
+    int nlisted = 0;
+    const bool listed = c->prm.precond == FS_PRECOND_MG && mg_level0_list(c, false, &ql, &nlisted);
     static const int rl = resident_blocks((const void *)k_spmv_list<PoisOp>, 0);  // one wave of the list apply
     if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_liquid;  // list entry and flags per quad
     const TileMap &tm = c->tm_cell;
@@ -936,7 +922,7 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
             const float *zsrc = jac ? c->pr : c->pz;
             if (listed)
                 k_spmv_list<PoisOp><<<wave_blocks(c, nlisted, rl), TH, 0, c->stream>>>(
-                    qls, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
+                    ql, nlisted, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
             else if (tiled)
                 k_spmv_z<PoisOp><<<tg.spmv, tdim, zmarch_smem(), c->stream>>>(
                     jac ? c->tmz_pr : c->tmz_pz, c->tmz_pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, c->items_cell,
@@ -1198,11 +1184,10 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     double by_spmv = (double)L.nF + 16.0 * (double)c->n_fluid;
     const double by_upd = (double)L.nF + 24.0 * (double)c->n_fluid;
     const bool tiled = c->act_face != nullptr;
-    // with multigrid, the operator apply walks the V-cycles' lists of active quads
-    QuadLists qls{};
-    qls.nv = 3;
-    const bool listed = mg && mg_level0_lists(c, true, qls.ql, qls.n, qls.base);
-    const long long nlisted = listed ? (long long)qls.n[0] + qls.n[1] + qls.n[2] : 0;
+    // with multigrid, the operator apply walks the V-cycles' list of active quads
+    const int *ql = nullptr;
+    int nlisted = 0;
+    const bool listed = mg && mg_level0_list(c, true, &ql, &nlisted);
     static const int rl = resident_blocks((const void *)k_spmv_list<HelmOp>, 0);  // one wave of the list apply
     if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_fluid;  // list entry and flags per quad
     const TileMap &tm = c->tm_face;
@@ -1217,7 +1202,7 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             if (listed)
                 k_spmv_list<HelmOp><<<wave_blocks(c, nlisted, rl), TH, 0, c->stream>>>(
-                    qls, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
+                    ql, nlisted, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
             else if (tiled)
                 k_spmv_z<HelmOp><<<tg.spmv, tdim, zmarch_smem(), c->stream>>>(
                     mg ? c->tmz_vz : c->tmz_vr, c->tmz_vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, c->items_face,
