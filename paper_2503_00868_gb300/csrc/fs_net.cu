@@ -22,8 +22,9 @@
 //                  cells of the liquid (the output on liquid cells depends on
 //                  nothing farther), from a tile list sorted by that distance;
 //   k_bwd_last     gradient through layer 5 to its input;
-//   k_wgrad<CIN,COUT>  weight and bias gradients (FP32 CUDA cores, per-block
-//                  partial sums, one atomicAdd per weight per block);
+//   k_wgrad<CIN,COUT>  weight and bias gradients as contractions over the cells on
+//                  the tensor cores (per-block sums, one atomicAdd per weight per
+//                  block);
 //   k_adam         Adam on the FP32 master weights, then the bf16 copies.
 // Layout: activations are channel-last, [cell][16] bf16 (32 bytes per cell) in
 // cell space; a neighbour outside the grid reads zero (checked per cell).
@@ -696,67 +697,191 @@ __global__ void __launch_bounds__(256) k_bwd_last(const float *__restrict__ gy, 
 
 // Weight and bias gradients of one layer: gW[co][ci][tap] += sum_cells
 // g[cell][co] * a[cell + tap][ci]; gB[co] += sum_cells g[cell][co]. g is bf16
-// [cell][16] (COUT = 16) or FP32 [cell] (COUT = 1); a is bf16 [cell][16].
-template <int CIN, int COUT, bool GF32>
-__global__ void __launch_bounds__(256) k_wgrad(const void *__restrict__ gptr, const __nv_bfloat16 *__restrict__ a,
-                                               float *gW, float *gB, Layout L)
+// [cell][16] (COUT = 16) or FP32 [cell] (COUT = 1); a is bf16 [cell][16], of which
+// the first CIN channels count.
+//
+// A contraction over the cells: per tap M = 16 output channels, N = 16 (or 8)
+// input channels, K = cells, on mma.sync m16n8k16 (bf16 products, FP32 sums). A
+// tile is 32 x 8 cells of one plane; warp w takes the taps of dz = w / 4 on rows
+// 2 (w % 4) and the next, whose g operand it loads once per 16 cells for its nine
+// taps. Each tile's sums start from zero and are added to FP32 totals in
+// registers, as few terms in a row as before (a tile had been one chain of 256).
+// An FP32 g (the last layer) enters as three bf16 rows of M whose sum it is
+// exactly (8 + 8 + 8 significant bits). The next tile is copied (cp.async) while
+// this one is worked on. At 64^3 a 16 x 16 layer takes 27 us (FP32 cores, one
+// thread per weight walking the tile's cells: 3.09 ms), the last layer 26 (247);
+// the copies of the tiles' halos (4 times the cells) and their latency bound it.
+constexpr int WG_TH = 384;
+constexpr int WG_A = TCELLS * 32, WG_G = NT_X * NT_Y * 32;  // bytes of a tile's two operands
+constexpr size_t WG_SMEM = 2 * (size_t)(WG_A + WG_G);
+
+__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3)
 {
-    constexpr int NOUT = COUT * CIN * 27;
-    extern __shared__ float wg_smem[];
-    float(*sg)[COUT] = reinterpret_cast<float(*)[COUT]>(wg_smem);
-    float(*sa)[CIN] = reinterpret_cast<float(*)[CIN]>(wg_smem + NT_X * NT_Y * COUT);
-    float part[(NOUT + 255) / 256];
-    float bpart = 0.f;
-#pragma unroll
-    for (int u = 0; u < (NOUT + 255) / 256; u++) part[u] = 0.f;
-    const int tid = threadIdx.x;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(addr));
+}
+
+// 16 bytes from global to shared memory, or zeros
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <int CIN, int COUT, bool GF32>
+__global__ void __launch_bounds__(WG_TH, 1) k_wgrad(const void *__restrict__ gptr, const __nv_bfloat16 *__restrict__ a,
+                                                    float *gW, float *gB, Layout L)
+{
+    constexpr int NB = CIN > 8 ? 2 : 1;  // tiles of 8 input channels
+    extern __shared__ __align__(128) unsigned char wg_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int dz = warp >> 2, y0 = 2 * (warp & 3);
     const int ntx = (L.nx + NT_X - 1) / NT_X, nty = (L.ny + NT_Y - 1) / NT_Y;
     const int ntiles = ntx * nty * L.nz;
-    for (int tb = blockIdx.x; tb < ntiles; tb += gridDim.x) {
+    auto stage = [&](int tb, unsigned char *buf) {
         const int tx = tb % ntx, ty = (tb / ntx) % nty, tk = tb / (ntx * nty);
         const int i0 = tx * NT_X, j0 = ty * NT_Y;
-        __syncthreads();
-        for (int e = tid; e < NT_X * NT_Y * COUT; e += blockDim.x) {
-            const int cl = e / COUT, o = e % COUT;
-            const int gi = i0 + cl % NT_X, gj = j0 + cl / NT_X;
-            float v = 0.f;
-            if (gi < L.nx && gj < L.ny) {
-                const size_t t = (size_t)cell_t(L, gi, gj, tk);
-                v = GF32 ? static_cast<const float *>(gptr)[t]
-                         : __bfloat162float(static_cast<const __nv_bfloat16 *>(gptr)[t * 16 + o]);
-            }
-            sg[cl][o] = v;
-        }
-        for (int e = tid; e < TCELLS * CIN; e += blockDim.x) {
-            const int cidx = e / CIN, ci = e % CIN;
+        const uint32_t sa = (uint32_t)__cvta_generic_to_shared(buf), sg = sa + WG_A;
+        for (int e = tid; e < TCELLS * 2; e += WG_TH) {
+            const int cidx = e >> 1, half = e & 1;
             const int xx = cidx % TXH, yy = (cidx / TXH) % TYH, zz = cidx / (TXH * TYH);
             const int gi = i0 - 1 + xx, gj = j0 - 1 + yy, gk = tk - 1 + zz;
-            sa[cidx][ci] = in_grid(L, gi, gj, gk) ? __bfloat162float(a[(size_t)cell_t(L, gi, gj, gk) * 16 + ci]) : 0.f;
+            const bool in = in_grid(L, gi, gj, gk);
+            const int t = in ? cell_t(L, gi, gj, gk) : L.PL;
+            cp_async16(sa + swz_off(cidx, half), a + (size_t)t * 16 + half * 8, in);
+        }
+        if (!GF32) {
+            for (int e = tid; e < NT_X * NT_Y * 2; e += WG_TH) {
+                const int cl = e >> 1, half = e & 1;
+                const int gi = i0 + cl % NT_X, gj = j0 + cl / NT_X;
+                const bool in = gi < L.nx && gj < L.ny;
+                const int t = in ? cell_t(L, gi, gj, tk) : L.PL;
+                cp_async16(sg + swz_off(cl, half), static_cast<const __nv_bfloat16 *>(gptr) + (size_t)t * 16 + half * 8,
+                           in);
+            }
+        } else {  // rows 0, 1, 2 of M: the leading, middle and last bf16 of g
+            for (int cl = tid; cl < NT_X * NT_Y; cl += WG_TH) {
+                const int gi = i0 + cl % NT_X, gj = j0 + cl / NT_X;
+                const float g = gi < L.nx && gj < L.ny ? static_cast<const float *>(gptr)[cell_t(L, gi, gj, tk)] : 0.f;
+                const __nv_bfloat16 h = __float2bfloat16(g);
+                const float g1 = g - __bfloat162float(h);
+                const __nv_bfloat16 m = __float2bfloat16(g1);
+                const __nv_bfloat16 l = __float2bfloat16(g1 - __bfloat162float(m));
+                __nv_bfloat162 hm, lz;
+                hm.x = h;
+                hm.y = m;
+                lz.x = l;
+                lz.y = __float2bfloat16(0.f);
+                unsigned char *dst = buf + WG_A;
+                *reinterpret_cast<uint4 *>(dst + swz_off(cl, 0)) =
+                    make_uint4(*reinterpret_cast<uint32_t *>(&hm), *reinterpret_cast<uint32_t *>(&lz), 0u, 0u);
+                *reinterpret_cast<uint4 *>(dst + swz_off(cl, 1)) = make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+        cp_async_commit();
+    };
+    float tot[9][NB][4], btot[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int p = 0; p < 9; p++)
+#pragma unroll
+        for (int n = 0; n < NB; n++)
+#pragma unroll
+            for (int e = 0; e < 4; e++) tot[p][n][e] = 0.f;
+    const uint32_t one2 = 0x3f803f80u;  // two bf16 ones: the bias sums g itself
+    int buf = 0;
+    if ((int)blockIdx.x < ntiles) stage(blockIdx.x, wg_smem);
+    for (int tb = blockIdx.x; tb < ntiles; tb += gridDim.x, buf ^= 1) {
+        if (tb + (int)gridDim.x < ntiles) {
+            stage(tb + gridDim.x, wg_smem + (buf ^ 1) * (WG_A + WG_G));
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
         }
         __syncthreads();
+        const uint32_t sa = (uint32_t)__cvta_generic_to_shared(wg_smem + buf * (WG_A + WG_G)), sg = sa + WG_A;
+        float acc[9][NB][4], bacc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int u = 0; u < (NOUT + 255) / 256; u++) {
-            const int o = tid + u * 256;
-            if (o >= NOUT) break;
-            const int tp = o % 27, ci = (o / 27) % CIN, co = o / (27 * CIN);
-            const int dz = tp / 9, dy = (tp / 3) % 3, dx = tp % 3;
-            float acc = 0.f;
-            for (int cl = 0; cl < NT_X * NT_Y; cl++) {
-                const float g = sg[cl][co];
-                const int cx = cl % NT_X, cy = cl / NT_X;
-                acc += g * sa[(dz * TYH + cy + dy) * TXH + cx + dx][ci];
+        for (int p = 0; p < 9; p++)
+#pragma unroll
+            for (int n = 0; n < NB; n++)
+#pragma unroll
+                for (int e = 0; e < 4; e++) acc[p][n][e] = 0.f;
+#pragma unroll 1
+        for (int ch = 0; ch < 4; ch++) {  // two rows of two groups of 16 cells
+            const int y = y0 + (ch >> 1), x = (ch & 1) * 16;
+            // g transposed: matrices (cells 0-7, channels 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15)
+            uint32_t g0, g1, g2, g3;
+            {
+                const int cl = y * NT_X + x + (lane & 7) + ((lane >> 4) << 3);
+                ldsm_x4_t(sg + swz_off(cl, (lane >> 3) & 1), g0, g1, g2, g3);
             }
-            part[u] += acc;
-        }
-        if (tid < COUT)
-            for (int cl = 0; cl < NT_X * NT_Y; cl++) bpart += sg[cl][tid];
-    }
+            if (dz == 0) mma_bf16(bacc, g0, g1, g2, g3, one2, one2);
 #pragma unroll
-    for (int u = 0; u < (NOUT + 255) / 256; u++) {
-        const int o = tid + u * 256;
-        if (o < NOUT) atomicAdd(gW + o, part[u]);
+            for (int p = 0; p < 9; p++) {
+                // a: matrices (cells 0-7, channels 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15)
+                const int cidx = (dz * TYH + y + p / 3) * TXH + x + p % 3 + (lane & 15);
+                uint32_t b0, b1, b2, b3;
+                ldsm_x4_t(sa + swz_off(cidx, lane >> 4), b0, b1, b2, b3);
+                mma_bf16(acc[p][0], g0, g1, g2, g3, b0, b1);
+                if (NB == 2) mma_bf16(acc[p][NB - 1], g0, g1, g2, g3, b2, b3);
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < 9; p++)
+#pragma unroll
+            for (int n = 0; n < NB; n++)
+#pragma unroll
+                for (int e = 0; e < 4; e++) tot[p][n][e] += acc[p][n][e];
+#pragma unroll
+        for (int e = 0; e < 4; e++) btot[e] += bacc[e];
+        __syncthreads();  // this buffer is staged again
     }
-    if (tid < COUT) atomicAdd(gB + tid, bpart);
+    // the four warps of a dz added in order, then one atomic per weight and block
+    constexpr int PER = 9 * NB * 4 + 4;
+    float *red = reinterpret_cast<float *>(wg_smem);  // [3 dz][PER][32]
+    for (int w = 0; w < 4; w++) {
+        if ((warp & 3) == w) {
+            float *r = red + (size_t)dz * PER * 32 + lane;
+#pragma unroll
+            for (int p = 0; p < 9; p++)
+#pragma unroll
+                for (int n = 0; n < NB; n++)
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        float &v = r[((p * NB + n) * 4 + e) * 32];
+                        v = w ? v + tot[p][n][e] : tot[p][n][e];
+                    }
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                float &v = r[(9 * NB * 4 + e) * 32];
+                v = w ? v + btot[e] : btot[e];
+            }
+        }
+        __syncthreads();
+    }
+    // accumulator element e of lane l: row l / 4 (+ 8 for e >= 2), column 2 (l % 4) + (e & 1)
+    auto sum_at = [&](int z, int slot, int row, int col) {
+        const int e = ((row >> 3) << 1) | (col & 1), l = (row & 7) * 4 + (col >> 1);
+        return red[((size_t)z * PER + slot * 4 + e) * 32 + l];
+    };
+    for (int o = tid; o < COUT * CIN * 27; o += WG_TH) {
+        const int tp = o % 27, ci = (o / 27) % CIN, co = o / (27 * CIN);
+        const int slot = (tp % 9) * NB + (ci >> 3);
+        float v = sum_at(tp / 9, slot, co, ci & 7);
+        if (GF32) v += sum_at(tp / 9, slot, 1, ci & 7) + sum_at(tp / 9, slot, 2, ci & 7);
+        atomicAdd(gW + o, v);
+    }
+    if (tid < COUT) {
+        float v = sum_at(0, 9 * NB, tid, 0);
+        if (GF32) v += sum_at(0, 9 * NB, 1, 0) + sum_at(0, 9 * NB, 2, 0);
+        atomicAdd(gB + tid, v);
+    }
 }
 
 // A parameter that does not depend on the residual: a bias, or a weight of the
@@ -828,9 +953,6 @@ static size_t conv_smem() { return (size_t)TCELLS * 32 + 27 * 16 * 32; }
 
 static int conv_tiles(const Layout &L) { return ((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) * L.nz; }
 
-template <int CIN, int COUT>
-static size_t wgrad_smem() { return ((size_t)NT_X * NT_Y * COUT + (size_t)TCELLS * CIN) * 4; }
-
 static int conv_tiles_tc(const Layout &L)
 {
     return ((L.nx + TC_M - 1) / TC_M) * ((L.ny + TC_NY - 1) / TC_NY) * L.nz;
@@ -892,11 +1014,11 @@ int net_alloc(fs_ctx *c, bool training)
         FS_CUDA(cudaFuncSetAttribute(k_conv_tc<IN_ACT, OUT_Z>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)TC_SMEM));
         FS_CUDA(cudaFuncSetAttribute(k_wgrad<16, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)wgrad_smem<16, 16>()));
+                                     (int)WG_SMEM));
         FS_CUDA(cudaFuncSetAttribute(k_wgrad<16, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)wgrad_smem<16, 1>()));
+                                     (int)WG_SMEM));
         FS_CUDA(cudaFuncSetAttribute(k_wgrad<2, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)wgrad_smem<2, 16>()));
+                                     (int)WG_SMEM));
         attr_done = true;
     }
     return FS_OK;
@@ -1159,8 +1281,8 @@ int net_grad(fs_ctx *c, const float *b, const float *q, double *loss)
         c->n_launches += 3;
     }
     // layer 5
-    const int wg = std::max(1, std::min(((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) * L.nz, c->num_sms * 2));
-    k_wgrad<16, 1, true><<<wg, 256, wgrad_smem<16, 1>(), c->stream>>>(n->gy, A[4], n->grad + OW5, n->grad + OB5, L);
+    const int wg = std::max(1, std::min(((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) * L.nz, c->num_sms));
+    k_wgrad<16, 1, true><<<wg, WG_TH, WG_SMEM, c->stream>>>(n->gy, A[4], n->grad + OW5, n->grad + OB5, L);
     __nv_bfloat16 *G[2] = {n->gact, n->gact + nC * 16};
     k_bwd_last<<<gb, 256, 0, c->stream>>>(n->gy, n->w5f, A[4], G[0], L);
     // layers 4, 3, 2: weight gradient, then the gradient of the layer input
@@ -1168,7 +1290,7 @@ int net_grad(fs_ctx *c, const float *b, const float *q, double *loss)
     int gi = 0;
     for (int l = 2; l >= 0; l--) {
         // G[gi] = dL/d(output of layer l+2) (post-ReLU mask applied); input = A[l+1]
-        k_wgrad<16, 16, false><<<wg, 256, wgrad_smem<16, 16>(), c->stream>>>(G[gi], A[l + 1], n->grad + woff[l], n->grad + boff[l], L);
+        k_wgrad<16, 16, false><<<wg, WG_TH, WG_SMEM, c->stream>>>(G[gi], A[l + 1], n->grad + woff[l], n->grad + boff[l], L);
         ConvArgs bw{};
         bw.in = G[gi];
         bw.wts = n->wt + (size_t)l * NWM;
@@ -1179,7 +1301,7 @@ int net_grad(fs_ctx *c, const float *b, const float *q, double *loss)
         gi ^= 1;
     }
     // layer 1: gradient w.r.t. W1 from the stored input x (2 channels used)
-    k_wgrad<2, 16, false><<<wg, 256, wgrad_smem<2, 16>(), c->stream>>>(G[gi], A[0], n->grad + OW1, n->grad + OB1, L);
+    k_wgrad<2, 16, false><<<wg, WG_TH, WG_SMEM, c->stream>>>(G[gi], A[0], n->grad + OW1, n->grad + OB1, L);
     c->n_launches += 2 + 6 + 1;
     FS_CUDA(cudaGetLastError());
     SolveScal h;
