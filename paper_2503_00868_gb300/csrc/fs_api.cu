@@ -358,7 +358,7 @@ int fs_init_grid(fs_ctx **out, int nx, int ny, int nz, const fs_params *p, void 
     ALLOC(c->partials, (size_t)red_blocks * 8 * sizeof(double));
     ALLOC(c->err_word, 16);
 #undef ALLOC
-    if (cudaHostAlloc((void **)&c->scal_host, 4 * sizeof(SolveScal), cudaHostAllocDefault) != cudaSuccess) {
+    if (cudaHostAlloc((void **)&c->scal_host, 5 * sizeof(SolveScal), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
         c->scal_host = nullptr;
         free_ctx(c);

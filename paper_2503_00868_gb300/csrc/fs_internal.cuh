@@ -162,7 +162,7 @@ struct fs_ctx {
 
     // reductions
     fs::SolveScal *scal;        // device [4]: 0 pressure, 1 viscosity, 2 misc, 3 misc
-    fs::SolveScal *scal_host;   // pinned mirror
+    fs::SolveScal *scal_host;   // pinned mirror [4], then the error word
     double *partials;           // device [max_blocks * 8]
     int max_blocks;
     unsigned *err_word;         // device error word of bounded waits
@@ -445,6 +445,8 @@ __device__ __forceinline__ bool grid_reduce(KSum (&v)[K], double *partials, unsi
 int build_mask(fs_ctx *c, const uint8_t *types_dense, const fs_mac *bc);
 TileMap make_tilemap(const Layout &L, int nvol, int num_sms);
 int make_tensor_maps(fs_ctx *c);   // fs_mask.cu, once per context
+// fs_mask.cu: 16-channel bf16 cells (cell space) as a 4-D tensor, boxes of bx x by x bz cells, 32-byte swizzle
+int encode_cells16(CUtensorMap *m, const void *cells, const Layout &L, int bx, int by, int bz);
 int zmarch_slots(const fs_ctx *c, bool face);  // fs_pcg.cu: resident blocks of the operator apply
 // fs_pcg.cu
 int solve_pressure(fs_ctx *c, fs_stats *st);             // pb -> px
@@ -512,7 +514,8 @@ bool net_loaded(const fs_ctx *c);
 int cell_in(fs_ctx *c, const float *src, float *dst);
 int cell_out(fs_ctx *c, const float *src, float *dst);  // cell space -> public cell array
 
-int read_scal(fs_ctx *c, int which, SolveScal *out);
+// scalars of a slot (and, with err, the error word of bounded waits), after the stream's work
+int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err = nullptr);
 // mean-free preconditioned residual over the liquid when the operator is singular
 int remove_null_mode(fs_ctx *c, float *z);
 // fs_fcg.cu: flexible CG with the network, pb -> px (warm: from the current x);

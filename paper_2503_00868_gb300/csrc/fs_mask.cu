@@ -224,6 +224,23 @@ static int encode_map(CUtensorMap *m, float *base, const Layout &L, long long le
     return FS_OK;
 }
 
+// x, y, z run over the grid's cells only, so that a box reads zeros off the grid.
+int encode_cells16(CUtensorMap *m, const void *cells, const Layout &L, int bx, int by, int bz)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    if (!enc) return set_error(FS_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    const cuuint64_t dims[4] = {16, (cuuint64_t)L.nx, (cuuint64_t)L.ny, (cuuint64_t)L.nz};
+    const cuuint64_t strides[3] = {32, (cuuint64_t)L.P * 32, (cuuint64_t)L.PL * 32};
+    const cuuint32_t box[4] = {16, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    uint8_t *origin = static_cast<uint8_t *>(const_cast<void *>(cells)) + (size_t)L.PL * 32;  // cell (0, 0, 0)
+    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, origin, dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return set_error(FS_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+    return FS_OK;
+}
+
 int make_tensor_maps(fs_ctx *c)
 {
     const Layout &L = c->L;

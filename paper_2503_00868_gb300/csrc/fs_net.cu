@@ -10,17 +10,17 @@
 // activation is stored as bf16, every sum accumulates in FP32.
 //
 // Kernels:
-//   k_conv<IN, OUT>  every layer as an implicit GEMM per 3x3x3 tap on the tensor
-//                  cores (mma.sync m16n8k16 bf16 x bf16 -> f32, operands via
-//                  ldmatrix from a swizzled shared-memory tile); layer 1 builds
-//                  its (r/s, cell type) input tile on the fly with the weights
-//                  zero-padded to 16 input channels, layer 5 uses one 8-wide
-//                  n-tile and writes z = s y on liquid cells; the same kernel
-//                  runs the backward-data pass of layers 2-4 with flipped,
-//                  transposed weights and a ReLU-derivative epilogue. For
-//                  inference layer l visits only the conv tiles within 5 - l
-//                  cells of the liquid (the output on liquid cells depends on
-//                  nothing farther), from a tile list sorted by that distance;
+//   k_conv<OUT>    layers 2-5, layer 1 of training and the backward-data pass of
+//                  layers 2-4 (flipped, transposed weights, ReLU-derivative
+//                  epilogue) as an implicit GEMM per 3x3x3 tap on the tensor cores
+//                  (mma.sync m16n8k16 bf16 x bf16 -> f32), tiles by tensor copy,
+//                  weights in registers; layer 5 uses one 8-wide n-tile and writes
+//                  z = s y on liquid cells. For inference layer l visits only the
+//                  tiles within 5 - l cells of the liquid (the output on liquid
+//                  cells depends on nothing farther), from a list sorted by that
+//                  distance;
+//   k_conv1        layer 1 of inference from r itself, three taps per MMA;
+//   k_conv_tc      the inference layers on tcgen05 (fs_net_kernel);
 //   k_bwd_last     gradient through layer 5 to its input;
 //   k_wgrad<CIN,COUT>  weight and bias gradients as contractions over the cells on
 //                  the tensor cores (per-block sums, one atomicAdd per weight per
@@ -57,8 +57,8 @@ struct NetState {
     __nv_bfloat16 *wf;    // layers 2-4 forward: [3][27 tap][16 co][16 ci]
     __nv_bfloat16 *wf1;   // layer 1 forward: [27 tap][16 co][16 ci], ci >= 2 zero
     __nv_bfloat16 *wf5;   // layer 5 forward: [27 tap][16 co][16 ci], co >= 1 zero
-    int *tlist;           // conv tiles sorted by distance to the liquid (0 .. 5 = farther)
-    uint8_t *tdist;       // per conv tile: Chebyshev distance to the nearest liquid cell, capped at 5
+    int *tlist;           // 32 x 8 x 4 tiles sorted by distance to the liquid (0 .. 5 = farther)
+    uint8_t *tdist;       // per 32 x 8 x 1 tile: Chebyshev distance to the nearest liquid cell, capped at 5
     int tcount[6];        // tiles within distance d of the liquid
     int *tlist_tc;        // tiles of the tensor-core layer (TC_M x TC_NY of one plane), sorted the same way
     int tcount_tc[6];
@@ -91,7 +91,7 @@ __device__ __forceinline__ float type_code(uint8_t f) { return (f & CF_LIQ) ? 1.
 
 __device__ __forceinline__ float bfr(float x) { return __bfloat162float(__float2bfloat16(x)); }
 
-// ---- layers 2-4 (16 -> 16), tensor cores ------------------------------------------
+// ---- the shared tile of the weight gradients -----------------------------------------
 // Shared tile: 3 planes x (NT_Y + 2) rows x (NT_X + 2) cells x 16 bf16. The two
 // 16-byte halves of a cell are swapped when bit 2 of its tile index is set, so
 // the 8 rows of an ldmatrix phase fall in distinct banks.
@@ -119,8 +119,9 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-enum : int { IN_ACT = 0, IN_R = 1 };                  // input: bf16 activations / built from r
+enum : int { IN_ACT = 0, IN_R = 1 };                  // input (tcgen05 layers): bf16 activations / built from r
 enum : int { OUT_RELU = 0, OUT_BWD = 1, OUT_Z = 2 };  // epilogue
+constexpr unsigned ERR_NET = 8u;  // error word: a bounded wait of a network kernel ran out
 
 struct ConvArgs {
     const __nv_bfloat16 *in;    // IN_ACT: [cell][16]
@@ -131,129 +132,397 @@ struct ConvArgs {
     const float *bias;          // OUT_RELU: [16]; OUT_Z: [1]
     const __nv_bfloat16 *aref;  // OUT_BWD: the layer input whose ReLU derivative masks
     __nv_bfloat16 *out;         // OUT_RELU, OUT_BWD: [cell][16]
-    __nv_bfloat16 *xin;         // IN_R (optional): the bf16 input, channels 0 and 1
     float *y, *z;               // OUT_Z (each optional): network output; z = s y on liquid, else 0
     const int *tiles;           // optional list of conv tiles (else every tile)
     int ntiles;                 // entries of `tiles`
     Layout L;
 };
 
-// IN_ACT/OUT_RELU: out = relu(conv(in) + bias). OUT_BWD (backward data):
-// out = conv(in) * [aref > 0]. OUT_Z: y = conv(in) + bias, z = s y on liquid
-// cells. IN_R: the input is (bf16(r/s) on liquid, cell-type code), channels 2-15
-// zero. Outputs only on grid cells.
-template <int IN, int OUT>
-__global__ void __launch_bounds__(256) k_conv(ConvArgs a)
+// ---- layers 2-5 and the backward-data pass -----------------------------------------
+// OUT_RELU: out = relu(conv(in) + bias). OUT_BWD (backward data): out = conv(in) *
+// [aref > 0]. OUT_Z: y = conv(in) + bias, z = s y on liquid cells. Outputs only on
+// grid cells.
+//
+// A block computes 32 x 8 x 4 cells, a warp 16 x 8 cells of one plane: 8 M-tiles of
+// 16 cells, one per row, whose sums it holds in registers with the weights of all 27
+// taps (108 registers). An input row of a plane is read once per x shift and serves
+// the three output rows it touches, so a warp issues 90 ldmatrix for 432 MMAs; with
+// one row per warp and the weights read beside the cells it was 108 for 108, and
+// shared-memory bandwidth bound the layer (264 us on a union of spheres at 256^3; now
+// 154, with the MMA pipe near its rate, and the last layer 89 from 240). Per
+// output the taps are summed in the order dz, dy, dx, one MMA each, as before. The
+// next tile comes by one tensor copy (zeros off the grid) while this one is worked
+// on: with 2 warps per scheduler, cp.async and its index arithmetic in the computing
+// warps left the MMA pipe idle half the time. The copy's 32-byte swizzle swaps the
+// two halves of a cell when bit 2 of its index is set, so that the 8 rows of an
+// ldmatrix phase fall in distinct banks; rows are 36 cells apart, so the swap flips
+// with the row's parity. Output channels are dealt to the MMA columns so that a lane
+// holds four neighbouring ones and stores 8 bytes.
+constexpr int CV_Z = 4, CV_P = 36, CV_PL = CV_P * TYH, CV_CELLS = CV_PL * (CV_Z + 2);
+constexpr int CV_BUF = CV_CELLS * 32;                    // bytes of a tile, a multiple of 256
+constexpr size_t CV_SMEM = 1024 + 2 * (size_t)CV_BUF;
+constexpr unsigned CV_SPIN = 1u << 24;                   // try_wait rounds before a wait gives up
+static_assert(CV_P >= TXH && CV_P % 4 == 0 && CV_PL % 8 == 0 && CV_BUF % 256 == 0, "the swizzle of the tile");
+
+// 32 x 8 x 4 tiles of the grid: index (kz * nty + ty) * ntx + tx
+__device__ __forceinline__ void conv_tile(int tb, const Layout &L, int &i0, int &j0, int &k0)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char *tile = smem;                          // TCELLS * 32 bytes
-    unsigned char *wsm = smem + TCELLS * 32;             // 27 * 16 rows * 32 bytes
+    const int ntx = (L.nx + NT_X - 1) / NT_X, nty = (L.ny + NT_Y - 1) / NT_Y;
+    i0 = (tb % ntx) * NT_X;
+    j0 = ((tb / ntx) % nty) * NT_Y;
+    k0 = tb / (ntx * nty) * CV_Z;
+}
+
+// 16 bytes from global to shared memory, or zeros
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// an mbarrier's phase, waited for within a bound
+__device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        " .reg .pred p;\n"
+        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity)
+{
+    for (unsigned n = 0; n < CV_SPIN; n++)
+        if (bar_try_wait(bar, parity)) return true;
+    return false;
+}
+__device__ __forceinline__ void bar_init(uint32_t bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(1) : "memory");
+}
+
+// a box of cells (16 channels, from cell (x, y, z)) global -> shared, completing on `bar`
+__device__ __forceinline__ void tma_cells(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar,
+                                          uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+        "[%6];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+// the output channel of MMA column n (0 .. 15, two n-tiles of 8)
+__device__ __forceinline__ int conv_channel(int n) { return 4 * ((n & 7) >> 1) + (n & 1) + 2 * (n >> 3); }
+
+template <int OUT>
+__global__ void __launch_bounds__(256, 1) k_conv(const __grid_constant__ CUtensorMap map,
+                                                 const __grid_constant__ ConvArgs a, unsigned *err)
+{
+    constexpr int NT = OUT == OUT_Z ? 1 : 2;  // n-tiles of 8 output channels
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ __align__(8) uint64_t mbar[2];
     const Layout &L = a.L;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // weights once per block (rows n = tap * 16 + co, swizzled like the tile)
-    for (int e = tid; e < 27 * 16 * 2; e += blockDim.x) {
-        const int row = e >> 1, half = e & 1;
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(a.wts) + row * 2 + half);
-        *reinterpret_cast<uint4 *>(wsm + swz_off(row, half)) = v;
+    const int xh = (warp & 1) * 16, pz = warp >> 1;
+    const uint32_t sm = ((uint32_t)__cvta_generic_to_shared(smem) + 1023u) & ~1023u;
+    const uint32_t bar[2] = {(uint32_t)__cvta_generic_to_shared(mbar), (uint32_t)__cvta_generic_to_shared(mbar + 1)};
+    const int total = a.tiles ? a.ntiles : ((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) *
+                                               ((L.nz + CV_Z - 1) / CV_Z);
+    auto tile_at = [&](int idx) { return a.tiles ? __ldg(a.tiles + idx) : idx; };
+    auto stage = [&](int idx, int buf) {
+        int i0, j0, k0;
+        conv_tile(tile_at(idx), L, i0, j0, k0);
+        tma_cells(sm + buf * CV_BUF, &map, i0 - 1, j0 - 1, k0 - 1, bar[buf], CV_BUF);
+    };
+    if (tid == 0) {
+        bar_init(bar[0]);
+        bar_init(bar[1]);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if ((int)blockIdx.x < total) stage(blockIdx.x, 0);
     }
-    float bv[4] = {0.f, 0.f, 0.f, 0.f};  // bias of this lane's output channels
+    uint32_t wreg[27][NT][2];  // lane's B fragments: input channels 2 (lane % 4) + {0, 1} (+ 8) of column lane / 4
+#pragma unroll
+    for (int tp = 0; tp < 27; tp++)
+#pragma unroll
+        for (int n = 0; n < NT; n++) {
+            const int co = OUT == OUT_Z ? lane >> 2 : conv_channel(8 * n + (lane >> 2));
+            const __nv_bfloat16 *w = a.wts + (tp * 16 + co) * 16 + 2 * (lane & 3);
+            wreg[tp][n][0] = __ldg(reinterpret_cast<const uint32_t *>(w));
+            wreg[tp][n][1] = __ldg(reinterpret_cast<const uint32_t *>(w + 8));
+        }
+    float bv[4] = {0.f, 0.f, 0.f, 0.f};  // bias of the lane's four channels
     if (OUT == OUT_RELU) {
-        const int co = (lane & 3) * 2;
-        bv[0] = a.bias[co];
-        bv[1] = a.bias[co + 1];
-        bv[2] = a.bias[8 + co];
-        bv[3] = a.bias[8 + co + 1];
+#pragma unroll
+        for (int e = 0; e < 4; e++) bv[e] = a.bias[4 * (lane & 3) + e];
     } else if (OUT == OUT_Z) {
         bv[0] = a.bias[0];
     }
-    float sc = 1.f, inv = 0.f;
-    if (IN == IN_R || OUT == OUT_Z) {
-        sc = __uint_as_float(*a.smax);
-        inv = sc > 0.f ? 1.f / sc : 0.f;
-    }
-    const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
-    const uint32_t w_s = (uint32_t)__cvta_generic_to_shared(wsm);
-    const int ntx = (L.nx + NT_X - 1) / NT_X, nty = (L.ny + NT_Y - 1) / NT_Y;
-    const int total = a.tiles ? a.ntiles : ntx * nty * L.nz;
-    for (int idx = blockIdx.x; idx < total; idx += gridDim.x) {
-        const int tb = a.tiles ? __ldg(a.tiles + idx) : idx;
-        const int tx = tb % ntx, ty = (tb / ntx) % nty, tk = tb / (ntx * nty);
-        const int i0 = tx * NT_X, j0 = ty * NT_Y;
-        __syncthreads();  // previous tile done with the shared tile (and weights stored)
-        for (int e = tid; e < TCELLS * 2; e += blockDim.x) {
-            const int cidx = e >> 1, half = e & 1;
-            const int xx = cidx % TXH, yy = (cidx / TXH) % TYH, zz = cidx / (TXH * TYH);
-            const int gi = i0 - 1 + xx, gj = j0 - 1 + yy, gk = tk - 1 + zz;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (in_grid(L, gi, gj, gk)) {
-                const int t = cell_t(L, gi, gj, gk);
-                if (IN == IN_ACT) {
-                    v = __ldg(reinterpret_cast<const uint4 *>(a.in + (size_t)t * 16) + half);
-                } else if (half == 0) {
-                    const uint8_t f = a.cf[t];
-                    const __nv_bfloat162 x = __floats2bfloat162_rn((f & CF_LIQ) ? a.r[t] * inv : 0.f, type_code(f));
-                    v.x = *reinterpret_cast<const uint32_t *>(&x);
+    const float sc = OUT == OUT_Z ? __uint_as_float(*a.smax) : 1.f;
+    // the lane's ldmatrix row for each x shift (rows of odd index have the halves swapped)
+    uint32_t off[3];
+#pragma unroll
+    for (int dx = 0; dx < 3; dx++) off[dx] = swz_off(pz * CV_PL + xh + dx + (lane & 15), lane >> 4);
+    __syncthreads();
+    int buf = 0;
+    uint32_t phase = 0;  // bit b: parity of buffer b's next phase
+    for (int idx = blockIdx.x; idx < total; idx += gridDim.x, buf ^= 1) {
+        if (tid == 0 && idx + (int)gridDim.x < total) stage(idx + gridDim.x, buf ^ 1);
+        int i0, j0, k0;
+        conv_tile(tile_at(idx), L, i0, j0, k0);
+        const bool ok = bar_wait(bar[buf], (phase >> buf) & 1u);
+        phase ^= 1u << buf;
+        if (__syncthreads_or(!ok)) {  // a copy that never came: note it, wait (bounded) for the one in flight, leave
+            if (tid == 0) {
+                atomicOr(err, ERR_NET);
+                if (idx + (int)gridDim.x < total) bar_wait(bar[buf ^ 1], (phase >> (buf ^ 1)) & 1u);
+            }
+            __syncthreads();
+            break;
+        }
+        const int gk = k0 + pz;
+        if (gk < L.nz) {
+            float acc[NT_Y][NT][4];
+#pragma unroll
+            for (int y = 0; y < NT_Y; y++)
+#pragma unroll
+                for (int n = 0; n < NT; n++)
+#pragma unroll
+                    for (int e = 0; e < 4; e++) acc[y][n][e] = 0.f;
+            const uint32_t base = sm + buf * CV_BUF;
+#pragma unroll
+            for (int dz = 0; dz < 3; dz++)
+#pragma unroll
+                for (int r = 0; r < TYH; r++)
+#pragma unroll
+                    for (int dx = 0; dx < 3; dx++) {
+                        uint32_t a0, a1, a2, a3;
+                        ldsm_x4(base + (off[dx] ^ ((r & 1) << 4)) + (dz * CV_PL + r * CV_P) * 32, a0, a1, a2, a3);
+#pragma unroll
+                        for (int dy = 2; dy >= 0; dy--) {
+                            const int y = r - dy, tp = dz * 9 + dy * 3 + dx;
+                            if (y < 0 || y >= NT_Y) continue;
+#pragma unroll
+                            for (int n = 0; n < NT; n++)
+                                mma_bf16(acc[y][n], a0, a1, a2, a3, wreg[tp][n][0], wreg[tp][n][1]);
+                        }
+                    }
+            // cells lane / 4 (accumulators 0, 1) and lane / 4 + 8 (2, 3) of each row
+            const int gi = i0 + xh + (lane >> 2);
+            const size_t t0 = (size_t)cell_t(L, gi, j0, gk);
+            if (OUT == OUT_Z) {
+                // column 0 sits in one lane of four; the four share the rows (their flags are read at once)
+                const int c = lane & 3;
+                float y4[2][2];
+                uint8_t f4[2][2];
+#pragma unroll
+                for (int q = 0; q < 2; q++)
+#pragma unroll
+                    for (int hr = 0; hr < 2; hr++) {
+                        float v = 0.f;
+#pragma unroll
+                        for (int e = 0; e < 4; e++) {
+                            const float w = __shfl_sync(0xffffffffu, acc[4 * q + e][0][hr * 2], lane & ~3);
+                            if (e == c) v = w;
+                        }
+                        y4[q][hr] = v + bv[0];
+                        const int y = 4 * q + c;
+                        f4[q][hr] = gi + hr * 8 < L.nx && j0 + y < L.ny ? __ldg(a.cf + t0 + y * L.P + hr * 8) : 0;
+                    }
+#pragma unroll
+                for (int q = 0; q < 2; q++)
+#pragma unroll
+                    for (int hr = 0; hr < 2; hr++) {
+                        const int y = 4 * q + c;
+                        if (gi + hr * 8 >= L.nx || j0 + y >= L.ny) continue;
+                        const size_t t = t0 + y * L.P + hr * 8;
+                        if (a.y) a.y[t] = y4[q][hr];
+                        if (a.z) a.z[t] = (f4[q][hr] & CF_LIQ) ? sc * y4[q][hr] : 0.f;
+                    }
+            } else {
+#pragma unroll
+                for (int y2 = 0; y2 < NT_Y; y2 += 2) {
+                    uint2 m[2][2];
+                    if (OUT == OUT_BWD) {  // four rows' masks in flight before the first store
+#pragma unroll
+                        for (int y = 0; y < 2; y++)
+#pragma unroll
+                            for (int hr = 0; hr < 2; hr++)
+                                m[y][hr] = gi + hr * 8 < L.nx && j0 + y2 + y < L.ny
+                                               ? __ldg(reinterpret_cast<const uint2 *>(
+                                                     a.aref + (t0 + (y2 + y) * L.P + hr * 8) * 16 + 4 * (lane & 3)))
+                                               : make_uint2(0u, 0u);
+                    }
+#pragma unroll
+                    for (int yy = 0; yy < 2; yy++)
+#pragma unroll
+                        for (int hr = 0; hr < 2; hr++) {
+                            const int y = y2 + yy;
+                            if (gi + hr * 8 >= L.nx || j0 + y >= L.ny) continue;
+                            float v[4] = {acc[y][0][hr * 2], acc[y][0][hr * 2 + 1], acc[y][NT - 1][hr * 2],
+                                          acc[y][NT - 1][hr * 2 + 1]};
+                            if (OUT == OUT_RELU) {
+#pragma unroll
+                                for (int e = 0; e < 4; e++) v[e] = fmaxf(v[e] + bv[e], 0.f);
+                            } else {
+                                const __nv_bfloat162 m0 = *reinterpret_cast<const __nv_bfloat162 *>(&m[yy][hr].x);
+                                const __nv_bfloat162 m1 = *reinterpret_cast<const __nv_bfloat162 *>(&m[yy][hr].y);
+                                v[0] = __bfloat162float(m0.x) > 0.f ? v[0] : 0.f;
+                                v[1] = __bfloat162float(m0.y) > 0.f ? v[1] : 0.f;
+                                v[2] = __bfloat162float(m1.x) > 0.f ? v[2] : 0.f;
+                                v[3] = __bfloat162float(m1.y) > 0.f ? v[3] : 0.f;
+                            }
+                            const __nv_bfloat162 o0 = __floats2bfloat162_rn(v[0], v[1]);
+                            const __nv_bfloat162 o1 = __floats2bfloat162_rn(v[2], v[3]);
+                            *reinterpret_cast<uint2 *>(a.out + (t0 + y * L.P + hr * 8) * 16 + 4 * (lane & 3)) =
+                                make_uint2(*reinterpret_cast<const uint32_t *>(&o0),
+                                           *reinterpret_cast<const uint32_t *>(&o1));
+                        }
                 }
             }
-            *reinterpret_cast<uint4 *>(tile + swz_off(cidx, half)) = v;
+        }
+        __syncthreads();  // this buffer is copied into again
+    }
+}
+
+// ---- layer 1 of inference ------------------------------------------------------------
+// The input (bf16(r / s) on liquid, cell-type code) is one 32-bit word per cell, and a
+// row of three taps along x is one m16n8k8 MMA: k = 2 dx + channel, so lane l of an A
+// fragment reads the word of the cell l % 4 to the right of its row's first tap (the
+// fourth has weight zero). 9 MMAs pairs per 16 cells in place of 27 of K = 16 on
+// channels padded from 2 to 16 (319 us on a union of spheres at 256^3, most of it the
+// padded tile; now 85, bound by its loads and the 32 bytes it writes per cell).
+__device__ __forceinline__ void mma_bf16_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0)
+{
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(b0));
+}
+
+// the input word of a cell of flags f and right-hand side r
+__device__ __forceinline__ uint32_t net_input(float r, uint8_t f, float inv)
+{
+    const __nv_bfloat162 x = __floats2bfloat162_rn((f & CF_LIQ) ? r * inv : 0.f, type_code(f));
+    return *reinterpret_cast<const uint32_t *>(&x);
+}
+
+__global__ void __launch_bounds__(256, 2) k_conv1(const __grid_constant__ ConvArgs a)
+{
+    __shared__ uint32_t sx[CV_CELLS];
+    const Layout &L = a.L;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int xh = (warp & 1) * 16, pz = warp >> 1;
+    uint32_t wreg[9][2];
+#pragma unroll
+    for (int q = 0; q < 9; q++)
+#pragma unroll
+        for (int n = 0; n < 2; n++)
+            wreg[q][n] = (lane & 3) == 3 ? 0u
+                                         : __ldg(reinterpret_cast<const uint32_t *>(
+                                               a.wts + ((q * 3 + (lane & 3)) * 16 + conv_channel(8 * n + (lane >> 2))) * 16));
+    float bv[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) bv[e] = a.bias[4 * (lane & 3) + e];
+    const float sc = __uint_as_float(*a.smax);
+    const float inv = sc > 0.f ? 1.f / sc : 0.f;
+    for (int e = tid; e < CV_CELLS; e += 256) sx[e] = 0u;  // the padding of the rows stays zero
+    // the next tile's cells are read into registers while this tile is worked on
+    constexpr int PER = ((CV_Z + 2) * TYH * TXH + 255) / 256;
+    float rv[PER];
+    uint8_t fv[PER];
+    auto fetch = [&](int idx) {
+        int i0, j0, k0;
+        conv_tile(__ldg(a.tiles + idx), L, i0, j0, k0);
+#pragma unroll
+        for (int q = 0; q < PER; q++) {
+            const int e = tid + q * 256;
+            const int xx = e % TXH, yy = (e / TXH) % TYH, zz = e / (TXH * TYH);
+            const int gi = i0 - 1 + xx, gj = j0 - 1 + yy, gk = k0 - 1 + zz;
+            const bool in = zz < CV_Z + 2 && in_grid(L, gi, gj, gk);
+            const int t = in ? cell_t(L, gi, gj, gk) : 0;
+            fv[q] = in ? __ldg(a.cf + t) : 0xff;
+            rv[q] = in ? __ldg(a.r + t) : 0.f;
+        }
+    };
+    if ((int)blockIdx.x < a.ntiles) fetch(blockIdx.x);
+    for (int idx = blockIdx.x; idx < a.ntiles; idx += gridDim.x) {
+        int i0, j0, k0;
+        conv_tile(__ldg(a.tiles + idx), L, i0, j0, k0);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < PER; q++) {
+            const int e = tid + q * 256;
+            if (e < (CV_Z + 2) * TYH * TXH) {
+                const int xx = e % TXH, yy = (e / TXH) % TYH, zz = e / (TXH * TYH);
+                sx[zz * CV_PL + yy * CV_P + xx] = fv[q] == 0xff ? 0u : net_input(rv[q], fv[q], inv);
+            }
         }
         __syncthreads();
-        // warp w: row y = w of the tile, two M-tiles of 16 cells (x 0-15, 16-31)
-        for (int mt = 0; mt < 2; mt++) {
-            float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
-            const int row = lane & 15, khalf = lane >> 4;
-            for (int dz = 0; dz < 3; dz++)
-                for (int dy = 0; dy < 3; dy++)
-                    for (int dx = 0; dx < 3; dx++) {
-                        const int cidx = (dz * TYH + warp + dy) * TXH + mt * 16 + dx + row;
-                        uint32_t a0, a1, a2, a3;
-                        ldsm_x4(tile_s + swz_off(cidx, khalf), a0, a1, a2, a3);
-                        const int tp = dz * 9 + dy * 3 + dx;
-                        const int wrow = tp * 16 + (lane & 7) + ((lane >> 4) << 3);
-                        const int wh = (lane >> 3) & 1;
-                        uint32_t b0, b1, b2, b3;
-                        ldsm_x4(w_s + swz_off(wrow, wh), b0, b1, b2, b3);
-                        mma_bf16(acc0, a0, a1, a2, a3, b0, b1);
-                        if (OUT != OUT_Z) mma_bf16(acc1, a0, a1, a2, a3, b2, b3);
-                    }
-            // epilogue: cells (lane/4) and (lane/4 + 8); channels (lane%4)*2 (+1), +8
-            const int gj = j0 + warp;
+        if (idx + (int)gridDim.x < a.ntiles) fetch(idx + gridDim.x);
+        const int gk = k0 + pz;
+        if (gk >= L.nz) continue;
+        float acc[NT_Y][2][4];
+#pragma unroll
+        for (int y = 0; y < NT_Y; y++)
+#pragma unroll
+            for (int n = 0; n < 2; n++)
+#pragma unroll
+                for (int e = 0; e < 4; e++) acc[y][n][e] = 0.f;
+        const uint32_t *row0 = sx + pz * CV_PL + xh + (lane >> 2) + (lane & 3);
+#pragma unroll
+        for (int dz = 0; dz < 3; dz++)
+#pragma unroll
+            for (int r = 0; r < TYH; r++) {
+                const uint32_t a0 = row0[dz * CV_PL + r * CV_P], a1 = row0[dz * CV_PL + r * CV_P + 8];
+#pragma unroll
+                for (int dy = 2; dy >= 0; dy--) {
+                    const int y = r - dy;
+                    if (y < 0 || y >= NT_Y) continue;
+#pragma unroll
+                    for (int n = 0; n < 2; n++) mma_bf16_k8(acc[y][n], a0, a1, wreg[dz * 3 + dy][n]);
+                }
+            }
+#pragma unroll
+        for (int y = 0; y < NT_Y; y++) {
+            const int gj = j0 + y;
+#pragma unroll
             for (int hr = 0; hr < 2; hr++) {
-                const int gi = i0 + mt * 16 + (lane >> 2) + hr * 8;
+                const int gi = i0 + xh + (lane >> 2) + hr * 8;
                 if (gi >= L.nx || gj >= L.ny) continue;
-                const size_t t = (size_t)cell_t(L, gi, gj, tk);
-                const int co = (lane & 3) * 2;
-                if (OUT == OUT_Z) {
-                    if (co == 0) {
-                        const float yv = acc0[hr * 2] + bv[0];
-                        if (a.y) a.y[t] = yv;
-                        if (a.z) a.z[t] = (a.cf[t] & CF_LIQ) ? sc * yv : 0.f;
-                    }
-                    continue;
-                }
-                if (IN == IN_R && a.xin && co == 0) {
-                    const uint8_t f = a.cf[t];
-                    *reinterpret_cast<__nv_bfloat162 *>(a.xin + t * 16) =
-                        __floats2bfloat162_rn((f & CF_LIQ) ? a.r[t] * inv : 0.f, type_code(f));
-                }
-                float v0 = acc0[hr * 2], v1 = acc0[hr * 2 + 1], v2 = acc1[hr * 2], v3 = acc1[hr * 2 + 1];
-                if (OUT == OUT_RELU) {
-                    v0 = fmaxf(v0 + bv[0], 0.f);
-                    v1 = fmaxf(v1 + bv[1], 0.f);
-                    v2 = fmaxf(v2 + bv[2], 0.f);
-                    v3 = fmaxf(v3 + bv[3], 0.f);
-                } else {
-                    const __nv_bfloat162 r0 = *reinterpret_cast<const __nv_bfloat162 *>(a.aref + t * 16 + co);
-                    const __nv_bfloat162 r1 = *reinterpret_cast<const __nv_bfloat162 *>(a.aref + t * 16 + 8 + co);
-                    v0 = __bfloat162float(r0.x) > 0.f ? v0 : 0.f;
-                    v1 = __bfloat162float(r0.y) > 0.f ? v1 : 0.f;
-                    v2 = __bfloat162float(r1.x) > 0.f ? v2 : 0.f;
-                    v3 = __bfloat162float(r1.y) > 0.f ? v3 : 0.f;
-                }
-                *reinterpret_cast<__nv_bfloat162 *>(a.out + t * 16 + co) = __floats2bfloat162_rn(v0, v1);
-                *reinterpret_cast<__nv_bfloat162 *>(a.out + t * 16 + 8 + co) = __floats2bfloat162_rn(v2, v3);
+                const __nv_bfloat162 o0 = __floats2bfloat162_rn(fmaxf(acc[y][0][hr * 2] + bv[0], 0.f),
+                                                                fmaxf(acc[y][0][hr * 2 + 1] + bv[1], 0.f));
+                const __nv_bfloat162 o1 = __floats2bfloat162_rn(fmaxf(acc[y][1][hr * 2] + bv[2], 0.f),
+                                                                fmaxf(acc[y][1][hr * 2 + 1] + bv[3], 0.f));
+                *reinterpret_cast<uint2 *>(a.out + (size_t)cell_t(L, gi, gj, gk) * 16 + 4 * (lane & 3)) =
+                    make_uint2(*reinterpret_cast<const uint32_t *>(&o0), *reinterpret_cast<const uint32_t *>(&o1));
             }
         }
+    }
+}
+
+// The network's input on every grid cell, 16 channels (training: layer 1 then runs as
+// the others do, and its weight gradient reads it).
+__global__ void k_net_x(const float *__restrict__ r, const uint8_t *__restrict__ cf, const unsigned *smax, Layout L,
+                        __nv_bfloat16 *x)
+{
+    const float sc = __uint_as_float(*smax);
+    const float inv = sc > 0.f ? 1.f / sc : 0.f;
+    for (int t = L.PL + blockIdx.x * blockDim.x + threadIdx.x; t < L.PL + L.S; t += gridDim.x * blockDim.x) {
+        uint4 *o = reinterpret_cast<uint4 *>(x + (size_t)t * 16);
+        o[0] = make_uint4(net_input(r[t], cf[t], inv), 0u, 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -281,7 +550,6 @@ constexpr int TC_A_BYTES = 3 * TC_ROWS * TC_ROWB;            // 49920 per buffer
 constexpr int TC_B_BYTES = 27 * 512;                         // 13824
 constexpr size_t TC_SMEM = 128 + 2 * (size_t)TC_A_BYTES + TC_B_BYTES;
 constexpr unsigned TC_SPIN = 1u << 24;
-constexpr unsigned ERR_TC = 8u;
 static_assert(TC_THREADS == 2 * TC_M, "one thread per accumulator row lane in the epilogue");
 
 __device__ __forceinline__ uint32_t tc_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -460,7 +728,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(ConvArgs a, unsigned *er
         bool ok = false;
         for (unsigned n = 0; n < TC_SPIN && !ok; n++) ok = tc_try_wait(bar_u, phase);
         if (!ok) {
-            if (lane == 0) atomicOr(err, ERR_TC);
+            if (lane == 0) atomicOr(err, ERR_NET);
             stop = 1;
         }
         phase ^= 1u;
@@ -722,18 +990,6 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t 
                  : "r"(addr));
 }
 
-// 16 bytes from global to shared memory, or zeros
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 template <int CIN, int COUT, bool GF32>
 __global__ void __launch_bounds__(WG_TH, 1) k_wgrad(const void *__restrict__ gptr, const __nv_bfloat16 *__restrict__ a,
                                                     float *gW, float *gB, Layout L)
@@ -949,9 +1205,12 @@ __global__ void k_fill_zero(float *p, int n)
 
 static NetState *net(fs_ctx *c) { return static_cast<NetState *>(c->net); }
 
-static size_t conv_smem() { return (size_t)TCELLS * 32 + 27 * 16 * 32; }
-
-static int conv_tiles(const Layout &L) { return ((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) * L.nz; }
+// 32 x 8 tiles of one plane, and 32 x 8 x 4 tiles
+static int plane_tiles(const Layout &L) { return ((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) * L.nz; }
+static int conv_tiles(const Layout &L)
+{
+    return ((L.nx + NT_X - 1) / NT_X) * ((L.ny + NT_Y - 1) / NT_Y) * ((L.nz + CV_Z - 1) / CV_Z);
+}
 
 static int conv_tiles_tc(const Layout &L)
 {
@@ -986,7 +1245,7 @@ int net_alloc(fs_ctx *c, bool training)
         (rc = alloc((void **)&n->wf, 3 * NWM * 2)) || (rc = alloc((void **)&n->wt, 3 * NWM * 2)) ||
         (rc = alloc((void **)&n->smax, 16)) || (rc = alloc((void **)&n->y, nC * 4)) ||
         (rc = alloc((void **)&n->wf1, 27 * 16 * 16 * 2)) || (rc = alloc((void **)&n->wf5, 27 * 16 * 16 * 2)) ||
-        (rc = alloc((void **)&n->tdist, (size_t)conv_tiles(c->L))) ||
+        (rc = alloc((void **)&n->tdist, (size_t)plane_tiles(c->L))) ||
         (rc = alloc((void **)&n->tlist, (size_t)conv_tiles(c->L) * sizeof(int))) ||
         (rc = alloc((void **)&n->tlist_tc, (size_t)conv_tiles_tc(c->L) * sizeof(int))))
         return rc;
@@ -1002,11 +1261,9 @@ int net_alloc(fs_ctx *c, bool training)
     }
     static bool attr_done = false;
     if (!attr_done) {
-        const int cs = (int)conv_smem();
-        FS_CUDA(cudaFuncSetAttribute(k_conv<IN_R, OUT_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, cs));
-        FS_CUDA(cudaFuncSetAttribute(k_conv<IN_ACT, OUT_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, cs));
-        FS_CUDA(cudaFuncSetAttribute(k_conv<IN_ACT, OUT_Z>, cudaFuncAttributeMaxDynamicSharedMemorySize, cs));
-        FS_CUDA(cudaFuncSetAttribute(k_conv<IN_ACT, OUT_BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, cs));
+        FS_CUDA(cudaFuncSetAttribute(k_conv<OUT_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CV_SMEM));
+        FS_CUDA(cudaFuncSetAttribute(k_conv<OUT_Z>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CV_SMEM));
+        FS_CUDA(cudaFuncSetAttribute(k_conv<OUT_BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CV_SMEM));
         FS_CUDA(cudaFuncSetAttribute(k_conv_tc<IN_R, OUT_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)TC_SMEM));
         FS_CUDA(cudaFuncSetAttribute(k_conv_tc<IN_ACT, OUT_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1061,46 +1318,37 @@ int net_read(fs_ctx *c, float *params_host)
     return FS_OK;
 }
 
-// Persistent grid of the conv kernel: as many blocks as fit on the SMs.
-static int conv_grid(const fs_ctx *c, int tiles)
-{
-    static int per_sm = 0;
-    if (!per_sm) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_conv<IN_ACT, OUT_RELU>, 256, conv_smem()) !=
-                cudaSuccess ||
-            per_sm < 1) {
-            cudaGetLastError();
-            per_sm = 1;
-        }
-    }
-    return std::max(1, std::min(tiles, c->num_sms * per_sm));
-}
-
 // The conv tiles sorted by their distance to the liquid, for the current mask.
 static int net_tile_list(fs_ctx *c)
 {
     NetState *n = net(c);
     if (n->tlist_epoch == c->mask_epoch) return FS_OK;
     const Layout &L = c->L;
-    const int nt = conv_tiles(L);
+    const int nt = plane_tiles(L);
     k_conv_tile_dist<<<nt, 256, 0, c->stream>>>(c->cflag, L, n->tdist);
     c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
     std::vector<uint8_t> d((size_t)nt);
     FS_CUDA(cudaMemcpyAsync(d.data(), n->tdist, (size_t)nt, cudaMemcpyDeviceToHost, c->stream));
     FS_CUDA(cudaStreamSynchronize(c->stream));
+    // a 32 x 8 x 4 tile is as near as the nearest of its four planes' tiles
+    const int ntx = (L.nx + NT_X - 1) / NT_X, nty = (L.ny + NT_Y - 1) / NT_Y, nxy = ntx * nty, n4 = conv_tiles(L);
+    std::vector<uint8_t> d4((size_t)n4, 5);
+    for (int t = 0; t < nt; t++) {
+        uint8_t &m = d4[(size_t)(t / nxy / CV_Z * nxy + t % nxy)];
+        m = std::min(m, d[(size_t)t]);
+    }
     std::vector<int> list;
-    list.reserve((size_t)nt);
+    list.reserve((size_t)n4);
     for (int dd = 0; dd <= 5; dd++) {
-        for (int t = 0; t < nt; t++)
-            if (d[(size_t)t] == dd) list.push_back(t);
+        for (int t = 0; t < n4; t++)
+            if (d4[(size_t)t] == dd) list.push_back(t);
         n->tcount[dd] = (int)list.size();
     }
     FS_CUDA(cudaMemcpy(n->tlist, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice));
     // the tensor-core layer's tiles (TC_M x TC_NY of one plane, inside one row of
     // conv tiles since NT_Y is a multiple of TC_NY): the distance of the nearest
     // conv tile they overlap
-    const int ntx = (L.nx + NT_X - 1) / NT_X, nty = (L.ny + NT_Y - 1) / NT_Y;
     const int ntxc = (L.nx + TC_M - 1) / TC_M, ntyc = (L.ny + TC_NY - 1) / TC_NY, ntc = conv_tiles_tc(L);
     std::vector<uint8_t> dc((size_t)ntc, 5);
     for (int t = 0; t < ntc; t++) {
@@ -1123,19 +1371,20 @@ static int net_tile_list(fs_ctx *c)
     return FS_OK;
 }
 
-static void conv_launch(fs_ctx *c, int in, int out, const ConvArgs &a, int tiles)
+// Persistent grids: one block of k_conv per SM (its two tiles fill the shared memory).
+static int conv_launch(fs_ctx *c, int out, const ConvArgs &a, int tiles)
 {
-    const int g = conv_grid(c, tiles);
-    const size_t sm = conv_smem();
-    if (in == IN_R)
-        k_conv<IN_R, OUT_RELU><<<g, 256, sm, c->stream>>>(a);
-    else if (out == OUT_RELU)
-        k_conv<IN_ACT, OUT_RELU><<<g, 256, sm, c->stream>>>(a);
+    CUtensorMap map;
+    if (int rc = encode_cells16(&map, a.in, c->L, CV_P, TYH, CV_Z + 2)) return rc;
+    const int g = std::max(1, std::min(tiles, c->num_sms));
+    if (out == OUT_RELU)
+        k_conv<OUT_RELU><<<g, 256, CV_SMEM, c->stream>>>(map, a, c->err_word);
     else if (out == OUT_Z)
-        k_conv<IN_ACT, OUT_Z><<<g, 256, sm, c->stream>>>(a);
+        k_conv<OUT_Z><<<g, 256, CV_SMEM, c->stream>>>(map, a, c->err_word);
     else
-        k_conv<IN_ACT, OUT_BWD><<<g, 256, sm, c->stream>>>(a);
+        k_conv<OUT_BWD><<<g, 256, CV_SMEM, c->stream>>>(map, a, c->err_word);
     c->n_launches += 1;
+    return FS_OK;
 }
 
 // The tensor-core layer: two blocks per SM (two input tiles and the weights each).
@@ -1173,28 +1422,38 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
     auto tiles_for = [&](int layer) {         // layer 1 .. 5
         return keep ? all : (tc ? n->tcount_tc[5 - layer] : n->tcount[5 - layer]);
     };
-    auto launch = [&](int in, int out, const ConvArgs &ca) {
-        if (tc)
+    auto launch = [&](int in, int out, const ConvArgs &ca) -> int {
+        if (tc) {
             conv_launch_tc(c, in, out, ca, ca.ntiles);
-        else
-            conv_launch(c, in, out, ca, ca.ntiles);
+        } else if (in == IN_R) {
+            k_conv1<<<std::max(1, std::min(ca.ntiles, c->num_sms * 2)), 256, 0, c->stream>>>(ca);
+            c->n_launches += 1;
+        } else {
+            return conv_launch(c, out, ca, ca.ntiles);
+        }
+        return FS_OK;
     };
     ConvArgs a{};
     a.cf = c->cflag;
     a.smax = n->smax;
     a.tiles = keep ? nullptr : (tc ? n->tlist_tc : n->tlist);
     a.L = L;
-    // layer 1: input built from r; keep: x -> A[0], a1 -> A[1]
-    a.r = r;
+    // layer 1: inference builds its input from r; training stores it, x -> A[0], a1 -> A[1]
     a.wts = n->wf1;
     a.bias = n->master + OB1;
-    a.xin = keep ? A[0] : nullptr;
     a.out = keep ? A[1] : A[0];
     a.ntiles = tiles_for(1);
-    launch(IN_R, OUT_RELU, a);
+    if (keep) {
+        k_net_x<<<grid_blocks(c, L.S, 256), 256, 0, c->stream>>>(r, c->cflag, n->smax, L, A[0]);
+        c->n_launches += 1;
+        a.in = A[0];
+        if ((rc = launch(IN_ACT, OUT_RELU, a))) return rc;
+    } else {
+        a.r = r;
+        if ((rc = launch(IN_R, OUT_RELU, a))) return rc;
+        a.r = nullptr;
+    }
     __nv_bfloat16 *cur = a.out;
-    a.xin = nullptr;
-    a.r = nullptr;
     const int bias_off[3] = {OB2, OB3, OB4};
     for (int l = 0; l < 3; l++) {
         __nv_bfloat16 *nxt = keep ? A[2 + l] : (cur == A[0] ? A[1] : A[0]);
@@ -1203,7 +1462,7 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
         a.bias = n->master + bias_off[l];
         a.out = nxt;
         a.ntiles = tiles_for(2 + l);
-        launch(IN_ACT, OUT_RELU, a);
+        if ((rc = launch(IN_ACT, OUT_RELU, a))) return rc;
         cur = nxt;
     }
     a.in = cur;
@@ -1213,13 +1472,13 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
     a.y = y;
     a.z = z;
     a.ntiles = tiles_for(5);
-    launch(IN_ACT, OUT_Z, a);
+    if ((rc = launch(IN_ACT, OUT_Z, a))) return rc;
     FS_CUDA(cudaGetLastError());
-    // the useful flops of the layers, on the cells of the tiles they visit (both
-    // tilings hold 256 cells a tile): 2 x 27 x (2 x 16 + 3 x 16 x 16 + 16 x 1) per cell
+    // the useful flops of the layers, on the cells of the tiles they visit:
+    // 2 x 27 x (2 x 16 + 3 x 16 x 16 + 16 x 1) per cell
     n->last_flops = 0.0;
     const double fl[5] = {2.0 * 27 * 2 * 16, 2.0 * 27 * 16 * 16, 2.0 * 27 * 16 * 16, 2.0 * 27 * 16 * 16, 2.0 * 27 * 16};
-    for (int l = 1; l <= 5; l++) n->last_flops += fl[l - 1] * 256.0 * (double)tiles_for(l);
+    for (int l = 1; l <= 5; l++) n->last_flops += fl[l - 1] * (tc ? 256.0 : 256.0 * CV_Z) * (double)tiles_for(l);
     return FS_OK;
 }
 
@@ -1253,6 +1512,7 @@ int net_grad(fs_ctx *c, const float *b, const float *q, double *loss)
     const size_t nC = (size_t)L.nC;
     const int ncell = L.nx * L.ny * L.nz;
     const int gb = std::max(1, std::min((ncell + 255) / 256, c->num_sms * 8));
+    FS_CUDA(cudaMemsetAsync(c->err_word, 0, sizeof(unsigned), c->stream));
     // b, q into cell space (zero off liquid): pb <- b, px <- q
     if ((rc = cell_in(c, b, c->pb)) || (rc = cell_in(c, q, c->px))) return rc;
     if ((rc = net_forward(c, c->pb, nullptr, n->y, true))) return rc;
@@ -1297,7 +1557,7 @@ int net_grad(fs_ctx *c, const float *b, const float *q, double *loss)
         bw.aref = A[l + 1];
         bw.out = G[gi ^ 1];
         bw.L = L;
-        conv_launch(c, IN_ACT, OUT_BWD, bw, conv_tiles(L));
+        if ((rc = conv_launch(c, OUT_BWD, bw, conv_tiles(L)))) return rc;
         gi ^= 1;
     }
     // layer 1: gradient w.r.t. W1 from the stored input x (2 channels used)
@@ -1305,7 +1565,9 @@ int net_grad(fs_ctx *c, const float *b, const float *q, double *loss)
     c->n_launches += 2 + 6 + 1;
     FS_CUDA(cudaGetLastError());
     SolveScal h;
-    if ((rc = read_scal(c, 3, &h))) return rc;
+    unsigned herr = 0;
+    if ((rc = read_scal(c, 3, &h, &herr))) return rc;
+    if (herr & ERR_NET) return set_error(FS_ETIMEOUT, "network: a bounded wait ran out");
     if (loss) *loss += h.aux[1] > 0.0 ? h.aux[0] / h.aux[1] : 0.0;
     return FS_OK;
 }

@@ -709,16 +709,19 @@ int check_wait_error(fs_ctx *c, const char *what)
                          c->prm.spin_limit);
     }
     if (herr & ERR_TMA) return set_error(FS_ETIMEOUT, "%s: a wait for a tensor copy ran out", what);
-    if (herr & 8u)  // the bit of the tensor-core network layer
-        return set_error(FS_ETIMEOUT, "%s: a wait for the network's tensor-core MMAs ran out", what);
+    if (herr & 8u)  // the bit of the network's kernels
+        return set_error(FS_ETIMEOUT, "%s: a bounded wait of the network ran out", what);
     return FS_OK;
 }
 
-int read_scal(fs_ctx *c, int which, SolveScal *out)
+int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err)
 {
+    unsigned *eh = reinterpret_cast<unsigned *>(c->scal_host + 4);
     FS_CUDA(cudaMemcpyAsync(c->scal_host + which, c->scal + which, sizeof(SolveScal), cudaMemcpyDeviceToHost,
                             c->stream));
+    if (err) FS_CUDA(cudaMemcpyAsync(eh, c->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     FS_CUDA(cudaStreamSynchronize(c->stream));
+    if (err) *err = *eh;
     prof_flush(c);
     *out = c->scal_host[which];
     return FS_OK;
@@ -1326,7 +1329,7 @@ int precond_apply_public(fs_ctx *c, const float *r, float *z)
         c->mic_ready = 0;  // the factor may be incomplete: refactor on the next use
         return set_error(FS_ETIMEOUT, "MIC(0) sweep: a wait on a predecessor tile ran out");
     }
-    if (herr & 8u) return set_error(FS_ETIMEOUT, "network: a wait for the tensor-core MMAs ran out");
+    if (herr & 8u) return set_error(FS_ETIMEOUT, "network: a bounded wait ran out");
     return FS_OK;
 }
 
