@@ -176,7 +176,7 @@ static void free_ctx(fs_ctx *c)
                     c->fg[2], c->gc[0], c->gc[1], c->gc[2], c->mic_prec, c->scal, c->partials, c->err_word, c->pw[0], c->pw[1],
                     c->act_cell, c->act_face, c->list_cell, c->list_face, c->items_cell, c->items_face, c->qmask_cell, c->qmask_face,
                     c->py, c->mic_order,
-                    c->mic_tact, c->mic_tflag, c->mic_next};
+                    c->mic_tact, c->mic_tflag, c->mic_next, c->cq};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->scal_host) cudaFreeHost(c->scal_host);

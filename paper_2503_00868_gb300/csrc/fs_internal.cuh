@@ -159,6 +159,11 @@ struct fs_ctx {
     void *percnn;         // recurrent convolutional pressure solver (fs_percnn.cu)
     void *splat;          // splatting scratch (fs_splat.cu)
     void *mg;             // multigrid hierarchy of the pressure preconditioner (fs_mg.cu)
+    // the quads of cell space that hold a liquid cell, in order, for the mask of
+    // cq_epoch (fs_mg.cu cell_quads, built on first use)
+    int *cq;
+    int ncq;
+    long long cq_epoch;
 
     // reductions
     fs::SolveScal *scal;        // device [4]: 0 pressure, 1 viscosity, 2 misc, 3 misc
@@ -440,6 +445,15 @@ __device__ __forceinline__ bool grid_reduce(KSum (&v)[K], double *partials, unsi
     return true;
 }
 
+// Walks a list of quads (or other entries): each thread strides through it with the
+// next entry fetched one step ahead, so no list load stands between a thread and its
+// data loads.
+#define FS_FOR_LIST(list, na)                                                                            \
+    for (int fl_i = blockIdx.x * blockDim.x + threadIdx.x, fl_st = gridDim.x * blockDim.x,               \
+             q = fl_i < (na) ? __ldg((list) + fl_i) : 0, fl_next = 0;                                    \
+         fl_i < (na) && ((fl_next = fl_i + fl_st < (na) ? __ldg((list) + fl_i + fl_st) : 0), true);     \
+         fl_i += fl_st, q = fl_next)
+
 // ---- launchers implemented in the .cu files --------------------------------
 // fs_mask.cu
 int build_mask(fs_ctx *c, const uint8_t *types_dense, const fs_mac *bc);
@@ -463,6 +477,7 @@ int launch_loss(fs_ctx *c, CF3 u, CF3 t, int kind, double alpha, double beta, F3
 // fs_mg.cu
 int mg_apply(fs_ctx *c, const float *r, float *z, const int *done);
 int mg_apply_faces(fs_ctx *c, const float *r, float *z, float cc, const int *done);
+int cell_quads(fs_ctx *c, const int **ql, int *n);  // fs_mg.cu: the list of the current mask's active quads
 void mg_free(fs_ctx *c);
 void mg_count(fs_ctx *c, long long vcycles, bool faces);  // fs_mg.cu: launch counts for fs_profile
 int mg_levels(const fs_ctx *c);
@@ -500,7 +515,9 @@ int net_load(fs_ctx *c, const float *params, int count, bool host);
 int net_read(fs_ctx *c, float *params_host);
 int net_kernel(fs_ctx *c, int which);  // fs_net.cu: inference layers, 0 mma.sync, 1 tcgen05
 int check_wait_error(fs_ctx *c, const char *what);  // fs_pcg.cu: bounded-wait errors of the last solve
-int net_apply(fs_ctx *c, const float *r, float *z);   // cell space
+// cell space; z (zero off the liquid before) is written on the tiles that hold liquid; every kernel returns at
+// once when *done != 0 (done nullable)
+int net_apply(fs_ctx *c, const float *r, float *z, const int *done);
 int net_grad(fs_ctx *c, const float *b, const float *q, double *loss);  // public layout
 int net_adam(fs_ctx *c, double lr, double beta1, double beta2, double eps, int step, double gscale,
              int fix_offsets);
@@ -520,7 +537,10 @@ int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err = nullptr);
 int remove_null_mode(fs_ctx *c, float *z);
 // fs_fcg.cu: flexible CG with the network, pb -> px (warm: from the current x);
 // final scalars in *h
-int learned_apply(fs_ctx *c, const float *r, float *z, const int *done);  // fs_pcg.cu: network (+ V-cycle)
+// fs_pcg.cu: the network (+ V-cycle). learned_begin zeroes the buffers it keeps its
+// parts in; with e_out the result is z + *e_out (*e_out null: z alone), not yet added
+int learned_begin(fs_ctx *c);
+int learned_apply(fs_ctx *c, const float *r, float *z, const int *done, const float **e_out);
 int solve_pressure_fcg(fs_ctx *c, SolveScal *h, bool warm);
 int pressure_restart(fs_ctx *c);  // fs_pcg.cu: r = b - A x, p = 0 (scalars of slot 0)
 void fcg_release(fs_ctx *c);

@@ -115,6 +115,7 @@ struct MgSet {
     MgSetLevel lev[MG_MAX_LEVELS];
     uint8_t *blob = nullptr;  // flags and lists of the single-block levels, volume after volume
     bool one = false;         // one smoothing sweep each side on level 0 (the face volumes)
+    bool shared0 = false;     // level 0's list belongs to the context
     long long calls = 0;      // applies so far (profiling samples every prof_period-th)
     // algorithmic bytes of the level-0 kernels, in the order of K_MG0_SMOOTH2 ..
     // K_MG0_SMOOTH_Z (counted when first profiled; negative before)
@@ -179,14 +180,8 @@ __device__ __forceinline__ float sweep1(uint8_t f, float c, float nb, float rv, 
 }
 
 // The kernels below walk a level's list of active quads (those holding an
-// unknown, built with the hierarchy), each thread striding through it with the
-// next entry fetched one step ahead: no flag load stands between a thread and its
+// unknown, built with the hierarchy): no flag load stands between a thread and its
 // data loads, and the quads without an unknown cost nothing.
-#define MG_FOR_LIST(list, na)                                                                            \
-    for (int mg_i = blockIdx.x * blockDim.x + threadIdx.x, mg_st = gridDim.x * blockDim.x,               \
-             q = mg_i < (na) ? __ldg((list) + mg_i) : 0, mg_next = 0;                                    \
-         mg_i < (na) && ((mg_next = mg_i + mg_st < (na) ? __ldg((list) + mg_i + mg_st) : 0), true);     \
-         mg_i += mg_st, q = mg_next)
 
 // Vector loads through the non-coherent path: no launch writes what it reads.
 __device__ __forceinline__ float4 ldv4(const float *p, int t) { return __ldg(reinterpret_cast<const float4 *>(p + t)); }
@@ -393,7 +388,7 @@ __global__ void __launch_bounds__(256) k_mg0_smooth(const MgSpace S, const int *
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
     KSum acc;
-    MG_FOR_LIST(qlist, na) acc.add(smooth_q(S.g[vol_of(S, 4 * q)], fl, r, ein, eout, wt, scale, m, q));
+    FS_FOR_LIST(qlist, na) acc.add(smooth_q(S.g[vol_of(S, 4 * q)], fl, r, ein, eout, wt, scale, m, q));
     if (!rzs || *(volatile const int *)&rzs->done) return;  // (a timed sweep runs after convergence too)
     KSum v[1] = {acc};
     double tot[1];
@@ -415,7 +410,7 @@ __global__ void __launch_bounds__(256) k_mg0_pre1(const MgSpace S, const int *__
     if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
-    MG_FOR_LIST(qlist, na) pre1_q(S.g[vol_of(S, 4 * q)], fl, r, eb, res, wt, scale, m, q);
+    FS_FOR_LIST(qlist, na) pre1_q(S.g[vol_of(S, 4 * q)], fl, r, eb, res, wt, scale, m, q);
 }
 
 __global__ void __launch_bounds__(256, 8) k_mg0_residual(const MgSpace S, const int *__restrict__ qlist, int na,
@@ -424,7 +419,7 @@ __global__ void __launch_bounds__(256, 8) k_mg0_residual(const MgSpace S, const 
                                                       const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    MG_FOR_LIST(qlist, na) resid_q(S.g[vol_of(S, 4 * q)], fl, r, ev, res, scale, m, q);
+    FS_FOR_LIST(qlist, na) resid_q(S.g[vol_of(S, 4 * q)], fl, r, ev, res, scale, m, q);
 }
 
 __global__ void __launch_bounds__(256) k_mg0_smooth2(const MgSpace S, const int *__restrict__ qlist, int na,
@@ -434,7 +429,7 @@ __global__ void __launch_bounds__(256) k_mg0_smooth2(const MgSpace S, const int 
     if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
-    MG_FOR_LIST(qlist, na) smooth2_q(S.g[vol_of(S, 4 * q)], fl, r, eo, wt, scale, m, q);
+    FS_FOR_LIST(qlist, na) smooth2_q(S.g[vol_of(S, 4 * q)], fl, r, eo, wt, scale, m, q);
 }
 
 __global__ void __launch_bounds__(256) k_mg0_prolong(const MgSpace S, const MgSpace Sc, const int *__restrict__ qlist,
@@ -442,7 +437,7 @@ __global__ void __launch_bounds__(256) k_mg0_prolong(const MgSpace S, const MgSp
                                                      const float *__restrict__ ec, const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    MG_FOR_LIST(qlist, na)
+    FS_FOR_LIST(qlist, na)
     {
         const int v = vol_of(S, 4 * q), base = S.base[v];
         prolong_q(S.g[v], fl + base, ef + base, Sc.g[v], ec + Sc.base[v], q - (base >> 2));
@@ -455,7 +450,7 @@ __global__ void __launch_bounds__(256) k_mg0_restrict(const MgSpace S, const flo
                                                       const uint8_t *__restrict__ flc, float *rc, const int *done)
 {
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    MG_FOR_LIST(plist, np)
+    FS_FOR_LIST(plist, np)
     {
         const int v = vol_of(Sc, q), base = Sc.base[v];
         restrict_pair(S.g[v], res + S.base[v], Sc.g[v], flc + base, rc + base, q - base);
@@ -591,7 +586,7 @@ __global__ void __launch_bounds__(TH) k_mg_rz(const int *__restrict__ qlist, int
     if (s->done) return;
     KSum acc;
     const float4 *r4 = reinterpret_cast<const float4 *>(r), *z4 = reinterpret_cast<const float4 *>(z);
-    MG_FOR_LIST(qlist, na)
+    FS_FOR_LIST(qlist, na)
     {
         const float4 a = __ldg(r4 + q), b = __ldg(z4 + q);
         acc.add(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
@@ -666,8 +661,8 @@ void free_set(MgSet *t)
 {
     for (int l = 0; l < MG_MAX_LEVELS; l++) {
         MgSetLevel &v = t->lev[l];
-        cudaFree(v.ql);
         cudaFree(v.pl);
+        if (l > 0 || !t->shared0) cudaFree(v.ql);
         if (l > 0) {  // level 0 lies in the context's arrays and in MgAll's
             cudaFree(v.fl);
             for (float *p : {v.r, v.a, v.b, v.c}) cudaFree(p);
@@ -984,8 +979,10 @@ int make_list(fs_ctx *c, const MgSetLevel &v, long long (*items)(const MgGrid &)
     return rc;
 }
 
+long long quad_items(const MgGrid &g) { return g.n / 4; }
+
 // Arrays, flags and lists of a set whose volumes' levels are planned and whose
-// level 0 is given (flags, work arrays, bases).
+// level 0 is given (flags, work arrays, bases, and the list where it is shared).
 int build_set(fs_ctx *c, MgSet &t)
 {
     int nlev = 1, minlb = MG_MAX_LEVELS;
@@ -1060,8 +1057,8 @@ int build_set(fs_ctx *c, MgSet &t)
     for (int l = 0; l <= t.lf; l++) {
         MgSetLevel &x = t.lev[l];
         int rc = FS_OK;
-        if (l < t.lf)
-            rc = make_list<QuadPred>(c, x, [](const MgGrid &g) { return (long long)(g.n / 4); }, &x.ql, &x.nq);
+        if (l < t.lf && !x.ql)
+            rc = make_list<QuadPred>(c, x, quad_items, &x.ql, &x.nq);
         if (!rc && l > 0)
             rc = make_list<PairPred>(
                 c, x, [](const MgGrid &g) { return (long long)((g.nx + 1) >> 1) * g.ny * g.nz; }, &x.pl, &x.np);
@@ -1122,6 +1119,25 @@ void mg_free(fs_ctx *c)
     c->mg = nullptr;
 }
 
+int cell_quads(fs_ctx *c, const int **ql, int *n)
+{
+    if (c->cq_epoch != c->mask_epoch || !c->cq) {
+        cudaFree(c->cq);
+        c->cq = nullptr;
+        MgSetLevel v;
+        v.sp.nv = 1;
+        v.sp.g[0] = level0_grid(c->L, c->L.nx, c->L.ny, c->L.nz);
+        v.sp.base[0] = 0;
+        v.fl = c->cflag;
+        if (int rc = make_list<QuadPred>(c, v, quad_items, &c->cq, &c->ncq))
+            return rc == FS_ENOMEM ? set_error(FS_ENOMEM, "list of active quads") : rc;
+        c->cq_epoch = c->mask_epoch;
+    }
+    *ql = c->cq;
+    *n = c->ncq;
+    return FS_OK;
+}
+
 // z = M r on the cell space (r and z of length nC, zero off the liquid); with
 // rzs, r.z in the last level-0 sweep when the hierarchy has one (*fused tells)
 static int apply_cell(fs_ctx *c, const float *r, float *z, const int *done, SolveScal *rzs, int first, bool *fused)
@@ -1142,6 +1158,13 @@ static int apply_cell(fs_ctx *c, const float *r, float *z, const int *done, Solv
         t.lev[0].fl = c->cflag;
         t.lev[0].b = m->cb;
         t.lev[0].c = m->cc;
+        t.shared0 = true;
+        const int *ql = nullptr;
+        if ((rc = cell_quads(c, &ql, &t.lev[0].nq))) {
+            free_set(&t);
+            return rc;
+        }
+        t.lev[0].ql = const_cast<int *>(ql);
         if ((rc = build_set(c, t))) {
             free_set(&t);
             return rc;

@@ -135,6 +135,7 @@ struct ConvArgs {
     float *y, *z;               // OUT_Z (each optional): network output; z = s y on liquid, else 0
     const int *tiles;           // optional list of conv tiles (else every tile)
     int ntiles;                 // entries of `tiles`
+    const int *done;            // k_conv, k_conv1: return at once when *done != 0 (nullable)
     Layout L;
 };
 
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(256, 1) k_conv(const __grid_constant__ CUtenso
                                                  const __grid_constant__ ConvArgs a, unsigned *err)
 {
     constexpr int NT = OUT == OUT_Z ? 1 : 2;  // n-tiles of 8 output channels
+    if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t mbar[2];
     const Layout &L = a.L;
@@ -420,6 +422,7 @@ __device__ __forceinline__ uint32_t net_input(float r, uint8_t f, float inv)
 
 __global__ void __launch_bounds__(256, 2) k_conv1(const __grid_constant__ ConvArgs a)
 {
+    if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     __shared__ uint32_t sx[CV_CELLS];
     const Layout &L = a.L;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -801,12 +804,18 @@ __global__ void __launch_bounds__(256) k_conv_tile_dist(const uint8_t *__restric
     if (threadIdx.x == 0) dist[tb] = (uint8_t)best;
 }
 
-// max |r| over the liquid, as float bits (non-negative floats order like ints)
-__global__ void k_absmax(const float *__restrict__ r, const uint8_t *__restrict__ cf, int n, unsigned *smax)
+// max |r| over the liquid, as float bits (non-negative floats order like ints), over
+// the list of quads that hold liquid (r is zero on their other cells)
+__global__ void __launch_bounds__(256) k_absmax(const int *__restrict__ ql, int nq, const float *__restrict__ r,
+                                                unsigned *smax, const int *done)
 {
+    if (done && *(volatile const int *)done) return;  // the solve has converged
     float m = 0.f;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
-        if (cf[t] & CF_LIQ) m = fmaxf(m, fabsf(r[t]));
+    FS_FOR_LIST(ql, nq)
+    {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(r) + q);
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(smax, __float_as_uint(m));
 }
@@ -1400,11 +1409,11 @@ static void conv_launch_tc(fs_ctx *c, int in, int out, const ConvArgs &a, int ti
     c->n_launches += 1;
 }
 
-// z = s Net(r / s) on liquid cells, 0 elsewhere (cell space). Training (`keep`)
+// z = s Net(r / s) on liquid cells (cell space; z is zero elsewhere before). Training (`keep`)
 // runs every layer on every tile and keeps the layer inputs in act[0..4] and the
 // output in y; inference runs layer l on the tiles within 5 - l cells of the
 // liquid, with activations ping-ponging in act[0..1].
-static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
+static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep, const int *done = nullptr)
 {
     NetState *n = net(c);
     const Layout &L = c->L;
@@ -1412,9 +1421,11 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
     int rc;
     if (!keep && (rc = net_tile_list(c))) return rc;
     FS_CUDA(cudaMemsetAsync(n->smax, 0, sizeof(unsigned), c->stream));
-    k_absmax<<<grid_blocks(c, L.nC, 256), 256, 0, c->stream>>>(r, c->cflag, L.nC, n->smax);
+    const int *ql = nullptr;
+    int nq = 0;
+    if ((rc = cell_quads(c, &ql, &nq))) return rc;
+    k_absmax<<<grid_blocks(c, nq, 256), 256, 0, c->stream>>>(ql, nq, r, n->smax, done);
     c->n_launches += 1;
-    if (z) FS_CUDA(cudaMemsetAsync(z, 0, nC * sizeof(float), c->stream));
     __nv_bfloat16 *A[6];
     for (int l = 0; l < 6; l++) A[l] = n->act + (keep ? (size_t)l : (size_t)(l & 1)) * nC * 16;
     const int all = conv_tiles(L);
@@ -1436,6 +1447,7 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
     ConvArgs a{};
     a.cf = c->cflag;
     a.smax = n->smax;
+    a.done = done;
     a.tiles = keep ? nullptr : (tc ? n->tlist_tc : n->tlist);
     a.L = L;
     // layer 1: inference builds its input from r; training stores it, x -> A[0], a1 -> A[1]
@@ -1482,12 +1494,12 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep)
     return FS_OK;
 }
 
-int net_apply(fs_ctx *c, const float *r, float *z)
+int net_apply(fs_ctx *c, const float *r, float *z, const int *done)
 {
     NetState *n = net(c);
     if (!n || !n->loaded) return set_error(FS_ESTATE, "the learned preconditioner has no network loaded");
     cudaEvent_t e0 = prof_mark(c);
-    int rc = net_forward(c, r, z, nullptr, false);
+    int rc = net_forward(c, r, z, nullptr, false, done);
     prof_add(c, K_NET_APPLY, e0, prof_mark(c), n->last_flops);  // flops, not bytes: a tensor-core entry
     return rc;
 }

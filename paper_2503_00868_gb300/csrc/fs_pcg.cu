@@ -378,19 +378,30 @@ __global__ void __launch_bounds__(TH) k_pois_true_res(const float *b, const floa
     }
 }
 
-// res = r - A e on the liquid, zero elsewhere (guard planes included); e is zero
+// res = r - A e on the liquid, over the list of active quads; e and res are zero
 // off the liquid
-__global__ void __launch_bounds__(TH) k_pois_resid(const float *__restrict__ r, const float *__restrict__ e,
-                                                   const uint8_t *__restrict__ fl, int n, int P, int PL, float *res)
+__global__ void __launch_bounds__(TH) k_pois_resid(const int *__restrict__ ql, int nq, const float *__restrict__ r,
+                                                   const float *__restrict__ e, const uint8_t *__restrict__ fl, int P,
+                                                   int PL, float *res, const int *done)
 {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const uint8_t f = fl[t];
-        float v = 0.f;
-        if (f & CF_LIQ) {
-            const float nb = (e[t - 1] + e[t + 1]) + (e[t - P] + e[t + P]) + (e[t - PL] + e[t + PL]);
-            v = r[t] - (PoisOp::diag(f, 0.f) * e[t] - nb);
-        }
-        res[t] = v;
+    if (done && *(volatile const int *)done) return;  // the solve has converged
+    FS_FOR_LIST(ql, nq)
+    {
+        const int t = 4 * q;
+        const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
+        auto e4 = [&](int u) { return __ldg(reinterpret_cast<const float4 *>(e + u)); };
+        const float4 c = e4(t), dn = e4(t - P), up = e4(t + P), bk = e4(t - PL), fw = e4(t + PL);
+        const float4 rv = __ldg(reinterpret_cast<const float4 *>(r + t));
+        const float lf = __ldg(e + t - 1), rt = __ldg(e + t + 4);
+        auto one = [&](uint8_t fe, float rc, float ce, float nb) {
+            return (fe & CF_LIQ) ? rc - (PoisOp::diag(fe, 0.f) * ce - nb) : 0.f;
+        };
+        float4 v;
+        v.x = one(f.x, rv.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x));
+        v.y = one(f.y, rv.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y));
+        v.z = one(f.z, rv.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z));
+        v.w = one(f.w, rv.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w));
+        *reinterpret_cast<float4 *>(res + t) = v;
     }
 }
 
@@ -769,16 +780,32 @@ int remove_null_mode(fs_ctx *c, float *z)
 // leaves (FS_PRECOND_LEARNED_MG): z = e + M(r - A e), e = s Net(r/s). The network
 // smooths, the V-cycle corrects the error it cannot reach. pp[0] and pp[1] are
 // free while flexible CG runs (it keeps its directions in its own ring).
-int learned_apply(fs_ctx *c, const float *r, float *z, const int *done)
+int learned_begin(fs_ctx *c)
 {
-    if (c->prm.precond != FS_PRECOND_LEARNED_MG) return net_apply(c, r, z);
+    if (c->prm.precond != FS_PRECOND_LEARNED_MG) return FS_OK;
+    for (float *p : c->pp) FS_CUDA(cudaMemsetAsync(p, 0, (size_t)c->L.nC * sizeof(float), c->stream));
+    return FS_OK;
+}
+
+int learned_apply(fs_ctx *c, const float *r, float *z, const int *done, const float **e_out)
+{
+    if (e_out) *e_out = nullptr;
+    if (c->prm.precond != FS_PRECOND_LEARNED_MG) return net_apply(c, r, z, done);
     const Layout &L = c->L;
     float *e = c->pp[0], *res = c->pp[1];
-    if (int rc = net_apply(c, r, e)) return rc;
-    k_pois_resid<<<grid_blocks(c, L.nC, TH), TH, 0, c->stream>>>(r, e, c->cflag, L.nC, L.P, L.PL, res);
+    if (int rc = net_apply(c, r, e, done)) return rc;
+    const int *ql = nullptr;
+    int nq = 0;
+    if (int rc = cell_quads(c, &ql, &nq)) return rc;
+    static const int rb = resident_blocks((const void *)k_pois_resid, 0);
+    k_pois_resid<<<wave_blocks(c, nq, rb), TH, 0, c->stream>>>(ql, nq, r, e, c->cflag, L.P, L.PL, res, done);
     c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
     if (int rc = mg_apply(c, res, z, done)) return rc;
+    if (e_out) {
+        *e_out = e;
+        return FS_OK;
+    }
     k_add4<<<grid_blocks(c, L.nC / 4, TH), TH, 0, c->stream>>>(z, e, L.nC / 4);
     c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
@@ -1316,7 +1343,8 @@ int precond_apply_public(fs_ctx *c, const float *r, float *z)
         int rc = mic0_apply(c, c->pr, c->pz);
         if (rc) return rc;
     } else {
-        int rc = learned_apply(c, c->pr, c->pz, nullptr);
+        int rc = learned_begin(c);
+        if (!rc) rc = learned_apply(c, c->pr, c->pz, nullptr, nullptr);
         if (rc) return rc;
     }
     k_cell_out<<<bs, TH, 0, c->stream>>>(c->pz, z, L);
