@@ -170,6 +170,7 @@ static void free_ctx(fs_ctx *c)
     fcg_release(c);
     percnn_free(c);
     splat_free(c);
+    apic_free(c);
     mg_free(c);
     void *ptrs[] = {c->cflag, c->fflag, c->bc, c->dsum, c->pb, c->pr, c->pp[0], c->pp[1], c->pq, c->px, c->pz,
                     c->pxh, c->pxt, c->pbr, c->vx, c->vr, c->vp[0], c->vp[1], c->vq, c->vz, c->fu[0], c->fu[1], c->fu[2], c->fg[0], c->fg[1],

@@ -158,6 +158,7 @@ struct fs_ctx {
     void *fcg;
     void *percnn;         // recurrent convolutional pressure solver (fs_percnn.cu)
     void *splat;          // splatting scratch (fs_splat.cu)
+    void *apic;           // particle ordering scratch (fs_apic.cu)
     void *mg;             // multigrid hierarchy of the pressure preconditioner (fs_mg.cu)
     // the quads of cell space that hold a liquid cell, in order, for the mask of
     // cq_epoch (fs_mg.cu cell_quads, built on first use)
@@ -497,6 +498,7 @@ void splat_free(fs_ctx *c);
 void splat_stats(const fs_ctx *c, unsigned long long *entries, unsigned long long *max_tile);
 // fs_apic.cu
 int launch_p2g(fs_ctx *c, int np, const float *x, const float *v, const float *C, const float *m, F3 u, F3 mass);
+void apic_free(fs_ctx *c);
 int launch_g2p(fs_ctx *c, int np, float *x, float *v, float *C, float *F, const float *A0, float *A, CF3 u,
                double dt, int advance, double lo, double hi);
 // fs_volume.cu
