@@ -446,6 +446,36 @@ __device__ __forceinline__ bool grid_reduce(KSum (&v)[K], double *partials, unsi
     return true;
 }
 
+// ---- dependent launches ------------------------------------------------------
+// The kernels of the solvers' loops are a few microseconds long, and between two
+// ordinary launches on a stream the GPU stands idle for about 2 (drain, launch,
+// first instructions). launch_dep starts a kernel while the one before it still runs
+// (programmatic dependent launch): its blocks take the slots that fall free and wait
+// in dep_wait until that kernel has completed and its writes are visible. Every
+// kernel launched so calls dep_wait in all its threads before it touches memory that
+// a launch before it may write (or may still read), and dep_go to let the next one
+// start: since each of them completes only after its own dep_wait, completion is
+// transitive along the stream. Anything launched otherwise (copies, other kernels)
+// waits for full completion on either side.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // an error stays for the caller's cudaGetLastError
+}
+
 // Walks a list of quads (or other entries): each thread strides through it with the
 // next entry fetched one step ahead, so no list load stands between a thread and its
 // data loads.

@@ -62,6 +62,8 @@ __global__ void __launch_bounds__(TH) k_pc_res(const int *__restrict__ ql, int n
                                                const float *__restrict__ p, float *__restrict__ r,
                                                const uint8_t *__restrict__ cf, int P, int PL)
 {
+    dep_go();
+    dep_wait();
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
@@ -88,6 +90,8 @@ __global__ void __launch_bounds__(TH) k_pc_conv(const int *__restrict__ ql, int 
                                                 const float *base, float *out, const uint8_t *__restrict__ cf, int P,
                                                 int PL, const __grid_constant__ PercnnW W)
 {
+    dep_go();
+    dep_wait();
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
@@ -291,8 +295,8 @@ int solve_pressure_percnn(fs_ctx *c, SolveScal *h)
     FS_CUDA(cudaMemsetAsync(c->px, 0, (size_t)L.nC * sizeof(float), c->stream));
     FS_CUDA(cudaMemsetAsync(c->pr, 0, (size_t)L.nC * sizeof(float), c->stream));
     for (int k = 0; k < s->K; k++) {
-        k_pc_res<<<br, TH, 0, c->stream>>>(ql, nq, c->pb, c->px, c->pr, c->cflag, L.P, L.PL);
-        k_pc_conv<<<bv, TH, 0, c->stream>>>(ql, nq, c->pr, c->px, c->px, c->cflag, L.P, L.PL, s->w);
+        launch_dep(k_pc_res, br, TH, 0, c->stream, ql, nq, c->pb, c->px, c->pr, c->cflag, L.P, L.PL);
+        launch_dep(k_pc_conv, bv, TH, 0, c->stream, ql, nq, c->pr, c->px, c->px, c->cflag, L.P, L.PL, s->w);
         c->n_launches += 2;
     }
     FS_CUDA(cudaGetLastError());

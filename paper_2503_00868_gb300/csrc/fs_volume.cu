@@ -126,9 +126,11 @@ __global__ void __launch_bounds__(TH) k_pbd_iterate(const int *__restrict__ ql, 
                                                     const float *__restrict__ div, const uint8_t *__restrict__ fl,
                                                     float *__restrict__ out, int P, int PL, float inv_dx2, float eps)
 {
+    dep_go();
     __shared__ float w[8];  // 1 / (n / dx^2 + eps); a cell without a free face moves nothing
     if (threadIdx.x < 8) w[threadIdx.x] = threadIdx.x ? 1.f / ((float)threadIdx.x * inv_dx2 + eps) : 0.f;
     __syncthreads();
+    dep_wait();
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
@@ -199,8 +201,8 @@ int launch_pbd_project(fs_ctx *c, F3 u, int hold, int iters, double eps, double 
         static const int rb = resident_blocks((const void *)k_pbd_iterate, 0);
         for (float *p : lam) FS_CUDA(cudaMemsetAsync(p, 0, (size_t)L.nC * sizeof(float), c->stream));
         for (int it = 0; it < iters; it++)
-            k_pbd_iterate<<<wave_blocks(c, nq, rb), TH, 0, c->stream>>>(ql, nq, lam[it & 1], div, nfree, lam[(it & 1) ^ 1],
-                                                                        L.P, L.PL, inv_dx * inv_dx, (float)eps);
+            launch_dep(k_pbd_iterate, wave_blocks(c, nq, rb), TH, 0, c->stream, ql, nq, lam[it & 1], div, nfree,
+                       lam[(it & 1) ^ 1], L.P, L.PL, inv_dx * inv_dx, (float)eps);
         k_pbd_update<<<bf, TH, 0, c->stream>>>(u, c->cflag, c->fflag, L, hold, inv_dx, lam[iters & 1]);
         c->n_launches += iters + 1;
         divergence();
