@@ -41,16 +41,17 @@ __global__ void __launch_bounds__(TH) k_fcg_dots(const int *__restrict__ ql, int
                                                  const float *__restrict__ r, Ring ring, int nvalid, SolveScal *s,
                                                  double *beta, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     KSum acc[FCG_M + 1];
     float4 *z4 = reinterpret_cast<float4 *>(z);
-    const float4 *r4 = reinterpret_cast<const float4 *>(r);
     FS_FOR_LIST(ql, nq)
     {
-        float4 a = z4[q];
-        const float4 b = __ldg(r4 + q);
+        float4 a = ldd4(z + 4 * q);
+        const float4 b = ldd4(r + 4 * q);
         if (e) {
-            const float4 w = __ldg(reinterpret_cast<const float4 *>(e) + q);
+            const float4 w = ldd4(e + 4 * q);
             a.x += w.x; a.y += w.y; a.z += w.z; a.w += w.w;
             z4[q] = a;
         }
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(TH) k_fcg_dots(const int *__restrict__ ql, int
 #pragma unroll
         for (int j = 0; j < FCG_M; j++) {
             if (j < nvalid) {
-                const float4 c = __ldg(reinterpret_cast<const float4 *>(ring.q[j]) + q);
+                const float4 c = ldd4(ring.q[j] + 4 * q);
                 acc[j].add(a.x * c.x + a.y * c.y + a.z * c.z + a.w * c.w);
             }
         }
@@ -84,6 +85,8 @@ __global__ void __launch_bounds__(TH) k_fcg_dir(const int *__restrict__ ql, int 
                                                 int nvalid, float *__restrict__ p, const SolveScal *s,
                                                 const double *__restrict__ beta)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     float b[FCG_M];
 #pragma unroll
@@ -91,11 +94,11 @@ __global__ void __launch_bounds__(TH) k_fcg_dir(const int *__restrict__ ql, int 
     float4 *p4 = reinterpret_cast<float4 *>(p);
     FS_FOR_LIST(ql, nq)
     {
-        float4 v = __ldg(reinterpret_cast<const float4 *>(z) + q);
+        float4 v = ldd4(z + 4 * q);
 #pragma unroll
         for (int j = 0; j < FCG_M; j++) {
             if (j < nvalid) {
-                const float4 w = __ldg(reinterpret_cast<const float4 *>(ring.p[j]) + q);
+                const float4 w = ldd4(ring.p[j] + 4 * q);
                 v.x += b[j] * w.x; v.y += b[j] * w.y; v.z += b[j] * w.z; v.w += b[j] * w.w;
             }
         }
@@ -109,15 +112,17 @@ __global__ void __launch_bounds__(TH) k_fcg_apply(const int *__restrict__ ql, in
                                                   float *__restrict__ qo, const uint8_t *__restrict__ cf, int P, int PL,
                                                   SolveScal *s, double *pq_out, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     KSum acc;
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
         const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(cf + t));
-        auto p4 = [&](int u) { return __ldg(reinterpret_cast<const float4 *>(p + u)); };
+        auto p4 = [&](int u) { return ldd4(p + u); };
         const float4 c = p4(t), dn = p4(t - P), up = p4(t + P), bk = p4(t - PL), fw = p4(t + PL);
-        const float lf = __ldg(p + t - 1), rt = __ldg(p + t + 4);
+        const float lf = ldd1(p + t - 1), rt = ldd1(p + t + 4);
         auto one = [&](uint8_t fe, float ce, float nb) { return (fe & CF_LIQ) ? (float)(fe & CF_D) * ce - nb : 0.f; };
         float4 v;
         v.x = one(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x));
@@ -144,6 +149,8 @@ __global__ void __launch_bounds__(TH) k_fcg_update(const int *__restrict__ ql, i
                                                    float *__restrict__ r, const float *__restrict__ p,
                                                    const float *__restrict__ ap, SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     const float alpha = (float)s->alpha;
     KSum rr;
@@ -151,9 +158,9 @@ __global__ void __launch_bounds__(TH) k_fcg_update(const int *__restrict__ ql, i
     float4 *r4 = reinterpret_cast<float4 *>(r);
     FS_FOR_LIST(ql, nq)
     {
-        const float4 pv = __ldg(reinterpret_cast<const float4 *>(p) + q);
-        const float4 qv = __ldg(reinterpret_cast<const float4 *>(ap) + q);
-        float4 xv = x4[q], rv = r4[q];
+        const float4 pv = ldd4(p + 4 * q);
+        const float4 qv = ldd4(ap + 4 * q);
+        float4 xv = ldd4(x + 4 * q), rv = ldd4(r + 4 * q);
         xv.x += alpha * pv.x; xv.y += alpha * pv.y; xv.z += alpha * pv.z; xv.w += alpha * pv.w;
         rv.x -= alpha * qv.x; rv.y -= alpha * qv.y; rv.z -= alpha * qv.z; rv.w -= alpha * qv.w;
         x4[q] = xv;
@@ -317,12 +324,12 @@ int solve_pressure_fcg(fs_ctx *c, SolveScal *h, bool warm)
             if ((rc = remove_null_mode(c, c->pz))) return rc;
             const bool samp = c->prof_on && (b % c->prof_period) == 0;
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
-            k_fcg_dots<<<wave_blocks(c, nq, rd), TH, 0, c->stream>>>(ql, nq, c->pz, e, c->pr, ring, nvalid, s, f->beta,
+            launch_dep(k_fcg_dots, wave_blocks(c, nq, rd), TH, 0, c->stream, ql, nq, c->pz, e, c->pr, ring, nvalid, s, f->beta,
                                                                      c->partials);
-            k_fcg_dir<<<wave_blocks(c, nq, ri), TH, 0, c->stream>>>(ql, nq, c->pz, ring, nvalid, f->p[slot], s, f->beta);
-            k_fcg_apply<<<wave_blocks(c, nq, ra), TH, 0, c->stream>>>(ql, nq, f->p[slot], f->q[slot], c->cflag, L.P,
+            launch_dep(k_fcg_dir, wave_blocks(c, nq, ri), TH, 0, c->stream, ql, nq, c->pz, ring, nvalid, f->p[slot], s, f->beta);
+            launch_dep(k_fcg_apply, wave_blocks(c, nq, ra), TH, 0, c->stream, ql, nq, f->p[slot], f->q[slot], c->cflag, L.P,
                                                                       L.PL, s, f->pq + slot, c->partials);
-            k_fcg_update<<<wave_blocks(c, nq, ru), TH, 0, c->stream>>>(ql, nq, c->px, c->pr, f->p[slot], f->q[slot], s,
+            launch_dep(k_fcg_update, wave_blocks(c, nq, ru), TH, 0, c->stream, ql, nq, c->px, c->pr, f->p[slot], f->q[slot], s,
                                                                        c->partials);
             cudaEvent_t e1 = samp ? prof_mark(c) : nullptr;
             // vectors streamed: dots 2 + nvalid, direction 2 + nvalid, operator ~3, update 6

@@ -183,9 +183,8 @@ __device__ __forceinline__ float sweep1(uint8_t f, float c, float nb, float rv, 
 // unknown, built with the hierarchy): no flag load stands between a thread and its
 // data loads, and the quads without an unknown cost nothing.
 
-// Vector loads through the non-coherent path: no launch writes what it reads.
-__device__ __forceinline__ float4 ldv4(const float *p, int t) { return __ldg(reinterpret_cast<const float4 *>(p + t)); }
-__device__ __forceinline__ float ldv1(const float *p, int t) { return __ldg(p + t); }
+__device__ __forceinline__ float4 ldv4(const float *p, int t) { return ldd4(p + t); }
+__device__ __forceinline__ float ldv1(const float *p, int t) { return ldd1(p + t); }
 
 // one damped Jacobi sweep on quad q: eout from ein; returns r.eout over the quad
 __device__ __forceinline__ float smooth_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
@@ -285,7 +284,7 @@ __device__ __forceinline__ void prolong_q(const MgGrid &gf, const uint8_t *__res
             s2 += w * (0.75f * c1 + 0.25f * c0);
             s3 += w * (0.75f * c1 + 0.25f * c2);
         }
-    float4 v = *reinterpret_cast<const float4 *>(ef + t);
+    float4 v = ldv4(ef, t);
     if (liq(f.x)) v.x += s0;
     if (liq(f.y)) v.y += s1;
     if (liq(f.z)) v.z += s2;
@@ -384,9 +383,11 @@ __global__ void __launch_bounds__(256) k_mg0_smooth(const MgSpace S, const int *
                                                     const float *__restrict__ ein, float *eout, float scale, float m,
                                                     const int *done, SolveScal *rzs, double *partials, int first)
 {
-    if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
+    dep_wait();
+    dep_go();
+    if (done && *(volatile const int *)done) return;  // the solve has converged
     KSum acc;
     FS_FOR_LIST(qlist, na) acc.add(smooth_q(S.g[vol_of(S, 4 * q)], fl, r, ein, eout, wt, scale, m, q));
     if (!rzs || *(volatile const int *)&rzs->done) return;  // (a timed sweep runs after convergence too)
@@ -407,9 +408,11 @@ __global__ void __launch_bounds__(256) k_mg0_pre1(const MgSpace S, const int *__
                                                   const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                   float *eb, float *res, float scale, float m, const int *done)
 {
-    if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
+    dep_wait();
+    dep_go();
+    if (done && *(volatile const int *)done) return;  // the solve has converged
     FS_FOR_LIST(qlist, na) pre1_q(S.g[vol_of(S, 4 * q)], fl, r, eb, res, wt, scale, m, q);
 }
 
@@ -418,6 +421,8 @@ __global__ void __launch_bounds__(256, 8) k_mg0_residual(const MgSpace S, const 
                                                       const float *__restrict__ ev, float *res, float scale, float m,
                                                       const int *done)
 {
+    dep_wait();
+    dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
     FS_FOR_LIST(qlist, na) resid_q(S.g[vol_of(S, 4 * q)], fl, r, ev, res, scale, m, q);
 }
@@ -426,9 +431,11 @@ __global__ void __launch_bounds__(256) k_mg0_smooth2(const MgSpace S, const int 
                                                      const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                      float *eo, float scale, float m, const int *done)
 {
-    if (done && *(volatile const int *)done) return;  // the solve has converged
     __shared__ float wt[8];
     fill_wtab(wt, scale, m);
+    dep_wait();
+    dep_go();
+    if (done && *(volatile const int *)done) return;  // the solve has converged
     FS_FOR_LIST(qlist, na) smooth2_q(S.g[vol_of(S, 4 * q)], fl, r, eo, wt, scale, m, q);
 }
 
@@ -436,6 +443,8 @@ __global__ void __launch_bounds__(256) k_mg0_prolong(const MgSpace S, const MgSp
                                                      int na, const uint8_t *__restrict__ fl, float *ef,
                                                      const float *__restrict__ ec, const int *done)
 {
+    dep_wait();
+    dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
     FS_FOR_LIST(qlist, na)
     {
@@ -449,6 +458,8 @@ __global__ void __launch_bounds__(256) k_mg0_restrict(const MgSpace S, const flo
                                                       const int *__restrict__ plist, int np,
                                                       const uint8_t *__restrict__ flc, float *rc, const int *done)
 {
+    dep_wait();
+    dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
     FS_FOR_LIST(plist, np)
     {
@@ -583,12 +594,13 @@ __global__ void k_mg_count(MgGrid g, uint8_t *fl)
 __global__ void __launch_bounds__(TH) k_mg_rz(const int *__restrict__ qlist, int na, const float *__restrict__ r,
                                              const float *__restrict__ z, int first, SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     KSum acc;
-    const float4 *r4 = reinterpret_cast<const float4 *>(r), *z4 = reinterpret_cast<const float4 *>(z);
     FS_FOR_LIST(qlist, na)
     {
-        const float4 a = __ldg(r4 + q), b = __ldg(z4 + q);
+        const float4 a = ldd4(r + 4 * q), b = ldd4(z + 4 * q);
         acc.add(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
     }
     KSum v[1] = {acc};
@@ -718,9 +730,9 @@ int launch_leg(fs_ctx *c, const MgSet &t, int l, bool down, const int *done)
     }
     if (!nv) return FS_OK;
     if (down)
-        k_mg_down<<<dim3(tiles, nv), MGT_TH, sm, c->stream>>>(a);
+        launch_dep(k_mg_down, dim3(tiles, nv), MGT_TH, sm, c->stream, a);
     else
-        k_mg_up<<<dim3(tiles, nv), MGT_TH, sm, c->stream>>>(a);
+        launch_dep(k_mg_up, dim3(tiles, nv), MGT_TH, sm, c->stream, a);
     c->n_launches += 1;
     return FS_OK;
 }
@@ -771,7 +783,7 @@ int launch_bottom(fs_ctx *c, const MgSet &t, const float *r0, float *z0, const i
             a.v[v].lev[0].l.r = const_cast<float *>(r0) + t.lev[0].sp.base[v];
             a.v[v].lev[0].l.a = z0 + t.lev[0].sp.base[v];
         }
-    k_mg_bottom<<<t.nv, MGB_TH, sm, c->stream>>>(a);
+    launch_dep(k_mg_bottom, t.nv, MGB_TH, sm, c->stream, a);
     c->n_launches += 1;
     return FS_OK;
 }
@@ -828,22 +840,22 @@ int vcycle(fs_ctx *c, MgSet &t, const float *r, float *z, const int *done_, bool
         const float *rl = l == 0 ? r : v.r, scale = s0.lev[l].scale, mass = s0.lev[l].mass;
         const int *done = sample && l == 0 ? nullptr : done_;
         if (l == 0 && t.one) {  // the sweep from zero and the residual it leaves, in one pass
-            k_mg0_pre1<<<wave_blocks(c, v.nq, res.pre1), TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass,
+            launch_dep(k_mg0_pre1, wave_blocks(c, v.nq, res.pre1), TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass,
                                                                       done);
             c->n_launches += 1;
         } else {
             begin(l);
-            k_mg0_smooth2<<<wave_blocks(c, v.nq, res.smooth2), TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, scale,
+            launch_dep(k_mg0_smooth2, wave_blocks(c, v.nq, res.smooth2), TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, scale,
                                                                             mass, done);
             end(l, K_MG0_SMOOTH2, t.by0[0]);
             begin(l);
-            k_mg0_residual<<<wave_blocks(c, v.nq, res.residual), TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c,
+            launch_dep(k_mg0_residual, wave_blocks(c, v.nq, res.residual), TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c,
                                                                               scale, mass, done);
             end(l, K_MG0_RESIDUAL, t.by0[1]);
             c->n_launches += 2;
         }
         begin(l);
-        k_mg0_restrict<<<wave_blocks(c, w.np, res.restrict_), TH, 0, st>>>(v.sp, v.c, w.sp, w.pl, w.np, w.fl, w.r,
+        launch_dep(k_mg0_restrict, wave_blocks(c, w.np, res.restrict_), TH, 0, st, v.sp, v.c, w.sp, w.pl, w.np, w.fl, w.r,
                                                                            done);
         end(l, K_MG0_RESTRICT, t.by0[2]);
         c->n_launches += 1;
@@ -863,20 +875,20 @@ int vcycle(fs_ctx *c, MgSet &t, const float *r, float *z, const int *done_, bool
         const int nb = wave_blocks(c, v.nq, res.smooth);
         end(l, K_MG_COARSE, 0.0);
         begin(l);
-        k_mg0_prolong<<<wave_blocks(c, v.nq, res.prolong), TH, 0, st>>>(v.sp, w.sp, v.ql, v.nq, v.fl, v.b, w.a, done);
+        launch_dep(k_mg0_prolong, wave_blocks(c, v.nq, res.prolong), TH, 0, st, v.sp, w.sp, v.ql, v.nq, v.fl, v.b, w.a, done);
         end(l, K_MG0_PROLONG, t.by0[3]);
         const float *ez = v.c;  // the input of the last sweep
         if (l == 0 && t.one) {
             ez = v.b;
         } else {
             begin(l);
-            k_mg0_smooth<<<nb, TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass, done, nullptr, nullptr,
+            launch_dep(k_mg0_smooth, nb, TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass, done, nullptr, nullptr,
                                             0);
             end(l, K_MG0_SMOOTH, t.by0[4]);
             c->n_launches += 1;
         }
         begin(l);
-        k_mg0_smooth<<<nb, TH, 0, st>>>(v.sp, v.ql, v.nq, v.fl, rl, ez, l == 0 ? z : v.a, scale, mass, done,
+        launch_dep(k_mg0_smooth, nb, TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, ez, l == 0 ? z : v.a, scale, mass, done,
                                         l == 0 ? rzs : nullptr, c->partials, first);
         end(l, K_MG0_SMOOTH_Z, t.by0[5]);
         c->n_launches += 2;
@@ -1306,7 +1318,7 @@ bool mg_rz(fs_ctx *c, bool faces, const float *r, const float *z, int first, Sol
 {
     const MgSet *t = listed_set(c, faces);
     if (!t) return false;
-    k_mg_rz<<<grid_blocks(c, t->lev[0].nq, TH), TH, 0, c->stream>>>(t->lev[0].ql, t->lev[0].nq, r, z, first, s, c->partials);
+    launch_dep(k_mg_rz, grid_blocks(c, t->lev[0].nq, TH), TH, 0, c->stream, t->lev[0].ql, t->lev[0].nq, r, z, first, s, c->partials);
     c->n_launches += 1;
     return cudaPeekAtLastError() == cudaSuccess;
 }

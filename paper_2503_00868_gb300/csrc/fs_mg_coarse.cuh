@@ -195,14 +195,16 @@ __device__ __forceinline__ bool leg_tile(const MgTiles &T, int &q0, int &j0, int
 // the restriction of r - A b. A tile without an unknown returns after its flags.
 __global__ void __launch_bounds__(MGT_TH, 2) k_mg_down(const __grid_constant__ MgLegArgs a)
 {
-    if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     extern __shared__ __align__(16) float mg_sm[];
     __shared__ float wt[8];
     const MgLegVol &V = a.v[blockIdx.y];
     const MgTiles &T = V.t;
     const MgcLevel &L = V.f;
     int q0, j0, k0;
-    if (!leg_tile(T, q0, j0, k0)) return;
+    const bool mine = leg_tile(T, q0, j0, k0);
+    dep_wait();
+    dep_go();
+    if (!mine || (a.done && *(volatile const int *)a.done)) return;  // (or the solve has converged)
     if (threadIdx.x < 8) wt[threadIdx.x] = wtab_entry(L.scale, L.mass, threadIdx.x);
     const int nq = T.tqx + 2, ny = T.ty + 6, nz = T.tz + 6;
     const int P = nq * 4, PL = P * ny, n = PL * nz;
@@ -284,14 +286,16 @@ __global__ void __launch_bounds__(MGT_TH, 2) k_mg_down(const __grid_constant__ M
 // Up one level: the coarse result prolonged onto b, then two sweeps, into a.
 __global__ void __launch_bounds__(MGT_TH, 2) k_mg_up(const __grid_constant__ MgLegArgs a)
 {
-    if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     extern __shared__ __align__(16) float mg_sm[];
     __shared__ float wt[8];
     const MgLegVol &V = a.v[blockIdx.y];
     const MgTiles &T = V.t;
     const MgcLevel &L = V.f, &W = V.c;
     int q0, j0, k0;
-    if (!leg_tile(T, q0, j0, k0)) return;
+    const bool mine = leg_tile(T, q0, j0, k0);
+    dep_wait();
+    dep_go();
+    if (!mine || (a.done && *(volatile const int *)a.done)) return;  // (or the solve has converged)
     if (threadIdx.x < 8) wt[threadIdx.x] = wtab_entry(L.scale, L.mass, threadIdx.x);
     const int nq = T.tqx + 2, ny = T.ty + 4, nz = T.tz + 4;
     const int P = nq * 4, PL = P * ny, n = PL * nz;
@@ -323,7 +327,7 @@ __global__ void __launch_bounds__(MGT_TH, 2) k_mg_up(const __grid_constant__ MgL
     for (int s = threadIdx.x; s < cn; s += MGT_TH) {
         const int x = s % CP, y = (s / CP) % (T.ty / 2 + 4), z = s / CPL;
         const int I = 2 * q0 - 3 + x, J = j0 / 2 - 2 + y, K = k0 / 2 - 2 + z;
-        EC[s] = I >= 0 && J >= 0 && K >= 0 && I < W.g.nx && J < W.g.ny && K < W.g.nz ? __ldg(W.a + W.g.idx(I, J, K))
+        EC[s] = I >= 0 && J >= 0 && K >= 0 && I < W.g.nx && J < W.g.ny && K < W.g.nz ? ldd1(W.a + W.g.idx(I, J, K))
                                                                                       : 0.f;
     }
     if (!__syncthreads_or(any)) return;
@@ -445,6 +449,8 @@ __device__ __forceinline__ void bar_some(int threads) { asm volatile("bar.sync 1
 
 __global__ void __launch_bounds__(MGB_TH, 1) k_mg_bottom(const __grid_constant__ MgBottomArgs a)
 {
+    dep_wait();
+    dep_go();
     if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     extern __shared__ __align__(16) float mg_sm[];
     __shared__ float wts[MGB_MAXLEV][8];

@@ -232,6 +232,8 @@ __global__ void __launch_bounds__(256, 1) k_conv(const __grid_constant__ CUtenso
                                                  const __grid_constant__ ConvArgs a, unsigned *err)
 {
     constexpr int NT = OUT == OUT_Z ? 1 : 2;  // n-tiles of 8 output channels
+    dep_wait();
+    dep_go();
     if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t mbar[2];
@@ -422,6 +424,8 @@ __device__ __forceinline__ uint32_t net_input(float r, uint8_t f, float inv)
 
 __global__ void __launch_bounds__(256, 2) k_conv1(const __grid_constant__ ConvArgs a)
 {
+    dep_wait();
+    dep_go();
     if (a.done && *(volatile const int *)a.done) return;  // the solve has converged
     __shared__ uint32_t sx[CV_CELLS];
     const Layout &L = a.L;
@@ -1387,11 +1391,11 @@ static int conv_launch(fs_ctx *c, int out, const ConvArgs &a, int tiles)
     if (int rc = encode_cells16(&map, a.in, c->L, CV_P, TYH, CV_Z + 2)) return rc;
     const int g = std::max(1, std::min(tiles, c->num_sms));
     if (out == OUT_RELU)
-        k_conv<OUT_RELU><<<g, 256, CV_SMEM, c->stream>>>(map, a, c->err_word);
+        launch_dep(k_conv<OUT_RELU>, g, 256, CV_SMEM, c->stream, map, a, c->err_word);
     else if (out == OUT_Z)
-        k_conv<OUT_Z><<<g, 256, CV_SMEM, c->stream>>>(map, a, c->err_word);
+        launch_dep(k_conv<OUT_Z>, g, 256, CV_SMEM, c->stream, map, a, c->err_word);
     else
-        k_conv<OUT_BWD><<<g, 256, CV_SMEM, c->stream>>>(map, a, c->err_word);
+        launch_dep(k_conv<OUT_BWD>, g, 256, CV_SMEM, c->stream, map, a, c->err_word);
     c->n_launches += 1;
     return FS_OK;
 }
@@ -1437,7 +1441,7 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep,
         if (tc) {
             conv_launch_tc(c, in, out, ca, ca.ntiles);
         } else if (in == IN_R) {
-            k_conv1<<<std::max(1, std::min(ca.ntiles, c->num_sms * 2)), 256, 0, c->stream>>>(ca);
+            launch_dep(k_conv1, std::max(1, std::min(ca.ntiles, c->num_sms * 2)), 256, 0, c->stream, ca);
             c->n_launches += 1;
         } else {
             return conv_launch(c, out, ca, ca.ntiles);

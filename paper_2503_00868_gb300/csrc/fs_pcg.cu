@@ -53,6 +53,8 @@ __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, in
                                                   float *__restrict__ q, const uint8_t *__restrict__ fl, int P,
                                                   int PL, float cc, SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     const float beta = (float)s->beta;
     const float off = Op::offc(cc);
@@ -65,11 +67,10 @@ __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, in
         qn = i + st < na ? __ldg(ql + i + st) : 0;
         const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
         auto pn4 = [&](int u) {
-            const float4 a = __ldg(reinterpret_cast<const float4 *>(src + u));
-            const float4 b = __ldg(reinterpret_cast<const float4 *>(pold + u));
+            const float4 a = ldd4(src + u), b = ldd4(pold + u);
             return make_float4(a.x + beta * b.x, a.y + beta * b.y, a.z + beta * b.z, a.w + beta * b.w);
         };
-        auto pn1 = [&](int u) { return __ldg(src + u) + beta * __ldg(pold + u); };
+        auto pn1 = [&](int u) { return ldd1(src + u) + beta * ldd1(pold + u); };
         const float4 c = pn4(t), dn = pn4(t - P), up = pn4(t + P), bk = pn4(t - PL), fw = pn4(t + PL);
         const float lf = pn1(t - 1), rt = pn1(t + 4);
         auto one = [&](uint8_t fe, float ce, float nb) {
@@ -105,6 +106,8 @@ __global__ void __launch_bounds__(TH) k_spmv(const float *__restrict__ src, cons
                                              const uint8_t *__restrict__ fl, int n, int P, int PL, float cc,
                                              SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     const float beta = (float)s->beta;
     KSum acc;
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(TH) k_spmv(const float *__restrict__ src, cons
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         const uint8_t f = fl[t];
         if (!(f & Op::ACTIVE)) continue;
-        auto pn = [&](int u) -> float { return __ldg(src + u) + beta * __ldg(pold + u); };
+        auto pn = [&](int u) -> float { return ldd1(src + u) + beta * ldd1(pold + u); };
         const float pc = pn(t);
         const float nb = (pn(t - 1) + pn(t + 1)) + (pn(t - P) + pn(t + P)) + (pn(t - PL) + pn(t + PL));
         const float qv = Op::diag(f, cc) * pc - Op::offc(cc) * nb;
@@ -140,20 +143,20 @@ __global__ void __launch_bounds__(TH) k_update(float *__restrict__ x, float *__r
                                                const uint8_t *__restrict__ fl, int n4, float cc,
                                                SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     const float alpha = (float)s->alpha;
     KSum rz, rr;
     float4 *x4 = reinterpret_cast<float4 *>(x);
     float4 *r4 = reinterpret_cast<float4 *>(r);
-    const float4 *p4 = reinterpret_cast<const float4 *>(p);
-    const float4 *q4 = reinterpret_cast<const float4 *>(q);
     const uchar4 *f4 = reinterpret_cast<const uchar4 *>(fl);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += gridDim.x * blockDim.x) {
         const uchar4 fv = f4[t];
         // four inactive elements: p = q = 0 there, nothing changes
         if (!((fv.x | fv.y | fv.z | fv.w) & Op::ACTIVE)) continue;
-        float4 xv = x4[t], rv = r4[t];
-        const float4 pv = __ldg(p4 + t), qv = __ldg(q4 + t);
+        float4 xv = ldd4(x + 4 * t), rv = ldd4(r + 4 * t);
+        const float4 pv = ldd4(p + 4 * t), qv = ldd4(q + 4 * t);
         xv.x += alpha * pv.x; xv.y += alpha * pv.y; xv.z += alpha * pv.z; xv.w += alpha * pv.w;
         if (JAC) {
             // scaled residual z = D^-1 r: z -= alpha D^-1 Ap; r.z = sum d z^2, r.r = sum (d z)^2
@@ -189,12 +192,12 @@ __global__ void __launch_bounds__(TH) k_update(float *__restrict__ x, float *__r
 __global__ void __launch_bounds__(TH) k_rz(const float *__restrict__ r, const float *__restrict__ z, int n4,
                                            int first, SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     KSum acc;
-    const float4 *r4 = reinterpret_cast<const float4 *>(r);
-    const float4 *z4 = reinterpret_cast<const float4 *>(z);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += gridDim.x * blockDim.x) {
-        const float4 a = __ldg(r4 + t), b = __ldg(z4 + t);
+        const float4 a = ldd4(r + 4 * t), b = ldd4(z + 4 * t);
         acc.add(a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w);
     }
     KSum v[1] = {acc};
@@ -384,15 +387,17 @@ __global__ void __launch_bounds__(TH) k_pois_resid(const int *__restrict__ ql, i
                                                    const float *__restrict__ e, const uint8_t *__restrict__ fl, int P,
                                                    int PL, float *res, const int *done)
 {
+    dep_wait();
+    dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
         const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
-        auto e4 = [&](int u) { return __ldg(reinterpret_cast<const float4 *>(e + u)); };
+        auto e4 = [&](int u) { return ldd4(e + u); };
         const float4 c = e4(t), dn = e4(t - P), up = e4(t + P), bk = e4(t - PL), fw = e4(t + PL);
-        const float4 rv = __ldg(reinterpret_cast<const float4 *>(r + t));
-        const float lf = __ldg(e + t - 1), rt = __ldg(e + t + 4);
+        const float4 rv = ldd4(r + t);
+        const float lf = ldd1(e + t - 1), rt = ldd1(e + t + 4);
         auto one = [&](uint8_t fe, float rc, float ce, float nb) {
             return (fe & CF_LIQ) ? rc - (PoisOp::diag(fe, 0.f) * ce - nb) : 0.f;
         };
@@ -798,7 +803,7 @@ int learned_apply(fs_ctx *c, const float *r, float *z, const int *done, const fl
     int nq = 0;
     if (int rc = cell_quads(c, &ql, &nq)) return rc;
     static const int rb = resident_blocks((const void *)k_pois_resid, 0);
-    k_pois_resid<<<wave_blocks(c, nq, rb), TH, 0, c->stream>>>(ql, nq, r, e, c->cflag, L.P, L.PL, res, done);
+    launch_dep(k_pois_resid, wave_blocks(c, nq, rb), TH, 0, c->stream, ql, nq, r, e, c->cflag, L.P, L.PL, res, done);
     c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
     if (int rc = mg_apply(c, res, z, done)) return rc;
@@ -896,7 +901,7 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     // r.z: over the V-cycle's active quads with multigrid, else a dense pass
     auto rz = [&](int first) {
         if (!(c->prm.precond == FS_PRECOND_MG && mg_rz(c, false, c->pr, c->pz, first, s)))
-            k_rz<<<grid_blocks(c, n4, TH), TH, 0, c->stream>>>(c->pr, c->pz, n4, first, s, c->partials);
+            launch_dep(k_rz, grid_blocks(c, n4, TH), TH, 0, c->stream, c->pr, c->pz, n4, first, s, c->partials);
         c->n_launches += 1;
     };
     // z = M r and r.z: with multigrid (and no null mode to remove from z) r.z is
@@ -951,30 +956,26 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             const float *zsrc = jac ? c->pr : c->pz;
             if (listed)
-                k_spmv_list<PoisOp><<<wave_blocks(c, nlisted, rl), TH, 0, c->stream>>>(
-                    ql, nlisted, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
+                launch_dep(k_spmv_list<PoisOp>, wave_blocks(c, nlisted, rl), TH, 0, c->stream, ql, nlisted, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
             else if (tiled)
-                k_spmv_z<PoisOp><<<tg.spmv, tdim, zmarch_smem(), c->stream>>>(
-                    jac ? c->tmz_pr : c->tmz_pz, c->tmz_pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, c->items_cell,
+                launch_dep(k_spmv_z<PoisOp>, tg.spmv, tdim, zmarch_smem(), c->stream, jac ? c->tmz_pr : c->tmz_pz, c->tmz_pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, c->items_cell,
                     c->nitems_cell, tm, 0.f, s, c->partials, c->err_word);
             else
-                k_spmv<PoisOp><<<bs, TH, 0, c->stream>>>(zsrc, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.nC,
+                launch_dep(k_spmv<PoisOp>, bs, TH, 0, c->stream, zsrc, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.nC,
                                                          L.P, L.PL, 0.f, s, c->partials);
             cudaEvent_t e1 = samp ? prof_mark(c) : nullptr, e2 = samp ? prof_mark(c) : nullptr;
             if (tiled) {
                 if (jac)
-                    k_update_q<PoisOp, true><<<tg.upd, tdim, 0, c->stream>>>(
-                        c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag, c->list_cell, c->qmask_cell, c->nact_cell, tm,
+                    launch_dep(k_update_q<PoisOp, true>, tg.upd, tdim, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag, c->list_cell, c->qmask_cell, c->nact_cell, tm,
                         0.f, s, c->partials);
                 else
-                    k_update_q<PoisOp, false><<<tg.upd, tdim, 0, c->stream>>>(
-                        c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag, c->list_cell, c->qmask_cell, c->nact_cell, tm,
+                    launch_dep(k_update_q<PoisOp, false>, tg.upd, tdim, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag, c->list_cell, c->qmask_cell, c->nact_cell, tm,
                         0.f, s, c->partials);
             } else if (jac)
-                k_update<PoisOp, true><<<b4, TH, 0, c->stream>>>(c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag,
+                launch_dep(k_update<PoisOp, true>, b4, TH, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag,
                                                                  n4, 0.f, s, c->partials);
             else
-                k_update<PoisOp, false><<<b4, TH, 0, c->stream>>>(c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag,
+                launch_dep(k_update<PoisOp, false>, b4, TH, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag,
                                                                   n4, 0.f, s, c->partials);
             cudaEvent_t e3 = samp ? prof_mark(c) : nullptr;
             prof_add(c, K_P_SPMV, e0, e1, by_spmv);
@@ -1199,7 +1200,7 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
         int rc = FS_OK;
         if (mg_apply_faces_rz(c, c->vr, c->vz, cc, &s->done, s, first, rc) || rc) return rc;  // r.z in the V-cycle
         if (!mg_rz(c, true, c->vr, c->vz, first, s))  // over the active quads, else a dense pass
-            k_rz<<<b4, TH, 0, c->stream>>>(c->vr, c->vz, n4, first, s, c->partials);
+            launch_dep(k_rz, b4, TH, 0, c->stream, c->vr, c->vz, n4, first, s, c->partials);
         c->n_launches += 1;
         FS_CUDA(cudaGetLastError());
         return FS_OK;
@@ -1231,30 +1232,26 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
             const bool samp = c->prof_on && ((launched + b) % c->prof_period) == 0;  // every prof_period-th
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             if (listed)
-                k_spmv_list<HelmOp><<<wave_blocks(c, nlisted, rl), TH, 0, c->stream>>>(
-                    ql, nlisted, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
+                launch_dep(k_spmv_list<HelmOp>, wave_blocks(c, nlisted, rl), TH, 0, c->stream, ql, nlisted, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
             else if (tiled)
-                k_spmv_z<HelmOp><<<tg.spmv, tdim, zmarch_smem(), c->stream>>>(
-                    mg ? c->tmz_vz : c->tmz_vr, c->tmz_vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, c->items_face,
+                launch_dep(k_spmv_z<HelmOp>, tg.spmv, tdim, zmarch_smem(), c->stream, mg ? c->tmz_vz : c->tmz_vr, c->tmz_vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, c->items_face,
                     c->nitems_face, tm, cc, s, c->partials, c->err_word);
             else
-                k_spmv<HelmOp><<<bs, TH, 0, c->stream>>>(mg ? c->vz : c->vr, c->vp[cur], c->vp[cur ^ 1], c->vq,
+                launch_dep(k_spmv<HelmOp>, bs, TH, 0, c->stream, mg ? c->vz : c->vr, c->vp[cur], c->vp[cur ^ 1], c->vq,
                                                          c->fflag, L.nF, L.P, L.PL, cc, s, c->partials);
             cudaEvent_t e1 = samp ? prof_mark(c) : nullptr, e2 = samp ? prof_mark(c) : nullptr;
             if (tiled) {
                 if (mg)
-                    k_update_q<HelmOp, false><<<tg.upd, tdim, 0, c->stream>>>(
-                        c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, c->list_face, c->qmask_face, c->nact_face, tm,
+                    launch_dep(k_update_q<HelmOp, false>, tg.upd, tdim, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, c->list_face, c->qmask_face, c->nact_face, tm,
                         cc, s, c->partials);
                 else
-                    k_update_q<HelmOp, true><<<tg.upd, tdim, 0, c->stream>>>(
-                        c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, c->list_face, c->qmask_face, c->nact_face, tm,
+                    launch_dep(k_update_q<HelmOp, true>, tg.upd, tdim, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, c->list_face, c->qmask_face, c->nact_face, tm,
                         cc, s, c->partials);
             } else if (mg) {
-                k_update<HelmOp, false><<<b4, TH, 0, c->stream>>>(c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, n4,
+                launch_dep(k_update<HelmOp, false>, b4, TH, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, n4,
                                                                   cc, s, c->partials);
             } else {
-                k_update<HelmOp, true><<<b4, TH, 0, c->stream>>>(c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, n4,
+                launch_dep(k_update<HelmOp, true>, b4, TH, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, n4,
                                                                  cc, s, c->partials);
             }
             cudaEvent_t e3 = samp ? prof_mark(c) : nullptr;

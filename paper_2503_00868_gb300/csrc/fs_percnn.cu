@@ -62,16 +62,16 @@ __global__ void __launch_bounds__(TH) k_pc_res(const int *__restrict__ ql, int n
                                                const float *__restrict__ p, float *__restrict__ r,
                                                const uint8_t *__restrict__ cf, int P, int PL)
 {
-    dep_go();
     dep_wait();
+    dep_go();
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
         const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(cf + t));
-        auto p4 = [&](int u) { return __ldg(reinterpret_cast<const float4 *>(p + u)); };
+        auto p4 = [&](int u) { return ldd4(p + u); };
         const float4 c = p4(t), dn = p4(t - P), up = p4(t + P), bk = p4(t - PL), fw = p4(t + PL);
-        const float4 bv = __ldg(reinterpret_cast<const float4 *>(b + t));
-        const float lf = __ldg(p + t - 1), rt = __ldg(p + t + 4);
+        const float4 bv = ldd4(b + t);
+        const float lf = ldd1(p + t - 1), rt = ldd1(p + t + 4);
         auto one = [&](uint8_t fe, float ce, float nb, float be) {
             return (fe & CF_LIQ) ? be - ((float)(fe & CF_D) * ce - nb) : 0.f;
         };
@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(TH) k_pc_conv(const int *__restrict__ ql, int 
                                                 const float *base, float *out, const uint8_t *__restrict__ cf, int P,
                                                 int PL, const __grid_constant__ PercnnW W)
 {
-    dep_go();
     dep_wait();
+    dep_go();
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
@@ -100,14 +100,14 @@ __global__ void __launch_bounds__(TH) k_pc_conv(const int *__restrict__ ql, int 
 #pragma unroll
         for (int row = 0; row < 9; row++) {
             const int u = t + (row / 3 - 1) * PL + (row % 3 - 1) * P;
-            const float4 c = __ldg(reinterpret_cast<const float4 *>(x + u));
-            const float lf = __ldg(x + u - 1), rt = __ldg(x + u + 4);
+            const float4 c = ldd4(x + u);
+            const float lf = ldd1(x + u - 1), rt = ldd1(x + u + 4);
             const float w0 = W.w[3 * row], w1 = W.w[3 * row + 1], w2 = W.w[3 * row + 2];
             v.x += w0 * lf; v.y += w0 * c.x; v.z += w0 * c.y; v.w += w0 * c.z;
             v.x += w1 * c.x; v.y += w1 * c.y; v.z += w1 * c.z; v.w += w1 * c.w;
             v.x += w2 * c.y; v.y += w2 * c.z; v.z += w2 * c.w; v.w += w2 * rt;
         }
-        float4 o = base ? *reinterpret_cast<const float4 *>(base + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 o = base ? ldd4(base + t) : make_float4(0.f, 0.f, 0.f, 0.f);
         if (f.x & CF_LIQ) o.x += v.x;
         if (f.y & CF_LIQ) o.y += v.y;
         if (f.z & CF_LIQ) o.z += v.z;

@@ -9,10 +9,7 @@
 namespace fs {
 namespace {
 
-__device__ __forceinline__ float4 ld4(const float *__restrict__ p, int t)
-{
-    return __ldg(reinterpret_cast<const float4 *>(p + t));
-}
+__device__ __forceinline__ float4 ld4(const float *p, int t) { return ldd4(p + t); }
 
 __device__ __forceinline__ float4 fma4(float4 a, float b, float4 c)  // a + b c
 {
@@ -45,6 +42,8 @@ __global__ void __launch_bounds__(256) k_update_q(float *x, float *r, const floa
                                                   const int *__restrict__ list, const unsigned *__restrict__ qmask,
                                                   int nact, TileMap M, float cc, SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     if (s->done) return;
     __shared__ float dtab[8], itab[8];
     if (JAC) {
@@ -66,8 +65,7 @@ __global__ void __launch_bounds__(256) k_update_q(float *x, float *r, const floa
             M.decode(b, v, k, tyi, txi);
             const int t = M.origin0 + v * M.vstride + k * M.PL + (tyi * TILE_Y + ty) * M.P + txi * TILE_X + 4 * tx;
             const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
-            const float4 cx = *reinterpret_cast<const float4 *>(x + t);
-            const float4 cr = *reinterpret_cast<const float4 *>(r + t);
+            const float4 cx = ld4(x, t), cr = ld4(r, t);
             const float4 cp = ld4(p, t), cq = ld4(q, t);
             const float4 xv = fma4(cx, alpha, cp);
             float4 rv = cr;

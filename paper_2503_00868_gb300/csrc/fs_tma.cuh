@@ -110,7 +110,6 @@ __global__ void __launch_bounds__(256) k_spmv_z(const __grid_constant__ CUtensor
                                                 const int4 *__restrict__ items, int nitems, TileMap M, float cc,
                                                 SolveScal *s, double *partials, unsigned *err)
 {
-    if (s->done) return;
     extern __shared__ unsigned char dyn_smem[];
     unsigned char *base = align128(dyn_smem);
     float *ring = reinterpret_cast<float *>(base + Z_NS * 2 * ZB_PITCH);
@@ -123,6 +122,9 @@ __global__ void __launch_bounds__(256) k_spmv_z(const __grid_constant__ CUtensor
         mbar_fence_init();
     }
     __syncthreads();
+    dep_wait();
+    dep_go();
+    if (s->done) return;
     const float beta = (float)s->beta;
     const float oc = Op::offc(cc);
     KSum acc;

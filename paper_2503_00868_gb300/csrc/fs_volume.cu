@@ -122,23 +122,23 @@ __global__ void __launch_bounds__(TH) k_pbd_div(F3 u, const uint8_t *__restrict_
 
 // One iteration on Lambda over the active quads; fl holds CF_LIQ and the number of
 // free faces of a liquid cell, 0 elsewhere.
-__global__ void __launch_bounds__(TH) k_pbd_iterate(const int *__restrict__ ql, int nq, const float *__restrict__ lam,
-                                                    const float *__restrict__ div, const uint8_t *__restrict__ fl,
-                                                    float *__restrict__ out, int P, int PL, float inv_dx2, float eps)
+__global__ void __launch_bounds__(TH) k_pbd_iterate(const int *__restrict__ ql, int nq, const float *lam,
+                                                    const float *div, const uint8_t *fl,
+                                                    float *out, int P, int PL, float inv_dx2, float eps)
 {
-    dep_go();
     __shared__ float w[8];  // 1 / (n / dx^2 + eps); a cell without a free face moves nothing
     if (threadIdx.x < 8) w[threadIdx.x] = threadIdx.x ? 1.f / ((float)threadIdx.x * inv_dx2 + eps) : 0.f;
     __syncthreads();
     dep_wait();
+    dep_go();
     FS_FOR_LIST(ql, nq)
     {
         const int t = 4 * q;
-        const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
-        auto l4 = [&](int u) { return __ldg(reinterpret_cast<const float4 *>(lam + u)); };
+        const uchar4 f = *reinterpret_cast<const uchar4 *>(fl + t);
+        auto l4 = [&](int u) { return ldd4(lam + u); };
         const float4 c = l4(t), dn = l4(t - P), up = l4(t + P), bk = l4(t - PL), fw = l4(t + PL);
-        const float4 d = __ldg(reinterpret_cast<const float4 *>(div + t));
-        const float lf = __ldg(lam + t - 1), rt = __ldg(lam + t + 4);
+        const float4 d = ldd4(div + t);
+        const float lf = ldd1(lam + t - 1), rt = ldd1(lam + t + 4);
         auto one = [&](uint8_t fe, float ce, float nb, float de) {
             return (fe & CF_LIQ) ? ce - w[fe & CF_D] * (de + ((float)(fe & CF_D) * ce - nb) * inv_dx2) : 0.f;
         };
