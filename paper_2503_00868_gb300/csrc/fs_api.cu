@@ -180,7 +180,7 @@ static void free_ctx(fs_ctx *c)
                     c->mic_tact, c->mic_tflag, c->mic_next, c->cq};
     for (void *p : ptrs)
         if (p) cudaFree(p);
-    if (c->scal_host) cudaFreeHost(c->scal_host);
+    if (c->post) cudaFreeHost(c->post);
     delete c;
 }
 
@@ -359,12 +359,13 @@ int fs_init_grid(fs_ctx **out, int nx, int ny, int nz, const fs_params *p, void 
     ALLOC(c->partials, (size_t)red_blocks * 8 * sizeof(double));
     ALLOC(c->err_word, 16);
 #undef ALLOC
-    if (cudaHostAlloc((void **)&c->scal_host, 5 * sizeof(SolveScal), cudaHostAllocDefault) != cudaSuccess) {
+    if (cudaHostAlloc((void **)&c->post, sizeof(HostPost), cudaHostAllocMapped) != cudaSuccess) {
         cudaGetLastError();
-        c->scal_host = nullptr;
+        c->post = nullptr;
         free_ctx(c);
         return set_error(FS_ENOMEM, "pinned allocation failed");
     }
+    std::memset((void *)c->post, 0, sizeof(HostPost));
     if (int rc = make_tensor_maps(c)) {
         free_ctx(c);
         return rc;

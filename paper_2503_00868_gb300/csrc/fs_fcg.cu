@@ -295,9 +295,10 @@ int solve_pressure_fcg(fs_ctx *c, SolveScal *h, bool warm)
     }
     FS_CUDA(cudaGetLastError());
     long long k = 0;
+    unsigned herr = 0;
     std::vector<std::pair<int, double>> hist;  // (iteration, r.r) at the host checks
     for (;;) {
-        if ((rc = read_scal(c, 0, h))) return rc;
+        if ((rc = read_scal(c, 0, h, &herr))) return rc;
         if (h->done) break;
         if (k > (long long)c->prm.maxit_p + c->prm.check_every)
             return set_error(FS_ECUDA, "flexible CG: iteration flag never set");
@@ -338,7 +339,7 @@ int solve_pressure_fcg(fs_ctx *c, SolveScal *h, bool warm)
         }
         FS_CUDA(cudaGetLastError());
     }
-    return check_wait_error(c, "flexible CG");
+    return check_wait_error(c, "flexible CG", herr);
 }
 
 }  // namespace fs

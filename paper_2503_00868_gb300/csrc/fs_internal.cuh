@@ -50,6 +50,12 @@ struct SolveScal {
     int pad;
 };
 
+// Scalars posted to the host (pinned memory), complete when seq is the number waited for.
+struct HostPost {
+    SolveScal s;
+    unsigned err, seq;
+};
+
 struct Layout {
     int nx, ny, nz;
     int P;      // pitch
@@ -168,7 +174,8 @@ struct fs_ctx {
 
     // reductions
     fs::SolveScal *scal;        // device [4]: 0 pressure, 1 viscosity, 2 misc, 3 misc
-    fs::SolveScal *scal_host;   // pinned mirror [4], then the error word
+    fs::HostPost *post;         // pinned: what read_scal waits for
+    unsigned post_seq;
     double *partials;           // device [max_blocks * 8]
     int max_blocks;
     unsigned *err_word;         // device error word of bounded waits
@@ -567,7 +574,8 @@ void net_free(fs_ctx *c);
 int net_load(fs_ctx *c, const float *params, int count, bool host);
 int net_read(fs_ctx *c, float *params_host);
 int net_kernel(fs_ctx *c, int which);  // fs_net.cu: inference layers, 0 mma.sync, 1 tcgen05
-int check_wait_error(fs_ctx *c, const char *what);  // fs_pcg.cu: bounded-wait errors of the last solve
+// fs_pcg.cu: the status of a solve whose error word (bounded waits) is herr
+int check_wait_error(fs_ctx *c, const char *what, unsigned herr);
 // cell space; z (zero off the liquid before) is written on the tiles that hold liquid; every kernel returns at
 // once when *done != 0 (done nullable)
 int net_apply(fs_ctx *c, const float *r, float *z, const int *done);

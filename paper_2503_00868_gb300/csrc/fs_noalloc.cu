@@ -112,8 +112,7 @@ extern "C" int fs_project_noalloc(int nx, int ny, int nz, const uint8_t *cell_ty
     c.scal = reinterpret_cast<SolveScal *>(take(4 * sizeof(SolveScal)));
     c.partials = reinterpret_cast<double *>(take((size_t)c.max_blocks * 8 * sizeof(double)));
     c.err_word = reinterpret_cast<unsigned *>(take(16));
-    SolveScal host_scal[4];
-    c.scal_host = host_scal;
+    c.post = nullptr;  // no pinned memory: the scalars are copied
 
     fs_default_params(&c.prm);
     c.prm.dx = dx;

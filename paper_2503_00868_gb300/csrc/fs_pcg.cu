@@ -10,7 +10,9 @@
 // host round trip; the host reads the convergence flag every `check_every`
 // iterations. Once `done` is set every later kernel of the batch returns at once.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <cstring>
 #include <utility>
 #include <vector>
 
@@ -690,17 +692,18 @@ struct TmaGrids {
 };
 
 // Iterations launched before each read of the convergence flag. A read costs a
-// host round trip with the GPU idle, and every iteration launched after
-// convergence costs its launches (each returns at once). With the count of the
-// last pass of the same kind known, the first batch runs one fewer than it and
-// later batches two at a time; otherwise `check` at a time.
+// host round trip with the GPU idle (5 us), and every iteration launched after
+// convergence its launches (each returns at once; about 1 us each, 15 in a multigrid
+// iteration). With the count of the last pass of the same kind known, the first batch
+// runs one fewer than it; later batches are one multigrid iteration, or two others.
+// Without it, `check` at a time.
 struct CgBatches {
     int first, later;
-    CgBatches(int last, int check, long long maxit)
+    CgBatches(int last, int check, long long maxit, bool mg)
     {
         const long long f = std::min<long long>((long long)last - 1, maxit);
         first = last > 1 ? (int)std::max<long long>(f, 1) : check;
-        later = last > 1 ? std::min(check, 2) : check;
+        later = last > 1 ? std::min(check, mg ? 1 : 2) : check;
     }
     int size(long long launched) const { return launched == 0 ? first : later; }
 };
@@ -712,13 +715,65 @@ int zmarch_slots(const fs_ctx *c, bool face)
     return c->num_sms * r;
 }
 
+namespace {
+// The scalars of a slot and the error word into pinned host memory, then the
+// sequence number that the host waits for.
+__global__ void k_post(const SolveScal *s, const unsigned *err, HostPost *out, unsigned seq)
+{
+    dep_wait();
+    const int t = threadIdx.x;
+    volatile unsigned *dst = reinterpret_cast<volatile unsigned *>(&out->s);
+    const volatile unsigned *src = reinterpret_cast<const volatile unsigned *>(s);
+    if (t < (int)(sizeof(SolveScal) / 4)) dst[t] = src[t];
+    if (t == 0) out->err = *(const volatile unsigned *)err;
+    __threadfence_system();
+    __syncthreads();
+    if (t == 0) *(volatile unsigned *)&out->seq = seq;
+}
+static_assert(sizeof(SolveScal) % 4 == 0 && sizeof(SolveScal) / 4 <= 128, "one word per thread of k_post");
+}  // namespace
+
+// A host read of the scalars happens several times per solve with the GPU idle
+// meanwhile. A copy and a stream synchronisation take about 17 us; a kernel that
+// writes the values and a sequence number to pinned memory, which the host polls,
+// about 5. Everything enqueued before it has then completed. The stream is queried
+// now and then, so that a failed launch ends the wait.
+int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err)
+{
+    HostPost *h = c->post;
+    if (!h) {  // a context without pinned memory
+        unsigned e = 0;
+        FS_CUDA(cudaMemcpyAsync(out, c->scal + which, sizeof(SolveScal), cudaMemcpyDeviceToHost, c->stream));
+        if (err) FS_CUDA(cudaMemcpyAsync(&e, c->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+        FS_CUDA(cudaStreamSynchronize(c->stream));
+        if (err) *err = e;
+        return FS_OK;
+    }
+    const unsigned seq = ++c->post_seq;
+    launch_dep(k_post, 1, 128, 0, c->stream, c->scal + which, c->err_word, h, seq);
+    FS_CUDA(cudaGetLastError());
+    volatile unsigned *flag = &h->seq;
+    for (unsigned n = 1; *flag != seq; n++) {
+        if (n % 4096) continue;
+        const cudaError_t e = cudaStreamQuery(c->stream);
+        if (e == cudaErrorNotReady) continue;
+        FS_CUDA(e);
+        if (*flag != seq) {  // the stream is empty: its writes are here, or the launch did not run
+            FS_CUDA(cudaStreamSynchronize(c->stream));
+            if (*flag != seq) return set_error(FS_ECUDA, "the solver's scalars were not posted");
+        }
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    std::memcpy(out, &h->s, sizeof(SolveScal));
+    if (err) *err = h->err;
+    prof_flush(c);
+    return FS_OK;
+}
+
 // A bounded wait of a TMA-fed kernel or of the MIC(0) wavefront that ran out
 // leaves a bit in the error word.
-int check_wait_error(fs_ctx *c, const char *what)
+int check_wait_error(fs_ctx *c, const char *what, unsigned herr)
 {
-    unsigned herr = 0;
-    FS_CUDA(cudaMemcpyAsync(&herr, c->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-    FS_CUDA(cudaStreamSynchronize(c->stream));
     if (herr & 1u) {
         c->mic_ready = 0;  // the factor may be incomplete: refactor on the next use
         return set_error(FS_ETIMEOUT, "MIC(0) sweep: a wait on a predecessor tile ran out (spin_limit %d)",
@@ -727,19 +782,6 @@ int check_wait_error(fs_ctx *c, const char *what)
     if (herr & ERR_TMA) return set_error(FS_ETIMEOUT, "%s: a wait for a tensor copy ran out", what);
     if (herr & 8u)  // the bit of the network's kernels
         return set_error(FS_ETIMEOUT, "%s: a bounded wait of the network ran out", what);
-    return FS_OK;
-}
-
-int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err)
-{
-    unsigned *eh = reinterpret_cast<unsigned *>(c->scal_host + 4);
-    FS_CUDA(cudaMemcpyAsync(c->scal_host + which, c->scal + which, sizeof(SolveScal), cudaMemcpyDeviceToHost,
-                            c->stream));
-    if (err) FS_CUDA(cudaMemcpyAsync(eh, c->err_word, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-    FS_CUDA(cudaStreamSynchronize(c->stream));
-    if (err) *err = *eh;
-    prof_flush(c);
-    *out = c->scal_host[which];
     return FS_OK;
 }
 
@@ -925,13 +967,12 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
             c->pb, c->px, c->pr, c->pp[0], c->pp[1], c->cflag, n4, tol2, c->prm.maxit_p, s, c->partials);
     if (!c->refining)
         if (int rc = try_warm_start(c, jac)) return rc;
-    if (!jac)
-        if (int rc = precondition(1)) return rc;
     c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
     const int bs = grid_blocks(c, L.nC, TH);
     const int b4 = grid_blocks(c, n4, TH);
     int cur = 0;
+    unsigned herr = 0;
     long long launched = 0;
     double by_spmv = (double)L.nC + 16.0 * (double)c->n_liquid;
     const double by_upd = (double)L.nC + 24.0 * (double)c->n_liquid;
@@ -948,10 +989,13 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     // a multigrid iteration costs several operator applies: check convergence more often
     const int check = c->prm.precond == FS_PRECOND_MG ? std::min(c->prm.check_every, 4) : c->prm.check_every;
     int &last = c->it_last_p[c->solve_kind & 1][c->refining ? 1 : 0];
-    const CgBatches batches(last, check, c->prm.maxit_p);
+    const CgBatches batches(last, check, c->prm.maxit_p, c->prm.precond == FS_PRECOND_MG);
     for (;;) {
         const int nb = batches.size(launched);
         for (int b = 0; b < nb; b++) {
+            // (at an iteration's start, so that none follows the last one)
+            if (!jac)
+                if (int rc = precondition(launched + b == 0)) return rc;
             const bool samp = c->prof_on && ((launched + b) % c->prof_period) == 0;  // every prof_period-th
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             const float *zsrc = jac ? c->pr : c->pz;
@@ -981,13 +1025,11 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
             prof_add(c, K_P_SPMV, e0, e1, by_spmv);
             prof_add(c, K_P_UPDATE, e2, e3, by_upd);
             c->n_launches += 2;
-            if (!jac)
-                if (int rc = precondition(0)) return rc;
             cur ^= 1;
         }
         launched += nb;
         FS_CUDA(cudaGetLastError());
-        int rc = read_scal(c, 0, &h);
+        int rc = read_scal(c, 0, &h, &herr);
         if (rc) return rc;
         if (h.done) break;
         if (launched > (long long)c->prm.maxit_p + c->prm.check_every)
@@ -997,7 +1039,7 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     prof_count(c, K_P_SPMV, h.iter);
     prof_count(c, K_P_UPDATE, h.iter);
     if (c->prm.precond == FS_PRECOND_MG) mg_count(c, h.iter, false);
-    return check_wait_error(c, "pressure solve");
+    return check_wait_error(c, "pressure solve", herr);
 }
 
 // At most this many refinement steps per solve (one suffices unless CG itself
@@ -1205,11 +1247,10 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
         FS_CUDA(cudaGetLastError());
         return FS_OK;
     };
-    if (mg)
-        if (int rc = precondition(1)) return rc;
     // a multigrid iteration costs several operator applies: check convergence more often
     const int check = mg ? std::min(c->prm.check_every, 4) : c->prm.check_every;
     int cur = 0;
+    unsigned herr = 0;
     long long launched = 0;
     SolveScal h;
     double by_spmv = (double)L.nF + 16.0 * (double)c->n_fluid;
@@ -1225,10 +1266,12 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     const dim3 tdim(TILE_X / 4, TILE_Y);
     const TmaGrids<HelmOp> tg(c, c->nitems_face, c->nact_face);
     int &last = c->it_last_v[dirichlet ? 1 : 0];
-    const CgBatches batches(last, check, c->prm.maxit_v);
+    const CgBatches batches(last, check, c->prm.maxit_v, mg);
     for (;;) {
         const int nb = batches.size(launched);
         for (int b = 0; b < nb; b++) {
+            if (mg)
+                if (int rc = precondition(launched + b == 0)) return rc;
             const bool samp = c->prof_on && ((launched + b) % c->prof_period) == 0;  // every prof_period-th
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             if (listed)
@@ -1258,20 +1301,18 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
             prof_add(c, K_V_SPMV, e0, e1, by_spmv);
             prof_add(c, K_V_UPDATE, e2, e3, by_upd);
             c->n_launches += 2;
-            if (mg)
-                if (int rc = precondition(0)) return rc;
             cur ^= 1;
         }
         launched += nb;
         FS_CUDA(cudaGetLastError());
-        int rc = read_scal(c, 1, &h);
+        int rc = read_scal(c, 1, &h, &herr);
         if (rc) return rc;
         if (h.done) break;
         if (launched > (long long)c->prm.maxit_v + c->prm.check_every)
             return set_error(FS_ECUDA, "viscosity solve: iteration flag never set");
     }
     last = h.status == FS_OK ? (int)std::min<long long>(h.iter, 1 << 20) : 0;
-    if (int rc = check_wait_error(c, "viscosity solve")) return rc;
+    if (int rc = check_wait_error(c, "viscosity solve", herr)) return rc;
     prof_count(c, K_V_SPMV, h.iter);
     prof_count(c, K_V_UPDATE, h.iter);
     if (mg) mg_count(c, h.iter, true);
