@@ -497,6 +497,12 @@ __device__ __forceinline__ float4 ldd4(const float *p)
     asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
+__device__ __forceinline__ float2 ldd2(const float *p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ float ldd1(const float *p)
 {
     float v;
@@ -506,12 +512,50 @@ __device__ __forceinline__ float ldd1(const float *p)
 
 // Walks a list of quads (or other entries): each thread strides through it with the
 // next entry fetched one step ahead, so no list load stands between a thread and its
-// data loads.
-#define FS_FOR_LIST(list, na)                                                                            \
-    for (int fl_i = blockIdx.x * blockDim.x + threadIdx.x, fl_st = gridDim.x * blockDim.x,               \
+// data loads. (PART: by the blk-th of nblk blocks.)
+#define FS_FOR_LIST_PART(list, na, blk, nblk)                                                            \
+    for (int fl_i = (blk) * blockDim.x + threadIdx.x, fl_st = (nblk) * blockDim.x,                       \
              q = fl_i < (na) ? __ldg((list) + fl_i) : 0, fl_next = 0;                                    \
-         fl_i < (na) && ((fl_next = fl_i + fl_st < (na) ? __ldg((list) + fl_i + fl_st) : 0), true);     \
+         fl_i < (na) && ((fl_next = fl_i + fl_st < (na) ? __ldg((list) + fl_i + fl_st) : 0), true);      \
          fl_i += fl_st, q = fl_next)
+#define FS_FOR_LIST(list, na) FS_FOR_LIST_PART(list, na, blockIdx.x, gridDim.x)
+
+// The same for stencils whose lanes take their x neighbours from one another. A list
+// is sorted, so a listed quad's neighbours in x are the entries before and after it,
+// and a quad that is not listed holds zeros. A warp therefore walks windows of 32
+// entries that overlap by two: lanes 1 to 30 own theirs (they alone store and sum),
+// lanes 0 and 31 only hold the neighbours of lanes 1 and 30. It spares the scalar
+// loads on each side of a quad, whose 32 lanes, 16 bytes apart, cost L1 as many
+// cycles as a whole float4. Every lane of a warp takes part in each step; past the
+// list's ends a lane repeats the end entry, which then links to nothing.
+constexpr unsigned FULL_WARP = 0xffffffffu;
+struct Links {
+    bool own, l, r;  // the lane's entry is its own; the left, right lane holds the quad before, after it
+    __device__ __forceinline__ float left(float last) const
+    {
+        const float v = __shfl_up_sync(FULL_WARP, last, 1);
+        return l ? v : 0.f;
+    }
+    __device__ __forceinline__ float right(float first) const
+    {
+        const float v = __shfl_down_sync(FULL_WARP, first, 1);
+        return r ? v : 0.f;
+    }
+};
+__device__ __forceinline__ Links links(int q, int i, int na)
+{
+    const int lane = threadIdx.x & 31;
+    const int a = __shfl_up_sync(FULL_WARP, q, 1), b = __shfl_down_sync(FULL_WARP, q, 1);
+    return {lane > 0 && lane < 31 && i < na, lane > 0 && a == q - 1, lane < 31 && b == q + 1};
+}
+inline long long linked_threads(long long na) { return (na + 29) / 30 * 32; }
+#define FS_FOR_LIST_LINKED(list, na, blk, nblk)                                                          \
+    for (int fl_b = (int)(((blk) * blockDim.x + threadIdx.x) >> 5) * 30,                                 \
+             fl_st = (int)(((nblk) * blockDim.x) >> 5) * 30, fl_i = fl_b + (int)(threadIdx.x & 31) - 1,  \
+             q = fl_b < (na) ? __ldg((list) + min(max(fl_i, 0), (na) - 1)) : 0, fl_next = 0;             \
+         fl_b < (na) &&                                                                                  \
+         ((fl_next = fl_b + fl_st < (na) ? __ldg((list) + min(fl_i + fl_st, (na) - 1)) : 0), true);      \
+         fl_b += fl_st, fl_i += fl_st, q = fl_next)
 
 // ---- launchers implemented in the .cu files --------------------------------
 // fs_mask.cu
@@ -534,6 +578,7 @@ int launch_nu_grad(fs_ctx *c, CF3 uv, double *dot);      // <vx, L~ uv>
 int launch_loss(fs_ctx *c, CF3 u, CF3 t, int kind, double alpha, double beta, F3 g,
                 double *loss);
 // fs_mg.cu
+int mg_prepare(fs_ctx *c, bool faces, float cc);
 int mg_apply(fs_ctx *c, const float *r, float *z, const int *done);
 int mg_apply_faces(fs_ctx *c, const float *r, float *z, float cc, const int *done);
 int cell_quads(fs_ctx *c, const int **ql, int *n);  // fs_mg.cu: the list of the current mask's active quads

@@ -27,7 +27,8 @@
 // The sweeps, the residual and the transfers take four elements per thread and
 // walk a list of a level's quads that hold an unknown (built with the hierarchy).
 // Every array a V-cycle writes is written only on those quads (with zeros on
-// their other elements) and is zero on every other quad: the work arrays are
+// their other elements) and is zero on every other quad (but for the residual's x
+// restriction, restrict_x): the work arrays are
 // zeroed when the hierarchy is built, and the level-0 output (the solver's z) is
 // a context buffer that is zeroed with each new mask and that every writer
 // leaves zero off the unknowns. So a stencil at the edge of the liquid reads
@@ -53,6 +54,29 @@ constexpr int MG_MAX_LEVELS = 16;
 constexpr int MG_COARSE_CELLS = 3072;  // padded cells of a level solved in shared memory
 constexpr int MG_COARSE_SWEEPS = 30;
 constexpr float MG_OMEGA = 0.8f;
+
+// n / d for n d < 2^32 by one high multiply (m = ceil(2^32 / d); d = 1 kept apart)
+struct FastDiv {
+    unsigned m, d;
+    __host__ __device__ FastDiv() : m(0), d(1) {}
+    __host__ __device__ explicit FastDiv(unsigned dv) : m(dv > 1 ? (unsigned)(((1ull << 32) + dv - 1) / dv) : 0u), d(dv) {}
+    __device__ __forceinline__ unsigned div(unsigned n) const { return d == 1 ? n : __umulhi(n, m); }
+    __device__ __forceinline__ void split(unsigned n, unsigned &q, unsigned &r) const
+    {
+        q = div(n);
+        r = n - q * d;
+    }
+    // any n: m exceeds 2^32 / d by less than 1, so the quotient is at most 1 too large
+    __device__ __forceinline__ void split_any(unsigned n, unsigned &q, unsigned &r) const
+    {
+        q = div(n);
+        r = n - q * d;
+        if (r >= d) {
+            q -= 1;
+            r += d;
+        }
+    }
+};
 
 // A level's array is `rows` rows of `sy` elements, `rpp` rows per plane; element
 // e of row w is cell (e - ioff, w % rpp - joff, w / rpp - koff). The set-up
@@ -93,6 +117,23 @@ struct MgSpace {
     MgGrid g[3];
     int base[3];
     int nv;
+    FastDiv dq[3], dr[3];  // by the quads of a row and the rows of a plane
+    void divisors()
+    {
+        for (int v = 0; v < nv; v++) {
+            dq[v] = FastDiv((unsigned)g[v].sy / 4);
+            dr[v] = FastDiv((unsigned)g[v].rpp);
+        }
+    }
+};
+
+// Where each volume's entries lie in a level's list: off[v] .. off[v + 1]. A launch
+// gives each volume the same number of blocks, so that its grid is uniform over a
+// block: picked per entry, its fields were loads from constant memory at a varying
+// index and sat among the instructions that bound the large levels' kernels.
+struct MgCut {
+    int off[4];
+    int blocks;  // per volume
 };
 
 // Volumes whose V-cycles run together, launch by launch: the cell space alone, or
@@ -106,8 +147,10 @@ struct MgSetLevel {
     MgSpace sp;
     uint8_t *fl = nullptr;
     float *r = nullptr, *a = nullptr, *b = nullptr, *c = nullptr;
+    float *d = nullptr;  // the residual's x restriction, half the level's length, behind b
     int *ql = nullptr, *pl = nullptr;
     int nq = 0, np = 0;
+    int qoff[4] = {0, 0, 0, 0}, poff[4] = {0, 0, 0, 0};
 };
 struct MgSet {
     int nv = 0, lf = 1;
@@ -123,12 +166,12 @@ struct MgSet {
 };
 
 // The pressure hierarchy and one per face volume (viscosity). The work arrays of
-// level 0 belong here: one pair of cell-space length, one of face-space length.
+// level 0 belong here (work_arrays), of cell-space and face-space length.
 struct MgAll {
     MgState cell, face[3];
     MgSet cset, fset[3];
     int nfset = 0;
-    float *cb = nullptr, *cc = nullptr, *fb = nullptr, *fc = nullptr;
+    float *cb = nullptr, *cc = nullptr, *fb = nullptr;
 };
 
 namespace {
@@ -138,12 +181,6 @@ const dim3 RT(32, 8);  // a warp along a row, 8 rows per block
 
 __device__ __forceinline__ bool liq(uint8_t f) { return f & CF_LIQ; }
 
-// A_l e at a liquid cell, without the scale
-__device__ __forceinline__ float lap(const float *__restrict__ e, int t, uint8_t f, const MgGrid &g)
-{
-    return (float)(f & CF_D) * e[t] - ((e[t - 1] + e[t + 1]) + (e[t - g.sy] + e[t + g.sy]) + (e[t - g.sz] + e[t + g.sz]));
-}
-
 // omega / (m + scale d), zero where the diagonal vanishes
 __device__ __forceinline__ float wtab_entry(float scale, float m, int d)
 {
@@ -151,13 +188,27 @@ __device__ __forceinline__ float wtab_entry(float scale, float m, int d)
     return dg > 0.f ? MG_OMEGA / dg : 0.f;
 }
 
-// the table for d = 0..7 in shared memory
-__device__ __forceinline__ void fill_wtab(float *wt, float scale, float m)
+// What a flag byte's low four bits (the count d and whether it is an unknown) stand
+// for, in shared memory: omega / (m + scale d), and that with m + scale d; zero off
+// the unknowns. The sweeps from zero form the first at five quads of r per quad, and
+// were bound by their instructions: a lookup takes a byte permute, the load and the
+// product, where testing and converting the byte took six.
+struct WTab {
+    float w[16];
+    float2 c[16];
+};
+__device__ __forceinline__ void fill_wtab(WTab &tab, float scale, float m)
 {
-    const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-    if (tid < 8) wt[tid] = wtab_entry(scale, m, tid);
+    const int i = threadIdx.x;
+    if (i < 16) {
+        const int d = i & CF_D;
+        const float w = i & CF_LIQ ? wtab_entry(scale, m, d) : 0.f;
+        tab.w[i] = w;
+        tab.c[i] = make_float2(w, i & CF_LIQ ? m + scale * (float)d : 0.f);
+    }
     __syncthreads();
 }
+static_assert((CF_D | CF_LIQ) == 15, "the table's index");
 
 // ---- four elements per thread -------------------------------------------------
 // Every level but the coarsest has a row pitch, plane stride and origin that are
@@ -171,12 +222,33 @@ __device__ __forceinline__ uchar4 ldf4(const uint8_t *__restrict__ p, int t)
 {
     return __ldg(reinterpret_cast<const uchar4 *>(p + t));
 }
+__device__ __forceinline__ unsigned ldw4(const uint8_t *__restrict__ p, int t)
+{
+    return __ldg(reinterpret_cast<const unsigned *>(p + t));
+}
+// the entries of element k of a quad's flag word W
+__device__ __forceinline__ float w_of(const WTab &tab, unsigned W, int k)
+{
+    return *reinterpret_cast<const float *>(reinterpret_cast<const char *>(tab.w) +
+                                            __byte_perm((W << 2) & 0x3c3c3c3cu, 0, 0x4440 | k));
+}
+__device__ __forceinline__ float2 c_of(const WTab &tab, unsigned W, int k)
+{
+    return *reinterpret_cast<const float2 *>(reinterpret_cast<const char *>(tab.c) +
+                                             __byte_perm((W << 3) & 0x78787878u, 0, 0x4440 | k));
+}
 __device__ __forceinline__ bool any_liq(uchar4 f) { return ((f.x | f.y | f.z | f.w) & CF_LIQ) != 0; }
 
-// e_out on one element from e_in: c (centre), the sum of its six neighbours nb
-__device__ __forceinline__ float sweep1(uint8_t f, float c, float nb, float rv, const float *wt, float scale, float m)
+// e_out on element k of a quad from e_in: c (centre), the sum of its six neighbours nb
+__device__ __forceinline__ float sweep1(const WTab &tab, unsigned W, int k, float c, float nb, float rv, float scale)
 {
-    return liq(f) ? c + wt[f & CF_D] * (rv - m * c - scale * ((float)(f & CF_D) * c - nb)) : 0.f;
+    const float2 t = c_of(tab, W, k);
+    return W & (CF_LIQ << 8 * k) ? c + t.x * (rv - (t.y * c - scale * nb)) : 0.f;
+}
+// r - A e there
+__device__ __forceinline__ float resid1(const WTab &tab, unsigned W, int k, float c, float nb, float rv, float scale)
+{
+    return W & (CF_LIQ << 8 * k) ? rv - (c_of(tab, W, k).y * c - scale * nb) : 0.f;
 }
 
 // The kernels below walk a level's list of active quads (those holding an
@@ -188,212 +260,254 @@ __device__ __forceinline__ float ldv1(const float *p, int t) { return ldd1(p + t
 
 // one damped Jacobi sweep on quad q: eout from ein; returns r.eout over the quad
 __device__ __forceinline__ float smooth_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
-                                          const float *ein, float *eout, const float *wt, float scale, float m, int q)
+                                          const float *ein, float *eout, const WTab &tab, float scale, int q)
 {
     const int t = q << 2;
-    const uchar4 f = ldf4(fl, t);
+    const unsigned W = ldw4(fl, t);
     const float4 c = ldv4(ein, t), rv = ldv4(r, t);
     const float4 dn = ldv4(ein, t - g.sy), up = ldv4(ein, t + g.sy);
     const float4 bk = ldv4(ein, t - g.sz), fw = ldv4(ein, t + g.sz);
     const float lf = ldv1(ein, t - 1), rt = ldv1(ein, t + 4);
     float4 v;
-    v.x = sweep1(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, wt, scale, m);
-    v.y = sweep1(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, wt, scale, m);
-    v.z = sweep1(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z, wt, scale, m);
-    v.w = sweep1(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w, wt, scale, m);
+    v.x = sweep1(tab, W, 0, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, scale);
+    v.y = sweep1(tab, W, 1, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, scale);
+    v.z = sweep1(tab, W, 2, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z, scale);
+    v.w = sweep1(tab, W, 3, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w, scale);
     *reinterpret_cast<float4 *>(eout + t) = v;
     return rv.x * v.x + rv.y * v.y + rv.z * v.z + rv.w * v.w;
 }
 
-// res = r - A e on quad q
-__device__ __forceinline__ void resid_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
-                                        const float *ev, float *res, float scale, float m, int q)
+// The x part of the restriction of a residual, v on the quad at element t of a
+// volume's array: coarse cell 2m (fine 4m - 1 .. 4m + 2) and 2m + 1 (fine 4m + 1 ..
+// 4m + 4) of the quad 4m .. 4m + 3, to elements t / 2 and t / 2 + 1 of d. So a residual
+// is written and read at half its size, and the restriction needs no x neighbours.
+// A neighbour that is not listed gets what this quad's end adds to it from here: its
+// own elements add nothing, and its two cells each border one quad only. Nothing is
+// added across the ends of a row.
+__device__ __forceinline__ void restrict_x(const MgGrid &g, FastDiv dq, Links lk, float4 v, float *d, int t)
+{
+    unsigned row, e;
+    dq.split_any((unsigned)t >> 2, row, e);
+    const int i = (int)(4 * e) - g.ioff;
+    const bool lin = i > 0, rin = i + 4 < g.nx;
+    const float l = lk.left(v.w), r = lk.right(v.x);
+    if (!lk.own) return;
+    float *o = d + (t >> 1);
+    *reinterpret_cast<float2 *>(o) =
+        make_float2(0.25f * (lin ? l : 0.f) + 0.75f * v.x + 0.75f * v.y + 0.25f * v.z,
+                    0.25f * v.y + 0.75f * v.z + 0.75f * v.w + 0.25f * (rin ? r : 0.f));
+    if (lin && !lk.l) o[-1] = 0.25f * v.x;
+    if (rin && !lk.r) o[2] = 0.25f * v.w;
+}
+
+// r - A e on quad q
+__device__ __forceinline__ float4 resid_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
+                                          const float *ev, const WTab &tab, float scale, int q, Links lk)
 {
     const int t = q << 2;
-    const uchar4 f = ldf4(fl, t);
+    const unsigned W = ldw4(fl, t);
     const float4 c = ldv4(ev, t), rv = ldv4(r, t);
     const float4 dn = ldv4(ev, t - g.sy), up = ldv4(ev, t + g.sy);
     const float4 bk = ldv4(ev, t - g.sz), fw = ldv4(ev, t + g.sz);
-    const float lf = ldv1(ev, t - 1), rt = ldv1(ev, t + 4);
-    auto one = [&](uint8_t fe, float ce, float nb, float re) {
-        return liq(fe) ? re - m * ce - scale * ((float)(fe & CF_D) * ce - nb) : 0.f;
-    };
+    const float lf = lk.left(c.w), rt = lk.right(c.x);
     float4 v;
-    v.x = one(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x);
-    v.y = one(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y);
-    v.z = one(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z);
-    v.w = one(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w);
-    *reinterpret_cast<float4 *>(res + t) = v;
+    v.x = resid1(tab, W, 0, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, scale);
+    v.y = resid1(tab, W, 1, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, scale);
+    v.z = resid1(tab, W, 2, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z, scale);
+    v.w = resid1(tab, W, 3, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w, scale);
+    return v;
+}
+
+// omega D^-1 r on the quad at element u
+__device__ __forceinline__ float4 jacobi_q(const uint8_t *__restrict__ fl, const float *r, const WTab &tab, int u)
+{
+    const unsigned W = ldw4(fl, u);
+    const float4 v = ldv4(r, u);
+    return make_float4(w_of(tab, W, 0) * v.x, w_of(tab, W, 1) * v.y, w_of(tab, W, 2) * v.z, w_of(tab, W, 3) * v.w);
 }
 
 // the first two sweeps from e = 0 on quad q: e1 = omega D^-1 r on the fly, then one sweep
 __device__ __forceinline__ void smooth2_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r, float *eo,
-                                          const float *wt, float scale, float m, int q)
+                                          const WTab &tab, float scale, int q, Links lk)
 {
     const int t = q << 2;
-    const uchar4 f = ldf4(fl, t);
-    auto e1q = [&](int u) {  // e1 on the quad at u
-        const uchar4 fu = ldf4(fl, u);
-        const float4 ru = ldv4(r, u);
-        return make_float4(liq(fu.x) ? wt[fu.x & CF_D] * ru.x : 0.f, liq(fu.y) ? wt[fu.y & CF_D] * ru.y : 0.f,
-                           liq(fu.z) ? wt[fu.z & CF_D] * ru.z : 0.f, liq(fu.w) ? wt[fu.w & CF_D] * ru.w : 0.f);
-    };
-    auto e1s = [&](int u) {
-        const uint8_t fu = fl[u];
-        return liq(fu) ? wt[fu & CF_D] * ldv1(r, u) : 0.f;
-    };
-    const float4 c = e1q(t), rv = ldv4(r, t);
-    const float4 dn = e1q(t - g.sy), up = e1q(t + g.sy), bk = e1q(t - g.sz), fw = e1q(t + g.sz);
-    const float lf = e1s(t - 1), rt = e1s(t + 4);
+    const unsigned W = ldw4(fl, t);
+    const float4 c = jacobi_q(fl, r, tab, t), rv = ldv4(r, t);
+    const float4 dn = jacobi_q(fl, r, tab, t - g.sy), up = jacobi_q(fl, r, tab, t + g.sy);
+    const float4 bk = jacobi_q(fl, r, tab, t - g.sz), fw = jacobi_q(fl, r, tab, t + g.sz);
+    const float lf = lk.left(c.w), rt = lk.right(c.x);
     float4 v;
-    v.x = sweep1(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, wt, scale, m);
-    v.y = sweep1(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, wt, scale, m);
-    v.z = sweep1(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z, wt, scale, m);
-    v.w = sweep1(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w, wt, scale, m);
-    *reinterpret_cast<float4 *>(eo + t) = v;
+    v.x = sweep1(tab, W, 0, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, scale);
+    v.y = sweep1(tab, W, 1, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, scale);
+    v.z = sweep1(tab, W, 2, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z, scale);
+    v.w = sweep1(tab, W, 3, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w, scale);
+    if (lk.own) *reinterpret_cast<float4 *>(eo + t) = v;
+}
+
+// cell (i, j, k) of element t of a volume's array
+__device__ __forceinline__ void cell_of(const MgGrid &g, FastDiv dq, FastDiv dr, int t, int &i, int &j, int &k)
+{
+    unsigned row, e, pl, r;
+    dq.split_any((unsigned)t >> 2, row, e);
+    dr.split_any(row, pl, r);
+    i = (int)(4 * e + ((unsigned)t & 3u)) - g.ioff;
+    j = (int)r - g.joff;
+    k = (int)pl - g.koff;
 }
 
 // e_fine += P e_coarse on the unknowns of an active quad q (in place). The quad's
 // elements i .. i + 3 (i a multiple of 4) take their x samples from coarse
-// I0 - 1 .. I0 + 2 (I0 = i / 2); indices past the coarse halo are clamped to it
-// (a sample that only padding elements use).
-__device__ __forceinline__ void prolong_q(const MgGrid &gf, const uint8_t *__restrict__ fl, float *ef,
-                                          const MgGrid &gc, const float *ec, int q)
+// I0 - 1 .. I0 + 2 (I0 = i / 2, even, so that I0 and I0 + 1 are one aligned load;
+// the outer two are the neighbour lanes' where those hold the row's next quads).
+// I0 + 2 past the coarse halo is clamped to it (a sample that only padding
+// elements use). With FIRST, e_fine before it is the sweep from zero, omega D^-1 r,
+// formed here.
+template <bool FIRST>
+__device__ __forceinline__ void prolong_q(const MgGrid &gf, FastDiv dq, FastDiv dr, const uint8_t *__restrict__ fl,
+                                          float *ef, const MgGrid &gc, const float *ec, const float *r,
+                                          const WTab &tab, int q, Links lk)
 {
-    const int qrow = gf.sy >> 2;
     const int t = q << 2;
     const uchar4 f = ldf4(fl, t);
-    const int row = q / qrow, e = (q - row * qrow) << 2;
-    const int i = e - gf.ioff, j = row % gf.rpp - gf.joff, k = row / gf.rpp - gf.koff;
+    int i, j, k;
+    cell_of(gf, dq, dr, t, i, j, k);
     const int I0 = i >> 1, J = j >> 1, K = k >> 1;
     const int J2 = (j & 1) ? J + 1 : J - 1, K2 = (k & 1) ? K + 1 : K - 1;
-    const int xs[4] = {max(I0 - 1, -1), I0, min(I0 + 1, gc.nx), min(I0 + 2, gc.nx)};
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    const int jj[2] = {J, J2}, kk[2] = {K, K2};
-    const float wy[2] = {0.75f, 0.25f};
+    const int xr = min(I0 + 2, gc.nx);
+    const bool ll = lk.l && i > 0, lr = lk.r && i + 4 < gf.nx;  // the neighbour's quad is in this row
+    const int base[4] = {gc.idx(0, J, K), gc.idx(0, J2, K), gc.idx(0, J, K2), gc.idx(0, J2, K2)};
+    const float w[4] = {0.5625f, 0.1875f, 0.1875f, 0.0625f};
+    float4 v = FIRST ? jacobi_q(fl, r, tab, t) : ldv4(ef, t);
+    // the y and z parts first: the neighbour lanes' quads of the row share them
+    float c0 = 0.f, c1 = 0.f, cm = 0.f, c2 = 0.f;
 #pragma unroll
-    for (int b = 0; b < 2; b++)
+    for (int x = 0; x < 4; x++) {
+        const float2 c = ldd2(ec + base[x] + I0);
+        c0 += w[x] * c.x;
+        c1 += w[x] * c.y;
+    }
+    if (!ll)
 #pragma unroll
-        for (int a = 0; a < 2; a++) {
-            const int base = gc.idx(0, jj[a], kk[b]);
-            const float w = wy[a] * wy[b];
-            const float cm = ldv1(ec, base + xs[0]), c0 = ldv1(ec, base + xs[1]);
-            const float c1 = ldv1(ec, base + xs[2]), c2 = ldv1(ec, base + xs[3]);
-            s0 += w * (0.75f * c0 + 0.25f * cm);
-            s1 += w * (0.75f * c0 + 0.25f * c1);
-            s2 += w * (0.75f * c1 + 0.25f * c0);
-            s3 += w * (0.75f * c1 + 0.25f * c2);
-        }
-    float4 v = ldv4(ef, t);
+        for (int x = 0; x < 4; x++) cm += w[x] * ldv1(ec, base[x] + I0 - 1);
+    if (!lr)
+#pragma unroll
+        for (int x = 0; x < 4; x++) c2 += w[x] * ldv1(ec, base[x] + xr);
+    const float sl = __shfl_up_sync(FULL_WARP, c1, 1), sr = __shfl_down_sync(FULL_WARP, c0, 1);
+    if (ll) cm = sl;
+    if (lr) c2 = sr;
+    const float s0 = 0.75f * c0 + 0.25f * cm, s1 = 0.75f * c0 + 0.25f * c1;
+    const float s2 = 0.75f * c1 + 0.25f * c0, s3 = 0.75f * c1 + 0.25f * c2;
     if (liq(f.x)) v.x += s0;
     if (liq(f.y)) v.y += s1;
     if (liq(f.z)) v.z += s2;
     if (liq(f.w)) v.w += s3;
-    *reinterpret_cast<float4 *>(ef + t) = v;
+    if (lk.own) *reinterpret_cast<float4 *>(ef + t) = v;
 }
 
 // Restriction of an active pair of the coarse level: t0 is the element of coarse
-// cell (2m, J, K), and the pair (2m, 2m + 1) holds at least one unknown. Per fine
-// row of the 4 x 4 window it reads the aligned quad 4m .. 4m + 3 and the scalars
-// at 4m - 1 and 4m + 4 (excluded at or past nx, where the next row begins), and
-// forms both cells' x weights from them.
-__device__ __forceinline__ void restrict_pair(const MgGrid &gf, const float *res, const MgGrid &gc,
-                                              const uint8_t *__restrict__ flc, float *rc, int t0)
+// cell (2m, J, K), and the pair (2m, 2m + 1) holds at least one unknown. It weighs
+// the x parts (restrict_x) of a 4 x 4 window of fine rows: all of it (WHOLE), or the
+// plane c of each of four lanes, 8 apart, that share the pair.
+template <bool WHOLE>
+__device__ __forceinline__ void restrict_pair(const MgGrid &gf, const float *d, const MgGrid &gc, FastDiv dq,
+                                              FastDiv dr, const uint8_t *__restrict__ flc, float *rc, int t0, int c,
+                                              bool own)
 {
-    const float w[4] = {0.25f, 0.75f, 0.75f, 0.25f};
-    const int rel = t0 - gc.origin;
-    const int K = rel / gc.sz, J = (rel - K * gc.sz) / gc.sy, I0 = rel - K * gc.sz - J * gc.sy;
-    const int m = I0 >> 1;
+    int I0, J, K;
+    cell_of(gc, dq, dr, t0, I0, J, K);
     const bool l0 = liq(flc[t0]), l1 = I0 + 1 < gc.nx && liq(flc[t0 + 1]);
-    float a0 = 0.f, a1 = 0.f;
     // A row off the grid counts nothing: its weight is zero and the pair's own row
-    // is read in its place, so that no branch stands between the 16 rows' loads
-    // (with a skip per row each waited for the one before it: 12 us for the 64^3
-    // level of the three face volumes of 128^3, and the sweeps 4).
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        const int k = 2 * K - 1 + c;
-        const bool kin = k >= 0 && k < gf.nz;
-#pragma unroll
-        for (int b = 0; b < 4; b++) {
-            const int j = 2 * J - 1 + b;
-            const bool in = kin && j >= 0 && j < gf.ny;
-            const int row = gf.idx(0, in ? j : 2 * J, in ? k : 2 * K) + 4 * m;  // a multiple of 4
-            const float4 qd = ldv4(res, row);
-            const float lf = ldv1(res, row - 1), rt = ldv1(res, row + 4);
-            const float wyz = in ? w[c] * w[b] : 0.f;
-            // coarse 2m: fine 4m - 1 .. 4m + 2; coarse 2m + 1: fine 4m + 1 .. 4m + 4
-            a0 += wyz * (0.25f * (m > 0 ? lf : 0.f) + 0.75f * qd.x + 0.75f * qd.y + 0.25f * qd.z);
-            a1 += wyz * (0.25f * qd.y + 0.75f * qd.z + 0.75f * qd.w + 0.25f * (4 * m + 4 < gf.nx ? rt : 0.f));
-        }
+    // is read in its place, so that no branch stands between the rows' loads (with a
+    // skip per row each waited for the one before it: 12 us for the 64^3 level of
+    // the three face volumes of 128^3, and the sweeps 4). Rows -1 and ny, planes -1
+    // and nz are the only ones off the grid.
+    const float wy0 = J > 0 ? 0.25f : 0.f, wy2 = 2 * J + 1 < gf.ny ? 0.75f : 0.f, wy3 = 2 * J + 2 < gf.ny ? 0.25f : 0.f;
+    const float wz0 = K > 0 ? 0.25f : 0.f, wz2 = 2 * K + 1 < gf.nz ? 0.75f : 0.f, wz3 = 2 * K + 2 < gf.nz ? 0.25f : 0.f;
+    const int y0 = J > 0 ? -gf.sy : 0, y2 = 2 * J + 1 < gf.ny ? gf.sy : 0, y3 = 2 * J + 2 < gf.ny ? 2 * gf.sy : 0;
+    const int z0 = K > 0 ? -gf.sz : 0, z2 = 2 * K + 1 < gf.nz ? gf.sz : 0, z3 = 2 * K + 2 < gf.nz ? 2 * gf.sz : 0;
+    const int own_row = gf.idx(0, 2 * J, 2 * K) + 2 * I0;  // a multiple of 4
+    float a0 = 0.f, a1 = 0.f;
+    auto plane = [&](int z, float wz) {
+        const int p = own_row + z;
+        const float2 x0 = ldd2(d + ((p + y0) >> 1)), x1 = ldd2(d + (p >> 1));
+        const float2 x2 = ldd2(d + ((p + y2) >> 1)), x3 = ldd2(d + ((p + y3) >> 1));
+        a0 += wz * (wy0 * x0.x + 0.75f * x1.x + wy2 * x2.x + wy3 * x3.x);
+        a1 += wz * (wy0 * x0.y + 0.75f * x1.y + wy2 * x2.y + wy3 * x3.y);
+    };
+    if (WHOLE) {
+        plane(z0, wz0);
+        plane(0, 0.75f);
+        plane(z2, wz2);
+        plane(z3, wz3);
+        if (own && l0) rc[t0] = 0.125f * a0;
+        if (own && l1) rc[t0 + 1] = 0.125f * a1;
+        return;
     }
-    if (l0) rc[t0] = 0.125f * a0;
-    if (l1) rc[t0 + 1] = 0.125f * a1;
+    plane(c == 0 ? z0 : c == 1 ? 0 : c == 2 ? z2 : z3, c == 0 ? wz0 : c == 1 ? 0.75f : c == 2 ? wz2 : wz3);
+#pragma unroll
+    for (int o = 8; o < 32; o *= 2) {
+        a0 += __shfl_xor_sync(FULL_WARP, a0, o);
+        a1 += __shfl_xor_sync(FULL_WARP, a1, o);
+    }
+    if (own && c == 0 && l0) rc[t0] = 0.125f * a0;
+    if (own && c == 1 && l1) rc[t0 + 1] = 0.125f * a1;
 }
 
-// one damped Jacobi sweep from zero and the residual it leaves, on quad q:
-// eb = e1 = omega D^-1 r at the quad, res = r - A e1 (e1 at the neighbours formed
-// on the fly)
-__device__ __forceinline__ void pre1_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r, float *eb,
-                                       float *res, const float *wt, float scale, float m, int q)
+// r - A e1 on quad q for the damped Jacobi sweep from zero, e1 = omega D^-1 r
+// (formed on the fly, here and where it is used again)
+__device__ __forceinline__ float4 pre1_q(const MgGrid &g, const uint8_t *__restrict__ fl, const float *r,
+                                         const WTab &tab, float scale, int q, Links lk)
 {
     const int t = q << 2;
-    const uchar4 f = ldf4(fl, t);
-    auto e1q = [&](int u) {  // e1 on the quad at u
-        const uchar4 fu = ldf4(fl, u);
-        const float4 ru = ldv4(r, u);
-        return make_float4(liq(fu.x) ? wt[fu.x & CF_D] * ru.x : 0.f, liq(fu.y) ? wt[fu.y & CF_D] * ru.y : 0.f,
-                           liq(fu.z) ? wt[fu.z & CF_D] * ru.z : 0.f, liq(fu.w) ? wt[fu.w & CF_D] * ru.w : 0.f);
-    };
-    auto e1s = [&](int u) {
-        const uint8_t fu = fl[u];
-        return liq(fu) ? wt[fu & CF_D] * ldv1(r, u) : 0.f;
-    };
-    const float4 c = e1q(t), rv = ldv4(r, t);
-    const float4 dn = e1q(t - g.sy), up = e1q(t + g.sy), bk = e1q(t - g.sz), fw = e1q(t + g.sz);
-    const float lf = e1s(t - 1), rt = e1s(t + 4);
-    auto one = [&](uint8_t fe, float ce, float nb, float re) {
-        return liq(fe) ? re - m * ce - scale * ((float)(fe & CF_D) * ce - nb) : 0.f;
-    };
+    const unsigned W = ldw4(fl, t);
+    const float4 c = jacobi_q(fl, r, tab, t), rv = ldv4(r, t);
+    const float4 dn = jacobi_q(fl, r, tab, t - g.sy), up = jacobi_q(fl, r, tab, t + g.sy);
+    const float4 bk = jacobi_q(fl, r, tab, t - g.sz), fw = jacobi_q(fl, r, tab, t + g.sz);
+    const float lf = lk.left(c.w), rt = lk.right(c.x);
     float4 v;
-    v.x = one(f.x, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x);
-    v.y = one(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y);
-    v.z = one(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z);
-    v.w = one(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w);
-    *reinterpret_cast<float4 *>(eb + t) = c;
-    *reinterpret_cast<float4 *>(res + t) = v;
+    v.x = resid1(tab, W, 0, c.x, (lf + c.y) + (dn.x + up.x) + (bk.x + fw.x), rv.x, scale);
+    v.y = resid1(tab, W, 1, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y), rv.y, scale);
+    v.z = resid1(tab, W, 2, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z), rv.z, scale);
+    v.w = resid1(tab, W, 3, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w), rv.w, scale);
+    return v;
 }
 
 // ---- one launch per step ------------------------------------------------------
-// Each walks one list over every volume of a level.
+// Each walks one list over every volume of a level, with blocks of its own for
+// each volume.
 
-// the volume of an element of a level's arrays
-__device__ __forceinline__ int vol_of(const MgSpace &S, int t)
-{
-    return S.nv > 1 ? (t >= S.base[1]) + (t >= S.base[2]) : 0;
-}
+// What bounds them (measured one by one): above a few million unknowns the bytes,
+// and for the kernels that form a sweep on the fly or take two grids the
+// instructions; below, latency (a launch, the list, the loads). The three face
+// volumes at 256^3, 28 M unknowns: pre1 66 us (with a test and a conversion of each
+// flag byte 73), prolong 51 (56), smooth 59, near its bytes at 6.9 TB/s.
+// The sweeps that are not followed by a restriction keep the plain walk: windows of
+// 30 quads start off a 128-byte line, which cost a sweep 4% there.
 
 // One sweep over the active quads. With rzs (the last sweep of a V-cycle's level
 // 0), it also forms r.eout, which is the solver's r.z: each block's compensated
 // sum goes to the partials as block boff + blockIdx.x of btot (the blocks of the
 // face volumes' launches together), and the last block to arrive sets beta =
 // rz_new / rz (first: 0) and rz, as the solver's separate r.z pass does.
-__global__ void __launch_bounds__(256) k_mg0_smooth(const MgSpace S, const int *__restrict__ qlist, int na,
+__global__ void __launch_bounds__(256) k_mg0_smooth(const __grid_constant__ MgSpace S, const int *__restrict__ qlist, const __grid_constant__ MgCut cut,
                                                     const uint8_t *__restrict__ fl, const float *__restrict__ r,
                                                     const float *__restrict__ ein, float *eout, float scale, float m,
                                                     const int *done, SolveScal *rzs, double *partials, int first)
 {
-    __shared__ float wt[8];
-    fill_wtab(wt, scale, m);
+    __shared__ WTab tab;
+    fill_wtab(tab, scale, m);
     dep_wait();
     dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
     KSum acc;
-    FS_FOR_LIST(qlist, na) acc.add(smooth_q(S.g[vol_of(S, 4 * q)], fl, r, ein, eout, wt, scale, m, q));
+    const int v = blockIdx.x / cut.blocks, blk = blockIdx.x - v * cut.blocks;
+    const int na = cut.off[v + 1] - cut.off[v];
+    FS_FOR_LIST_PART(qlist + cut.off[v], na, blk, cut.blocks)
+    acc.add(smooth_q(S.g[v], fl, r, ein, eout, tab, scale, q));
     if (!rzs || *(volatile const int *)&rzs->done) return;  // (a timed sweep runs after convergence too)
-    KSum v[1] = {acc};
+    KSum sum[1] = {acc};
     double tot[1];
-    if (grid_reduce<1>(v, partials, &rzs->ticket, tot) && threadIdx.x == 0) {
+    if (grid_reduce<1>(sum, partials, &rzs->ticket, tot) && threadIdx.x == 0) {
         if (!isfinite(tot[0])) {
             rzs->done = 1;
             rzs->status = FS_ENONFINITE;
@@ -404,67 +518,108 @@ __global__ void __launch_bounds__(256) k_mg0_smooth(const MgSpace S, const int *
     }
 }
 
-__global__ void __launch_bounds__(256) k_mg0_pre1(const MgSpace S, const int *__restrict__ qlist, int na,
+__global__ void __launch_bounds__(256, 6) k_mg0_pre1(const __grid_constant__ MgSpace S, const int *__restrict__ qlist, const __grid_constant__ MgCut cut,
                                                   const uint8_t *__restrict__ fl, const float *__restrict__ r,
-                                                  float *eb, float *res, float scale, float m, const int *done)
+                                                  float *d, float scale, float m, const int *done)
 {
-    __shared__ float wt[8];
-    fill_wtab(wt, scale, m);
+    __shared__ WTab tab;
+    fill_wtab(tab, scale, m);
     dep_wait();
     dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    FS_FOR_LIST(qlist, na) pre1_q(S.g[vol_of(S, 4 * q)], fl, r, eb, res, wt, scale, m, q);
-}
-
-__global__ void __launch_bounds__(256, 8) k_mg0_residual(const MgSpace S, const int *__restrict__ qlist, int na,
-                                                      const uint8_t *__restrict__ fl, const float *__restrict__ r,
-                                                      const float *__restrict__ ev, float *res, float scale, float m,
-                                                      const int *done)
-{
-    dep_wait();
-    dep_go();
-    if (done && *(volatile const int *)done) return;  // the solve has converged
-    FS_FOR_LIST(qlist, na) resid_q(S.g[vol_of(S, 4 * q)], fl, r, ev, res, scale, m, q);
-}
-
-__global__ void __launch_bounds__(256) k_mg0_smooth2(const MgSpace S, const int *__restrict__ qlist, int na,
-                                                     const uint8_t *__restrict__ fl, const float *__restrict__ r,
-                                                     float *eo, float scale, float m, const int *done)
-{
-    __shared__ float wt[8];
-    fill_wtab(wt, scale, m);
-    dep_wait();
-    dep_go();
-    if (done && *(volatile const int *)done) return;  // the solve has converged
-    FS_FOR_LIST(qlist, na) smooth2_q(S.g[vol_of(S, 4 * q)], fl, r, eo, wt, scale, m, q);
-}
-
-__global__ void __launch_bounds__(256) k_mg0_prolong(const MgSpace S, const MgSpace Sc, const int *__restrict__ qlist,
-                                                     int na, const uint8_t *__restrict__ fl, float *ef,
-                                                     const float *__restrict__ ec, const int *done)
-{
-    dep_wait();
-    dep_go();
-    if (done && *(volatile const int *)done) return;  // the solve has converged
-    FS_FOR_LIST(qlist, na)
+    const int v = blockIdx.x / cut.blocks, blk = blockIdx.x - v * cut.blocks, base = S.base[v];
+    const int na = cut.off[v + 1] - cut.off[v];
+    FS_FOR_LIST_LINKED(qlist + cut.off[v], na, blk, cut.blocks)
     {
-        const int v = vol_of(S, 4 * q), base = S.base[v];
-        prolong_q(S.g[v], fl + base, ef + base, Sc.g[v], ec + Sc.base[v], q - (base >> 2));
+        const Links lk = links(q, fl_i, na);
+        const float4 res = pre1_q(S.g[v], fl, r, tab, scale, q, lk);
+        restrict_x(S.g[v], S.dq[v], lk, res, d + (base >> 1), 4 * q - base);
     }
 }
 
-// restriction over the coarse level's list of active pairs
-__global__ void __launch_bounds__(256) k_mg0_restrict(const MgSpace S, const float *__restrict__ res, const MgSpace Sc,
-                                                      const int *__restrict__ plist, int np,
+__global__ void __launch_bounds__(256, 6) k_mg0_residual(const __grid_constant__ MgSpace S, const int *__restrict__ qlist, const __grid_constant__ MgCut cut,
+                                                      const uint8_t *__restrict__ fl, const float *__restrict__ r,
+                                                      const float *__restrict__ ev, float *d, float scale, float m,
+                                                      const int *done)
+{
+    __shared__ WTab tab;
+    fill_wtab(tab, scale, m);
+    dep_wait();
+    dep_go();
+    if (done && *(volatile const int *)done) return;  // the solve has converged
+    const int v = blockIdx.x / cut.blocks, blk = blockIdx.x - v * cut.blocks, base = S.base[v];
+    const int na = cut.off[v + 1] - cut.off[v];
+    FS_FOR_LIST_LINKED(qlist + cut.off[v], na, blk, cut.blocks)
+    {
+        const Links lk = links(q, fl_i, na);
+        const float4 res = resid_q(S.g[v], fl, r, ev, tab, scale, q, lk);
+        restrict_x(S.g[v], S.dq[v], lk, res, d + (base >> 1), 4 * q - base);
+    }
+}
+
+__global__ void __launch_bounds__(256, 6) k_mg0_smooth2(const __grid_constant__ MgSpace S, const int *__restrict__ qlist, const __grid_constant__ MgCut cut,
+                                                     const uint8_t *__restrict__ fl, const float *__restrict__ r,
+                                                     float *eo, float scale, float m, const int *done)
+{
+    __shared__ WTab tab;
+    fill_wtab(tab, scale, m);
+    dep_wait();
+    dep_go();
+    if (done && *(volatile const int *)done) return;  // the solve has converged
+    const int v = blockIdx.x / cut.blocks, blk = blockIdx.x - v * cut.blocks;
+    const int na = cut.off[v + 1] - cut.off[v];
+    FS_FOR_LIST_LINKED(qlist + cut.off[v], na, blk, cut.blocks)
+    smooth2_q(S.g[v], fl, r, eo, tab, scale, q, links(q, fl_i, na));
+}
+
+template <bool FIRST>
+__global__ void __launch_bounds__(256) k_mg0_prolong(const __grid_constant__ MgSpace S, const __grid_constant__ MgSpace Sc, const int *__restrict__ qlist,
+                                                     const __grid_constant__ MgCut cut, const uint8_t *__restrict__ fl, float *ef,
+                                                     const float *__restrict__ ec, const float *r, float scale, float m,
+                                                     const int *done)
+{
+    __shared__ WTab tab;
+    if (FIRST) fill_wtab(tab, scale, m);
+    dep_wait();
+    dep_go();
+    if (done && *(volatile const int *)done) return;  // the solve has converged
+    const int v = blockIdx.x / cut.blocks, blk = blockIdx.x - v * cut.blocks, base = S.base[v];
+    const int na = cut.off[v + 1] - cut.off[v];
+    FS_FOR_LIST_LINKED(qlist + cut.off[v], na, blk, cut.blocks)
+    {
+        prolong_q<FIRST>(S.g[v], S.dq[v], S.dr[v], fl + base, ef + base, Sc.g[v], ec + Sc.base[v], r + base, tab,
+                         q - (base >> 2), links(q, fl_i, na));
+    }
+}
+
+// Restriction over the coarse level's list of active pairs. Pairs take a thread each
+// (WHOLE): the index arithmetic bounds the large levels (the three face volumes,
+// 28 M unknowns at 256^3: 20 us against 37 with four lanes per pair, and 45 over whole
+// residuals with their x neighbours; 3.4 M at 128^3: 7.4 against 9.3 and 13.5). Where
+// four lanes per pair fit in one wave they are used, for four times the loads in
+// flight (the 64^3 level below a pressure blob: 4.7 us against 6.0 and 9.1).
+template <bool WHOLE>
+__global__ void __launch_bounds__(256) k_mg0_restrict(const __grid_constant__ MgSpace S, const float *__restrict__ d,
+                                                      const __grid_constant__ MgSpace Sc,
+                                                      const int *__restrict__ plist, const __grid_constant__ MgCut cut,
                                                       const uint8_t *__restrict__ flc, float *rc, const int *done)
 {
     dep_wait();
     dep_go();
     if (done && *(volatile const int *)done) return;  // the solve has converged
-    FS_FOR_LIST(plist, np)
-    {
-        const int v = vol_of(Sc, q), base = Sc.base[v];
-        restrict_pair(S.g[v], res + S.base[v], Sc.g[v], flc + base, rc + base, q - base);
+    const int v = blockIdx.x / cut.blocks, blk = blockIdx.x - v * cut.blocks, base = Sc.base[v];
+    const int np = cut.off[v + 1] - cut.off[v];
+    plist += cut.off[v];
+    // a warp takes 32 or 8 consecutive pairs, all lanes in each step
+    constexpr int PER = WHOLE ? 32 : 8;
+    const int lane = threadIdx.x & 31, st = cut.blocks * (int)(blockDim.x >> 5) * PER;
+    int i = (int)((blk * blockDim.x + threadIdx.x) >> 5) * PER + (lane & (PER - 1));
+    int next = (i & ~(PER - 1)) < np ? __ldg(plist + min(i, np - 1)) : 0;
+    for (; (i & ~(PER - 1)) < np; i += st) {
+        const int q = next;
+        next = (i & ~(PER - 1)) + st < np ? __ldg(plist + min(i + st, np - 1)) : 0;
+        restrict_pair<WHOLE>(S.g[v], d + (S.base[v] >> 1), Sc.g[v], Sc.dq[v], Sc.dr[v], flc + base, rc + base, q - base,
+                             lane >> 3, i < np);
     }
 }
 
@@ -691,15 +846,17 @@ void free_set(MgSet *t)
 
 // Resident blocks per SM of the list-walking kernels, for one-wave grids.
 struct MgResidency {
-    int smooth2, residual, pre1, restrict_, prolong, smooth;
+    int smooth2, residual, pre1, whole, split, prolong, first, smooth;
 };
 const MgResidency &mg_residency()
 {
     static const MgResidency r{resident_blocks((const void *)k_mg0_smooth2, 0),
                                resident_blocks((const void *)k_mg0_residual, 0),
                                resident_blocks((const void *)k_mg0_pre1, 0),
-                               resident_blocks((const void *)k_mg0_restrict, 0),
-                               resident_blocks((const void *)k_mg0_prolong, 0),
+                               resident_blocks((const void *)k_mg0_restrict<true>, 0),
+                               resident_blocks((const void *)k_mg0_restrict<false>, 0),
+                               resident_blocks((const void *)k_mg0_prolong<false>, 0),
+                               resident_blocks((const void *)k_mg0_prolong<true>, 0),
                                resident_blocks((const void *)k_mg0_smooth, 0)};
     return r;
 }
@@ -805,8 +962,8 @@ int count_bytes(fs_ctx *c, MgSet &t)
     FS_CUDA(cudaStreamSynchronize(c->stream));
     const double u0 = (double)nl[0], u1 = (double)nl[1], q0 = (double)t.lev[0].nq, p1 = (double)t.lev[1].np;
     t.by0[0] = 8.0 * q0 + 8.0 * u0;             // smooth2: read r, write e
-    t.by0[1] = 8.0 * q0 + 12.0 * u0;            // residual: read r, e, write res
-    t.by0[2] = 6.0 * p1 + 4.0 * u0 + 4.0 * u1;  // restrict: pair list and flags, read res, write level-1 r
+    t.by0[1] = 8.0 * q0 + 10.0 * u0;            // residual: read r, e, write its x restriction
+    t.by0[2] = 6.0 * p1 + 2.0 * u0 + 4.0 * u1;  // restrict: pair list and flags, read that, write level-1 r
     t.by0[3] = 8.0 * q0 + 8.0 * u0 + 4.0 * u1;  // prolong: read and write e, read the level-1 e
     t.by0[4] = 8.0 * q0 + 12.0 * u0;            // smooth: read r, e, write e
     t.by0[5] = 8.0 * q0 + 12.0 * u0;            // last smooth: read r, e, write z
@@ -835,27 +992,44 @@ int vcycle(fs_ctx *c, MgSet &t, const float *r, float *z, const int *done_, bool
     // its resident blocks (the volumes of a set share their scale)
     const MgResidency &res = mg_residency();
     cudaStream_t st = c->stream;
+    auto cut = [&](const int *off, int kind, int resident) {  // kind: threads per entry, or 0 for linked quads
+        MgCut m;
+        long long most = 0;
+        for (int v = 0; v < 4; v++) m.off[v] = off[v];
+        for (int v = 0; v < t.nv; v++) {
+            const long long n = off[v + 1] - off[v];
+            most = std::max(most, kind ? kind * n : linked_threads(n));
+        }
+        m.blocks = (int)std::max(1LL, std::min((most + TH - 1) / TH, (long long)c->num_sms * std::max(resident, 1) / t.nv));
+        return m;
+    };
+    MgCut k;
     for (int l = 0; l < t.lf; l++) {
         MgSetLevel &v = t.lev[l], &w = t.lev[l + 1];
         const float *rl = l == 0 ? r : v.r, scale = s0.lev[l].scale, mass = s0.lev[l].mass;
         const int *done = sample && l == 0 ? nullptr : done_;
         if (l == 0 && t.one) {  // the sweep from zero and the residual it leaves, in one pass
-            launch_dep(k_mg0_pre1, wave_blocks(c, v.nq, res.pre1), TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass,
-                                                                      done);
+            k = cut(v.qoff, 0, res.pre1);
+            launch_dep(k_mg0_pre1, k.blocks * t.nv, TH, 0, st, v.sp, v.ql, k, v.fl, rl, v.d, scale, mass,
+                       done);
             c->n_launches += 1;
         } else {
+            k = cut(v.qoff, 0, res.smooth2);
             begin(l);
-            launch_dep(k_mg0_smooth2, wave_blocks(c, v.nq, res.smooth2), TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, scale,
-                                                                            mass, done);
+            launch_dep(k_mg0_smooth2, k.blocks * t.nv, TH, 0, st, v.sp, v.ql, k, v.fl, rl, v.b, scale,
+                       mass, done);
             end(l, K_MG0_SMOOTH2, t.by0[0]);
+            k = cut(v.qoff, 0, res.residual);
             begin(l);
-            launch_dep(k_mg0_residual, wave_blocks(c, v.nq, res.residual), TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c,
-                                                                              scale, mass, done);
+            launch_dep(k_mg0_residual, k.blocks * t.nv, TH, 0, st, v.sp, v.ql, k, v.fl, rl, v.b, v.d,
+                       scale, mass, done);
             end(l, K_MG0_RESIDUAL, t.by0[1]);
             c->n_launches += 2;
         }
+        const bool whole = 4LL * w.np > (long long)c->num_sms * res.split * TH;
+        k = cut(w.poff, whole ? 1 : 4, whole ? res.whole : res.split);
         begin(l);
-        launch_dep(k_mg0_restrict, wave_blocks(c, w.np, res.restrict_), TH, 0, st, v.sp, v.c, w.sp, w.pl, w.np, w.fl, w.r,
+        launch_dep(whole ? k_mg0_restrict<true> : k_mg0_restrict<false>, k.blocks * t.nv, TH, 0, st, v.sp, v.d, w.sp, w.pl, k, w.fl, w.r,
                                                                            done);
         end(l, K_MG0_RESTRICT, t.by0[2]);
         c->n_launches += 1;
@@ -872,23 +1046,26 @@ int vcycle(fs_ctx *c, MgSet &t, const float *r, float *z, const int *done_, bool
         MgSetLevel &v = t.lev[l], &w = t.lev[l + 1];
         const float *rl = l == 0 ? r : v.r, scale = s0.lev[l].scale, mass = s0.lev[l].mass;
         const int *done = sample && l == 0 ? nullptr : done_;
-        const int nb = wave_blocks(c, v.nq, res.smooth);
         end(l, K_MG_COARSE, 0.0);
         begin(l);
-        launch_dep(k_mg0_prolong, wave_blocks(c, v.nq, res.prolong), TH, 0, st, v.sp, w.sp, v.ql, v.nq, v.fl, v.b, w.a, done);
+        const bool one = l == 0 && t.one;
+        k = cut(v.qoff, 0, one ? res.first : res.prolong);
+        launch_dep(one ? k_mg0_prolong<true> : k_mg0_prolong<false>, k.blocks * t.nv, TH, 0, st, v.sp, w.sp, v.ql,
+                   k, v.fl, v.b, w.a, rl, scale, mass, done);
         end(l, K_MG0_PROLONG, t.by0[3]);
         const float *ez = v.c;  // the input of the last sweep
+        k = cut(v.qoff, 1, res.smooth);
         if (l == 0 && t.one) {
             ez = v.b;
         } else {
             begin(l);
-            launch_dep(k_mg0_smooth, nb, TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, v.b, v.c, scale, mass, done, nullptr, nullptr,
+            launch_dep(k_mg0_smooth, k.blocks * t.nv, TH, 0, st, v.sp, v.ql, k, v.fl, rl, v.b, v.c, scale, mass, done, nullptr, nullptr,
                                             0);
             end(l, K_MG0_SMOOTH, t.by0[4]);
             c->n_launches += 1;
         }
         begin(l);
-        launch_dep(k_mg0_smooth, nb, TH, 0, st, v.sp, v.ql, v.nq, v.fl, rl, ez, l == 0 ? z : v.a, scale, mass, done,
+        launch_dep(k_mg0_smooth, k.blocks * t.nv, TH, 0, st, v.sp, v.ql, k, v.fl, rl, ez, l == 0 ? z : v.a, scale, mass, done,
                                         l == 0 ? rzs : nullptr, c->partials, first);
         end(l, K_MG0_SMOOTH_Z, t.by0[5]);
         c->n_launches += 2;
@@ -934,9 +1111,10 @@ int plan_levels(fs_ctx *c, MgState *s, const MgGrid &g0, float coef, float mass)
     return FS_OK;
 }
 
-// A list over the volumes of a level of a set, in order: counted, allocated, filled.
+// A list over the volumes of a level of a set, in order: counted, allocated, filled;
+// off[v] is where volume v begins (the whole count past the last).
 template <class P>
-int make_list(fs_ctx *c, const MgSetLevel &v, long long (*items)(const MgGrid &), int **list, int *count)
+int make_list(fs_ctx *c, const MgSetLevel &v, long long (*items)(const MgGrid &), int **list, int *count, int *off)
 {
     int *dcnt = nullptr;
     std::vector<int> hcnt;
@@ -974,6 +1152,7 @@ int make_list(fs_ctx *c, const MgSetLevel &v, long long (*items)(const MgGrid &)
         total += n;
     }
     *count = total;
+    for (int k = 0; k < 4; k++) off[k] = k < v.sp.nv ? hcnt[boff[k]] : total;
     if (cudaMalloc(list, sizeof(int) * (size_t)std::max(total, 1)) != cudaSuccess) {
         cudaGetLastError();
         *list = nullptr;
@@ -1012,17 +1191,21 @@ int build_set(fs_ctx *c, MgSet &t)
             x.sp.base[v] = (int)n;
             if (l < t.s[v]->nlev) n += (size_t)x.sp.g[v].n;
         }
+        x.sp.divisors();
         if (l == 0) {
             for (int v = 0; v < t.nv; v++) t.s[v]->lev[0].fl = x.fl + x.sp.base[v];
             continue;
         }
         bool ok = cudaMalloc(&x.fl, n) == cudaSuccess;
-        for (float **p : {&x.r, &x.a, &x.b, &x.c}) ok = ok && cudaMalloc(p, n * 4) == cudaSuccess;
+        for (float **p : {&x.r, &x.a, &x.c}) ok = ok && cudaMalloc(p, n * 4) == cudaSuccess;
+        ok = ok && cudaMalloc(&x.b, n * 6) == cudaSuccess;
         if (!ok) {
             cudaGetLastError();
             return set_error(FS_ENOMEM, "multigrid level arrays");
         }
-        for (float *p : {x.r, x.a, x.b, x.c}) FS_CUDA(cudaMemsetAsync(p, 0, n * 4, c->stream));
+        for (float *p : {x.r, x.a, x.c}) FS_CUDA(cudaMemsetAsync(p, 0, n * 4, c->stream));
+        FS_CUDA(cudaMemsetAsync(x.b, 0, n * 6, c->stream));
+        x.d = x.b + n;
         for (int v = 0; v < t.nv; v++) {
             if (l >= t.s[v]->nlev) continue;
             MgLevel &L = t.s[v]->lev[l];
@@ -1070,10 +1253,10 @@ int build_set(fs_ctx *c, MgSet &t)
         MgSetLevel &x = t.lev[l];
         int rc = FS_OK;
         if (l < t.lf && !x.ql)
-            rc = make_list<QuadPred>(c, x, quad_items, &x.ql, &x.nq);
+            rc = make_list<QuadPred>(c, x, quad_items, &x.ql, &x.nq, x.qoff);
         if (!rc && l > 0)
             rc = make_list<PairPred>(
-                c, x, [](const MgGrid &g) { return (long long)((g.nx + 1) >> 1) * g.ny * g.nz; }, &x.pl, &x.np);
+                c, x, [](const MgGrid &g) { return (long long)((g.nx + 1) >> 1) * g.ny * g.nz; }, &x.pl, &x.np, x.poff);
         if (rc == FS_ENOMEM) return set_error(FS_ENOMEM, "multigrid active lists");
         if (rc) return rc;
     }
@@ -1099,22 +1282,20 @@ int coarse_attributes()
     return FS_OK;
 }
 
-// two zeroed work arrays of n floats, allocated once
-int work_arrays(fs_ctx *c, float **a, float **b, size_t n, bool zero)
+// level 0's zeroed work arrays, allocated once: *a with the half-length one behind
+// it (MgSetLevel::b and d), and where b is given a second one of n floats
+int work_arrays(fs_ctx *c, float **a, float **b, size_t n)
 {
     if (!*a) {
-        if (cudaMalloc(a, n * 4) != cudaSuccess || cudaMalloc(b, n * 4) != cudaSuccess) {
+        if (cudaMalloc(a, n * 6) != cudaSuccess || (b && cudaMalloc(b, n * 4) != cudaSuccess)) {
             cudaGetLastError();
             cudaFree(*a);
             *a = nullptr;
             return set_error(FS_ENOMEM, "multigrid level-0 work arrays");
         }
-        zero = true;
     }
-    if (zero) {
-        FS_CUDA(cudaMemsetAsync(*a, 0, n * 4, c->stream));
-        FS_CUDA(cudaMemsetAsync(*b, 0, n * 4, c->stream));
-    }
+    FS_CUDA(cudaMemsetAsync(*a, 0, n * 6, c->stream));
+    if (b) FS_CUDA(cudaMemsetAsync(*b, 0, n * 4, c->stream));
     return FS_OK;
 }
 
@@ -1126,7 +1307,7 @@ void mg_free(fs_ctx *c)
     if (!m) return;
     free_set(&m->cset);
     for (MgSet &t : m->fset) free_set(&t);
-    for (float *p : {m->cb, m->cc, m->fb, m->fc}) cudaFree(p);
+    for (float *p : {m->cb, m->cc, m->fb}) cudaFree(p);
     delete m;
     c->mg = nullptr;
 }
@@ -1141,7 +1322,7 @@ int cell_quads(fs_ctx *c, const int **ql, int *n)
         v.sp.g[0] = level0_grid(c->L, c->L.nx, c->L.ny, c->L.nz);
         v.sp.base[0] = 0;
         v.fl = c->cflag;
-        if (int rc = make_list<QuadPred>(c, v, quad_items, &c->cq, &c->ncq))
+        if (int rc = make_list<QuadPred>(c, v, quad_items, &c->cq, &c->ncq, v.qoff))
             return rc == FS_ENOMEM ? set_error(FS_ENOMEM, "list of active quads") : rc;
         c->cq_epoch = c->mask_epoch;
     }
@@ -1150,38 +1331,104 @@ int cell_quads(fs_ctx *c, const int **ql, int *n)
     return FS_OK;
 }
 
+// The pressure hierarchy and its set for the current mask.
+static int build_cell(fs_ctx *c, MgAll *m)
+{
+    const Layout &L = c->L;
+    int rc;
+    MgSet &t = m->cset;
+    free_set(&t);
+    if ((rc = coarse_attributes()) || (rc = work_arrays(c, &m->cb, &m->cc, (size_t)L.nC)) ||
+        (rc = plan_levels(c, &m->cell, level0_grid(L, L.nx, L.ny, L.nz), 1.f, 0.f)))
+        return rc;
+    t.nv = 1;
+    t.s[0] = &m->cell;
+    t.lev[0].fl = c->cflag;
+    t.lev[0].b = m->cb;
+    t.lev[0].c = m->cc;
+    t.lev[0].d = m->cb + L.nC;
+    t.shared0 = true;
+    const int *ql = nullptr;
+    if ((rc = cell_quads(c, &ql, &t.lev[0].nq))) {
+        free_set(&t);
+        return rc;
+    }
+    t.lev[0].ql = const_cast<int *>(ql);
+    for (int v = 1; v < 4; v++) t.lev[0].qoff[v] = t.lev[0].nq;
+    if ((rc = build_set(c, t))) {
+        free_set(&t);
+        return rc;
+    }
+    return FS_OK;
+}
+
+// The three face hierarchies and their sets for the current mask.
+static int build_faces(fs_ctx *c, MgAll *m, float cc)
+{
+    const Layout &L = c->L;
+    int rc;
+    for (MgSet &t : m->fset) free_set(&t);
+    m->nfset = 0;
+    if ((rc = coarse_attributes()) || (rc = work_arrays(c, &m->fb, nullptr, (size_t)L.nF))) return rc;
+    bool all = true;
+    for (int k = 0; k < 3; k++) {
+        if ((rc = plan_levels(c, &m->face[k], level0_grid(L, L.nx + (k == 0), L.ny + (k == 1), L.nz + (k == 2)), cc,
+                              1.f)))
+            return rc;
+        all = all && m->face[k].nlev >= 2;
+    }
+    const int nset = all ? 1 : 3;
+    for (int n = 0; n < nset; n++) {
+        MgSet &t = m->fset[n];
+        t.nv = all ? 3 : 1;
+        t.lev[0].fl = c->fflag;
+        t.lev[0].b = m->fb;
+        t.lev[0].d = m->fb + L.nF;
+        t.one = true;
+        for (int v = 0; v < t.nv; v++) {
+            const int k = all ? v : n;
+            t.s[v] = &m->face[k];
+            t.lev[0].sp.base[v] = L.face_origin(k) - L.PL;  // the volume's leading guard plane
+        }
+        if ((rc = build_set(c, t))) {
+            for (MgSet &f : m->fset) free_set(&f);
+            return rc;
+        }
+    }
+    m->nfset = nset;
+    return FS_OK;
+}
+
+// The hierarchy of the pressure, or of the face volumes for the operator's
+// coefficient cc, for the current mask.
+int mg_prepare(fs_ctx *c, bool faces, float cc)
+{
+    MgAll *m = state(c);
+    if (!m) return set_error(FS_ENOMEM, "host allocation failed");
+    if (!faces) return m->cell.epoch != c->mask_epoch ? build_cell(c, m) : FS_OK;
+    if (m->nfset == 0 || m->face[0].epoch != c->mask_epoch) {
+        if (int rc = build_faces(c, m, cc)) {
+            m->nfset = 0;
+            return rc;
+        }
+    } else if (m->face[0].coef != cc) {  // a new viscosity or time step: rescale the levels only
+        for (MgState &s : m->face) {
+            float sc = cc;
+            for (int l = 0; l < s.nlev; l++, sc *= 0.25f) s.lev[l].scale = sc;
+            s.coef = cc;
+        }
+    }
+    return FS_OK;
+}
+
 // z = M r on the cell space (r and z of length nC, zero off the liquid); with
 // rzs, r.z in the last level-0 sweep when the hierarchy has one (*fused tells)
 static int apply_cell(fs_ctx *c, const float *r, float *z, const int *done, SolveScal *rzs, int first, bool *fused)
 {
     if (fused) *fused = false;
+    int rc = mg_prepare(c, false, 1.f);
+    if (rc) return rc;
     MgAll *m = state(c);
-    if (!m) return set_error(FS_ENOMEM, "host allocation failed");
-    const Layout &L = c->L;
-    int rc;
-    if (m->cell.epoch != c->mask_epoch) {
-        MgSet &t = m->cset;
-        free_set(&t);
-        if ((rc = coarse_attributes()) || (rc = work_arrays(c, &m->cb, &m->cc, (size_t)L.nC, true)) ||
-            (rc = plan_levels(c, &m->cell, level0_grid(L, L.nx, L.ny, L.nz), 1.f, 0.f)))
-            return rc;
-        t.nv = 1;
-        t.s[0] = &m->cell;
-        t.lev[0].fl = c->cflag;
-        t.lev[0].b = m->cb;
-        t.lev[0].c = m->cc;
-        t.shared0 = true;
-        const int *ql = nullptr;
-        if ((rc = cell_quads(c, &ql, &t.lev[0].nq))) {
-            free_set(&t);
-            return rc;
-        }
-        t.lev[0].ql = const_cast<int *>(ql);
-        if ((rc = build_set(c, t))) {
-            free_set(&t);
-            return rc;
-        }
-    }
     const bool fuse = rzs && m->cell.nlev >= 2;
     const bool sample = c->prof_on && (m->cset.calls++ % std::max(1, c->prof_period)) == 0;
     cudaEvent_t e0 = sample ? prof_mark(c) : nullptr;
@@ -1203,43 +1450,6 @@ bool mg_apply_rz(fs_ctx *c, const float *r, float *z, const int *done, SolveScal
     return fused;
 }
 
-// The three face hierarchies and their sets for the current mask.
-static int build_faces(fs_ctx *c, MgAll *m, float cc)
-{
-    const Layout &L = c->L;
-    int rc;
-    for (MgSet &t : m->fset) free_set(&t);
-    m->nfset = 0;
-    if ((rc = coarse_attributes()) || (rc = work_arrays(c, &m->fb, &m->fc, (size_t)L.nF, true))) return rc;
-    bool all = true;
-    for (int k = 0; k < 3; k++) {
-        if ((rc = plan_levels(c, &m->face[k], level0_grid(L, L.nx + (k == 0), L.ny + (k == 1), L.nz + (k == 2)), cc,
-                              1.f)))
-            return rc;
-        all = all && m->face[k].nlev >= 2;
-    }
-    const int nset = all ? 1 : 3;
-    for (int n = 0; n < nset; n++) {
-        MgSet &t = m->fset[n];
-        t.nv = all ? 3 : 1;
-        t.lev[0].fl = c->fflag;
-        t.lev[0].b = m->fb;
-        t.lev[0].c = m->fc;
-        t.one = true;
-        for (int v = 0; v < t.nv; v++) {
-            const int k = all ? v : n;
-            t.s[v] = &m->face[k];
-            t.lev[0].sp.base[v] = L.face_origin(k) - L.PL;  // the volume's leading guard plane
-        }
-        if ((rc = build_set(c, t))) {
-            for (MgSet &f : m->fset) free_set(&f);
-            return rc;
-        }
-    }
-    m->nfset = nset;
-    return FS_OK;
-}
-
 // z = M r on the face space for the Helmholtz operator I + cc L of the viscosity
 // solve (r and z of length nF, zero off the unknown faces), the three velocity
 // components' V-cycles launch by launch together. With `done` set, every kernel
@@ -1248,20 +1458,8 @@ static int apply_faces(fs_ctx *c, const float *r, float *z, float cc, const int 
                        bool *fused)
 {
     if (fused) *fused = false;
+    if (int rc = mg_prepare(c, true, cc)) return rc;
     MgAll *m = state(c);
-    if (!m) return set_error(FS_ENOMEM, "host allocation failed");
-    if (m->nfset == 0 || m->face[0].epoch != c->mask_epoch) {
-        if (int rc = build_faces(c, m, cc)) {
-            m->nfset = 0;
-            return rc;
-        }
-    } else if (m->face[0].coef != cc) {  // a new viscosity or time step: rescale the levels only
-        for (MgState &s : m->face) {
-            float sc = cc;
-            for (int l = 0; l < s.nlev; l++, sc *= 0.25f) s.lev[l].scale = sc;
-            s.coef = cc;
-        }
-    }
     const bool fuse = rzs && m->nfset == 1;
     const bool sample = c->prof_on && (m->fset[0].calls++ % std::max(1, c->prof_period)) == 0;
     cudaEvent_t e0 = sample ? prof_mark(c) : nullptr;

@@ -25,19 +25,6 @@ struct MgcLevel {
     float scale, mass;
 };
 
-// n / d for n d < 2^32 by one high multiply (m = ceil(2^32 / d); d = 1 kept apart)
-struct FastDiv {
-    unsigned m, d;
-    __host__ __device__ FastDiv() : m(0), d(1) {}
-    __host__ __device__ explicit FastDiv(unsigned dv) : m(dv > 1 ? (unsigned)(((1ull << 32) + dv - 1) / dv) : 0u), d(dv) {}
-    __device__ __forceinline__ unsigned div(unsigned n) const { return d == 1 ? n : __umulhi(n, m); }
-    __device__ __forceinline__ void split(unsigned n, unsigned &q, unsigned &r) const
-    {
-        q = div(n);
-        r = n - q * d;
-    }
-};
-
 // Tiles of a level: tqx quads x ty rows x tz planes (ty, tz even, so that a tile
 // holds whole 2 x 2 x 2 children of its coarse cells).
 struct MgTiles {
@@ -87,6 +74,12 @@ inline MgTiles make_tiles(const MgGrid &g, int nv, int num_sms)
     t.dyd = FastDiv(t.ty + 6);
     t.dyu = FastDiv(t.ty + 4);
     return t;
+}
+
+// e_out on one element from e_in: c (centre), the sum of its six neighbours nb
+__device__ __forceinline__ float sweep1(uint8_t f, float c, float nb, float rv, const float *wt, float scale, float m)
+{
+    return liq(f) ? c + wt[f & CF_D] * (rv - m * c - scale * ((float)(f & CF_D) * c - nb)) : 0.f;
 }
 
 // omega D^-1 r on a quad

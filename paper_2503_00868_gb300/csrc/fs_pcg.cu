@@ -49,10 +49,13 @@ __device__ __forceinline__ float inv_diag(uint8_t f, float cc)
 // there), q = A p_new on the quad, both written whole, and p_new . q. A thread
 // strides through the list with the next entry fetched a step ahead, so only quads
 // with an unknown are read or written, where a 128 x 8 tile carries many without.
+// The x neighbours come from the neighbouring lanes (FS_FOR_LIST_LINKED). Bound by
+// its bytes on large grids: 28 M unknown faces at 256^3 in 76 us (92 with scalar
+// loads, 114 by tiles), 29 us for the pressure there (34, 43).
 template <class Op>
 __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, int na, const float *__restrict__ src,
                                                   const float *__restrict__ pold, float *__restrict__ pnew,
-                                                  float *__restrict__ q, const uint8_t *__restrict__ fl, int P,
+                                                  float *__restrict__ aq, const uint8_t *__restrict__ fl, int P,
                                                   int PL, float cc, SolveScal *s, double *partials)
 {
     dep_wait();
@@ -61,20 +64,17 @@ __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, in
     const float beta = (float)s->beta;
     const float off = Op::offc(cc);
     KSum acc;
-    const int st = gridDim.x * blockDim.x;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int qn = i < na ? __ldg(ql + i) : 0;
-    for (; i < na; i += st) {
-        const int t = 4 * qn;
-        qn = i + st < na ? __ldg(ql + i + st) : 0;
+    FS_FOR_LIST_LINKED(ql, na, blockIdx.x, gridDim.x)
+    {
+        const int t = 4 * q;
+        const Links lk = links(q, fl_i, na);
         const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(fl + t));
         auto pn4 = [&](int u) {
             const float4 a = ldd4(src + u), b = ldd4(pold + u);
             return make_float4(a.x + beta * b.x, a.y + beta * b.y, a.z + beta * b.z, a.w + beta * b.w);
         };
-        auto pn1 = [&](int u) { return ldd1(src + u) + beta * ldd1(pold + u); };
         const float4 c = pn4(t), dn = pn4(t - P), up = pn4(t + P), bk = pn4(t - PL), fw = pn4(t + PL);
-        const float lf = pn1(t - 1), rt = pn1(t + 4);
+        const float lf = lk.left(c.w), rt = lk.right(c.x);
         auto one = [&](uint8_t fe, float ce, float nb) {
             return (fe & Op::ACTIVE) ? Op::diag(fe, cc) * ce - off * nb : 0.f;
         };
@@ -83,9 +83,10 @@ __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, in
         qv.y = one(f.y, c.y, (c.x + c.z) + (dn.y + up.y) + (bk.y + fw.y));
         qv.z = one(f.z, c.z, (c.y + c.w) + (dn.z + up.z) + (bk.z + fw.z));
         qv.w = one(f.w, c.w, (c.z + rt) + (dn.w + up.w) + (bk.w + fw.w));
+        if (!lk.own) continue;
         acc.add(c.x * qv.x + c.y * qv.y + c.z * qv.z + c.w * qv.w);
         *reinterpret_cast<float4 *>(pnew + t) = c;
-        *reinterpret_cast<float4 *>(q + t) = qv;
+        *reinterpret_cast<float4 *>(aq + t) = qv;
     }
     KSum vv[1] = {acc};
     double tot[1];
@@ -980,6 +981,8 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     // with multigrid, the operator apply walks the V-cycle's list of active quads
     const int *ql = nullptr;
     int nlisted = 0;
+    if (c->prm.precond == FS_PRECOND_MG)
+        if (int rc = mg_prepare(c, false, 1.f)) return rc;
     const bool listed = c->prm.precond == FS_PRECOND_MG && mg_level0_list(c, false, &ql, &nlisted);
     static const int rl = resident_blocks((const void *)k_spmv_list<PoisOp>, 0);  // one wave of the list apply
     if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_liquid;  // list entry and flags per quad
@@ -1000,7 +1003,7 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             const float *zsrc = jac ? c->pr : c->pz;
             if (listed)
-                launch_dep(k_spmv_list<PoisOp>, wave_blocks(c, nlisted, rl), TH, 0, c->stream, ql, nlisted, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
+                launch_dep(k_spmv_list<PoisOp>, wave_blocks(c, linked_threads(nlisted), rl), TH, 0, c->stream, ql, nlisted, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
             else if (tiled)
                 launch_dep(k_spmv_z<PoisOp>, tg.spmv, tdim, zmarch_smem(), c->stream, jac ? c->tmz_pr : c->tmz_pz, c->tmz_pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, c->items_cell,
                     c->nitems_cell, tm, 0.f, s, c->partials, c->err_word);
@@ -1259,6 +1262,8 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     // with multigrid, the operator apply walks the V-cycles' list of active quads
     const int *ql = nullptr;
     int nlisted = 0;
+    if (mg)
+        if (int rc = mg_prepare(c, true, cc)) return rc;
     const bool listed = mg && mg_level0_list(c, true, &ql, &nlisted);
     static const int rl = resident_blocks((const void *)k_spmv_list<HelmOp>, 0);  // one wave of the list apply
     if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_fluid;  // list entry and flags per quad
@@ -1275,7 +1280,7 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
             const bool samp = c->prof_on && ((launched + b) % c->prof_period) == 0;  // every prof_period-th
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             if (listed)
-                launch_dep(k_spmv_list<HelmOp>, wave_blocks(c, nlisted, rl), TH, 0, c->stream, ql, nlisted, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
+                launch_dep(k_spmv_list<HelmOp>, wave_blocks(c, linked_threads(nlisted), rl), TH, 0, c->stream, ql, nlisted, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
             else if (tiled)
                 launch_dep(k_spmv_z<HelmOp>, tg.spmv, tdim, zmarch_smem(), c->stream, mg ? c->tmz_vz : c->tmz_vr, c->tmz_vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, c->items_face,
                     c->nitems_face, tm, cc, s, c->partials, c->err_word);
