@@ -72,7 +72,7 @@ NCU_TRAFFIC = {
     "mg0_smooth_z": {"bytes_per_launch": 83167232 + 5408384, "source": "5ebc55d1e28ef6ee",
                      "files": ("fs_mg.cu", "fs_internal.cuh", "fs_mask.cu")},
 }
-KERNEL_FILES = ("fs_stencil.cuh", "fs_tma.cuh", "fs_mask.cu")
+KERNEL_FILES = ("fs_pcg.cu", "fs_mask.cu")
 
 
 def args_parse():

@@ -175,9 +175,8 @@ static void free_ctx(fs_ctx *c)
     void *ptrs[] = {c->cflag, c->fflag, c->bc, c->dsum, c->pb, c->pr, c->pp[0], c->pp[1], c->pq, c->px, c->pz,
                     c->pxh, c->pxt, c->pbr, c->vx, c->vr, c->vp[0], c->vp[1], c->vq, c->vz, c->fu[0], c->fu[1], c->fu[2], c->fg[0], c->fg[1],
                     c->fg[2], c->gc[0], c->gc[1], c->gc[2], c->mic_prec, c->scal, c->partials, c->err_word, c->pw[0], c->pw[1],
-                    c->act_cell, c->act_face, c->list_cell, c->list_face, c->items_cell, c->items_face, c->qmask_cell, c->qmask_face,
                     c->py, c->mic_order,
-                    c->mic_tact, c->mic_tflag, c->mic_next, c->cq};
+                    c->mic_tact, c->mic_tflag, c->mic_next, c->cq, c->fq};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->post) cudaFreeHost(c->post);
@@ -344,19 +343,8 @@ int fs_init_grid(fs_ctx **out, int nx, int ny, int nz, const fs_params *p, void 
     ALLOC(c->mic_tact, (size_t)c->mic_ntiles);
     ALLOC(c->mic_tflag, (size_t)c->mic_ntiles * sizeof(int));
     ALLOC(c->mic_next, 16);
-    c->tm_cell = make_tilemap(L, 1, c->num_sms);
-    c->tm_face = make_tilemap(L, 3, c->num_sms);
-    ALLOC(c->act_cell, (size_t)c->tm_cell.nblocks);
-    ALLOC(c->act_face, (size_t)c->tm_face.nblocks);
-    ALLOC(c->list_cell, (size_t)c->tm_cell.nblocks * sizeof(int));
-    ALLOC(c->list_face, (size_t)c->tm_face.nblocks * sizeof(int));
-    ALLOC(c->qmask_cell, (size_t)c->tm_cell.nblocks * 8 * sizeof(unsigned));
-    ALLOC(c->qmask_face, (size_t)c->tm_face.nblocks * 8 * sizeof(unsigned));
-    ALLOC(c->items_cell, (size_t)c->tm_cell.nblocks * sizeof(int4));
-    ALLOC(c->items_face, (size_t)c->tm_face.nblocks * sizeof(int4));
-    const int red_blocks = std::max(c->max_blocks, std::max(c->tm_cell.nblocks, c->tm_face.nblocks));
     ALLOC(c->scal, 4 * sizeof(SolveScal));
-    ALLOC(c->partials, (size_t)red_blocks * 8 * sizeof(double));
+    ALLOC(c->partials, (size_t)c->max_blocks * 8 * sizeof(double));
     ALLOC(c->err_word, 16);
 #undef ALLOC
     if (cudaHostAlloc((void **)&c->post, sizeof(HostPost), cudaHostAllocMapped) != cudaSuccess) {
@@ -366,10 +354,6 @@ int fs_init_grid(fs_ctx **out, int nx, int ny, int nz, const fs_params *p, void 
         return set_error(FS_ENOMEM, "pinned allocation failed");
     }
     std::memset((void *)c->post, 0, sizeof(HostPost));
-    if (int rc = make_tensor_maps(c)) {
-        free_ctx(c);
-        return rc;
-    }
     *out = c;
     return FS_OK;
 }

@@ -68,29 +68,6 @@ struct Layout {
     __host__ __device__ int face_origin(int c) const { return PL + c * (S + PL); }
 };
 
-// Tiling of a guarded space for the z-marching stencil kernels: `nvol` volumes
-// (1 for cell space, 3 for face space) of P x R x Z elements starting at
-// origin0 + v * vstride; tiles of TILE_X x TILE_Y columns, `tz` planes per chunk.
-// Block b covers tile (tx, ty) of chunk ch of volume v, x fastest.
-constexpr int TILE_X = 128;  // elements (32 threads x 4)
-constexpr int TILE_Y = 8;
-
-struct TileMap {
-    int ntx, nty, tz, nch, nvol;
-    int P, R, Z, PL;
-    int origin0, vstride;
-    int nblocks;
-    __host__ __device__ void decode(int b, int &v, int &ch, int &ty, int &tx) const
-    {
-        tx = b % ntx;
-        b /= ntx;
-        ty = b % nty;
-        b /= nty;
-        ch = b % nch;
-        v = b / nch;
-    }
-};
-
 struct F3 {
     float *c[3];
 };
@@ -171,6 +148,10 @@ struct fs_ctx {
     int *cq;
     int ncq;
     long long cq_epoch;
+    // the same for the unknown faces of the three face volumes (face_quads)
+    int *fq;
+    int nfq, fq_off[4];
+    long long fq_epoch;
 
     // reductions
     fs::SolveScal *scal;        // device [4]: 0 pressure, 1 viscosity, 2 misc, 3 misc
@@ -180,19 +161,7 @@ struct fs_ctx {
     int max_blocks;
     unsigned *err_word;         // device error word of bounded waits
     long long n_fluid;          // fluid faces
-    fs::TileMap tm_cell, tm_face;    // z-marching tilings of cell and face space
-    uint8_t *act_cell, *act_face;    // per tile block: 1 if it holds an active element
-    int *list_cell, *list_face;      // the active tiles, in tile order
-    int nact_cell, nact_face;
-    // per listed tile, 8 words (one per tile row) with bit q set when quad q of
-    // that row holds an active element
-    unsigned *qmask_cell, *qmask_face;
-    // z-marching work of the operator apply: {column, k0, k1, 0} chunks of active planes
-    int4 *items_cell, *items_face;
-    int nitems_cell, nitems_face;
-    // tensor maps of the vectors the operator apply reads (3-D: pitch x rows x
-    // planes of the guarded space, 136 x 10 x 1 boxes)
-    CUtensorMap tmz_pr, tmz_pz, tmz_pp[2], tmz_vr, tmz_vp[2], tmz_vz;
+    int noalloc;                // a context in the caller's memory (fs_noalloc.cu): no lists, no pinned memory
 
     // per-kernel timing (fs_profile)
     int prof_on;
@@ -560,11 +529,8 @@ inline long long linked_threads(long long na) { return (na + 29) / 30 * 32; }
 // ---- launchers implemented in the .cu files --------------------------------
 // fs_mask.cu
 int build_mask(fs_ctx *c, const uint8_t *types_dense, const fs_mac *bc);
-TileMap make_tilemap(const Layout &L, int nvol, int num_sms);
-int make_tensor_maps(fs_ctx *c);   // fs_mask.cu, once per context
 // fs_mask.cu: 16-channel bf16 cells (cell space) as a 4-D tensor, boxes of bx x by x bz cells, 32-byte swizzle
 int encode_cells16(CUtensorMap *m, const void *cells, const Layout &L, int bx, int by, int bz);
-int zmarch_slots(const fs_ctx *c, bool face);  // fs_pcg.cu: resident blocks of the operator apply
 // fs_pcg.cu
 int solve_pressure(fs_ctx *c, fs_stats *st);             // pb -> px
 int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st);  // vx (guess, rhs) -> vx
@@ -582,10 +548,10 @@ int mg_prepare(fs_ctx *c, bool faces, float cc);
 int mg_apply(fs_ctx *c, const float *r, float *z, const int *done);
 int mg_apply_faces(fs_ctx *c, const float *r, float *z, float cc, const int *done);
 int cell_quads(fs_ctx *c, const int **ql, int *n);  // fs_mg.cu: the list of the current mask's active quads
+int face_quads(fs_ctx *c, const int **ql, int *n, int *off = nullptr);  // fs_mg.cu
 void mg_free(fs_ctx *c);
 void mg_count(fs_ctx *c, long long vcycles, bool faces);  // fs_mg.cu: launch counts for fs_profile
 int mg_levels(const fs_ctx *c);
-bool mg_level0_list(const fs_ctx *c, bool faces, const int **ql, int *n);  // fs_mg.cu
 int pressure_pair(fs_ctx *c, float *q_hi, float *q_lo);  // fs_pcg.cu
 bool mg_rz(fs_ctx *c, bool faces, const float *r, const float *z, int first, SolveScal *s);  // fs_mg.cu
 // z = M r with r.z formed in the V-cycle's last level-0 sweep (beta = rz_new / rz,

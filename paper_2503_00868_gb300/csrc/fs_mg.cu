@@ -1331,6 +1331,31 @@ int cell_quads(fs_ctx *c, const int **ql, int *n)
     return FS_OK;
 }
 
+// the same over the three face volumes, in the face space's quads; off: where each
+// volume begins
+int face_quads(fs_ctx *c, const int **ql, int *n, int *off)
+{
+    if (c->fq_epoch != c->mask_epoch || !c->fq) {
+        cudaFree(c->fq);
+        c->fq = nullptr;
+        MgSetLevel v;
+        v.sp.nv = 3;
+        for (int k = 0; k < 3; k++) {
+            v.sp.g[k] = level0_grid(c->L, c->L.nx + (k == 0), c->L.ny + (k == 1), c->L.nz + (k == 2));
+            v.sp.base[k] = c->L.face_origin(k) - c->L.PL;
+        }
+        v.fl = c->fflag;
+        if (int rc = make_list<QuadPred>(c, v, quad_items, &c->fq, &c->nfq, c->fq_off))
+            return rc == FS_ENOMEM ? set_error(FS_ENOMEM, "list of active face quads") : rc;
+        c->fq_epoch = c->mask_epoch;
+    }
+    *ql = c->fq;
+    *n = c->nfq;
+    if (off)
+        for (int k = 0; k < 4; k++) off[k] = c->fq_off[k];
+    return FS_OK;
+}
+
 // The pressure hierarchy and its set for the current mask.
 static int build_cell(fs_ctx *c, MgAll *m)
 {
@@ -1385,6 +1410,12 @@ static int build_faces(fs_ctx *c, MgAll *m, float cc)
         t.lev[0].b = m->fb;
         t.lev[0].d = m->fb + L.nF;
         t.one = true;
+        if (all) {  // the context's list; one volume at a time, lists of their own
+            const int *ql = nullptr;
+            if ((rc = face_quads(c, &ql, &t.lev[0].nq, t.lev[0].qoff))) return rc;
+            t.lev[0].ql = const_cast<int *>(ql);
+        }
+        t.shared0 = all;
         for (int v = 0; v < t.nv; v++) {
             const int k = all ? v : n;
             t.s[v] = &m->face[k];
@@ -1519,18 +1550,6 @@ bool mg_rz(fs_ctx *c, bool faces, const float *r, const float *z, int first, Sol
     launch_dep(k_mg_rz, grid_blocks(c, t->lev[0].nq, TH), TH, 0, c->stream, t->lev[0].ql, t->lev[0].nq, r, z, first, s, c->partials);
     c->n_launches += 1;
     return cudaPeekAtLastError() == cudaSuccess;
-}
-
-// The level-0 list of active quads of the pressure hierarchy, or of the three
-// face volumes together (quads of the whole face space); false when a hierarchy
-// has no list for the current mask.
-bool mg_level0_list(const fs_ctx *c, bool faces, const int **ql, int *n)
-{
-    const MgSet *t = listed_set(c, faces);
-    if (!t) return false;
-    *ql = t->lev[0].ql;
-    *n = t->lev[0].nq;
-    return true;
 }
 
 int mg_levels(const fs_ctx *c)

@@ -113,6 +113,7 @@ extern "C" int fs_project_noalloc(int nx, int ny, int nz, const uint8_t *cell_ty
     c.partials = reinterpret_cast<double *>(take((size_t)c.max_blocks * 8 * sizeof(double)));
     c.err_word = reinterpret_cast<unsigned *>(take(16));
     c.post = nullptr;  // no pinned memory: the scalars are copied
+    c.noalloc = 1;
 
     fs_default_params(&c.prm);
     c.prm.dx = dx;

@@ -48,10 +48,12 @@ __device__ __forceinline__ float inv_diag(uint8_t f, float cc)
 // quad and its six neighbours (inactive elements hold z = p_old = 0, so p_new = 0
 // there), q = A p_new on the quad, both written whole, and p_new . q. A thread
 // strides through the list with the next entry fetched a step ahead, so only quads
-// with an unknown are read or written, where a 128 x 8 tile carries many without.
+// with an unknown are read or written.
 // The x neighbours come from the neighbouring lanes (FS_FOR_LIST_LINKED). Bound by
 // its bytes on large grids: 28 M unknown faces at 256^3 in 76 us (92 with scalar
-// loads, 114 by tiles), 29 us for the pressure there (34, 43).
+// loads, 114 by columns of TMA tiles marched along z), 29 us for the pressure there
+// (34, 43). On small ones by latency: the march was a chain of planes, and an
+// iteration on 101 x 75 x 90 took 22 us with it, 12 with the lists of both kernels.
 template <class Op>
 __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, int na, const float *__restrict__ src,
                                                   const float *__restrict__ pold, float *__restrict__ pnew,
@@ -99,7 +101,7 @@ __global__ void __launch_bounds__(TH) k_spmv_list(const int *__restrict__ ql, in
     }
 }
 
-// Flat versions of the two CG kernels, for a context without tile maps.
+// The flat operator apply, for a context without lists (fs_noalloc.cu).
 // p_new = z + beta p_old (z the stored preconditioned residual; for Jacobi the
 // solver keeps z = D^-1 r itself), then q = A p_new and the partial sums of
 // p_new . q. alpha = r.z / p.q at the end.
@@ -139,11 +141,16 @@ __global__ void __launch_bounds__(TH) k_spmv(const float *__restrict__ src, cons
 }
 
 // x += alpha p, r -= alpha q; partial sums of r.r (and r.z for Jacobi); the
-// last block counts the iteration and decides convergence.
+// last block counts the iteration and decides convergence. Over the list of active
+// quads, or (ql null) over all n4 quads of the space. With the Jacobi preconditioner
+// r holds the scaled residual z = D^-1 r, so the direction update needs no division.
+// Bound by its bytes on large grids (28 M unknown faces at 256^3 in 94 us, as the
+// walk over active 128 x 8 tiles before it), by latency on small ones.
 template <class Op, bool JAC>
 __global__ void __launch_bounds__(TH) k_update(float *__restrict__ x, float *__restrict__ r,
                                                const float *__restrict__ p, const float *__restrict__ q,
-                                               const uint8_t *__restrict__ fl, int n4, float cc,
+                                               const uint8_t *__restrict__ fl, const int *__restrict__ ql,
+                                               int n4, float cc,
                                                SolveScal *s, double *partials)
 {
     dep_wait();
@@ -154,7 +161,12 @@ __global__ void __launch_bounds__(TH) k_update(float *__restrict__ x, float *__r
     float4 *x4 = reinterpret_cast<float4 *>(x);
     float4 *r4 = reinterpret_cast<float4 *>(r);
     const uchar4 *f4 = reinterpret_cast<const uchar4 *>(fl);
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += gridDim.x * blockDim.x) {
+    const int st = gridDim.x * blockDim.x;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int next = ql && i < n4 ? __ldg(ql + i) : i;
+    for (; i < n4; i += st) {
+        const int t = next;
+        next = ql ? (i + st < n4 ? __ldg(ql + i + st) : 0) : i + st;
         const uchar4 fv = f4[t];
         // four inactive elements: p = q = 0 there, nothing changes
         if (!((fv.x | fv.y | fv.z | fv.w) & Op::ACTIVE)) continue;
@@ -673,24 +685,7 @@ __global__ void __launch_bounds__(TH) k_loss_face(CF3 u, CF3 tg, const uint8_t *
 }  // namespace
 }  // namespace fs
 
-#include "fs_stencil.cuh"
-#include "fs_tma.cuh"
-
 namespace fs {
-
-// Persistent grid sizes of the two CG kernels for one operator.
-template <class Op>
-struct TmaGrids {
-    int spmv, upd;
-    TmaGrids(const fs_ctx *c, int nitems, int nact)
-    {
-        static const int rs = resident_blocks((const void *)k_spmv_z<Op>, zmarch_smem());
-        static const int ru = resident_blocks((const void *)k_update_q<Op, true>, 0);
-        static const int ru2 = resident_blocks((const void *)k_update_q<Op, false>, 0);
-        spmv = std::max(1, std::min(nitems, c->num_sms * rs));
-        upd = std::max(1, std::min(nact, c->num_sms * std::min(ru, ru2)));
-    }
-};
 
 // Iterations launched before each read of the convergence flag. A read costs a
 // host round trip with the GPU idle (5 us), and every iteration launched after
@@ -708,13 +703,6 @@ struct CgBatches {
     }
     int size(long long launched) const { return launched == 0 ? first : later; }
 };
-
-int zmarch_slots(const fs_ctx *c, bool face)
-{
-    const int r = face ? resident_blocks((const void *)k_spmv_z<HelmOp>, zmarch_smem())
-                       : resident_blocks((const void *)k_spmv_z<PoisOp>, zmarch_smem());
-    return c->num_sms * r;
-}
 
 namespace {
 // The scalars of a slot and the error word into pinned host memory, then the
@@ -780,7 +768,6 @@ int check_wait_error(fs_ctx *c, const char *what, unsigned herr)
         return set_error(FS_ETIMEOUT, "MIC(0) sweep: a wait on a predecessor tile ran out (spin_limit %d)",
                          c->prm.spin_limit);
     }
-    if (herr & ERR_TMA) return set_error(FS_ETIMEOUT, "%s: a wait for a tensor copy ran out", what);
     if (herr & 8u)  // the bit of the network's kernels
         return set_error(FS_ETIMEOUT, "%s: a bounded wait of the network ran out", what);
     return FS_OK;
@@ -977,18 +964,18 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     long long launched = 0;
     double by_spmv = (double)L.nC + 16.0 * (double)c->n_liquid;
     const double by_upd = (double)L.nC + 24.0 * (double)c->n_liquid;
-    const bool tiled = c->act_cell != nullptr;
-    // with multigrid, the operator apply walks the V-cycle's list of active quads
+    // both kernels walk the list of active quads
     const int *ql = nullptr;
     int nlisted = 0;
     if (c->prm.precond == FS_PRECOND_MG)
         if (int rc = mg_prepare(c, false, 1.f)) return rc;
-    const bool listed = c->prm.precond == FS_PRECOND_MG && mg_level0_list(c, false, &ql, &nlisted);
+    const bool listed = !c->noalloc;
+    if (listed)
+        if (int rc = cell_quads(c, &ql, &nlisted)) return rc;
     static const int rl = resident_blocks((const void *)k_spmv_list<PoisOp>, 0);  // one wave of the list apply
+    static const int ru = std::min(resident_blocks((const void *)k_update<PoisOp, true>, 0),
+                                   resident_blocks((const void *)k_update<PoisOp, false>, 0));
     if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_liquid;  // list entry and flags per quad
-    const TileMap &tm = c->tm_cell;
-    const dim3 tdim(TILE_X / 4, TILE_Y);
-    const TmaGrids<PoisOp> tg(c, c->nitems_cell, c->nact_cell);
     // a multigrid iteration costs several operator applies: check convergence more often
     const int check = c->prm.precond == FS_PRECOND_MG ? std::min(c->prm.check_every, 4) : c->prm.check_every;
     int &last = c->it_last_p[c->solve_kind & 1][c->refining ? 1 : 0];
@@ -1003,27 +990,15 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             const float *zsrc = jac ? c->pr : c->pz;
             if (listed)
-                launch_dep(k_spmv_list<PoisOp>, wave_blocks(c, linked_threads(nlisted), rl), TH, 0, c->stream, ql, nlisted, c->pz, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
-            else if (tiled)
-                launch_dep(k_spmv_z<PoisOp>, tg.spmv, tdim, zmarch_smem(), c->stream, jac ? c->tmz_pr : c->tmz_pz, c->tmz_pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, c->items_cell,
-                    c->nitems_cell, tm, 0.f, s, c->partials, c->err_word);
+                launch_dep(k_spmv_list<PoisOp>, wave_blocks(c, linked_threads(nlisted), rl), TH, 0, c->stream, ql, nlisted, zsrc, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.P, L.PL, 0.f, s, c->partials);
             else
                 launch_dep(k_spmv<PoisOp>, bs, TH, 0, c->stream, zsrc, c->pp[cur], c->pp[cur ^ 1], c->pq, c->cflag, L.nC,
                                                          L.P, L.PL, 0.f, s, c->partials);
             cudaEvent_t e1 = samp ? prof_mark(c) : nullptr, e2 = samp ? prof_mark(c) : nullptr;
-            if (tiled) {
-                if (jac)
-                    launch_dep(k_update_q<PoisOp, true>, tg.upd, tdim, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag, c->list_cell, c->qmask_cell, c->nact_cell, tm,
-                        0.f, s, c->partials);
-                else
-                    launch_dep(k_update_q<PoisOp, false>, tg.upd, tdim, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag, c->list_cell, c->qmask_cell, c->nact_cell, tm,
-                        0.f, s, c->partials);
-            } else if (jac)
-                launch_dep(k_update<PoisOp, true>, b4, TH, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag,
-                                                                 n4, 0.f, s, c->partials);
-            else
-                launch_dep(k_update<PoisOp, false>, b4, TH, 0, c->stream, c->px, c->pr, c->pp[cur ^ 1], c->pq, c->cflag,
-                                                                  n4, 0.f, s, c->partials);
+            const int *uq = listed ? ql : nullptr;
+            const int un = listed ? nlisted : n4, ub = listed ? wave_blocks(c, nlisted, ru) : b4;
+            launch_dep(jac ? k_update<PoisOp, true> : k_update<PoisOp, false>, ub, TH, 0, c->stream, c->px, c->pr,
+                       c->pp[cur ^ 1], c->pq, c->cflag, uq, un, 0.f, s, c->partials);
             cudaEvent_t e3 = samp ? prof_mark(c) : nullptr;
             prof_add(c, K_P_SPMV, e0, e1, by_spmv);
             prof_add(c, K_P_UPDATE, e2, e3, by_upd);
@@ -1258,18 +1233,18 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     SolveScal h;
     double by_spmv = (double)L.nF + 16.0 * (double)c->n_fluid;
     const double by_upd = (double)L.nF + 24.0 * (double)c->n_fluid;
-    const bool tiled = c->act_face != nullptr;
-    // with multigrid, the operator apply walks the V-cycles' list of active quads
+    // both kernels walk the list of active quads of the face volumes
     const int *ql = nullptr;
     int nlisted = 0;
     if (mg)
         if (int rc = mg_prepare(c, true, cc)) return rc;
-    const bool listed = mg && mg_level0_list(c, true, &ql, &nlisted);
+    const bool listed = !c->noalloc;
+    if (listed)
+        if (int rc = face_quads(c, &ql, &nlisted)) return rc;
     static const int rl = resident_blocks((const void *)k_spmv_list<HelmOp>, 0);  // one wave of the list apply
+    static const int ru = std::min(resident_blocks((const void *)k_update<HelmOp, true>, 0),
+                                   resident_blocks((const void *)k_update<HelmOp, false>, 0));
     if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_fluid;  // list entry and flags per quad
-    const TileMap &tm = c->tm_face;
-    const dim3 tdim(TILE_X / 4, TILE_Y);
-    const TmaGrids<HelmOp> tg(c, c->nitems_face, c->nact_face);
     int &last = c->it_last_v[dirichlet ? 1 : 0];
     const CgBatches batches(last, check, c->prm.maxit_v, mg);
     for (;;) {
@@ -1280,28 +1255,15 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
             const bool samp = c->prof_on && ((launched + b) % c->prof_period) == 0;  // every prof_period-th
             cudaEvent_t e0 = samp ? prof_mark(c) : nullptr;
             if (listed)
-                launch_dep(k_spmv_list<HelmOp>, wave_blocks(c, linked_threads(nlisted), rl), TH, 0, c->stream, ql, nlisted, c->vz, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
-            else if (tiled)
-                launch_dep(k_spmv_z<HelmOp>, tg.spmv, tdim, zmarch_smem(), c->stream, mg ? c->tmz_vz : c->tmz_vr, c->tmz_vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, c->items_face,
-                    c->nitems_face, tm, cc, s, c->partials, c->err_word);
+                launch_dep(k_spmv_list<HelmOp>, wave_blocks(c, linked_threads(nlisted), rl), TH, 0, c->stream, ql, nlisted, mg ? c->vz : c->vr, c->vp[cur], c->vp[cur ^ 1], c->vq, c->fflag, L.P, L.PL, cc, s, c->partials);
             else
                 launch_dep(k_spmv<HelmOp>, bs, TH, 0, c->stream, mg ? c->vz : c->vr, c->vp[cur], c->vp[cur ^ 1], c->vq,
                                                          c->fflag, L.nF, L.P, L.PL, cc, s, c->partials);
             cudaEvent_t e1 = samp ? prof_mark(c) : nullptr, e2 = samp ? prof_mark(c) : nullptr;
-            if (tiled) {
-                if (mg)
-                    launch_dep(k_update_q<HelmOp, false>, tg.upd, tdim, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, c->list_face, c->qmask_face, c->nact_face, tm,
-                        cc, s, c->partials);
-                else
-                    launch_dep(k_update_q<HelmOp, true>, tg.upd, tdim, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, c->list_face, c->qmask_face, c->nact_face, tm,
-                        cc, s, c->partials);
-            } else if (mg) {
-                launch_dep(k_update<HelmOp, false>, b4, TH, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, n4,
-                                                                  cc, s, c->partials);
-            } else {
-                launch_dep(k_update<HelmOp, true>, b4, TH, 0, c->stream, c->vx, c->vr, c->vp[cur ^ 1], c->vq, c->fflag, n4,
-                                                                 cc, s, c->partials);
-            }
+            const int *uq = listed ? ql : nullptr;
+            const int un = listed ? nlisted : n4, ub = listed ? wave_blocks(c, nlisted, ru) : b4;
+            launch_dep(mg ? k_update<HelmOp, false> : k_update<HelmOp, true>, ub, TH, 0, c->stream, c->vx, c->vr,
+                       c->vp[cur ^ 1], c->vq, c->fflag, uq, un, cc, s, c->partials);
             cudaEvent_t e3 = samp ? prof_mark(c) : nullptr;
             prof_add(c, K_V_SPMV, e0, e1, by_spmv);
             prof_add(c, K_V_UPDATE, e2, e3, by_upd);

@@ -1,4 +1,4 @@
-"""MIC(0) substitution where its tiles can go wrong: one cell, one tile, one cell into a
+"""MIC(0) substitution where its tiles can go wrong: the smallest grid, one tile, one cell into a
 second tile on each axis, and scattered masks with empty tiles, against the oracle."""
 import numpy as np
 import pytest
@@ -18,7 +18,7 @@ def built():
     torch.cuda.set_device(0)
 
 
-@pytest.mark.parametrize("nx,ny,nz,liquid", [(1, 1, 1, 1.0), (8, 8, 8, 1.0), (9, 8, 8, 0.9), (8, 9, 17, 0.7), (17, 24, 9, 0.4),
+@pytest.mark.parametrize("nx,ny,nz,liquid", [(2, 2, 2, 1.0), (8, 8, 8, 1.0), (9, 8, 8, 0.9), (8, 9, 17, 0.7), (17, 24, 9, 0.4),
                                              (63, 41, 34, 0.02), (40, 64, 33, 0.8)])
 def test_mic0_tiles_match_oracle(nx, ny, nz, liquid):
     rng = np.random.default_rng(7)
