@@ -479,8 +479,8 @@ __device__ __forceinline__ float4 pre1_q(const MgGrid &g, const uint8_t *__restr
 // What bounds them (measured one by one): above a few million unknowns the bytes,
 // and for the kernels that form a sweep on the fly or take two grids the
 // instructions; below, latency (a launch, the list, the loads). The three face
-// volumes at 256^3, 28 M unknowns: pre1 66 us (with a test and a conversion of each
-// flag byte 73), prolong 51 (56), smooth 59, near its bytes at 6.9 TB/s.
+// volumes at 256^3, 20 M unknowns: pre1 66 us (with a test and a conversion of each
+// flag byte 73), prolong 51 (56), smooth 59 (4.8 TB/s of its bytes).
 // The sweeps that are not followed by a restriction keep the plain walk: windows of
 // 30 quads start off a 128-byte line, which cost a sweep 4% there.
 
@@ -594,8 +594,8 @@ __global__ void __launch_bounds__(256) k_mg0_prolong(const __grid_constant__ MgS
 
 // Restriction over the coarse level's list of active pairs. Pairs take a thread each
 // (WHOLE): the index arithmetic bounds the large levels (the three face volumes,
-// 28 M unknowns at 256^3: 20 us against 37 with four lanes per pair, and 45 over whole
-// residuals with their x neighbours; 3.4 M at 128^3: 7.4 against 9.3 and 13.5). Where
+// 20 M unknowns at 256^3: 20 us against 37 with four lanes per pair, and 45 over whole
+// residuals with their x neighbours; 2.5 M at 128^3: 7.4 against 9.3 and 13.5). Where
 // four lanes per pair fit in one wave they are used, for four times the loads in
 // flight (the 64^3 level below a pressure blob: 4.7 us against 6.0 and 9.1).
 template <bool WHOLE>

@@ -183,7 +183,7 @@ constexpr int MSTH = 128;          // threads: one per quad of the tile
 constexpr int MPY = 40, MPZ = 384; // pitches of the padded tile: a warp's 32 cells lie in 32 banks
 template <int MODE>
 __global__ void __launch_bounds__(MSTH) k_mic_solve(MicGrid G, const uint8_t *__restrict__ cf,
-                                                    const float *__restrict__ prec, const float *__restrict__ in,
+                                                    const float *__restrict__ prec, const float *in,
                                                     float *out, const int *__restrict__ order, int n,
                                                     const uint8_t *__restrict__ tact, int *tflag, int *next, int *other,
                                                     int epoch, int spin_limit, unsigned *err)
@@ -198,6 +198,8 @@ __global__ void __launch_bounds__(MSTH) k_mic_solve(MicGrid G, const uint8_t *__
     __shared__ int s_tile;
     __shared__ int s_abort;
     const int tid = threadIdx.x;
+    dep_wait();
+    dep_go();
     if (blockIdx.x == 0 && tid == 0) *other = 0;  // the next sweep's tile counter
     const int qx = (tid & 1) * 4, qy = (tid >> 1) % MT, qz = tid / (2 * MT);
     for (;;) {
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(MSTH) k_mic_solve(MicGrid G, const uint8_t *__
         float4 rv = make_float4(0.f, 0.f, 0.f, 0.f), pv = rv;
         if (qin) {
             const uchar4 f = __ldg(reinterpret_cast<const uchar4 *>(cf + qt));
-            const float4 r4 = *reinterpret_cast<const float4 *>(in + qt), p4 = *reinterpret_cast<const float4 *>(prec + qt);
+            const float4 r4 = ldd4(in + qt), p4 = *reinterpret_cast<const float4 *>(prec + qt);
             rv = make_float4(f.x & CF_LIQ ? r4.x : 0.f, f.y & CF_LIQ ? r4.y : 0.f, f.z & CF_LIQ ? r4.z : 0.f,
                              f.w & CF_LIQ ? r4.w : 0.f);
             pv = make_float4(f.x & CF_LIQ ? p4.x : 0.f, f.y & CF_LIQ ? p4.y : 0.f, f.z & CF_LIQ ? p4.z : 0.f,
@@ -374,9 +376,8 @@ static int mic_solve(fs_ctx *c, const float *in, float *out)
     int *next = c->mic_next + (MODE == MIC_FORWARD ? 0 : 1), *other = c->mic_next + (MODE == MIC_FORWARD ? 1 : 0);
     c->mic_epoch += 1;
     const int grid = std::max(1, std::min(c->mic_n, 4 * c->num_sms));
-    k_mic_solve<MODE><<<grid, MSTH, 0, c->stream>>>(mic_grid(c), c->cflag, c->mic_prec, in, out, c->mic_order, c->mic_n,
-                                                    c->mic_tact, c->mic_tflag, next, other, c->mic_epoch,
-                                                    c->prm.spin_limit, c->err_word);
+    launch_dep(k_mic_solve<MODE>, grid, MSTH, 0, c->stream, mic_grid(c), c->cflag, c->mic_prec, in, out, c->mic_order,
+               c->mic_n, c->mic_tact, c->mic_tflag, next, other, c->mic_epoch, c->prm.spin_limit, c->err_word);
     c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
     return FS_OK;

@@ -50,7 +50,7 @@ __device__ __forceinline__ float inv_diag(uint8_t f, float cc)
 // strides through the list with the next entry fetched a step ahead, so only quads
 // with an unknown are read or written.
 // The x neighbours come from the neighbouring lanes (FS_FOR_LIST_LINKED). Bound by
-// its bytes on large grids: 28 M unknown faces at 256^3 in 76 us (92 with scalar
+// its bytes on large grids: 20 M unknown faces at 256^3 in 76 us (92 with scalar
 // loads, 114 by columns of TMA tiles marched along z), 29 us for the pressure there
 // (34, 43). On small ones by latency: the march was a chain of planes, and an
 // iteration on 101 x 75 x 90 took 22 us with it, 12 with the lists of both kernels.
@@ -144,8 +144,9 @@ __global__ void __launch_bounds__(TH) k_spmv(const float *__restrict__ src, cons
 // last block counts the iteration and decides convergence. Over the list of active
 // quads, or (ql null) over all n4 quads of the space. With the Jacobi preconditioner
 // r holds the scaled residual z = D^-1 r, so the direction update needs no division.
-// Bound by its bytes on large grids (28 M unknown faces at 256^3 in 94 us, as the
-// walk over active 128 x 8 tiles before it), by latency on small ones.
+// Bound by its bytes on large grids (20 M unknown faces at 256^3 in 95 us, as the
+// walk over active 128 x 8 tiles before it, and 100 with the flags read for nothing),
+// by latency on small ones.
 template <class Op, bool JAC>
 __global__ void __launch_bounds__(TH) k_update(float *__restrict__ x, float *__restrict__ r,
                                                const float *__restrict__ p, const float *__restrict__ q,
@@ -167,9 +168,11 @@ __global__ void __launch_bounds__(TH) k_update(float *__restrict__ x, float *__r
     for (; i < n4; i += st) {
         const int t = next;
         next = ql ? (i + st < n4 ? __ldg(ql + i + st) : 0) : i + st;
-        const uchar4 fv = f4[t];
+        // (a listed quad needs its flags for the Jacobi diagonals only: p, q and r are
+        // zero off the unknowns)
+        const uchar4 fv = JAC || !ql ? f4[t] : make_uchar4(0, 0, 0, 0);
         // four inactive elements: p = q = 0 there, nothing changes
-        if (!((fv.x | fv.y | fv.z | fv.w) & Op::ACTIVE)) continue;
+        if (!ql && !((fv.x | fv.y | fv.z | fv.w) & Op::ACTIVE)) continue;
         float4 xv = ldd4(x + 4 * t), rv = ldd4(r + 4 * t);
         const float4 pv = ldd4(p + 4 * t), qv = ldd4(q + 4 * t);
         xv.x += alpha * pv.x; xv.y += alpha * pv.y; xv.z += alpha * pv.z; xv.w += alpha * pv.w;
@@ -493,9 +496,11 @@ __global__ void __launch_bounds__(TH) k_pois_restart(const float *__restrict__ b
 __global__ void __launch_bounds__(TH) k_liquid_sum(const float *__restrict__ x, const uint8_t *__restrict__ fl,
                                                    int n, SolveScal *s, double *partials)
 {
+    dep_wait();
+    dep_go();
     double a = 0.0, c = 0.0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
-        if (fl[t] & CF_LIQ) { a += x[t]; c += 1.0; }
+        if (fl[t] & CF_LIQ) { a += ldd1(x + t); c += 1.0; }
     double v[2] = {a, c}, tot[2];
     if (grid_reduce<2>(v, partials, &s->ticket, tot) && threadIdx.x == 0) {
         s->aux[0] = tot[0];
@@ -505,9 +510,12 @@ __global__ void __launch_bounds__(TH) k_liquid_sum(const float *__restrict__ x, 
 
 __global__ void k_sub_liquid_mean(float *x, const uint8_t *__restrict__ fl, int n, const SolveScal *s)
 {
-    const float mean = s->aux[1] > 0.0 ? (float)(s->aux[0] / s->aux[1]) : 0.f;
+    dep_wait();
+    dep_go();
+    const double sum = *(volatile const double *)&s->aux[0], cells = *(volatile const double *)&s->aux[1];
+    const float mean = cells > 0.0 ? (float)(sum / cells) : 0.f;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
-        if (fl[t] & CF_LIQ) x[t] -= mean;
+        if (fl[t] & CF_LIQ) x[t] = ldd1(x + t) - mean;
 }
 
 // b = -dx * div(u) on liquid cells (cell space), u a public-layout field.
@@ -803,8 +811,8 @@ int remove_null_mode(fs_ctx *c, float *z)
     if (!c->singular) return FS_OK;
     const Layout &L = c->L;
     const int bs = grid_blocks(c, L.nC, TH);
-    k_liquid_sum<<<bs, TH, 0, c->stream>>>(z, c->cflag, L.nC, c->scal + 3, c->partials);
-    k_sub_liquid_mean<<<bs, TH, 0, c->stream>>>(z, c->cflag, L.nC, c->scal + 3);
+    launch_dep(k_liquid_sum, bs, TH, 0, c->stream, z, c->cflag, L.nC, c->scal + 3, c->partials);
+    launch_dep(k_sub_liquid_mean, bs, TH, 0, c->stream, z, c->cflag, L.nC, c->scal + 3);
     c->n_launches += 2;
     FS_CUDA(cudaGetLastError());
     return FS_OK;
@@ -963,7 +971,7 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     unsigned herr = 0;
     long long launched = 0;
     double by_spmv = (double)L.nC + 16.0 * (double)c->n_liquid;
-    const double by_upd = (double)L.nC + 24.0 * (double)c->n_liquid;
+    double by_upd = (double)L.nC + 24.0 * (double)c->n_liquid;
     // both kernels walk the list of active quads
     const int *ql = nullptr;
     int nlisted = 0;
@@ -975,7 +983,10 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     static const int rl = resident_blocks((const void *)k_spmv_list<PoisOp>, 0);  // one wave of the list apply
     static const int ru = std::min(resident_blocks((const void *)k_update<PoisOp, true>, 0),
                                    resident_blocks((const void *)k_update<PoisOp, false>, 0));
-    if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_liquid;  // list entry and flags per quad
+    if (listed) {  // list entry and flags per quad (the update's flags with Jacobi only)
+        by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_liquid;
+        by_upd = (jac ? 8.0 : 4.0) * (double)nlisted + 24.0 * (double)c->n_liquid;
+    }
     // a multigrid iteration costs several operator applies: check convergence more often
     const int check = c->prm.precond == FS_PRECOND_MG ? std::min(c->prm.check_every, 4) : c->prm.check_every;
     int &last = c->it_last_p[c->solve_kind & 1][c->refining ? 1 : 0];
@@ -1232,7 +1243,7 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     long long launched = 0;
     SolveScal h;
     double by_spmv = (double)L.nF + 16.0 * (double)c->n_fluid;
-    const double by_upd = (double)L.nF + 24.0 * (double)c->n_fluid;
+    double by_upd = (double)L.nF + 24.0 * (double)c->n_fluid;
     // both kernels walk the list of active quads of the face volumes
     const int *ql = nullptr;
     int nlisted = 0;
@@ -1244,7 +1255,10 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     static const int rl = resident_blocks((const void *)k_spmv_list<HelmOp>, 0);  // one wave of the list apply
     static const int ru = std::min(resident_blocks((const void *)k_update<HelmOp, true>, 0),
                                    resident_blocks((const void *)k_update<HelmOp, false>, 0));
-    if (listed) by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_fluid;  // list entry and flags per quad
+    if (listed) {  // list entry and flags per quad (the update's flags with Jacobi only)
+        by_spmv = 8.0 * (double)nlisted + 16.0 * (double)c->n_fluid;
+        by_upd = (mg ? 4.0 : 8.0) * (double)nlisted + 24.0 * (double)c->n_fluid;
+    }
     int &last = c->it_last_v[dirichlet ? 1 : 0];
     const CgBatches batches(last, check, c->prm.maxit_v, mg);
     for (;;) {
