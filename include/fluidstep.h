@@ -126,7 +126,8 @@ typedef struct {
     int check_every;   /* iterations between host convergence checks, >= 1 (at most 4 with
                           the multigrid preconditioner). Once a pass of the same kind has
                           run on the context, the first check comes one iteration before
-                          that pass's count and later ones every two iterations */
+                          that pass's count and later ones every iteration with the
+                          multigrid preconditioner, every two without */
     int spin_limit;    /* cap on every device-side spin-wait (iterations), >= 1 */
     double mic_tau;    /* MIC(0) modification, in [0, 1] */
     double mic_sigma;  /* MIC(0) safety threshold, in [0, 1) */
