@@ -356,41 +356,59 @@ struct Sum2 {
 // change, is left out: sum e^2 - (sum e)^2 / N. With r_out, the residual is also
 // stored, rounded once to FP32, on the liquid (zero elsewhere, guard planes
 // included): the right-hand side of a refinement step. r_out may alias b: every
-// thread reads b only at the element it writes.
+// thread reads b only at the quad it writes. (Off the listed quads r_out is zero
+// already: b and the refinement's right-hand side are cleared with each mask.)
+//
+// It walks the list of active quads, or (ql null) all nq quads of the space. What it
+// costs beside its loads is the FP64 merge, a share per block: over all elements, with
+// a full grid at any size, it took 30 us at 101 x 75 x 90; over the list, 15.
 __global__ void __launch_bounds__(TH) k_pois_true_res(const float *b, const float *__restrict__ x,
-                                                      const uint8_t *__restrict__ fl, int n, int P, int PL,
-                                                      int singular, SolveScal *s, double *partials, float *r_out)
+                                                      const uint8_t *__restrict__ fl, const int *__restrict__ ql,
+                                                      int nq, int P, int PL, int singular, SolveScal *s,
+                                                      double *partials, float *r_out)
 {
     Sum2 acc, sum, bsq;
     int cnt = 0;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const uint8_t f = fl[t];
-        if (!(f & CF_LIQ)) {
-            if (r_out) r_out[t] = 0.f;
-            continue;
-        }
-        const float d = PoisOp::diag(f, 0.f), xc = x[t], bv = b[t];
+    auto cell = [&](uint8_t f, float bv, float xc, float x0, float x1, float x2, float x3, float x4, float x5) -> float {
+        if (!(f & CF_LIQ)) return 0.f;
+        const float d = PoisOp::diag(f, 0.f);
         const float dx = d * xc, dxe = fmaf(d, xc, -dx);  // d x = dx + dxe exactly
         Sum3 r;
         r.add(bv);
         r.add(-dx);
         r.add(-dxe);
-        r.add(x[t - 1]);
-        r.add(x[t + 1]);
-        r.add(x[t - P]);
-        r.add(x[t + P]);
-        r.add(x[t - PL]);
-        r.add(x[t + PL]);
+        r.add(x0);
+        r.add(x1);
+        r.add(x2);
+        r.add(x3);
+        r.add(x4);
+        r.add(x5);
         float el;
         const float eh = two_sum(r.hi, r.lo, el);
         el += r.rest;  // e = eh + el
-        if (r_out) r_out[t] = eh + el;
         const float sq = eh * eh;
         acc.add(sq, fmaf(eh, eh, -sq) + 2.f * eh * el);
         sum.add(eh, el);
         const float bb = bv * bv;
         bsq.add(bb, fmaf(bv, bv, -bb));
         cnt += 1;
+        return eh + el;
+    };
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nq; i += gridDim.x * blockDim.x) {
+        const int t = 4 * (ql ? __ldg(ql + i) : i);
+        const uchar4 f = *reinterpret_cast<const uchar4 *>(fl + t);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if ((f.x | f.y | f.z | f.w) & CF_LIQ) {
+            auto x4 = [&](int u) { return *reinterpret_cast<const float4 *>(x + u); };
+            const float4 c = x4(t), dn = x4(t - P), up = x4(t + P), bk = x4(t - PL), fw = x4(t + PL);
+            const float4 bv = *reinterpret_cast<const float4 *>(b + t);
+            const float lf = x[t - 1], rt = x[t + 4];
+            v.x = cell(f.x, bv.x, c.x, lf, c.y, dn.x, up.x, bk.x, fw.x);
+            v.y = cell(f.y, bv.y, c.y, c.x, c.z, dn.y, up.y, bk.y, fw.y);
+            v.z = cell(f.z, bv.z, c.z, c.y, c.w, dn.z, up.z, bk.z, fw.z);
+            v.w = cell(f.w, bv.w, c.w, c.z, rt, dn.w, up.w, bk.w, fw.w);
+        }
+        if (r_out) *reinterpret_cast<float4 *>(r_out + t) = v;
     }
     double v[4] = {acc.value(), sum.value(), (double)cnt, bsq.value()}, tot[4];
     if (grid_reduce<4>(v, partials, &s->ticket, tot) && threadIdx.x == 0) {
@@ -858,6 +876,20 @@ int learned_apply(fs_ctx *c, const float *r, float *z, const int *done, const fl
 static int pressure_tail(fs_ctx *c, const SolveScal &h, long long iters, double bb0, const SolveScal *known,
                          fs_stats *st);
 
+// b - A x over the liquid to FP64 accuracy: its sums to scal + 2, itself to r_out
+static int true_res(fs_ctx *c, const float *b, const float *x, float *r_out)
+{
+    const Layout &L = c->L;
+    const int *ql = nullptr;
+    int nq = L.nC / 4;
+    if (!c->noalloc)
+        if (int rc = cell_quads(c, &ql, &nq)) return rc;
+    k_pois_true_res<<<grid_blocks(c, nq, TH), TH, 0, c->stream>>>(b, x, c->cflag, ql, nq, L.P, L.PL, c->singular,
+                                                                 c->scal + 2, c->partials, r_out);
+    c->n_launches += 1;
+    return check_cuda(cudaGetLastError(), "k_pois_true_res");
+}
+
 // Warm start (fs_params.warm_start): after the x = 0 initialisation, start
 // instead from the last converged pressure of the same kind of projection when
 // its residual is below half of |b|^2; r = b - A x, p = 0, iteration count 0.
@@ -867,13 +899,9 @@ static int try_warm_start(fs_ctx *c, bool jac)
     if (!c->prm.warm_start || !c->pw_valid[k] || !c->pw[k]) return FS_OK;
     const Layout &L = c->L;
     const int bs = grid_blocks(c, L.nC, TH);
-    k_pois_true_res<<<bs, TH, 0, c->stream>>>(c->pb, c->pw[k], c->cflag, L.nC, L.P, L.PL, c->singular,
-                                              c->scal + 2, c->partials, nullptr);
-    c->n_launches += 1;
-    FS_CUDA(cudaGetLastError());
     SolveScal m, h0;
     int rc;
-    if ((rc = read_scal(c, 2, &m)) || (rc = read_scal(c, 0, &h0))) return rc;
+    if ((rc = true_res(c, c->pb, c->pw[k], nullptr)) || (rc = read_scal(c, 2, &m)) || (rc = read_scal(c, 0, &h0))) return rc;
     if (h0.done || !(m.aux[0] < 0.5 * m.aux[1])) return FS_OK;
     FS_CUDA(cudaMemcpyAsync(c->px, c->pw[k], (size_t)L.nC * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
     if (jac)
@@ -1054,7 +1082,6 @@ static int solve_pressure_once(fs_ctx *c, fs_stats *st)
         if (rc) return rc;
     }
     const Layout &L = c->L;
-    const int bs = grid_blocks(c, L.nC, TH);
     // Mixed-precision iterative refinement. CG runs on FP32 vectors, so its
     // recursively updated residual drifts from b - A x, and the rounding of the
     // FP32 iterate alone leaves |b - A x| ~ 2e-7 |A x| |x| / |x|: with a smooth
@@ -1089,10 +1116,7 @@ static int solve_pressure_once(fs_ctx *c, fs_stats *st)
         // the check of this pass's system (b0 and x, then each correction's); its
         // residual, rounded once to FP32, is the next correction's right-hand side,
         // stored in pbr (in place from the second pass on)
-        k_pois_true_res<<<bs, TH, 0, c->stream>>>(c->pb, c->px, c->cflag, L.nC, L.P, L.PL, c->singular,
-                                                  c->scal + 2, c->partials, c->pbr);
-        c->n_launches += 1;
-        if ((rc = check_cuda(cudaGetLastError(), "k_pois_true_res")) || (rc = read_scal(c, 2, &m))) break;
+        if ((rc = true_res(c, c->pb, c->px, c->pbr)) || (rc = read_scal(c, 2, &m))) break;
         checked = true;
         if (pass == 0) {
             bb0 = m.aux[1];
@@ -1130,10 +1154,7 @@ static int solve_pressure_once(fs_ctx *c, fs_stats *st)
         return rc;
     }
     if (!checked) {  // a pass that did not converge: the residual of its own system
-        k_pois_true_res<<<bs, TH, 0, c->stream>>>(c->pb, c->px, c->cflag, L.nC, L.P, L.PL, c->singular,
-                                                  c->scal + 2, c->partials, nullptr);
-        c->n_launches += 1;
-        if ((rc = check_cuda(cudaGetLastError(), "k_pois_true_res")) || (rc = read_scal(c, 2, &m))) {
+        if ((rc = true_res(c, c->pb, c->px, nullptr)) || (rc = read_scal(c, 2, &m))) {
             c->pb = b0;
             return rc;
         }
@@ -1157,11 +1178,8 @@ static int pressure_tail(fs_ctx *c, const SolveScal &h, long long iters, double 
 {
     const Layout &L = c->L;
     const int bs = grid_blocks(c, L.nC, TH);
-    if (!known) {
-        k_pois_true_res<<<bs, TH, 0, c->stream>>>(c->pb, c->px, c->cflag, L.nC, L.P, L.PL, c->singular,
-                                                  c->scal + 2, c->partials, nullptr);
-        c->n_launches += 1;
-    }
+    if (!known)
+        if (int rc = true_res(c, c->pb, c->px, nullptr)) return rc;
     if (c->singular) {  // the mean-free representative
         k_liquid_sum<<<bs, TH, 0, c->stream>>>(c->px, c->cflag, L.nC, c->scal + 3, c->partials);
         k_sub_liquid_mean<<<bs, TH, 0, c->stream>>>(c->px, c->cflag, L.nC, c->scal + 3);
