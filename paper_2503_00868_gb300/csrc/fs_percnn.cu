@@ -85,7 +85,9 @@ __global__ void __launch_bounds__(TH) k_pc_res(const int *__restrict__ ql, int n
 }
 
 // out = m (W * x) (+ base when base != null): 27-tap correlation on liquid cells. A
-// row of three taps is formed from one float4 and its two neighbours.
+// row of three taps is formed from one float4 and its two neighbours. One guard plane
+// stands before the cells, so for quads in the first two rows of the first plane some of
+// these taps lie before the vector: off the grid, they count zero without a load.
 __global__ void __launch_bounds__(TH) k_pc_conv(const int *__restrict__ ql, int nq, const float *__restrict__ x,
                                                 const float *base, float *out, const uint8_t *__restrict__ cf, int P,
                                                 int PL, const __grid_constant__ PercnnW W)
@@ -100,8 +102,9 @@ __global__ void __launch_bounds__(TH) k_pc_conv(const int *__restrict__ ql, int 
 #pragma unroll
         for (int row = 0; row < 9; row++) {
             const int u = t + (row / 3 - 1) * PL + (row % 3 - 1) * P;
-            const float4 c = ldd4(x + u);
-            const float lf = ldd1(x + u - 1), rt = ldd1(x + u + 4);
+            const bool in = row > 1 || u >= 0, lin = row > 1 || u > 0;
+            const float4 c = in ? ldd4(x + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float lf = lin ? ldd1(x + u - 1) : 0.f, rt = in ? ldd1(x + u + 4) : 0.f;
             const float w0 = W.w[3 * row], w1 = W.w[3 * row + 1], w2 = W.w[3 * row + 2];
             v.x += w0 * lf; v.y += w0 * c.x; v.z += w0 * c.y; v.w += w0 * c.z;
             v.x += w1 * c.x; v.y += w1 * c.y; v.z += w1 * c.z; v.w += w1 * c.w;
@@ -131,7 +134,8 @@ __global__ void __launch_bounds__(TH) k_pc_lapsub(float *g, const float *__restr
     }
 }
 
-// dw[q] += sum over liquid cells of g_i r(i + o_q)
+// dw[q] += sum over liquid cells of g_i r(i + o_q); a tap before the vector (k_pc_conv)
+// is off the grid and adds nothing
 __global__ void __launch_bounds__(TH) k_pc_wgrad(const float *__restrict__ g, const float *__restrict__ r,
                                                  const uint8_t *__restrict__ cf, Layout L, double *dw)
 {
@@ -147,7 +151,8 @@ __global__ void __launch_bounds__(TH) k_pc_wgrad(const float *__restrict__ g, co
         const float gv = g[t];
         if (gv == 0.f) continue;
 #pragma unroll
-        for (int q = 0; q < 27; q++) acc[q] += (double)(gv * r[t + off[q]]);
+        for (int q = 0; q < 27; q++)
+            if (q > 3 || t + off[q] >= 0) acc[q] += (double)(gv * r[t + off[q]]);
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
