@@ -185,9 +185,10 @@ int launch_pbd_project(fs_ctx *c, F3 u, int hold, int iters, double eps, double 
     const Layout &L = c->L;
     const float inv_dx = (float)(1.0 / c->prm.dx);
     const int bc_ = grid_blocks(c, L.S, TH), bf = grid_blocks(c, 3LL * L.S, TH);
-    // cell-space scratch (no solve runs meanwhile, and each starts its vectors anew)
+    // cell-space scratch (no solve runs meanwhile, and each starts its vectors anew; px
+    // and pxh hold the last projection's pressure, which fs_pressure_pair reads)
     float *div = c->pr, *lam[2] = {c->pp[0], c->pp[1]};
-    uint8_t *nfree = reinterpret_cast<uint8_t *>(c->pxh);
+    uint8_t *nfree = reinterpret_cast<uint8_t *>(c->pxt);
     SolveScal *s = c->scal + 2;
     auto divergence = [&]() {
         k_pbd_div<<<bc_, TH, 0, c->stream>>>(u, c->cflag, c->fflag, L, hold, inv_dx, div, nfree, s, c->partials);
