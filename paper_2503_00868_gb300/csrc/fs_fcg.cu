@@ -80,17 +80,18 @@ __global__ void __launch_bounds__(TH) k_fcg_dots(const int *__restrict__ ql, int
     }
 }
 
-// p = z + sum_j beta_j p_j
+// p = z + sum_j beta_j p_j (beta_j: written by the launch before, so read as the
+// vectors are, after dep_wait and not by the non-coherent path)
 __global__ void __launch_bounds__(TH) k_fcg_dir(const int *__restrict__ ql, int nq, const float *__restrict__ z, Ring ring,
                                                 int nvalid, float *__restrict__ p, const SolveScal *s,
-                                                const double *__restrict__ beta)
+                                                const double *beta)
 {
     dep_wait();
     dep_go();
     if (s->done) return;
     float b[FCG_M];
 #pragma unroll
-    for (int j = 0; j < FCG_M; j++) b[j] = j < nvalid ? (float)beta[j] : 0.f;
+    for (int j = 0; j < FCG_M; j++) b[j] = j < nvalid ? (float)*(const volatile double *)(beta + j) : 0.f;
     float4 *p4 = reinterpret_cast<float4 *>(p);
     FS_FOR_LIST(ql, nq)
     {
