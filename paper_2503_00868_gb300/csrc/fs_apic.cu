@@ -467,13 +467,17 @@ __global__ void __launch_bounds__(G2P_TH) k_g2p(int np, float *x, float *v, floa
     const float lim = (float)(max(L.nx, max(L.ny, L.nz)) + 8);
     float xp[3], vp[3], Cp[9];
     warp_load<3>(x, first, n, sm, xp);
+    // a particle whose position is not finite reaches no node: its offsets count as
+    // finite ones, since each is multiplied by the zero that stands for such a node
+    const bool placed = isfinite(xp[0]) && isfinite(xp[1]) && isfinite(xp[2]);
+    const float xo[3] = {placed ? xp[0] : 0.f, placed ? xp[1] : 0.f, placed ? xp[2] : 0.f};
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         const Spline s = spline(xp, c, inv_dx, lim);
         const float *uc = u.c[c];
         float dxv[3];
 #pragma unroll
-        for (int q = 0; q < 3; q++) dxv[q] = ((float)(s.base[0] + q) + (c == 0 ? 0.f : 0.5f)) * dx - xp[0];
+        for (int q = 0; q < 3; q++) dxv[q] = ((float)(s.base[0] + q) + (c == 0 ? 0.f : 0.5f)) * dx - xo[0];
         const bool inside = in_faces(L, c, s.base[0], s.base[1], s.base[2]) &&
                             in_faces(L, c, s.base[0] + 2, s.base[1] + 2, s.base[2] + 2);
         const int t0 = (s.base[2] * L.R + s.base[1]) * L.P + s.base[0];
@@ -487,8 +491,8 @@ __global__ void __launch_bounds__(G2P_TH) k_g2p(int np, float *x, float *v, floa
                                 a2 = s.w[0][2] * node(2, ky, kz);
                     const float r0 = a0 + a1 + a2, r1 = a0 * dxv[0] + a1 * dxv[1] + a2 * dxv[2];
                     const float wyz = s.w[1][ky] * s.w[2][kz];
-                    const float dyv = ((float)(s.base[1] + ky) + (c == 1 ? 0.f : 0.5f)) * dx - xp[1];
-                    const float dzv = ((float)(s.base[2] + kz) + (c == 2 ? 0.f : 0.5f)) * dx - xp[2];
+                    const float dyv = ((float)(s.base[1] + ky) + (c == 1 ? 0.f : 0.5f)) * dx - xo[1];
+                    const float dzv = ((float)(s.base[2] + kz) + (c == 2 ? 0.f : 0.5f)) * dx - xo[2];
                     const float w = wyz * r0;
                     vc += w;
                     g0 += wyz * r1;
