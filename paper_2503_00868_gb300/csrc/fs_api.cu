@@ -392,6 +392,15 @@ int fs_set_params(fs_ctx *c, const fs_params *p)
     int rc = check_params(p);
     if (rc) return rc;
     if (p->mic_tau != c->prm.mic_tau || p->mic_sigma != c->prm.mic_sigma) c->mic_ready = 0;
+    // The iteration counts that size the next solves' first batches hold for a
+    // preconditioner, a tolerance and about the same viscosity operator: a Jacobi
+    // count of hundreds would enqueue as many V-cycles before the first look at the
+    // flag. (A fit moves nu a little at a time, and its counts stay.)
+    const bool pc = p->precond != c->prm.precond;
+    auto cc = [](const fs_params &q) { return q.nu * q.dt / (q.dx * q.dx); };
+    if (pc || p->tol_p != c->prm.tol_p) std::memset(c->it_last_p, 0, sizeof(c->it_last_p));
+    if (pc || p->tol_v != c->prm.tol_v || cc(*p) > 2.0 * cc(c->prm) || cc(c->prm) > 2.0 * cc(*p))
+        std::memset(c->it_last_v, 0, sizeof(c->it_last_v));
     c->prm = *p;
     // a new problem: no warm start from earlier solves (the floor of the first
     // CG pass stays: it depends on the mask and the scale of the pressure, and a

@@ -113,8 +113,9 @@ struct fs_ctx {
     // not try to go below
     double p_floor2[2];
     // iterations of the last CG pass of each kind: pressure [kind][refining],
-    // viscosity [dirichlet]; 0 unknown. The host runs that many minus one before
-    // its first read of the convergence flag.
+    // viscosity [dirichlet]; 0 unknown (a new mask, or parameters that move the count:
+    // fs_set_params). The host runs that many minus one before its first read of the
+    // convergence flag.
     int it_last_p[2][2], it_last_v[2];
     int solve_kind;       // kind of the pressure solve being run
     // viscosity solve (face space)
