@@ -41,6 +41,15 @@ constexpr int TH = 256;
 constexpr int P2G_SORT = 1 << 16;  // particles from which P2G orders them by cell
 constexpr int P2G_PER = 32;        // most particles per thread of the march
 
+// A node coordinate of a component whose nodes lie `off` cells into them (0 or 1/2),
+// clamped to [-8, lim]. One rounding, spelled out: the passes that order the particles
+// and the march that relies on their order must agree on a particle's cell to the last
+// bit, whatever a compiler would fuse in each of them.
+__device__ __forceinline__ float node_coord(float x, float off, float inv_dx, float lim)
+{
+    return fminf(fmaxf(__fmaf_rn(x, inv_dx, -off), -8.f), lim);
+}
+
 struct Spline {
     int base[3];
     float w[3][3];
@@ -54,7 +63,7 @@ __device__ __forceinline__ Spline spline(const float x[3], int c, float inv_dx, 
     Spline s;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        const float sc = fminf(fmaxf(x[a] * inv_dx - (a == c ? 0.f : 0.5f), -8.f), lim);
+        const float sc = node_coord(x[a], a == c ? 0.f : 0.5f, inv_dx, lim);
         const int b = (int)floorf(sc - 0.5f);
         const float f = sc - (float)b;
         s.base[a] = b;
@@ -68,7 +77,7 @@ __device__ __forceinline__ Spline spline(const float x[3], int c, float inv_dx, 
 // one of the three weights of one axis
 __device__ __forceinline__ float spline_weight(float x, int a, int c, float inv_dx, float lim, int k)
 {
-    const float sc = fminf(fmaxf(x * inv_dx - (a == c ? 0.f : 0.5f), -8.f), lim);
+    const float sc = node_coord(x, a == c ? 0.f : 0.5f, inv_dx, lim);
     const float f = sc - floorf(sc - 0.5f);
     if (k == 1) return 0.75f - (f - 1.f) * (f - 1.f);
     const float g = k == 0 ? 1.5f - f : f - 0.5f;
@@ -141,7 +150,7 @@ __device__ __forceinline__ int particle_cell(const float x[3], const CellBox &B,
     int cell[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        const float sc = fminf(fmaxf(x[a] * inv_dx - 0.5f, -8.f), lim);
+        const float sc = node_coord(x[a], 0.5f, inv_dx, lim);
         cell[a] = (int)floorf(sc - 0.5f) + 3;  // base + 1, from -2
     }
     if (cell[0] < 0 || cell[1] < 0 || cell[2] < 0 || cell[0] >= B.nx || cell[1] >= B.ny || cell[2] >= B.nz) return -1;
@@ -304,14 +313,13 @@ __device__ __forceinline__ void red_add2(float2 *p, float a, float b)
 
 // One component: a thread takes particles [e, e1) in cell order. The window of nodes
 // moves along x with the particles' cell; acc[x][y][z] = {momentum, mass}. The next
-// particle is loaded while this one is added.
+// particle is loaded while this one is added. (inv_dx and lim as in the passes that
+// ordered the particles.)
 template <int c>
 __device__ __forceinline__ void p2g_march(const P2gItem *__restrict__ items, unsigned e, unsigned e1, float2 *out,
-                                          const Layout &L, float dx)
+                                          const Layout &L, float dx, float inv_dx, float lim)
 {
     constexpr int NX = c == 0 ? 4 : 3, NY = c == 1 ? 4 : 3, NZ = c == 2 ? 4 : 3;
-    const float inv_dx = 1.f / dx;
-    const float lim = (float)(max(L.nx, max(L.ny, L.nz)) + 8);
     float2 acc[NX][NY][NZ];
 #pragma unroll
     for (int a = 0; a < NX; a++)
@@ -367,7 +375,7 @@ __device__ __forceinline__ void p2g_march(const P2gItem *__restrict__ items, uns
         int lo[3];
 #pragma unroll
         for (int a = 0; a < 3; a++)
-            lo[a] = a == c ? (int)floorf(fminf(fmaxf(q.x[a] * inv_dx - 0.5f, -8.f), lim) - 0.5f) : s.base[a];
+            lo[a] = a == c ? (int)floorf(node_coord(q.x[a], 0.5f, inv_dx, lim) - 0.5f) : s.base[a];
         if (lo[1] != j0 || lo[2] != k0) {  // another row of cells
             while (live > 0) advance();
             j0 = lo[1];
@@ -418,18 +426,19 @@ __device__ __forceinline__ void p2g_march(const P2gItem *__restrict__ items, uns
 // blockIdx.y = component; the ordered particles end at *total (those that reach no
 // node are not among them)
 __global__ void __launch_bounds__(128) k_p2g_rows(const P2gItem *__restrict__ items, const unsigned *__restrict__ total,
-                                                  int per, float2 *s0, float2 *s1, float2 *s2, Layout L, float dx)
+                                                  int per, float2 *s0, float2 *s1, float2 *s2, Layout L, float dx,
+                                                  float inv_dx, float lim)
 {
     const unsigned n = *total;
     const unsigned long long e = (unsigned long long)(blockIdx.x * 128u + threadIdx.x) * (unsigned)per;
     if (e >= n) return;
     const unsigned e1 = (unsigned)min(e + per, (unsigned long long)n);
     if (blockIdx.y == 0)
-        p2g_march<0>(items, (unsigned)e, e1, s0, L, dx);
+        p2g_march<0>(items, (unsigned)e, e1, s0, L, dx, inv_dx, lim);
     else if (blockIdx.y == 1)
-        p2g_march<1>(items, (unsigned)e, e1, s1, L, dx);
+        p2g_march<1>(items, (unsigned)e, e1, s1, L, dx, inv_dx, lim);
     else
-        p2g_march<2>(items, (unsigned)e, e1, s2, L, dx);
+        p2g_march<2>(items, (unsigned)e, e1, s2, L, dx, inv_dx, lim);
 }
 
 // u = momentum / mass where mass > 0; mass copy when wanted
@@ -615,7 +624,8 @@ int launch_p2g(fs_ctx *c, int np, const float *x, const float *v, const float *C
         // particles per thread: enough threads for the GPU first, then long marches
         const int per = std::max(4, std::min(P2G_PER, np / (c->num_sms * 256)));
         const int gr = (int)(((long long)np + 128LL * per - 1) / (128LL * per));
-        k_p2g_rows<<<dim3(gr, 3), 128, 0, c->stream>>>(w->items, w->ends + n - 1, per, s2[0], s2[1], s2[2], L, dx);
+        k_p2g_rows<<<dim3(gr, 3), 128, 0, c->stream>>>(w->items, w->ends + n - 1, per, s2[0], s2[1], s2[2], L, dx,
+                                                     inv_dx, lim);
         k_p2g_norm2<<<dim3(grid_blocks(c, L.S, TH), 3), TH, 0, c->stream>>>(s2[0], s2[1], s2[2], u, mass, L.S);
         c->n_launches += 7;
         FS_CUDA(cudaGetLastError());
