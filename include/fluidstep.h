@@ -351,6 +351,10 @@ int fs_splat_stats(const fs_ctx *c, unsigned long long *entries, unsigned long l
  *   x, v: [np][3] metres and m/s; C: [np][3][3] row-major (row c = gradient of
  *   component c); m: [np]; u_out: overwritten; mass_out (nullable): sum_p w_ip m_p.
  * FP32 atomic accumulation: the last bits depend on the scheduling.
+ * From 65536 particles on, and one per 64 cells, they are put in the order of the cells
+ * first, in memory that the context keeps until fs_destroy: 64 bytes for each of 9/8 of
+ * the largest np so far, and 4 bytes per cell. Without that memory they are scattered as
+ * they come.
  * FS_EINVAL on a NULL array or np < 0. */
 int fs_p2g(fs_ctx *c, int np, const float *x, const float *v, const float *C, const float *m, fs_mac *u_out,
            fs_mac *mass_out);

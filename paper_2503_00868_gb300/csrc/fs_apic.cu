@@ -555,7 +555,10 @@ __global__ void __launch_bounds__(G2P_TH) k_g2p(int np, float *x, float *v, floa
 
 }  // namespace
 
-// Workspace of the cell-ordered P2G, kept on the context and grown on demand.
+// Workspace of the cell-ordered P2G, kept on the context and grown on demand: 64 bytes
+// per particle, with room for an eighth more than the largest call so far (where that
+// can be had), so that a count that rises from call to call does not free and allocate
+// it, and wait for the device, each time.
 struct ApicState {
     unsigned *ends = nullptr, *sums = nullptr;
     P2gItem *items = nullptr;
@@ -590,14 +593,17 @@ static bool apic_workspace(fs_ctx *c, long long np, long long n)
         *p = nullptr;
         return false;
     };
-    if (np > s->cap) {
-        cudaFree(s->items);
-        s->items = nullptr;
-        s->cap = 0;
-    }
-    if (!have(&s->ends, n) || !have(&s->sums, (n + SC_ITEMS - 1) / SC_ITEMS) || !have(&s->items, np)) return false;
-    s->cap = std::max(s->cap, np);
-    return true;
+    if (!have(&s->ends, n) || !have(&s->sums, (n + SC_ITEMS - 1) / SC_ITEMS)) return false;
+    if (np <= s->cap) return true;
+    cudaFree(s->items);
+    s->items = nullptr;
+    s->cap = 0;
+    for (long long cap : {np + np / 8, np})
+        if (have(&s->items, cap)) {
+            s->cap = cap;
+            return true;
+        }
+    return false;
 }
 
 int launch_p2g(fs_ctx *c, int np, const float *x, const float *v, const float *C, const float *m, F3 u, F3 mass)
