@@ -219,8 +219,7 @@ __global__ void __launch_bounds__(TH) k_pc_finish(const float *__restrict__ b, c
             rr.add(r[t] * r[t]);
             bb.add(b[t] * b[t]);
         }
-    KSum v[2] = {rr, bb};
-    double tot[2];
+    double v[2] = {rr.value(), bb.value()}, tot[2];
     if (grid_reduce<2>(v, partials, &s->ticket, tot) && threadIdx.x == 0) {
         s->rr = tot[0];
         s->bb = tot[1];
