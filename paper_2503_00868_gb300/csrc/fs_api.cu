@@ -97,7 +97,7 @@ static const char *kKernelNames[K_COUNT] = {"pressure_spmv", "pressure_update", 
 
 struct Prof {
     std::vector<cudaEvent_t> free_ev, all_ev;
-    struct Pending { int id; cudaEvent_t a, b; double bytes; };
+    struct Pending { int id; cudaEvent_t a, b; double bytes; long long it; };
     std::vector<Pending> pending;
     double ms[K_COUNT] = {};
     double bytes[K_COUNT] = {};
@@ -125,7 +125,7 @@ void prof_add(fs_ctx *c, int id, cudaEvent_t a, cudaEvent_t b, double bytes)
         if (b) p->free_ev.push_back(b);
         return;
     }
-    p->pending.push_back({id, a, b, bytes});
+    p->pending.push_back({id, a, b, bytes, c->prof_it});
 }
 
 void prof_count(fs_ctx *c, int id, long long launches)
@@ -134,13 +134,14 @@ void prof_count(fs_ctx *c, int id, long long launches)
     static_cast<Prof *>(c->prof)->all[id] += launches;
 }
 
-void prof_flush(fs_ctx *c)
+void prof_flush(fs_ctx *c, long long iters)
 {
     if (!c->prof) return;
     Prof *p = static_cast<Prof *>(c->prof);
     for (auto &q : p->pending) {
         float ms = 0.f;
-        if (cudaEventElapsedTime(&ms, q.a, q.b) == cudaSuccess) {
+        if (q.it > iters) {  // enqueued after convergence
+        } else if (cudaEventElapsedTime(&ms, q.a, q.b) == cudaSuccess) {
             p->ms[q.id] += ms;
             p->bytes[q.id] += q.bytes;
             p->n[q.id] += 1;

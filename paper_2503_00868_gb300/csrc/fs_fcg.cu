@@ -298,6 +298,7 @@ int solve_pressure_fcg(fs_ctx *c, SolveScal *h, bool warm)
     long long k = 0;
     unsigned herr = 0;
     std::vector<std::pair<int, double>> hist;  // (iteration, r.r) at the host checks
+    ProfIteration iteration(c);
     for (;;) {
         if ((rc = read_scal(c, 0, h, &herr))) return rc;
         if (h->done) break;
@@ -311,6 +312,7 @@ int solve_pressure_fcg(fs_ctx *c, SolveScal *h, bool warm)
             break;
         }
         for (int b = 0; b < c->prm.check_every; b++, k++) {
+            iteration(k);
             const int slot = (int)(k % FCG_M);
             const int nvalid = (int)std::min<long long>(k, FCG_M);
             Ring ring;

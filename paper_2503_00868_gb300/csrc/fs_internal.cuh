@@ -167,6 +167,7 @@ struct fs_ctx {
     // per-kernel timing (fs_profile)
     int prof_on;
     int prof_period;            // time every prof_period-th CG iteration
+    long long prof_it;          // 1 + the CG iteration being enqueued, 0 outside of one
     void *prof;                 // fs::Prof
     long long n_launches;       // kernels launched by this context since fs_profile(c, 1)
 };
@@ -652,6 +653,15 @@ enum KernelId : int {
 cudaEvent_t prof_mark(fs_ctx *c);   // records an event on the stream (nullptr when off)
 void prof_add(fs_ctx *c, int id, cudaEvent_t a, cudaEvent_t b, double bytes);
 void prof_count(fs_ctx *c, int id, long long launches);  // launches of a kind, timed or not
-void prof_flush(fs_ctx *c);         // call after the stream has been synchronised
+// Call after the stream has been synchronised. An entry made in a CG iteration counts
+// if that iteration was among the first `iters` (of the pass being run, those that did
+// work: the launches of a batch after convergence return at once).
+void prof_flush(fs_ctx *c, long long iters = 1LL << 62);
+struct ProfIteration {  // names the iterations of a pass to prof_add
+    fs_ctx *c;
+    explicit ProfIteration(fs_ctx *ctx) : c(ctx) {}
+    ~ProfIteration() { c->prof_it = 0; }
+    void operator()(long long it) { c->prof_it = it + 1; }
+};
 
 }  // namespace fs

@@ -781,7 +781,7 @@ int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err)
     std::atomic_thread_fence(std::memory_order_acquire);
     std::memcpy(out, &h->s, sizeof(SolveScal));
     if (err) *err = h->err;
-    prof_flush(c);
+    prof_flush(c, out->iter);
     return FS_OK;
 }
 
@@ -1019,9 +1019,11 @@ static int pcg_iterate(fs_ctx *c, SolveScal &h)
     const int check = c->prm.precond == FS_PRECOND_MG ? std::min(c->prm.check_every, 4) : c->prm.check_every;
     int &last = c->it_last_p[c->solve_kind & 1][c->refining ? 1 : 0];
     const CgBatches batches(last, check, c->prm.maxit_p, c->prm.precond == FS_PRECOND_MG);
+    ProfIteration iteration(c);
     for (;;) {
         const int nb = batches.size(launched);
         for (int b = 0; b < nb; b++) {
+            iteration(launched + b);
             // (at an iteration's start, so that none follows the last one)
             if (!jac)
                 if (int rc = precondition(launched + b == 0)) return rc;
@@ -1279,9 +1281,11 @@ int solve_viscosity(fs_ctx *c, bool dirichlet, fs_stats *st)
     }
     int &last = c->it_last_v[dirichlet ? 1 : 0];
     const CgBatches batches(last, check, c->prm.maxit_v, mg);
+    ProfIteration iteration(c);
     for (;;) {
         const int nb = batches.size(launched);
         for (int b = 0; b < nb; b++) {
+            iteration(launched + b);
             if (mg)
                 if (int rc = precondition(launched + b == 0)) return rc;
             const bool samp = c->prof_on && ((launched + b) % c->prof_period) == 0;  // every prof_period-th
