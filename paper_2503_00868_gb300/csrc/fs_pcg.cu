@@ -766,6 +766,7 @@ int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err)
     }
     const unsigned seq = ++c->post_seq;
     launch_dep(k_post, 1, 128, 0, c->stream, c->scal + which, c->err_word, h, seq);
+    c->n_launches += 1;
     FS_CUDA(cudaGetLastError());
     volatile unsigned *flag = &h->seq;
     for (unsigned n = 1; *flag != seq; n++) {
