@@ -63,8 +63,9 @@ struct NetState {
     int *tlist_tc;        // tiles of the tensor-core layer (TC_M x TC_NY of one plane), sorted the same way
     int tcount_tc[6];
     int kernel;           // inference layers: 0 mma.sync (k_conv), 1 tcgen05 (k_conv_tc)
-    double last_flops;    // useful flops of the last inference, on the tiles it visited
     long long tlist_epoch;  // mask epoch the list was built for (-1: none)
+    double flops;         // of one inference on the cells that each layer must compute (net_flops)
+    long long flops_epoch;  // mask epoch it was counted for (-1: none)
     __nv_bfloat16 *wt;    // layers 2-4 backward-data: [3][27 tap][16 ci][16 co], tap flipped
     __nv_bfloat16 *act;   // [6][nC][16]: x (2 ch used), a1, a2, a3, a4, spare
     __nv_bfloat16 *gact;  // [2][nC][16] gradient ping-pong
@@ -808,6 +809,32 @@ __global__ void __launch_bounds__(256) k_conv_tile_dist(const uint8_t *__restric
     if (threadIdx.x == 0) dist[tb] = (uint8_t)best;
 }
 
+// The cells of the grid within Chebyshev distance d of the liquid -> count[d], d = 0 .. 4
+// (once per mask, for the profiled flops).
+__global__ void __launch_bounds__(256) k_net_reach(const uint8_t *__restrict__ cf, Layout L, unsigned long long *count)
+{
+    const int ncell = L.nx * L.ny * L.nz;
+    unsigned long long near[5] = {0, 0, 0, 0, 0};
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ncell; e += gridDim.x * blockDim.x) {
+        const int i = e % L.nx, j = (e / L.nx) % L.ny, k = e / (L.nx * L.ny);
+        int d = cf[cell_t(L, i, j, k)] & CF_LIQ ? 0 : 5;
+        for (int z = -4; z <= 4 && d > 0; z++)
+            for (int y = -4; y <= 4; y++)
+                for (int x = -4; x <= 4; x++) {
+                    const int far = max(abs(z), max(abs(y), abs(x)));
+                    if (far < d && in_grid(L, i + x, j + y, k + z) && (cf[cell_t(L, i + x, j + y, k + z)] & CF_LIQ))
+                        d = far;
+                }
+#pragma unroll
+        for (int q = 0; q < 5; q++) near[q] += d <= q;
+    }
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+        for (int o = 16; o > 0; o >>= 1) near[q] += __shfl_xor_sync(0xffffffffu, near[q], o);
+        if ((threadIdx.x & 31) == 0 && near[q]) atomicAdd(count + q, near[q]);
+    }
+}
+
 // max |r| over the liquid, as float bits (non-negative floats order like ints), over
 // the list of quads that hold liquid (r is zero on their other cells)
 __global__ void __launch_bounds__(256) k_absmax(const int *__restrict__ ql, int nq, const float *__restrict__ r,
@@ -1237,7 +1264,7 @@ int net_alloc(fs_ctx *c, bool training)
     if (!n) {
         n = new (std::nothrow) NetState();
         if (!n) return set_error(FS_ENOMEM, "host allocation failed");
-        n->tlist_epoch = -1;
+        n->tlist_epoch = n->flops_epoch = -1;
         c->net = n;
     }
     auto alloc = [&](void **p, size_t bytes) -> int {
@@ -1490,11 +1517,28 @@ static int net_forward(fs_ctx *c, const float *r, float *z, float *y, bool keep,
     a.ntiles = tiles_for(5);
     if ((rc = launch(IN_ACT, OUT_Z, a))) return rc;
     FS_CUDA(cudaGetLastError());
-    // the useful flops of the layers, on the cells of the tiles they visit:
-    // 2 x 27 x (2 x 16 + 3 x 16 x 16 + 16 x 1) per cell
-    n->last_flops = 0.0;
-    const double fl[5] = {2.0 * 27 * 2 * 16, 2.0 * 27 * 16 * 16, 2.0 * 27 * 16 * 16, 2.0 * 27 * 16 * 16, 2.0 * 27 * 16};
-    for (int l = 1; l <= 5; l++) n->last_flops += fl[l - 1] * (tc ? 256.0 : 256.0 * CV_Z) * (double)tiles_for(l);
+    return FS_OK;
+}
+
+// The flops of one inference for the current mask: layer l must be computed on the cells
+// within 5 - l of the liquid, 2 x 27 x (channels in) x (channels out) each. What a tile
+// holds beside them, and the channels a kernel pads to, do not count.
+static int net_flops(fs_ctx *c)
+{
+    NetState *n = net(c);
+    if (n->flops_epoch == c->mask_epoch) return FS_OK;
+    const Layout &L = c->L;
+    unsigned long long *dev = reinterpret_cast<unsigned long long *>(c->partials), cells[5];
+    FS_CUDA(cudaMemsetAsync(dev, 0, sizeof(cells), c->stream));
+    k_net_reach<<<grid_blocks(c, (long long)L.nx * L.ny * L.nz, 256), 256, 0, c->stream>>>(c->cflag, L, dev);
+    c->n_launches += 1;
+    FS_CUDA(cudaGetLastError());
+    FS_CUDA(cudaMemcpyAsync(cells, dev, sizeof(cells), cudaMemcpyDeviceToHost, c->stream));
+    FS_CUDA(cudaStreamSynchronize(c->stream));
+    const double ch[5] = {2.0 * 16, 16.0 * 16, 16.0 * 16, 16.0 * 16, 16.0};
+    n->flops = 0.0;
+    for (int l = 1; l <= 5; l++) n->flops += 2.0 * 27 * ch[l - 1] * (double)cells[5 - l];
+    n->flops_epoch = c->mask_epoch;
     return FS_OK;
 }
 
@@ -1502,9 +1546,11 @@ int net_apply(fs_ctx *c, const float *r, float *z, const int *done)
 {
     NetState *n = net(c);
     if (!n || !n->loaded) return set_error(FS_ESTATE, "the learned preconditioner has no network loaded");
+    if (c->prof_on)
+        if (int rc = net_flops(c)) return rc;
     cudaEvent_t e0 = prof_mark(c);
     int rc = net_forward(c, r, z, nullptr, false, done);
-    prof_add(c, K_NET_APPLY, e0, prof_mark(c), n->last_flops);  // flops, not bytes: a tensor-core entry
+    prof_add(c, K_NET_APPLY, e0, prof_mark(c), n->flops);  // flops, not bytes: a tensor-core entry
     return rc;
 }
 

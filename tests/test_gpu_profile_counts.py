@@ -1,5 +1,7 @@
 """The profile counts what did work: with every iteration timed, an entry of a solve has
-as many launches as the solve has iterations, though a batch enqueues more."""
+as many launches as the solve has iterations, though a batch enqueues more; the network's
+flops are those of the cells that each layer must compute."""
+import numpy as np
 import pytest
 
 from paper_2503_00868_gb300 import fluidstep as F
@@ -7,6 +9,17 @@ from paper_2503_00868_gb300 import train_precond as T
 from paper_2503_00868_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
+
+
+def network_flops(types):
+    near, cells = types == 1, []
+    for _ in range(5):  # within 0 .. 4 cells of the liquid
+        cells.append(int(near.sum()))
+        for ax in range(3):
+            p = np.pad(near, [(1, 1) if a == ax else (0, 0) for a in range(3)])
+            lo, hi = (np.take(p, range(s, s + types.shape[ax]), ax) for s in (0, 2))
+            near = near | lo | hi
+    return sum(54.0 * c * n for c, n in zip((2 * 16, 256, 256, 256, 16), cells[::-1]))
 
 
 @pytest.mark.parametrize("role,precond", [("net", F.FS_PRECOND_LEARNED), ("net_mg", F.FS_PRECOND_LEARNED_MG)])
@@ -20,8 +33,9 @@ def test_network(role, precond):
     rc, st = g.project(g.pack(W.random_mac(nx, ny, nz, 5)))
     prof = g.profile_read()
     assert rc == F.FS_OK and st["iters_p"] % 8  # the last batch holds iterations after convergence
-    launches, _, _, every = prof["net_apply"]
+    launches, _, flops, every = prof["net_apply"]
     assert launches == every == st["iters_p"]
+    assert flops / launches == network_flops(types)
     assert prof["fcg_vectors"][0] == st["iters_p"]
 
 
