@@ -1548,8 +1548,7 @@ bool mg_rz(fs_ctx *c, bool faces, const float *r, const float *z, int first, Sol
     const MgSet *t = listed_set(c, faces);
     if (!t) return false;
     launch_dep(k_mg_rz, grid_blocks(c, t->lev[0].nq, TH), TH, 0, c->stream, t->lev[0].ql, t->lev[0].nq, r, z, first, s, c->partials);
-    c->n_launches += 1;
-    return cudaPeekAtLastError() == cudaSuccess;
+    return cudaPeekAtLastError() == cudaSuccess;  // (the caller counts the launch)
 }
 
 int mg_levels(const fs_ctx *c)
