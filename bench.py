@@ -47,32 +47,24 @@ PROFILE_PERIOD = 8   # time every 8th CG iteration inside the timed region
 METRIC = "fwd+adjoint cell-steps/s at 256^3"
 UNIT = "cell-steps/s"
 
-# ncu DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum,
-# bytes) of the kernels, keyed by the profile name; each entry holds the hash of
-# the files that define the kernel and the data layout it reads, and is reported
-# only while those files are unchanged (capture commands in profiles/).
+# ncu DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum, bytes) of
+# the kernels, keyed by the profile name, from one step of the benchmark's 256^3 blob with
+# the multigrid preconditioner (profiles/kernel_counters.md; writes still held dirty in L2
+# when a kernel ends are not counted). `source` is the hash of KERNEL_FILES at the capture:
+# the kernels, the list walks and grid sums they are made of, the code that builds their
+# lists and the mask layout they read. An entry is reported only while those files are
+# unchanged; one whose kernel has other files names them in `files`.
+KERNEL_FILES = ("fs_pcg.cu", "fs_internal.cuh", "fs_mg.cu", "fs_mask.cu")
+CAPTURED = "754c8d7550d0c6ed"
 NCU_TRAFFIC = {
-    # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum on the benchmark's 256^3 blob with the
-    # multigrid preconditioner (profiles/fwd_adjoint_256.md); DRAM writes still held dirty in L2
-    # when the kernel ends are not counted
-    "visc_spmv": {"bytes_per_launch": 342685440 + 134320896, "source": "5e31bb1c3ef8787b"},
-    "visc_update": {"bytes_per_launch": 387683584 + 125340416, "source": "5e31bb1c3ef8787b"},
-    # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:k_mg0_smooth2 on the
-    # benchmark's 256^3 blob, one level-0 launch (profiles/mg0_kernels_256_ncu.md); the entry
-    # names its own files: the V-cycle kernels and the mask layout they read
-    "mg0_smooth2": {"bytes_per_launch": 50603776 + 3720704, "source": "4cfc780494228df8",
-                    "files": ("fs_mg.cu", "fs_mask.cu")},
-    # the same metrics -k regex:^k_mg0_smooth$ on a 256^3 blob projection with the multigrid
-    # preconditioner: the last level-0 sweep of a pressure V-cycle, which forms r.z (the mean
-    # of two launches; profiles/mg0_kernels_256_ncu.md); its files include the grid sums
-    # the same metrics -k regex:k_spmv_list on that projection: the pressure operator apply over
-    # the multigrid level-0 list of active quads (the mean of four launches; profiles/spmv_list_256_ncu.md)
-    "pressure_spmv": {"bytes_per_launch": 85581312 + 35093888, "source": "83675cdd5bd4c57e",
-                      "files": ("fs_pcg.cu", "fs_internal.cuh", "fs_mg.cu", "fs_mask.cu")},
-    "mg0_smooth_z": {"bytes_per_launch": 83167232 + 5408384, "source": "5ebc55d1e28ef6ee",
-                     "files": ("fs_mg.cu", "fs_internal.cuh", "fs_mask.cu")},
+    "visc_spmv": {"bytes_per_launch": 255822000 + 135620000, "source": CAPTURED},
+    "visc_update": {"bytes_per_launch": 407085000 + 125030000, "source": CAPTURED},
+    "pressure_spmv": {"bytes_per_launch": 83889000 + 22773000, "source": CAPTURED},
+    "pressure_update": {"bytes_per_launch": 134928000 + 14142000, "source": CAPTURED},
+    "mg0_smooth2": {"bytes_per_launch": 50285000 + 1668000, "source": CAPTURED},
+    # the last sweep of a pressure V-cycle's level 0, which forms r.z
+    "mg0_smooth_z": {"bytes_per_launch": 83163000 + 5327000, "source": CAPTURED},
 }
-KERNEL_FILES = ("fs_pcg.cu", "fs_mask.cu")
 
 
 def args_parse():
