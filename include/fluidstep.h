@@ -494,14 +494,17 @@ int fs_net_train_step(fs_ctx *c, const float *b_batch, const float *q_batch, int
  * then on brackets launches of the solver kernels (every k-th CG iteration of
  * each batch), the advection kernels and the preconditioners with CUDA events on
  * the context's stream; fs_profile(c, 0) stops. It also counts every kernel the
- * context launches (reported as the entry "all_kernels"). Timing is collected when a call synchronises, so it adds no host
- * round trip. fs_profile_read copies up to `max` entries (one per kernel kind
- * that ran) into `out` and sets *count. `bytes` is the ALGORITHMIC traffic summed
- * over the launches: for the CG kernels the flag byte of every element of the
- * launch range plus, per active element (liquid cell or fluid face), 16 bytes for
- * the fused direction update and operator apply (read r or z and p, write p and
- * Ap) and 24 bytes for the iterate update (read x, r, p, Ap, write x, r); zero for
- * kernels without a stated figure. */
+ * context launches (reported as the entry "all_kernels"). Timing is collected when a
+ * call synchronises, so it adds no host round trip; an iteration that was enqueued after
+ * its solve had converged, whose launches return at once, does not count.
+ * fs_profile_read copies up to `max` entries (one per kernel kind that ran) into `out`
+ * and sets *count. `bytes` is the ALGORITHMIC traffic summed over the launches: for the
+ * CG kernels, per quad of four elements that holds an unknown, 8 bytes (its list entry
+ * and flags; the iterate update 4, but 8 with Jacobi), plus, per unknown (liquid cell or
+ * fluid face), 16 bytes for the fused direction update and operator apply (read r or z
+ * and p, write p and Ap) and 24 bytes for the iterate update (read x, r, p, Ap, write x,
+ * r). For "net_apply" it is the flops of the applications, on the cells that each layer
+ * must compute; zero for kernels without a stated figure. */
 typedef struct {
     char name[32];
     long long launches;      /* launches timed (every k-th of the sampled kinds) */

@@ -458,8 +458,9 @@ __global__ void __launch_bounds__(TH) k_p2g_norm2(const float2 *__restrict__ s0,
 // A thread per particle. The particles' 3 and 9 floats pass through shared memory,
 // warp by warp, so that global memory sees consecutive words (a thread reading its
 // own 36-byte record makes every access touch nine lines); a row of three nodes is
-// summed before its y and z weights apply. The gathers of the field from L1 and L2
-// bound it.
+// summed before its y and z weights apply. The latency of the gathers bounds it: at
+// 128^3 with 3.3 M particles (181 us) most stalls wait for them, with L1 at 64 % of its
+// rate, instructions on 60 % of the cycles and DRAM at 47 %.
 constexpr int G2P_TH = 128;
 
 __global__ void __launch_bounds__(G2P_TH) k_g2p(int np, float *x, float *v, float *C, float *F,

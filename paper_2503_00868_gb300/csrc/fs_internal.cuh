@@ -434,8 +434,8 @@ __device__ __forceinline__ bool grid_reduce(KSum (&v)[K], double *partials, unsi
 // a launch before it may write (or may still read), then dep_go to let the next one
 // start: since each of them completes only after its own dep_wait, completion is
 // transitive along the stream. (With dep_go first, six kernels of a small grid's
-// V-cycle waited at once, in each other's slots: 12 % slower there and on the TMA-fed
-// operator apply, 5 % at 128^3.) Anything launched otherwise (copies, other kernels)
+// V-cycle waited at once, in each other's slots: 12 % slower there, 5 % at 128^3.)
+// Anything launched otherwise (copies, other kernels)
 // waits for full completion on either side. A projection's 100 sub-steps of two
 // kernels at 128^3 went from 1.62 to 1.24 ms, a forward and a reverse step with
 // multigrid from 3.66 to 2.51 at 53 x 44 x 39 and from 28.2 to 25.7 at 256^3.
@@ -461,7 +461,10 @@ inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 // Loads of what a launch before this one writes, for kernels launched by launch_dep:
 // not the non-coherent path (its data may not change while the kernel runs, and this
 // kernel runs beside its predecessor), and not moved above dep_wait by the compiler
-// (volatile, as dep_wait is); stores may still move past them.
+// (volatile, as dep_wait is); stores may still move past them. The same goes for a
+// predecessor's scalars: through a volatile pointer, never a const __restrict__ one.
+// __ldg stays for what no launch of a solve writes (masks, lists, weights) or what an
+// ordinary launch in between has waited for.
 __device__ __forceinline__ float4 ldd4(const float *p)
 {
     float4 v;

@@ -27,7 +27,7 @@
 //                  block);
 //   k_adam         Adam on the FP32 master weights, then the bf16 copies.
 // Layout: activations are channel-last, [cell][16] bf16 (32 bytes per cell) in
-// cell space; a neighbour outside the grid reads zero (checked per cell).
+// cell space; a neighbour outside the grid reads zero (the tile copies fill zeros there).
 #include <cuda_bf16.h>
 
 #include <new>
@@ -149,10 +149,11 @@ struct ConvArgs {
 // 16 cells, one per row, whose sums it holds in registers with the weights of all 27
 // taps (108 registers). An input row of a plane is read once per x shift and serves
 // the three output rows it touches, so a warp issues 90 ldmatrix for 432 MMAs; with
-// one row per warp and the weights read beside the cells it was 108 for 108, and
-// shared-memory bandwidth bound the layer (264 us on a union of spheres at 256^3; now
-// 154, with the MMA pipe near its rate, and the last layer 89 from 240). Per
-// output the taps are summed in the order dz, dy, dx, one MMA each, as before. The
+// one row per warp and the weights read beside the cells it was 108 for 108 (264 us on
+// a union of spheres at 256^3; now 154, and the last layer 89 from 240). The tensor pipe
+// is active 68 % of the cycles there (the last layer: 53), and two warps per scheduler
+// wait for it or for the latency of an MMA most of the rest; L1 moves a third of its
+// rate. Per output the taps are summed in the order dz, dy, dx, one MMA each, as before. The
 // next tile comes by one tensor copy (zeros off the grid) while this one is worked
 // on: with 2 warps per scheduler, cp.async and its index arithmetic in the computing
 // warps left the MMA pipe idle half the time. The copy's 32-byte swizzle swaps the
@@ -408,7 +409,8 @@ __global__ void __launch_bounds__(256, 1) k_conv(const __grid_constant__ CUtenso
 // fragment reads the word of the cell l % 4 to the right of its row's first tap (the
 // fourth has weight zero). 9 MMAs pairs per 16 cells in place of 27 of K = 16 on
 // channels padded from 2 to 16 (319 us on a union of spheres at 256^3, most of it the
-// padded tile; now 85, bound by its loads and the 32 bytes it writes per cell).
+// padded tile; now 85, with the tensor pipe active 45 % of the cycles and every memory
+// below half its rate: four warps per scheduler that wait for an MMA's latency).
 __device__ __forceinline__ void mma_bf16_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0)
 {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
@@ -450,6 +452,8 @@ __global__ void __launch_bounds__(256, 2) k_conv1(const __grid_constant__ ConvAr
     constexpr int PER = ((CV_Z + 2) * TYH * TXH + 255) / 256;
     float rv[PER];
     uint8_t fv[PER];
+    // (r by __ldg: its writer is not the launch before, but k_absmax's predecessor, and
+    // k_absmax, an ordinary launch, has waited for it)
     auto fetch = [&](int idx) {
         int i0, j0, k0;
         conv_tile(__ldg(a.tiles + idx), L, i0, j0, k0);
@@ -1017,8 +1021,10 @@ __global__ void __launch_bounds__(256) k_bwd_last(const float *__restrict__ gy, 
 // An FP32 g (the last layer) enters as three bf16 rows of M whose sum it is
 // exactly (8 + 8 + 8 significant bits). The next tile is copied (cp.async) while
 // this one is worked on. At 64^3 a 16 x 16 layer takes 27 us (FP32 cores, one
-// thread per weight walking the tile's cells: 3.09 ms), the last layer 26 (247);
-// the copies of the tiles' halos (4 times the cells) and their latency bound it.
+// thread per weight walking the tile's cells: 3.09 ms), the last layer 26 (247).
+// One block of 12 warps fits an SM (its registers, and its copies of the tiles with
+// halo, 4 times the cells): the tensor pipe is active 25 % of the cycles, instructions
+// issue on 45 %, and warps wait for ldmatrix, an MMA's latency or the barrier.
 constexpr int WG_TH = 384;
 constexpr int WG_A = TCELLS * 32, WG_G = NT_X * NT_Y * 32;  // bytes of a tile's two operands
 constexpr size_t WG_SMEM = 2 * (size_t)(WG_A + WG_G);

@@ -8,7 +8,8 @@
 // The CG scalars (alpha, beta, r.z, r.r) stay on the device: the last block of
 // each reducing kernel updates them, so a batch of iterations runs without a
 // host round trip; the host reads the convergence flag every `check_every`
-// iterations. Once `done` is set every later kernel of the batch returns at once.
+// iterations. Once `done` is set every later kernel of the batch returns at once, but
+// for the MIC(0) sweeps and the removal of a null mode, which run in full.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -786,7 +787,7 @@ int read_scal(fs_ctx *c, int which, SolveScal *out, unsigned *err)
     return FS_OK;
 }
 
-// A bounded wait of a TMA-fed kernel or of the MIC(0) wavefront that ran out
+// A bounded wait of the MIC(0) wavefront or of the network's kernels that ran out
 // leaves a bit in the error word.
 int check_wait_error(fs_ctx *c, const char *what, unsigned herr)
 {

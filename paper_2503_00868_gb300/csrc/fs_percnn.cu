@@ -14,8 +14,8 @@
 // so the step's adjoint applies the same projection to the cotangent.
 // Per sub-step: one residual pass and one 27-point correlation pass over the list of
 // quads that hold liquid. At 128^3 (a blob, 40 %) the dense passes, with 27 scalar
-// loads per cell, took 5.6 and 21 us, these 3.6 and 6.2; both stay in L2, and the
-// launches' gaps (2 x 2.4 us) are next.
+// loads per cell, took 5.6 and 21 us, these 3.6 and 6.2; both stay in L2. The launches'
+// gaps (2 x 2.4 us) went with dependent launches: 12 us per sub-step for the two.
 //
 // Training (fs_percnn_grad): the energy-norm loss of Sec. 3.4.1's fit,
 //   e = p_K - q, loss = e^T L_p e / q^T L_p q,

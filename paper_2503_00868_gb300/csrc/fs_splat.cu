@@ -28,9 +28,10 @@
 //
 // Bitonic sorts of every segment and a radix sort of the longest by one block took
 // 407 and 126 us of a 650 us frame (835 k Gaussians at 1920 x 1080, 5.7 M pairs); this
-// step takes 178 of 275. The compositing's instructions bound it now: a warp has a
-// block of 8 x 4 pixels and walks only the records whose box meets it (208 us when it
-// walked them all), which leaves the order and every sum as they were.
+// step takes 178 of 275. The latency of the compositing's own instructions is most of
+// it now (issue on 62 % of the cycles, L1 below half its rate): a warp has a block of
+// 8 x 4 pixels and walks only the records whose box meets it (208 us when it walked
+// them all), which leaves the order and every sum as they were.
 #include <cmath>
 #include <new>
 

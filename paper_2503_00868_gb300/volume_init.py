@@ -67,11 +67,10 @@ def main():
     e1.record()
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1)
-    lay = F.fs_layout(g.ctx)
-    S = lay.nelems
-    # per iteration and element of the public layout: read 3 face arrays + cell flag,
-    # write lambda (17 B); read lambda, 3 face flags, 3 face arrays, write them (31 B)
-    bytes_iter = 48.0 * S
+    # per iteration and liquid cell: read Lambda, the constraint and the flag byte, write
+    # Lambda (13 B); on grids whose arrays stay in L2 the rate is L2's, not HBM's. The time
+    # per iteration includes its share of the passes over the faces at either end.
+    bytes_iter = 13.0 * float((types == 1).sum())
     per_it = ms / (a.iters + 1) * 1e-3
     print(json.dumps({"grid": [n, n, n], "occupancy": info["occupancy"], "iters": a.iters,
                       "ms": ms, "us_per_iteration": per_it * 1e6, "div_norm_after": norm,
