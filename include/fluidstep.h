@@ -220,7 +220,10 @@ int fs_set_mask(fs_ctx *c, const uint8_t *cell_type_dense, const fs_mac *bc);
  * u_in, u_out: DEVICE fields, must not alias. u_visc: nullable DEVICE field that
  * receives the field after viscosity (the input of the projection), which
  * fs_adjoint_step can reuse instead of recomputing it. st: nullable host stats.
- * Returns FS_ENOCONV/FS_ENONFINITE/FS_EBREAKDOWN from the solves. */
+ * Returns FS_ENOCONV/FS_ENONFINITE/FS_EBREAKDOWN from the solves, with u_out written.
+ * Where a solve could not run (FS_ENOMEM for its lists or scratch, FS_ESTATE without the
+ * network or the kernel it needs, FS_ETIMEOUT, FS_ECUDA) the call ends there and u_out is
+ * not a step; so too fs_project and fs_adjoint_step. */
 int fs_step(fs_ctx *c, const fs_mac *u_in, fs_mac *u_out, fs_mac *u_visc, fs_stats *st);
 
 /* Pressure projection alone (Sec. 3.2.2, Poisson pressure equation), in place on u.

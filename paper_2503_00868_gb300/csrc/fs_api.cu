@@ -421,6 +421,13 @@ int fs_set_mask(fs_ctx *c, const uint8_t *cell_type_dense, const fs_mac *bc)
     return build_mask(c, cell_type_dense, bc);
 }
 
+// A status of a solve that ends the call: the solve did not run, or not to an iterate.
+// (With the others the best iterate is written and the status is in the stats.)
+static bool ends_call(int rc)
+{
+    return rc != FS_OK && rc != FS_ENOCONV && rc != FS_ENONFINITE && rc != FS_EBREAKDOWN;
+}
+
 static int need_mask(const fs_ctx *c)
 {
     if (!c) return set_error(FS_EINVAL, "NULL context");
@@ -443,14 +450,14 @@ int fs_step(fs_ctx *c, const fs_mac *u_in, fs_mac *u_out, fs_mac *u_visc, fs_sta
     // advection + body force -> face space; implicit viscosity in place
     if ((rc = launch_advect(c, cf3(u_in)))) return rc;
     int rv = solve_viscosity(c, true, s);
-    if (rv == FS_ECUDA) return rv;
+    if (ends_call(rv)) return rv;
     // full field after viscosity, then the projection
     fs_mac *uv = u_visc ? u_visc : u_out;
     if ((rc = launch_compose(c, f3(uv)))) return rc;
     if ((rc = launch_divergence(c, cf3(uv)))) return rc;
     c->solve_kind = 0;
     int rp = solve_pressure(c, s);
-    if (rp == FS_ECUDA || rp == FS_EINVAL) return rp;
+    if (ends_call(rp)) return rp;
     if ((rc = launch_grad_subtract(c, cf3(uv), f3(u_out), nullptr))) return rc;
     FS_CUDA(cudaStreamSynchronize(c->stream));
     prof_flush(c);
@@ -469,7 +476,7 @@ int fs_project(fs_ctx *c, fs_mac *u, float *q_out, fs_stats *st)
     if ((rc = launch_divergence(c, cf3(u)))) return rc;
     c->solve_kind = 0;
     int rp = solve_pressure(c, s);
-    if (rp == FS_ECUDA || rp == FS_EINVAL) return rp;
+    if (ends_call(rp)) return rp;
     if ((rc = launch_grad_subtract(c, cf3(u), f3(u), q_out))) return rc;
     FS_CUDA(cudaStreamSynchronize(c->stream));
     prof_flush(c);
@@ -497,7 +504,7 @@ int fs_adjoint_step(fs_ctx *c, const fs_mac *u_in, const fs_mac *u_visc, const f
     } else {
         if ((rc = launch_advect(c, cf3(u_in)))) return rc;
         int rv = solve_viscosity(c, true, s);
-        if (rv == FS_ECUDA) return rv;
+        if (ends_call(rv)) return rv;
         F3 fu{{c->fu[0], c->fu[1], c->fu[2]}};
         if ((rc = launch_compose(c, fu))) return rc;
         uv = CF3{{c->fu[0], c->fu[1], c->fu[2]}};
@@ -509,12 +516,12 @@ int fs_adjoint_step(fs_ctx *c, const fs_mac *u_in, const fs_mac *u_visc, const f
     if ((rc = launch_divergence(c, fgc))) return rc;
     c->solve_kind = 1;
     int rp = solve_pressure(c, s);
-    if (rp == FS_ECUDA || rp == FS_EINVAL) return rp;
+    if (ends_call(rp)) return rp;
     if ((rc = launch_grad_subtract(c, fgc, fg, nullptr))) return rc;
     // viscosity adjoint: one more solve with the same operator, no Dirichlet part
     if ((rc = launch_to_face_space(c, fgc))) return rc;
     int rv = solve_viscosity(c, false, s);
-    if (rv == FS_ECUDA) return rv;
+    if (ends_call(rv)) return rv;
     if (g_nu) {
         double dot = 0.0;
         if ((rc = launch_nu_grad(c, uv, &dot))) return rc;
